@@ -76,6 +76,8 @@ def draw(rng):
     if kind in ("view", "stereo", "batch"):
         c["sh"] = rng.choice(("f32", "f32", "f16", "bf16") + (("cb",) if deg > 0 else ()))
         c["sr"] = rng.choice(("f32", "f32", "f16", "bf16"))
+    if kind == "stereo":                                         # an eye's image is upright, as in a headset
+        c.update(w=min(c["w"], c["h"]), h=max(c["w"], c["h"]))
     if kind == "batch":
         c.update(n=min(c["n"], 500_000), w=min(c["w"], 800), h=min(c["h"], 800), views=rng.randint(2, 8))
     if kind in ("frame", "train"):

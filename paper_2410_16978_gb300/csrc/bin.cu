@@ -13,16 +13,14 @@
 //     chunk of the depth order; a first pass counts each chunk's entries per
 //     row in shared memory, an exclusive scan over the chunks of every row
 //     (row-major count matrices [Ty][K] of entries and of pairs) gives each chunk its place, and a
-//     second pass writes the entries (Gaussian, x0 | x1 << 16) there.  Within
-//     a chunk the entries go out in depth order: a warp expands 32 Gaussians
-//     into their row pairs 32 at a time and ranks equal rows by lane
-//     (__match_any_sync or ballots), and lanes hold consecutive pairs in depth order.
-//  2. Tiles.  Every row list is cut into pieces of a fixed number of entries
+//     second pass writes the entries (Gaussian, x0 | x1 << 16) there, in depth
+//     order (emit_group).
+//  2. Tiles.  Every row list is cut into pieces of 256 to 1,024 entries
 //     (thousands of pieces per frame, so heavy rows spread over all SMs); a
 //     warp per piece counts its pairs per tile, a per-row scan over the
 //     pieces gives each (piece, tile) its first list position and each tile
-//     its range, and a second pass writes the Gaussian ids, again ranked in
-//     depth order within a warp.
+//     its range, and a warp per (piece, 16 tiles) writes the Gaussian ids in
+//     depth order (emit_group).
 //
 // Per pair this writes the row entry once (8 B, per row of the rectangle, not
 // per tile) and the final Gaussian id once (4 B); the count matrix is a few MB.
@@ -64,69 +62,59 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t *s_w, u
     return base + x - v;
 }
 
-__device__ __forceinline__ uint32_t shfl_payload(uint32_t v, int j) { return __shfl_sync(FULL, v, j); }
-__device__ __forceinline__ uint2 shfl_payload(uint2 v, int j) {
-    return make_uint2(__shfl_sync(FULL, v.x, j), __shfl_sync(FULL, v.y, j));
+// ---- ordered scatter of interval entries ----
+//
+// A warp streams list entries in order, entry e covering the buckets
+// [x0_e, x1_e) and carrying a payload, into kGroup consecutive buckets.  Every
+// covered (bucket, entry) pair stores the payload at the bucket's running
+// position, so each bucket receives its entries in order:
+//   * the entries that reach one of the warp's buckets are compacted, with a
+//     bit per bucket they cover;
+//   * 32 of them at a time, one per lane, are stored bucket by bucket: a
+//     ballot gives the lanes that cover the bucket, a lane's rank is the number
+//     of those below it, and they store to consecutive addresses.
+// Every lane works on every step and a store instruction covers one or two
+// lines.  Bound by instruction issue (66% of the slots, about three warp
+// instructions per pair).  The tile pass (count, scan and write) on the
+// 3M-Gaussian 2064x2208 close view (122M pairs) took 0.440 ms, 1.043 ms when
+// pairs were expanded 32 at a time and lanes with equal buckets ranked by
+// __match_any_sync or ballots, each 4-byte store a line of its own; 0.240
+// against 0.472 ms on the two eyes of a 3M-Gaussian stereo pair (26M pairs
+// each), 0.168 against 0.307 ms at 1920x1080 (36M pairs).  Also measured: a lane
+// per bucket walking the set bits of the transposed coverage matrix (0.490 ms
+// on the close view: a third of the lanes idle where the tile lists of a group
+// differ in length).
+// kGroup: narrower groups compact more often per entry, wider ones leave more
+// of a step's lanes without the bucket (0.29 of them store at 16 buckets and
+// splats 6.7 tiles wide, 0.17 at 32, 0.45 at 8); 8 took 0.535 ms on the close view.
+constexpr int kGroup = 16;
+
+// Bits [a, a + len) (bits at and above 32 fall away).
+__device__ __forceinline__ uint32_t bit_run(uint32_t a, uint32_t len) {
+    uint32_t m;
+    asm("bmsk.clamp.b32 %0, %1, %2;" : "=r"(m) : "r"(a), "r"(len));
+    return m;
 }
 
-// Lanes hold 32 consecutive list entries in order (the valid ones first),
-// entry j covering slots [start_j, start_j + w_j) of the expanded sequence.
-// Returns the entry that owns slot k0 + lane: entries starting before k0 plus
-// those starting in [k0, k0 + lane], minus one.  Valid entries have w > 0.
-__device__ __forceinline__ int window_owner(uint32_t start, uint32_t w, uint32_t k0, int lane) {
-    const unsigned before = __ballot_sync(FULL, w > 0 && start < k0);
-    const bool in = w > 0 && start >= k0 && start - k0 < 32u;
-    const unsigned mask = __reduce_or_sync(FULL, in ? 1u << (start - k0) : 0u);
-    return __popc(before) - 1 + __popc(mask & (0xFFFFFFFFu >> (31 - lane)));
+// The buckets of [c0, c0 + kGroup) that [x0, x1) covers, a bit each.
+__device__ __forceinline__ uint32_t coverage(uint32_t x0, uint32_t x1, uint32_t c0) {
+    const uint32_t a = static_cast<uint32_t>(max(static_cast<int>(x0 - c0), 0));
+    const uint32_t b = static_cast<uint32_t>(max(static_cast<int>(x1 - c0), 0));
+    return bit_run(a, b - a) & ((1u << kGroup) - 1u);
 }
 
-// Lanes with equal keys of nb bits (among the active ones), from nb + 1 ballots.
-__device__ __forceinline__ unsigned match_keyn(uint32_t key, bool act, int lane, int nb) {
-    unsigned m = __ballot_sync(FULL, act);
-#pragma unroll 8
-    for (int b = 0; b < nb; ++b) {
-        const unsigned bb = __ballot_sync(FULL, (key >> b) & 1u);
-        m &= ((key >> b) & 1u) ? bb : ~bb;
-    }
-    return act ? m : (1u << lane);
-}
-
-// The 32 lanes hold consecutive list entries in order; entry j covers the
-// buckets [b0_j, b0_j + n_j) (n_j = 0: no entry) and carries the payload v_j.
-// The (bucket, payload) items are expanded in that order, 32 per window, and
-// each is stored at its bucket's running position s_pos[bucket] (per-warp
-// counters in shared memory), so every bucket receives its items in order:
-// the lanes of a window that share a bucket are ranked by lane, and the first
-// of them moves the counter.  Windows go in pairs whose rankings run on
-// different pipes, __match_any_sync for the first and ballots on the nb key
-// bits for the second; either alone saturates its pipe on large frames.
-// store(pos, payload) writes one item.
-template <class V, class Store>
-__device__ __forceinline__ void expand_scatter(uint32_t b0, uint32_t n, V v, uint32_t *s_pos, int lane, int nb,
-                                               Store store) {
-    const unsigned lt = (1u << lane) - 1u;
-    const uint32_t incl = warp_incl_scan(n, lane);
-    const uint32_t total = __shfl_sync(FULL, incl, 31);
-    const uint32_t start = incl - n;
-    for (uint32_t k0 = 0; k0 < total; k0 += 64) {
+// Stores one entry per lane (cov: its buckets) at the running positions
+// pos[c] of the group's buckets (the same in every lane).
+template <class V, class Ok>
+__device__ __forceinline__ void emit_group(uint32_t cov, V v, uint32_t (&pos)[kGroup], V *__restrict__ dst,
+                                           unsigned lt, Ok ok) {
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const uint32_t kw = k0 + 32u * u;
-            const uint32_t k = kw + lane;
-            const bool act = k < total;
-            const int j = window_owner(start, n, kw, lane);
-            const uint32_t sj = __shfl_sync(FULL, start, j), bj = __shfl_sync(FULL, b0, j);
-            const V vj = shfl_payload(v, j);
-            const uint32_t bk = act ? bj + (k - sj) : 0u;
-            // the two windows rank on different pipes: __match_any_sync and ballots
-            const unsigned peers = u == 0 ? __match_any_sync(FULL, act ? bk : 0x10000u + lane)
-                                          : match_keyn(bk, act, lane, nb);
-            const uint32_t before = act ? s_pos[bk] : 0u;
-            __syncwarp();
-            if (act && (peers & lt) == 0) s_pos[bk] = before + __popc(peers);
-            if (act) store(before + __popc(peers & lt), vj);
-            __syncwarp();
-        }
+    for (int c = 0; c < kGroup; ++c) {
+        const bool in = (cov >> c) & 1u;
+        const unsigned b = __ballot_sync(FULL, in);
+        const uint32_t p = pos[c] + __popc(b & lt);
+        if (in && ok(p)) dst[p] = v;
+        pos[c] += __popc(b);
     }
 }
 
@@ -148,7 +136,12 @@ __device__ __forceinline__ void warp_prefix_inplace(uint32_t *a, int n, int lane
 // counts into kRowParts parts, one CTA each.
 constexpr int kRowParts = 2;
 constexpr int kPartChunks = kBinChunks / kRowParts;
-static_assert(kPartChunks % 1024 == 0 && kPartChunks / 1024 <= kBinChunksPerThread, "row-scan part shape");
+constexpr int kPartPerThread = (kPartChunks + 1023) / 1024;
+static_assert(kBinChunks % kRowParts == 0, "row-scan part shape");
+
+// Entries per piece of the tile pass (k_bin_rowscan chooses).
+constexpr uint32_t kPieceMin = 256, kPieceMax = 1024;
+constexpr uint32_t kPieceWarps = 12000;    // (piece, kGroup tiles) items below which pieces stay smaller
 
 struct RowInfo {           // per tile row, in the workspace
     uint32_t start;        // first row-list entry of the row
@@ -160,80 +153,156 @@ struct RowInfo {           // per tile row, in the workspace
     uint32_t pad_[4 - kRowParts];        // (32 bytes in all)
 };
 
-// Pass 1 (SCATTER = false: count, true: write) over the chunks of the depth order.
-template <bool SCATTER>
-__global__ void __launch_bounds__(256) k_bin_rows(const uint32_t *__restrict__ order, const Rec *__restrict__ rec,
-                                                  uint32_t n_cap, int Ty, uint32_t *__restrict__ M,
-                                                  RowInfo *__restrict__ rows, uint2 *__restrict__ rowlist,
-                                                  const Ctl *__restrict__ ctl) {
-    __shared__ uint32_t s_cnt[8][kBinMaxDim + 1];
-    __shared__ uint32_t s_px[SCATTER ? 1 : 8][kBinMaxDim + 1];
+// Chunk c of K of the depth order's n entries.
+__device__ __forceinline__ void chunk_range(uint32_t n, uint32_t c, uint32_t K, uint32_t &b, uint32_t &e) {
+    b = static_cast<uint32_t>(static_cast<uint64_t>(n) * c / K);
+    e = static_cast<uint32_t>(static_cast<uint64_t>(n) * (c + 1) / K);
+}
+
+// Rows, count: a warp per chunk of the depth order counts its entries and pairs per tile row.
+__global__ void __launch_bounds__(256) k_bin_rows_count(const uint32_t *__restrict__ order,
+                                                        const Rec *__restrict__ rec, uint32_t n_cap, int Ty,
+                                                        uint32_t *__restrict__ M, const Ctl *__restrict__ ctl) {
+    __shared__ uint32_t s_cnt[8][kBinMaxDim + 1], s_px[8][kBinMaxDim + 1];
     // an error before the binning (a depth sort that timed out) leaves the order unfinished: do not read it
     if (ctl->st.error != GS_OK) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t K = gridDim.x * 8u, c = blockIdx.x * 8u + warp;
-    const uint32_t n = min(ctl->n_vis, n_cap);
-    const uint32_t b = static_cast<uint32_t>(static_cast<uint64_t>(n) * c / K);
-    const uint32_t e = static_cast<uint32_t>(static_cast<uint64_t>(n) * (c + 1) / K);
+    const uint32_t K = gridDim.x * 8u;
+    uint32_t b, e;
+    chunk_range(min(ctl->n_vis, n_cap), blockIdx.x * 8u + warp, K, b, e);
+    for (int r = lane; r <= Ty; r += 32) s_cnt[warp][r] = s_px[warp][r] = 0u;
+    __syncwarp();
+    // ids two groups ahead and records one group ahead of the group being counted, so the gathers overlap
+    // the counting of the groups before them
+    const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    uint32_t gid = b + lane < e ? order[b + lane] : 0u;
+    float4 c_nx = b + lane < e ? rec[gid].c : z4;
+    gid = b + 32 + lane < e ? order[b + 32 + lane] : 0u;
+    for (uint32_t p0 = b; p0 < e; p0 += 32) {
+        const float4 cc = c_nx;
+        c_nx = p0 + 32 + lane < e ? rec[gid].c : z4;
+        gid = p0 + 64 + lane < e ? order[p0 + 64 + lane] : 0u;
+        // rows [y0, y1) each get one entry and w pairs: difference array
+        const uint32_t r0 = __float_as_uint(cc.z), r1 = __float_as_uint(cc.w);
+        const uint32_t y0 = r0 >> 16, y1 = r1 >> 16, w = (r1 & 0xFFFFu) - (r0 & 0xFFFFu);
+        if (y1 > y0) {
+            atomicAdd(&s_cnt[warp][y0], 1u);
+            atomicSub(&s_cnt[warp][y1], 1u);
+            atomicAdd(&s_px[warp][y0], w);
+            atomicSub(&s_px[warp][y1], w);
+        }
+    }
+    __syncwarp();
+    warp_prefix_inplace(s_cnt[warp], Ty, lane);
+    warp_prefix_inplace(s_px[warp], Ty, lane);
+    __syncthreads();
+    // the block's 8 chunks are 8 consecutive columns of the row-major count
+    // matrices, written as 32-byte row segments; the pairs matrix follows the
+    // entries matrix and is summed per row by the scan
+    for (int t = threadIdx.x; t < 8 * Ty; t += blockDim.x) {
+        const int r = t >> 3, w = t & 7;
+        const size_t at = static_cast<size_t>(r) * K + blockIdx.x * 8u + w;
+        M[at] = s_cnt[w][r];
+        M[static_cast<size_t>(Ty) * K + at] = s_px[w][r];
+    }
+}
+
+// Rows, write: the chunk's warp writes its row-list entries, 128 Gaussians at
+// a time (their ids and tile rectangles loaded while the block before them is
+// written), 16 tile rows at a time.  Four CTAs per SM with blocks of 128:
+// row pass of the 1.2M-Gaussian 1024x1024 frame 0.043 ms against 0.046 with
+// two CTAs per SM and blocks of 256 (0.219 against 0.224 ms on the close view).
+constexpr int kRowWords = 4;
+constexpr int kRowBlock = 32 * kRowWords;
+
+__global__ void __launch_bounds__(256) k_bin_rows_write(const uint32_t *__restrict__ order,
+                                                        const Rec *__restrict__ rec, uint32_t n_cap, int Ty,
+                                                        const uint32_t *__restrict__ M,
+                                                        const RowInfo *__restrict__ rows, uint2 *__restrict__ rowlist,
+                                                        const Ctl *__restrict__ ctl) {
+    __shared__ uint32_t s_pos[8][kBinMaxDim];
+    __shared__ uint2 s_val[8][kRowBlock];
+    __shared__ uint16_t s_cov[8][kRowBlock];
+    if (ctl->st.error != GS_OK) return;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned lt = (1u << lane) - 1u;
+    const uint32_t K = gridDim.x * 8u;
     // the block's 8 chunks are 8 consecutive columns of the row-major count
     // matrix: thread t moves (row t / 8, column t % 8), so every row segment
     // is one 32-byte transaction
-    for (int t = threadIdx.x; t < 8 * (Ty + 1); t += blockDim.x) {
+    for (int t = threadIdx.x; t < 8 * Ty; t += blockDim.x) {
         const int r = t >> 3, w = t & 7;
         const uint32_t ch = blockIdx.x * 8u + w, part = ch / (K / kRowParts);
-        s_cnt[w][r] = (SCATTER && r < Ty)
-                          ? rows[r].start + (part ? rows[r].part_base[part - 1] : 0u) + M[static_cast<size_t>(r) * K + ch]
-                          : 0u;
-        if (!SCATTER) s_px[w][r] = 0;
+        s_pos[w][r] = rows[r].start + (part ? rows[r].part_base[part - 1] : 0u) + M[static_cast<size_t>(r) * K + ch];
     }
     __syncthreads();
-    // ids two groups ahead and records one group ahead of the group being binned, so the gathers overlap
-    // the binning of the groups before them
-    const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
-    uint32_t g_nx = b + lane < e ? order[b + lane] : 0u;
-    float4 c_nx = b + lane < e ? rec[g_nx].c : z4;
-    uint32_t gid = b + 32 + lane < e ? order[b + 32 + lane] : 0u;
-    for (uint32_t p0 = b; p0 < e; p0 += 32) {
-        const bool valid = p0 + lane < e;
-        const uint32_t g = g_nx;
-        const float4 cc = c_nx;
-        g_nx = gid;
-        c_nx = p0 + 32 + lane < e ? rec[g_nx].c : z4;
-        gid = p0 + 64 + lane < e ? order[p0 + 64 + lane] : 0u;
-        uint32_t y0 = 0, x01 = 0, nrows = 0;
-        if (valid) {
-            const uint32_t r0 = __float_as_uint(cc.z), r1 = __float_as_uint(cc.w);
-            y0 = r0 >> 16;
-            nrows = (r1 >> 16) - y0;
-            x01 = (r0 & 0xFFFFu) | (r1 << 16);     // x0 | x1 << 16
+    uint32_t b, e;
+    chunk_range(min(ctl->n_vis, n_cap), blockIdx.x * 8u + warp, K, b, e);
+    // blocks of equal size, whole words
+    const uint32_t nblk = (e - b + kRowBlock - 1) / kRowBlock;
+    const uint32_t step = nblk ? ((e - b + nblk - 1) / nblk + 31u) & ~31u : 32u;
+    const int words = static_cast<int>(step / 32);
+    const auto ok = [&](uint32_t p) { return GS_CHECK(p < ctl->st.dup_capacity, ctl, kSiteRowList); };
+    constexpr uint32_t kNone = 0xFFFFFFFFu;
+    uint32_t gn[kRowWords];
+    float2 rn[kRowWords];
+    const auto load = [&](uint32_t p0) {
+#pragma unroll
+        for (int w = 0; w < kRowWords; ++w) {
+            const uint32_t p = p0 + 32 * w + lane;
+            gn[w] = w < words && p < e ? order[p] : kNone;
         }
-        if (!SCATTER) {
-            // rows [y0, y0 + nrows) each get one entry and w pairs: difference array
-            if (nrows) {
-                const uint32_t w = (x01 >> 16) - (x01 & 0xFFFFu);
-                atomicAdd(&s_cnt[warp][y0], 1u);
-                atomicSub(&s_cnt[warp][y0 + nrows], 1u);
-                atomicAdd(&s_px[warp][y0], w);
-                atomicSub(&s_px[warp][y0 + nrows], w);
+#pragma unroll
+        for (int w = 0; w < kRowWords; ++w)
+            rn[w] = gn[w] != kNone ? *reinterpret_cast<const float2 *>(&rec[gn[w]].c.z) : make_float2(0.f, 0.f);
+    };
+    load(b);
+    for (uint32_t p0 = b; p0 < e; p0 += step) {
+        uint32_t g[kRowWords], y01[kRowWords], x01[kRowWords];
+        uint32_t lo = 0xFFFFu, hi = 0;
+#pragma unroll
+        for (int w = 0; w < kRowWords; ++w) {
+            const uint32_t r0 = __float_as_uint(rn[w].x), r1 = __float_as_uint(rn[w].y);
+            g[w] = gn[w];
+            x01[w] = (r0 & 0xFFFFu) | (r1 << 16);
+            y01[w] = (r0 >> 16) | (r1 & 0xFFFF0000u);
+            if (gn[w] != kNone) {
+                lo = min(lo, r0 >> 16);
+                hi = max(hi, r1 >> 16);
             }
-            continue;
         }
-        expand_scatter(y0, nrows, make_uint2(g, x01), s_cnt[warp], lane, 32 - __clz(max(Ty - 1, 1)), [&](uint32_t pos, uint2 en) {
-            if (GS_CHECK(pos < ctl->st.dup_capacity, ctl, kSiteRowList)) rowlist[pos] = en;
-        });
-    }
-    if (!SCATTER) {
-        __syncwarp();
-        warp_prefix_inplace(s_cnt[warp], Ty, lane);
-        warp_prefix_inplace(s_px[warp], Ty, lane);
-        __syncthreads();
-        // entries and pairs per (row, chunk), written as 32-byte row segments; the
-        // pairs matrix follows the entries matrix and is summed per row by the scan
-        for (int t = threadIdx.x; t < 8 * Ty; t += blockDim.x) {
-            const int r = t >> 3, w = t & 7;
-            const size_t at = static_cast<size_t>(r) * K + blockIdx.x * 8u + w;
-            M[at] = s_cnt[w][r];
-            M[static_cast<size_t>(Ty) * K + at] = s_px[w][r];
+        load(p0 + step);
+        lo = __reduce_min_sync(FULL, lo);
+        hi = __reduce_max_sync(FULL, hi);
+        for (uint32_t c0 = lo & ~(kGroup - 1u); c0 < hi; c0 += kGroup) {
+            int fill = 0;
+#pragma unroll
+            for (int w = 0; w < kRowWords; ++w) {
+                if (w >= words) break;
+                const uint32_t cov = coverage(y01[w] & 0xFFFFu, y01[w] >> 16, c0);
+                const unsigned km = __ballot_sync(FULL, cov != 0);
+                if (cov) {
+                    const int slot = fill + __popc(km & lt);
+                    s_val[warp][slot] = make_uint2(g[w], x01[w]);
+                    s_cov[warp][slot] = static_cast<uint16_t>(cov);
+                }
+                fill += __popc(km);
+            }
+            if (fill == 0) continue;
+            __syncwarp();
+            const uint32_t mine = c0 + lane < static_cast<uint32_t>(Ty) && lane < kGroup ? s_pos[warp][c0 + lane] : 0u;
+            uint32_t pos[kGroup];
+#pragma unroll
+            for (int c = 0; c < kGroup; ++c) pos[c] = __shfl_sync(FULL, mine, c);
+            for (int k = 0; k < fill; k += 32) {
+                const bool in = k + lane < fill;
+                emit_group(in ? s_cov[warp][k + lane] : 0u, in ? s_val[warp][k + lane] : make_uint2(0u, 0u), pos,
+                           rowlist, lt, ok);
+            }
+#pragma unroll
+            for (int c = 0; c < kGroup; ++c)
+                if (lane == c && c0 + c < static_cast<uint32_t>(Ty)) s_pos[warp][c0 + c] = pos[c];
+            __syncwarp();
         }
     }
 }
@@ -248,7 +317,7 @@ __global__ void __launch_bounds__(256) k_bin_rows(const uint32_t *__restrict__ o
 // total and the capacity check.
 __global__ void __launch_bounds__(1024) k_bin_rowscan(uint32_t *__restrict__ M, int K, int Ty,
                                                       RowInfo *__restrict__ rows, uint2 *__restrict__ part_tot,
-                                                      Ctl *__restrict__ ctl, uint64_t cap, uint32_t piece) {
+                                                      Ctl *__restrict__ ctl, uint64_t cap, int Tx) {
     __shared__ uint32_t s_w[32];
     __shared__ uint32_t s_row[kPartChunks];
     __shared__ bool s_last;
@@ -264,19 +333,20 @@ __global__ void __launch_bounds__(1024) k_bin_rowscan(uint32_t *__restrict__ M, 
     }
     uint32_t ptot;
     block_excl_scan<1024>(psum, s_w, &ptot);             // synchronises the block, so s_row is complete
-    const int per = KP / 1024;
-    uint32_t v[kBinChunksPerThread];
+    uint32_t v[kPartPerThread];
     uint32_t sum = 0;
 #pragma unroll
-    for (int q = 0; q < kBinChunksPerThread; ++q) {
-        v[q] = q < per ? s_row[threadIdx.x * per + q] : 0u;
+    for (int q = 0; q < kPartPerThread; ++q) {
+        const int i = threadIdx.x * kPartPerThread + q;
+        v[q] = i < KP ? s_row[i] : 0u;
         sum += v[q];
     }
     uint32_t tot;
     uint32_t run = block_excl_scan<1024>(sum, s_w, &tot);
 #pragma unroll
-    for (int q = 0; q < kBinChunksPerThread; ++q) {
-        if (q < per) s_row[threadIdx.x * per + q] = run;
+    for (int q = 0; q < kPartPerThread; ++q) {
+        const int i = threadIdx.x * kPartPerThread + q;
+        if (i < KP) s_row[i] = run;
         run += v[q];
     }
     __syncthreads();
@@ -306,6 +376,10 @@ __global__ void __launch_bounds__(1024) k_bin_rowscan(uint32_t *__restrict__ M, 
     const bool in = threadIdx.x < Ty;
     const uint32_t s0 = block_excl_scan<1024>(in ? ent : 0u, s_w, &te);
     const uint32_t s1 = block_excl_scan<1024>(in ? prs : 0u, s_w, &tp);
+    // entries per piece: the largest that still gives every SM several warps of the scatter (piece, kGroup tiles)
+    uint32_t piece = kPieceMin;
+    const uint64_t groups = (Tx + kGroup - 1) / kGroup;
+    while (piece < kPieceMax && te / (2 * piece) * groups >= kPieceWarps) piece *= 2;
     const uint32_t s2 = block_excl_scan<1024>(in ? (ent + piece - 1) / piece : 0u, s_w, &tq);
     if (in) {
         rows[threadIdx.x].start = s0;
@@ -316,65 +390,137 @@ __global__ void __launch_bounds__(1024) k_bin_rowscan(uint32_t *__restrict__ M, 
         ctl->st.n_dup = tp;
         ctl->st.dup_capacity = cap;
         ctl->n_pieces = tq;
+        ctl->bin_piece = piece;
         if (tp > cap) ctl->st.error = GS_ERR_WORKSPACE;
     }
 }
 
-// Pass 2 (SCATTER = false: count, true: write), one warp per piece of a row
-// list.  Count: per-(piece, tile) counts into P[piece][Tx].  Write: P holds
-// the first list position of every (piece, tile) (k_bin_tiles_scan).
-template <bool SCATTER>
-__global__ void __launch_bounds__(256) k_bin_tiles(const uint2 *__restrict__ rowlist, const RowInfo *__restrict__ rows,
-                                                   int Tx, int Ty, uint32_t piece, uint32_t *__restrict__ P,
-                                                   uint32_t *__restrict__ list, const Ctl *__restrict__ ctl) {
+// The pieces of the row lists.  s_ps[r]: first piece of row r, s_ps[Ty]: their
+// number.  Row of piece p: the largest r with s_ps[r] <= p.
+__device__ __forceinline__ void load_piece_starts(uint32_t *s_ps, const RowInfo *rows, int Ty, const Ctl *ctl) {
+    for (int r = threadIdx.x; r < Ty; r += blockDim.x) s_ps[r] = rows[r].piece_start;
+    if (threadIdx.x == 0) s_ps[Ty] = ctl->n_pieces;
+    __syncthreads();
+}
+__device__ __forceinline__ int row_of_piece(const uint32_t *s_ps, int Ty, uint32_t p) {
+    int lo = 0, hi = Ty - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (s_ps[mid] <= p) lo = mid; else hi = mid - 1;
+    }
+    return lo;
+}
+
+// Tiles, count: a warp per piece counts its pairs per tile into P[piece][Tx].
+__global__ void __launch_bounds__(256) k_bin_tiles_count(const uint2 *__restrict__ rowlist,
+                                                         const RowInfo *__restrict__ rows, int Tx, int Ty,
+                                                         uint32_t *__restrict__ P, const Ctl *__restrict__ ctl) {
     __shared__ uint32_t s_cnt[8][kBinMaxDim + 1];
     __shared__ uint32_t s_ps[kBinMaxDim + 1];
     if (ctl->st.error != GS_OK) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t npieces = ctl->n_pieces;
-    for (int r = threadIdx.x; r < Ty; r += blockDim.x) s_ps[r] = rows[r].piece_start;
-    if (threadIdx.x == 0) s_ps[Ty] = npieces;
-    __syncthreads();
-    const uint32_t nwarps = gridDim.x * 8u;
-    for (uint32_t p = blockIdx.x * 8u + warp; p < npieces; p += nwarps) {
-        int lo = 0, hi = Ty - 1;                 // largest row r with s_ps[r] <= p
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (s_ps[mid] <= p) lo = mid; else hi = mid - 1;
-        }
-        const RowInfo ri = rows[lo];
-        const uint32_t e0 = ri.start + (p - s_ps[lo]) * piece;
+    const uint32_t npieces = ctl->n_pieces, piece = ctl->bin_piece;
+    load_piece_starts(s_ps, rows, Ty, ctl);
+    for (uint32_t p = blockIdx.x * 8u + warp; p < npieces; p += gridDim.x * 8u) {
+        const int row = row_of_piece(s_ps, Ty, p);
+        const RowInfo ri = rows[row];
+        const uint32_t e0 = ri.start + (p - s_ps[row]) * piece;
         const uint32_t e1 = min(e0 + piece, ri.start + ri.entries);
         uint32_t *Pp = P + static_cast<size_t>(p) * Tx;
-        for (int t = lane; t <= Tx; t += 32) s_cnt[warp][t] = (SCATTER && t < Tx) ? Pp[t] : 0u;
+        for (int t = lane; t <= Tx; t += 32) s_cnt[warp][t] = 0u;
         __syncwarp();
         uint2 en_nx = e0 + lane < e1 ? rowlist[e0 + lane] : make_uint2(0u, 0u);   // entries one group ahead
         for (uint32_t q0 = e0; q0 < e1; q0 += 32) {
             const uint2 en = en_nx;
             en_nx = q0 + 32 + lane < e1 ? rowlist[q0 + 32 + lane] : make_uint2(0u, 0u);
-            uint32_t g = 0, x0 = 0, w = 0;
-            if (q0 + lane < e1) {
-                g = en.x;
-                x0 = en.y & 0xFFFFu;
-                w = (en.y >> 16) - x0;
+            // tiles [x0, x1) each get one pair: difference array
+            const uint32_t x0 = en.y & 0xFFFFu, x1 = en.y >> 16;
+            if (x1 > x0) {
+                atomicAdd(&s_cnt[warp][x0], 1u);
+                atomicSub(&s_cnt[warp][x1], 1u);
             }
-            if (!SCATTER) {
-                // tiles [x0, x0 + w) each get one pair: difference array
-                if (w) {
-                    atomicAdd(&s_cnt[warp][x0], 1u);
-                    atomicSub(&s_cnt[warp][x0 + w], 1u);
+        }
+        __syncwarp();
+        warp_prefix_inplace(s_cnt[warp], Tx, lane);
+        for (int t = lane; t < Tx; t += 32) Pp[t] = s_cnt[warp][t];
+        __syncwarp();
+    }
+}
+
+// Tiles, write: a warp per (piece, 16 tiles) writes its Gaussian ids.  P holds
+// the first list position of every (piece, tile) (k_bin_tiles_scan).
+constexpr int kStepWords = 4;      // words of 32 entries loaded per step, one step ahead
+
+__global__ void __launch_bounds__(256) k_bin_tiles_write(const uint2 *__restrict__ rowlist,
+                                                         const RowInfo *__restrict__ rows, int Tx, int Ty,
+                                                         const uint32_t *__restrict__ P, uint32_t *__restrict__ list,
+                                                         const Ctl *__restrict__ ctl) {
+    __shared__ uint32_t s_val[8][64];              // compacted entries, a ring of two words of 32
+    __shared__ uint16_t s_cov[8][64];
+    __shared__ uint32_t s_ps[kBinMaxDim + 1];
+    if (ctl->st.error != GS_OK) return;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned lt = (1u << lane) - 1u;
+    const uint32_t npieces = ctl->n_pieces, piece = ctl->bin_piece;
+    load_piece_starts(s_ps, rows, Ty, ctl);
+    const uint32_t groups = (Tx + kGroup - 1) / kGroup;
+    const uint64_t items = static_cast<uint64_t>(npieces) * groups;
+    const auto ok = [&](uint32_t at) { return GS_CHECK(at < ctl->st.n_dup, ctl, kSitePairList); };
+    for (uint64_t it = blockIdx.x * 8u + warp; it < items; it += gridDim.x * 8u) {
+        const uint32_t p = static_cast<uint32_t>(it / groups);
+        const uint32_t c0 = kGroup * static_cast<uint32_t>(it - static_cast<uint64_t>(p) * groups), t = c0 + lane;
+        const int row = row_of_piece(s_ps, Ty, p);
+        uint32_t at = 0, next = 0;                 // next: the tile's position after this piece, where P holds it
+        if (lane < kGroup && t < static_cast<uint32_t>(Tx)) {
+            const uint32_t *Pp = P + static_cast<size_t>(p) * Tx + t;
+            at = Pp[0];
+            next = p + 1 < s_ps[row + 1] ? Pp[Tx] : at + 1;
+        }
+        if (!__any_sync(FULL, next != at)) continue;         // no entry of the piece reaches these tiles
+        const RowInfo ri = rows[row];
+        const uint32_t e0 = ri.start + (p - s_ps[row]) * piece;
+        const uint32_t e1 = min(e0 + piece, ri.start + ri.entries);
+        uint32_t pos[kGroup];
+#pragma unroll
+        for (int c = 0; c < kGroup; ++c) pos[c] = __shfl_sync(FULL, at, c);
+        int head = 0, fill = 0;
+        uint2 en_nx[kStepWords];                   // entries one step ahead
+        const auto entries = [&](uint32_t q0) {
+#pragma unroll
+            for (int w = 0; w < kStepWords; ++w)
+                en_nx[w] = q0 + 32 * w + lane < e1 ? rowlist[q0 + 32 * w + lane] : make_uint2(0u, 0u);
+        };
+        entries(e0);
+        for (uint32_t q0 = e0; q0 < e1; q0 += 32 * kStepWords) {
+            uint2 en[kStepWords];
+#pragma unroll
+            for (int w = 0; w < kStepWords; ++w) en[w] = en_nx[w];
+            entries(q0 + 32 * kStepWords);
+#pragma unroll 1
+            for (int w = 0; w < kStepWords; ++w) {
+                const uint2 now = en[0];
+#pragma unroll
+                for (int k = 0; k + 1 < kStepWords; ++k) en[k] = en[k + 1];
+                const uint32_t cov = coverage(now.y & 0xFFFFu, now.y >> 16, c0);
+                const unsigned km = __ballot_sync(FULL, cov != 0);
+                if (cov) {
+                    const int slot = (head + fill + __popc(km & lt)) & 63;
+                    s_val[warp][slot] = now.x;
+                    s_cov[warp][slot] = static_cast<uint16_t>(cov);
                 }
-                continue;
+                fill += __popc(km);
+                if (fill >= 32) {
+                    __syncwarp();
+                    emit_group<uint32_t>(s_cov[warp][head + lane], s_val[warp][head + lane], pos, list, lt, ok);
+                    head ^= 32;
+                    fill -= 32;
+                    __syncwarp();
+                }
             }
-            expand_scatter(x0, w, g, s_cnt[warp], lane, 32 - __clz(max(Tx - 1, 1)), [&](uint32_t pos, uint32_t id) {
-                if (GS_CHECK(pos < ctl->st.n_dup, ctl, kSitePairList)) list[pos] = id;
-            });
         }
-        if (!SCATTER) {
-            __syncwarp();
-            warp_prefix_inplace(s_cnt[warp], Tx, lane);
-            for (int t = lane; t < Tx; t += 32) Pp[t] = s_cnt[warp][t];
-        }
+        __syncwarp();
+        if (fill)
+            emit_group<uint32_t>(lane < fill ? s_cov[warp][head + lane] : 0u, s_val[warp][head + lane], pos, list, lt, ok);
         __syncwarp();
     }
 }
@@ -384,7 +530,7 @@ __global__ void __launch_bounds__(256) k_bin_tiles(const uint2 *__restrict__ row
 // thread (slice s, tile t) sums the counts of tile t over its share of the
 // row's pieces; the slice sums give each tile's total and range; then every
 // (piece, tile) count is replaced by its first list position.
-__global__ void __launch_bounds__(1024) k_bin_tiles_scan(const RowInfo *__restrict__ rows, int Tx, uint32_t piece,
+__global__ void __launch_bounds__(1024) k_bin_tiles_scan(const RowInfo *__restrict__ rows, int Tx,
                                                          uint32_t *__restrict__ P, uint2 *__restrict__ ranges,
                                                          const Ctl *__restrict__ ctl) {
     __shared__ uint32_t s_sum[1024];         // [slice][tile]
@@ -397,7 +543,7 @@ __global__ void __launch_bounds__(1024) k_bin_tiles_scan(const RowInfo *__restri
     const int r = blockIdx.x;
     const int t = threadIdx.x & (TW - 1), sl = threadIdx.x / TW;
     const RowInfo ri = rows[r];
-    const uint32_t npc = (ri.entries + piece - 1) / piece;
+    const uint32_t piece = ctl->bin_piece, npc = (ri.entries + piece - 1) / piece;
     const uint32_t per = (npc + S - 1) / S;
     const uint32_t p0 = ri.piece_start + min(npc, sl * per), p1 = ri.piece_start + min(npc, (sl + 1) * per);
     uint32_t sum = 0;
@@ -439,45 +585,34 @@ __global__ void __launch_bounds__(1024) k_bin_tiles_scan(const RowInfo *__restri
 
 }  // namespace
 
-cudaError_t launch_bin_rows(const uint32_t *order, const Rec *rec, uint32_t n_cap, int Ty, uint32_t *M,
-                            void *rows_buf, uint2 *rowlist, Ctl *ctl, uint64_t cap, uint32_t piece, cudaStream_t st) {
+cudaError_t launch_bin_rows(const uint32_t *order, const Rec *rec, uint32_t n_cap, int Tx, int Ty, uint32_t *M,
+                            void *rows_buf, uint2 *rowlist, Ctl *ctl, uint64_t cap, cudaStream_t st) {
     if (Ty > kBinMaxDim) return cudaErrorInvalidValue;
     RowInfo *rows = static_cast<RowInfo *>(rows_buf);   // zero on entry (cleared with the control block)
     uint2 *part_tot = reinterpret_cast<uint2 *>(static_cast<char *>(rows_buf) + bin_rows_bytes(Ty) -
                                                  static_cast<size_t>(Ty) * kRowParts * sizeof(uint2));
-    k_bin_rows<false><<<kBinBlocks, 256, 0, st>>>(order, rec, n_cap, Ty, M, rows, rowlist, ctl);
-    k_bin_rowscan<<<Ty * kRowParts, 1024, 0, st>>>(M, kBinBlocks * 8, Ty, rows, part_tot, ctl, cap, piece);
-    k_bin_rows<true><<<kBinBlocks, 256, 0, st>>>(order, rec, n_cap, Ty, M, rows, rowlist, ctl);
+    k_bin_rows_count<<<kBinBlocks, 256, 0, st>>>(order, rec, n_cap, Ty, M, ctl);
+    k_bin_rowscan<<<Ty * kRowParts, 1024, 0, st>>>(M, kBinChunks, Ty, rows, part_tot, ctl, cap, Tx);
+    k_bin_rows_write<<<kBinBlocks, 256, 0, st>>>(order, rec, n_cap, Ty, M, rows, rowlist, ctl);
     return cudaGetLastError();
 }
 
-cudaError_t launch_bin_tiles(const uint2 *rowlist, const void *rows_buf, int Tx, int Ty, uint32_t piece, uint32_t *P,
-                             uint32_t *list, uint2 *ranges, const Ctl *ctl, cudaStream_t st) {
+cudaError_t launch_bin_tiles(const uint2 *rowlist, const void *rows_buf, int Tx, int Ty, uint32_t *P, uint32_t *list,
+                             uint2 *ranges, const Ctl *ctl, cudaStream_t st) {
     if (Tx > kBinMaxDim || Ty > kBinMaxDim) return cudaErrorInvalidValue;
     const RowInfo *rows = static_cast<const RowInfo *>(rows_buf);
-    const int G = 4 * sort_blocks();
-    k_bin_tiles<false><<<G, 256, 0, st>>>(rowlist, rows, Tx, Ty, piece, P, list, ctl);
-    k_bin_tiles_scan<<<Ty, 1024, 0, st>>>(rows, Tx, piece, P, ranges, ctl);
-    k_bin_tiles<true><<<G, 256, 0, st>>>(rowlist, rows, Tx, Ty, piece, P, list, ctl);
+    const int G = 4 * sort_blocks();     // 16 CTAs per SM, several waves: pieces differ in pairs (half as many: 3% slower)
+    k_bin_tiles_count<<<G, 256, 0, st>>>(rowlist, rows, Tx, Ty, P, ctl);
+    k_bin_tiles_scan<<<Ty, 1024, 0, st>>>(rows, Tx, P, ranges, ctl);
+    k_bin_tiles_write<<<G, 256, 0, st>>>(rowlist, rows, Tx, Ty, P, list, ctl);
     return cudaGetLastError();
-}
-
-uint32_t bin_piece_entries(int64_t dup_cap, int Tx) {
-    // Pieces of 256 entries at every size: measured against 128, 512 and 1024 on the 1.2M-Gaussian 1024 x 1024
-    // frame and on 3M-Gaussian views of 1024 x 1024 and 2064 x 2208 (40M and 123M pairs), 256 was fastest or
-    // within 1% of it.  (Growing the pieces with the capacity, to keep the count matrix near 64 MB, made the pieces
-    // of the 2064 x 2208 view 2048 entries long and its tile pass 1.3 times slower.)  The count matrix then takes
-    // at most 4 B per pair of capacity.
-    (void)dup_cap;
-    (void)Tx;
-    return 256u;
 }
 
 size_t bin_piece_bytes(int64_t dup_cap, int Tx, int Ty) {
-    // A row list of E entries has ceil(E / piece) pieces and the row lists hold at most dup_cap entries, so
-    // dup_cap / piece + Ty rows of counts always suffice; the size grows with the capacity.
-    const uint32_t piece = bin_piece_entries(dup_cap, Tx);
-    return (static_cast<size_t>(dup_cap) / piece + Ty + 1) * Tx * 4;
+    // A row list of E entries has ceil(E / piece) pieces of at least kPieceMin entries and the row lists hold at
+    // most dup_cap entries, so dup_cap / kPieceMin + Ty rows of counts always suffice; the size grows with the
+    // capacity.
+    return (static_cast<size_t>(dup_cap) / kPieceMin + Ty + 1) * Tx * 4;
 }
 
 // The RowInfo of every row, then the (entries, pairs) totals of every (row, part) of the row scan.

@@ -44,7 +44,6 @@ bool make_layout(int64_t n, int W, int H, int64_t dup_cap, Layout *L) {
     o.sort_cnt = take(sort_count_bytes(n));
     o.sort_status = take(sort_status_bytes(n));
     o.bin_m = take(static_cast<size_t>(kBinChunks) * o.Ty * 8);   // entries and pairs per (row, chunk)
-    o.bin_piece = bin_piece_entries(dup_cap, o.Tx);
     o.bin_p = take(bin_piece_bytes(dup_cap, o.Tx, o.Ty));
     o.t_final = take(P * 4);
     o.n_contrib = take(P * 4);
@@ -406,14 +405,14 @@ int front_bin(FrontCtx &f, const uint32_t *order, cudaStream_t st, FwdJob *job) 
     uint2 *ranges = at<uint2>(ws, L.ranges);
     {
         Stage sg(GS_STAGE_BIN_ROWS, st, 3);
-        if ((rc = cuda_check(launch_bin_rows(order, f.rec, n, f.cv.Ty, at<uint32_t>(ws, L.bin_m),
-                                             at<void>(ws, L.bin_rows), rowlist, f.ctl, L.dup_cap, L.bin_piece, st),
+        if ((rc = cuda_check(launch_bin_rows(order, f.rec, n, f.cv.Tx, f.cv.Ty, at<uint32_t>(ws, L.bin_m),
+                                             at<void>(ws, L.bin_rows), rowlist, f.ctl, L.dup_cap, st),
                              "binning rows")) != GS_OK)
             return rc;
     }
     {
         Stage sg(GS_STAGE_BIN_TILES, st, 3);
-        if ((rc = cuda_check(launch_bin_tiles(rowlist, at<void>(ws, L.bin_rows), f.cv.Tx, f.cv.Ty, L.bin_piece,
+        if ((rc = cuda_check(launch_bin_tiles(rowlist, at<void>(ws, L.bin_rows), f.cv.Tx, f.cv.Ty,
                                               at<uint32_t>(ws, L.bin_p), list, ranges, f.ctl, st),
                              "binning tiles")) != GS_OK)
             return rc;

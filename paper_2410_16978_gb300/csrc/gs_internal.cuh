@@ -27,9 +27,8 @@ constexpr float kEigenFloor = 0.1f;            // floor of (mid^2 - det) under t
 constexpr uint32_t kSeg = 256;                 // list positions per backward segment (checkpoint stride)
 constexpr int kCbMaxDim = 48;                  // SH codebook: coordinates per row, 3(K-1) <= 45 padded
 constexpr int kBinMaxDim = 256;                // tile rows and columns the binning handles (4096 px)
-constexpr int kBinBlocks = 256;                // CTAs (of 8 chunk warps) of the row pass of the binning
+constexpr int kBinBlocks = 608;                // CTAs (of 8 chunk warps) of the row pass of the binning: four per SM
 constexpr int kBinChunks = kBinBlocks * 8;     // chunks of the depth order in the row pass
-constexpr int kBinChunksPerThread = kBinChunks / 1024;
 
 // Per-Gaussian record written by the preprocess and gathered by the compositor.
 // a = (u, v, A2, beta), b = (G2, opacity, r, g), c = (b, depth, rect01, rect23)
@@ -54,7 +53,8 @@ struct Ctl {
     uint32_t n_pieces;     // row-list pieces of the binning
     uint32_t sort_ticket[4];   // next tile of each digit kernel of the depth sort (after the first)
     uint32_t bin_scan_done;    // CTAs of the binning's per-row scan that have finished (the last one finishes)
-    uint32_t pad[11];
+    uint32_t bin_piece;        // row-list entries per piece of the binning
+    uint32_t pad[10];
 };
 static_assert(sizeof(Ctl) == 128, "Ctl layout");
 
@@ -91,7 +91,6 @@ __device__ __forceinline__ bool gs_check(bool ok, const Ctl *ctl, uint32_t site)
 struct Layout {
     int64_t n = 0, dup_cap = 0;
     int W = 0, H = 0, Tx = 0, Ty = 0, Tn = 0;
-    uint32_t bin_piece = 0;
     size_t ctl = 0, rec = 0, tiles = 0, depth = 0, sort_k[2] = {0, 0}, sort_v[2] = {0, 0}, order = 0, vis_index = 0,
            sort_hist = 0, sort_grp = 0, sort_cnt = 0, sort_status = 0, bin_m = 0,
            bin_rows = 0, bin_p = 0, rowlist = 0, list = 0, ranges = 0, t_final = 0, n_contrib = 0,
@@ -208,16 +207,15 @@ cudaError_t launch_sort_digits2(const uint32_t *tiles_a, const uint32_t *depth_a
 // (Gaussian, x0 | x1 << 16) in depth order; writes n_dup and the overflow
 // status (n_dup > cap).  M: 2 kBinChunks Ty words; rows_buf: bin_rows_bytes(Ty),
 // zero on entry.
-cudaError_t launch_bin_rows(const uint32_t *order, const Rec *rec, uint32_t n_cap, int Ty, uint32_t *M,
-                            void *rows_buf, uint2 *rowlist, Ctl *ctl, uint64_t cap, uint32_t piece, cudaStream_t st);
+cudaError_t launch_bin_rows(const uint32_t *order, const Rec *rec, uint32_t n_cap, int Tx, int Ty, uint32_t *M,
+                            void *rows_buf, uint2 *rowlist, Ctl *ctl, uint64_t cap, cudaStream_t st);
 // Tiles: splits every row list into its tiles; writes the final Gaussian list
 // (tile order, depth order within a tile) and every tile's [start, end).
 // Does nothing when the status holds an error.
-// P: bin_piece_bytes(cap, Tx, Ty) bytes; piece = bin_piece_entries(cap, Tx).
-cudaError_t launch_bin_tiles(const uint2 *rowlist, const void *rows_buf, int Tx, int Ty, uint32_t piece, uint32_t *P,
-                             uint32_t *list, uint2 *ranges, const Ctl *ctl, cudaStream_t st);
+// P: bin_piece_bytes(cap, Tx, Ty) bytes.
+cudaError_t launch_bin_tiles(const uint2 *rowlist, const void *rows_buf, int Tx, int Ty, uint32_t *P, uint32_t *list,
+                             uint2 *ranges, const Ctl *ctl, cudaStream_t st);
 size_t bin_rows_bytes(int Ty);
-uint32_t bin_piece_entries(int64_t dup_cap, int Tx);
 size_t bin_piece_bytes(int64_t dup_cap, int Tx, int Ty);
 // Training-step kernels (train.cu).
 size_t loss_workspace_bytes(int W, int H);

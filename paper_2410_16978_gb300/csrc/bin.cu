@@ -266,7 +266,7 @@ __global__ void __launch_bounds__(256) k_bin_rows_write(const uint32_t *__restri
             g[w] = gn[w];
             x01[w] = (r0 & 0xFFFFu) | (r1 << 16);
             y01[w] = (r0 >> 16) | (r1 & 0xFFFF0000u);
-            if (gn[w] != kNone) {
+            if (r0 >> 16 < r1 >> 16) {
                 lo = min(lo, r0 >> 16);
                 hi = max(hi, r1 >> 16);
             }

@@ -375,8 +375,8 @@ int front_sort(FrontCtx &f, const FrontCtx *other, cudaStream_t st, uint32_t **o
     int rc;
     {
         Stage sg(GS_STAGE_COMPACT, st, 1);
-        rc = other ? cuda_check(launch_sort_histograms2(f.tiles, f.depth, other->tiles, other->depth, f.sv.n, w,
-                                                        f.ctl, st),
+        rc = other ? cuda_check(launch_sort_histograms2(f.tiles, f.depth, f.rec, other->tiles, other->depth,
+                                                        other->rec, f.sv.n, w, f.ctl, st),
                                 "depth histograms (stereo)")
                    : cuda_check(launch_sort_histograms(f.tiles, f.depth, f.sv.n, w, f.ctl, st), "depth histograms");
         if (rc != GS_OK) return rc;

@@ -198,8 +198,11 @@ cudaError_t launch_sort_digits(const uint32_t *tiles, const uint32_t *depth, int
                                cudaStream_t st);
 // Two eyes: Gaussians visible to view a or view b, keyed by depth_a where
 // view a sees the Gaussian, else by depth_b (one depth order for both eyes).
-cudaError_t launch_sort_histograms2(const uint32_t *tiles_a, const uint32_t *depth_a, const uint32_t *tiles_b,
-                                    const uint32_t *depth_b, int n, const SortWork &work, Ctl *ctl, cudaStream_t st);
+// The histograms also give a Gaussian that only one view sees an empty tile
+// rectangle in the other view's records.
+cudaError_t launch_sort_histograms2(const uint32_t *tiles_a, const uint32_t *depth_a, Rec *rec_a,
+                                    const uint32_t *tiles_b, const uint32_t *depth_b, Rec *rec_b, int n,
+                                    const SortWork &work, Ctl *ctl, cudaStream_t st);
 cudaError_t launch_sort_digits2(const uint32_t *tiles_a, const uint32_t *depth_a, const uint32_t *tiles_b,
                                 const uint32_t *depth_b, int n, const SortWork &work, Ctl *ctl, cudaStream_t st);
 // Tile binning (bin.cu).  Rows: splits the depth-ordered visible Gaussians

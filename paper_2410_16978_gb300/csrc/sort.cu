@@ -164,9 +164,17 @@ struct VisSrc {             // one view: visible where its tile count is non-zer
     const uint32_t *tiles, *depth;
     __device__ __forceinline__ bool visible(uint32_t i) const { return tiles[i] > 0; }
     __device__ __forceinline__ uint32_t key(uint32_t i) const { return depth[i]; }
+    __device__ __forceinline__ void settle(uint32_t) const {}
 };
 struct VisSrc2 {            // two eyes: visible to either; keyed by view a's depth where view a sees it
     const uint32_t *tiles_a, *depth_a, *tiles_b, *depth_b;
+    Rec *rec_a, *rec_b;
+    // A visible Gaussian that one eye does not see is in both eyes' order, but that eye's record of it was not
+    // written: an empty tile rectangle there, so its binning passes the Gaussian over.
+    __device__ __forceinline__ void settle(uint32_t i) const {
+        if (tiles_a[i] == 0) rec_a[i].c.z = rec_a[i].c.w = 0.f;
+        if (tiles_b[i] == 0) rec_b[i].c.z = rec_b[i].c.w = 0.f;
+    }
     __device__ __forceinline__ bool visible(uint32_t i) const { return tiles_a[i] > 0 || tiles_b[i] > 0; }
     __device__ __forceinline__ uint32_t key(uint32_t i) const { return tiles_a[i] > 0 ? depth_a[i] : depth_b[i]; }
 };
@@ -278,6 +286,7 @@ __global__ void __launch_bounds__(256) k_sort_hist(Src src, uint32_t n, uint32_t
 #pragma unroll
         for (int r = 0; r < kSortItems; ++r) {
             if (vis[r]) {
+                src.settle(t0 + r * 256 + threadIdx.x);
                 kinv = max(kinv, ~key[r]);
                 kmax = max(kmax, key[r]);
                 ++cnt;
@@ -619,14 +628,15 @@ cudaError_t launch_sort_digits(const uint32_t *tiles, const uint32_t *depth, int
     return sort_digits(VisSrc{tiles, depth}, n, w, ctl, st);
 }
 
-cudaError_t launch_sort_histograms2(const uint32_t *tiles_a, const uint32_t *depth_a, const uint32_t *tiles_b,
-                                    const uint32_t *depth_b, int n, const SortWork &w, Ctl *ctl, cudaStream_t st) {
-    return sort_histograms(VisSrc2{tiles_a, depth_a, tiles_b, depth_b}, n, w, ctl, st);
+cudaError_t launch_sort_histograms2(const uint32_t *tiles_a, const uint32_t *depth_a, Rec *rec_a,
+                                    const uint32_t *tiles_b, const uint32_t *depth_b, Rec *rec_b, int n,
+                                    const SortWork &w, Ctl *ctl, cudaStream_t st) {
+    return sort_histograms(VisSrc2{tiles_a, depth_a, tiles_b, depth_b, rec_a, rec_b}, n, w, ctl, st);
 }
 
 cudaError_t launch_sort_digits2(const uint32_t *tiles_a, const uint32_t *depth_a, const uint32_t *tiles_b,
                                 const uint32_t *depth_b, int n, const SortWork &w, Ctl *ctl, cudaStream_t st) {
-    return sort_digits(VisSrc2{tiles_a, depth_a, tiles_b, depth_b}, n, w, ctl, st);
+    return sort_digits(VisSrc2{tiles_a, depth_a, tiles_b, depth_b, nullptr, nullptr}, n, w, ctl, st);
 }
 
 cudaError_t launch_activity_prune(const float *activity, const uint8_t *layer, uint32_t train_mask, int n,

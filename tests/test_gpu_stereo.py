@@ -143,3 +143,34 @@ def test_shared_sort_backward_per_eye(eye):
         assert np.abs(a - b).max() <= 1e-5 * np.abs(b).max(), (eye, f)
     vis = pre["vis"] > 0
     assert np.all(g["sh"].cpu().numpy()[~vis] == 0)
+
+
+def test_shared_sort_with_gaussians_only_one_eye_sees():
+    """A narrow view cuts off Gaussians at one eye's image border that the
+    other eye sees.  They are in the shared order of both eyes, but the eye
+    that does not see them has no record of them (its workspace holds whatever
+    was there before: here random bytes) and must not list them."""
+    sc = synth.scene_c4(scale=0.004)["scene"]
+    centre = synth.look_at_camera((0.0, 0.0, 4.0), fov_x_deg=9.0, width=208, height=80)
+    cams = list(synth.stereo_pair(centre, 0.064))
+    pre = [oracle.preprocess(sc, c, 0b11111, [], "f32") for c in cams]
+    vis = [p["vis"] > 0 for p in pre]
+    assert (vis[0] & ~vis[1]).sum() > 50 and (vis[1] & ~vis[0]).sum() > 50
+    ds = DeviceScene.from_host(sc)
+    g = torch.Generator("cuda").manual_seed(5)
+    r = [Rasterizer(sc.n, c.width, c.height) for c in cams]
+    for rr in r:
+        rr.workspace.random_(0, 256, generator=g)
+    imgs = [torch.empty((3, c.height, c.width), device="cuda") for c in cams]
+    _lib.gs_render_stereo(ds.c_struct(), _lib.make_camera(cams[0]), _lib.make_camera(cams[1]), 0b11111, [],
+                          (0.1, 0.2, 0.3), r[0].workspace, r[0].ws_bytes, r[1].workspace, r[1].ws_bytes, imgs[0],
+                          None, imgs[1], None, True, 0)
+    torch.cuda.synchronize()
+    for e in range(2):
+        keyed = dict(pre[e])
+        if e == 1:
+            keyed["depth"] = np.where(vis[0], pre[0]["depth"], pre[1]["depth"])
+        ranges, lst = oracle.bin_tiles(keyed)
+        ws = read_ws(r[e])
+        assert ws["status"].error == 0
+        compare_lists(ws, ranges, lst)

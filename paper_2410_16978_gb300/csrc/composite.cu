@@ -5,16 +5,16 @@
 //
 // Work decomposition (compositing is FP32 FMA + MUFU work, not a dense
 // contraction, so no tensor cores are involved):
-//  * Forward: persistent warps take work items (tile, 8x4 pixel block) from
-//    per-view device queues in heaviest-first tile order (the views of a
-//    batch in turn) and composite one pixel per lane until the block's 32
+//  * Forward: persistent warps take work items (tile, 8x4 or 8x8 pixel block)
+//    from per-view device queues in heaviest-first tile order (the views of a
+//    batch in turn) and composite one or two pixels per lane until the block's
 //    pixels are done.  The walk goes segment by segment (kSeg list
 //    positions), each segment blended from a local product that the
 //    transmittance at its start scales; at every segment boundary the warp
 //    stores each pixel's transmittance as a checkpoint, with the colour
 //    blended from there to the end of the pixel's walk (filled in when the
 //    walk ends).
-//  * Both passes drop, 32 records at a time, the splats that provably stay
+//  * Both passes drop, a chunk of records at a time, the splats that provably stay
 //    below alpha = 1/255 over the warp's whole pixel block (see
 //    splat_reaches_block); list positions are kept, so nothing changes.
 //  * Backward: the blended prefix of a pixel can be thousands of splats long,
@@ -36,10 +36,7 @@ namespace {
 
 constexpr unsigned FULL = 0xFFFFFFFFu;
 constexpr float kLn2 = 0x1.62e430p-1f;
-constexpr int kFwdThreads = 256;
-// One pixel per lane, an 8x4 block per warp.  (Two pixels per lane, an 8x8 block, gives each lane two blend
-// chains but culls on a larger block and needs 70 registers; on the 1.2M-Gaussian frame it measured 0.28 ms
-// against 0.22 ms.)
+constexpr int kFwdThreads = 128;
 constexpr int kBwdThreads = 128;
 // Backward pixels per lane: 2 (an 8x8 block per warp) or 4 (16x8).  4 halves the per-splat reduction and
 // atomics per pixel but needs 96 registers (5 blocks per SM instead of 7) and culls on a coarser block;
@@ -134,8 +131,11 @@ __device__ __forceinline__ int work_bucket(uint32_t w) {
 
 // One CTA (1024 threads) sorts the tiles heaviest first (by list length) into
 // order[] (ties in no particular order: tiles are independent, so the order
-// changes no result).
-__device__ void order_tiles(int Tn, uint32_t *order, uint32_t *s_cnt, uint32_t *s_w, const uint2 *ranges) {
+// changes no result), empty tiles last.  An entry holds what the compositor
+// needs to start on the tile: (tile, list start, list length, first checkpoint
+// segment).  Returns the number of tiles with a list.
+__device__ uint32_t order_tiles(int Tn, uint4 *order, uint32_t *s_cnt, uint32_t *s_w, const uint2 *ranges,
+                                const uint32_t *seg_base) {
     for (int b = threadIdx.x; b < kBuckets; b += blockDim.x) s_cnt[b] = 0;
     __syncthreads();
     for (int t = threadIdx.x; t < Tn; t += blockDim.x) atomicAdd(&s_cnt[work_bucket(ranges[t].y - ranges[t].x)], 1u);
@@ -147,9 +147,15 @@ __device__ void order_tiles(int Tn, uint32_t *order, uint32_t *s_cnt, uint32_t *
         if (threadIdx.x < kBuckets) s_cnt[threadIdx.x] = ex;
     }
     __syncthreads();
-    for (int t = threadIdx.x; t < Tn; t += blockDim.x)
-        order[atomicAdd(&s_cnt[work_bucket(ranges[t].y - ranges[t].x)], 1u)] = t;
+    const uint32_t live = s_cnt[kBuckets - 1];     // empty tiles are the last bucket
     __syncthreads();
+    for (int t = threadIdx.x; t < Tn; t += blockDim.x) {
+        const uint2 rg = ranges[t];
+        const uint32_t len = rg.y - rg.x;
+        order[atomicAdd(&s_cnt[work_bucket(len)], 1u)] =
+            make_uint4(static_cast<uint32_t>(t), rg.x, len, seg_base[t]);
+    }
+    return live;
 }
 
 // Forward set-up (one CTA): heaviest-first tile order by list length, the
@@ -161,12 +167,11 @@ __device__ void order_tiles(int Tn, uint32_t *order, uint32_t *s_cnt, uint32_t *
 constexpr int kSetupSmemTiles = 8192;
 
 __global__ void __launch_bounds__(1024) k_fwd_setup(const uint2 *__restrict__ g_ranges, int Tn,
-                                                    uint32_t *__restrict__ order, uint32_t *__restrict__ seg_base,
+                                                    uint4 *__restrict__ order, uint32_t *__restrict__ seg_base,
                                                     uint32_t *__restrict__ queue, uint32_t *__restrict__ qdone) {
     __shared__ uint32_t s_cnt[kBuckets];
     __shared__ uint32_t s_w[32];
     extern __shared__ uint2 s_ranges[];
-    if (threadIdx.x == 0) *queue = 0;
     const uint2 *ranges = g_ranges;
     if (Tn <= kSetupSmemTiles) {
         for (int t = threadIdx.x; t < Tn; t += blockDim.x) s_ranges[t] = g_ranges[t];
@@ -174,7 +179,6 @@ __global__ void __launch_bounds__(1024) k_fwd_setup(const uint2 *__restrict__ g_
         ranges = s_ranges;
     }
     for (int q = threadIdx.x; q < 8 * Tn; q += blockDim.x) qdone[q] = 0;   // 4 x 64-bit meeting words per tile
-    order_tiles(Tn, order, s_cnt, s_w, ranges);
     uint32_t carry = 0;
     for (int t0 = 0; t0 < Tn; t0 += 1024) {
         const int t = t0 + threadIdx.x;
@@ -184,6 +188,18 @@ __global__ void __launch_bounds__(1024) k_fwd_setup(const uint2 *__restrict__ g_
         if (t < Tn) seg_base[t] = carry + ex;
         carry += tot;
     }
+    __syncthreads();
+    const uint32_t live = order_tiles(Tn, order, s_cnt, s_w, ranges, seg_base);
+    if (threadIdx.x == 0) {
+        queue[0] = 0;
+        queue[1] = live;
+    }
+}
+
+__device__ __forceinline__ void load_geo(const Geo *g, float4 &a, float4 &b) {
+    asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
+                 : "l"(g));
 }
 
 struct Chunk {
@@ -256,7 +272,51 @@ struct FwdBatch {
 // Ts * P * (1 - alpha) < kTMin, the paper's T < 1e-4 on this factorisation.
 // The checkpoints store Ts and the colour blended from the segment on, which
 // is all the backward needs to start a segment's walk from its end.
+//
+// What bounds it, and what the kernel does about it:
+//  * A view whose longest walks set its time (up to about 1.5 Mpixels) waits
+//    on latencies.  One pixel per lane, and
+//    - the kept splats of a chunk are blended kFwdStep at a time: a step
+//      computes its alphas together and only the blends form a chain (a splat
+//      cost a lone warp 250 cycles of load, exponent, exponential and branch
+//      latency one at a time, 67 in steps of four);
+//    - chunks of 128 entries, four per lane, so that the records of the next
+//      chunk (about 700 cycles from L2) are on their way for as long as four
+//      32-entry chunks take to blend;
+//    - an item's successor is taken, and its tile's descriptor loaded, while
+//      the item is walked, and the exchange of the 8x4 blocks' prefixes is
+//      settled behind the next item's first loads: an item used to begin and
+//      end with about 2,500 cycles each of dependent L2 accesses;
+//    - tiles without a list are one item each, not eight.
+//  * Larger launches are bound by instruction issue and by the shared-memory /
+//    L1 pipe, where each gathered record costs a cycle per lane and load.  Two
+//    pixels per lane (8x8 blocks) halve the gathers, the tests and the items
+//    per pixel, and a record's geometry comes in one aligned 32-byte load (Geo);
+//    only kept entries fetch their last word (blue), by cp.async.
+// Measured (compositing stage, one at a time with 32-entry chunks before):
+// 1.2M-Gaussian 1024x1024 frame 0.154 -> 0.114 ms, 1.5M-Gaussian 1037x771 view
+// 0.177 -> 0.096, 500k-Gaussian 512x512 view 0.071 -> 0.053, 40k-Gaussian 397x243
+// view 0.061 -> 0.040; 3M-Gaussian 2064x2208 view 0.668 -> 0.452, both eyes of the
+// stereo pair 0.619 -> 0.380, 1920x1080 view 0.351 -> 0.211.
 constexpr int kFwdWarps = kFwdThreads / 32;
+constexpr int kFwdStep = 4;
+// A warp takes its next item before it walks the current one only where that
+// tile's list is at most this long: tiles come heaviest first, so what a
+// warp holds back is short too (taken early everywhere, the 1024x1024 frame took
+// 0.128 ms instead of 0.114).
+constexpr uint32_t kAheadLen = 1024;
+
+template <int PER>
+struct FwdKept {            // a chunk's entries that can reach the warp's block
+    float4 a[32 * PER + kFwdStep];     // u, v, A2, beta
+    float4 b[32 * PER + kFwdStep];     // G2, opacity, r, g
+    float blue[32 * PER + kFwdStep];   // (arrives by cp.async)
+    uint32_t pos[32 * PER];            // list position
+};
+template <int PER>
+struct FwdSmem {
+    FwdKept<PER> kept[kFwdWarps][2];
+};
 
 struct FwdLane {        // one pixel's walk
     float Ts;           // transmittance at the start of the current segment
@@ -267,71 +327,142 @@ struct FwdLane {        // one pixel's walk
     bool done;          // stopped (or outside the image)
 };
 
-struct FwdPipe {        // list ids and records fetched ahead of the walk
-    Chunk nxt;          // records of the 32 entries at pos
-    uint32_t gid;       // ids of the 32 entries at pos + 32
-    uint32_t pos;       // list position (from the tile's first entry) of nxt
-};
+__device__ __forceinline__ void cp_async4(void *dst, const void *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
+                 "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
 
-struct FwdSmem {
-    float4 a[kFwdWarps][32], b[kFwdWarps][32];
-    float c[kFwdWarps][32];
-    uint32_t pos[kFwdWarps][32];
-};
+// One tile list's entries on their way to a warp.
+template <int PER>
+struct FwdStream {
+    static constexpr uint32_t kChunk = 32 * PER;
+    const uint32_t *list;   // the tile's first entry
+    const Geo *geo;
+    const Rec *rec;
+    uint32_t len;
+    float4 a[PER], b[PER];    // this lane's entries of the next chunk
+    uint32_t cur[PER];     // their ids
+    uint32_t id[PER];      // this lane's ids of the chunk after it
+    uint32_t n;             // Gaussian count and status (bounds check of GS_DEBUG builds)
+    const Ctl *ctl;
 
-// Walks list positions [pp.pos, e) of the block at (bx0, by0) (an 8x4 block of
-// pixel centres), 32 entries at a time: the entries that can reach the block
-// are staged in shared memory, and each lane blends them into its pixel's
-// segment state.  Returns early once every lane has stopped.
-__device__ __forceinline__ void walk_segment(FwdPipe &pp, uint32_t e, const FwdJob &J, uint2 rg, float bx0, float by0,
-                                             float px, float py, FwdLane &L, int lane, int warp, FwdSmem &sm) {
-    const unsigned lt = (1u << lane) - 1u;
-    const uint32_t len = rg.y - rg.x;
-    bool mine = L.done;
-    for (; pp.pos < e; pp.pos += 32) {
-        if (__all_sync(FULL, mine)) break;
-        const uint32_t base = pp.pos;
-        const bool keep =
-            base + lane < len && splat_reaches_block(pp.nxt.a, pp.nxt.b, bx0, bx0 + 7.f, by0, by0 + 3.f);
-        const unsigned km = __ballot_sync(FULL, keep);
-        __syncwarp();
-        if (keep) {
-            const int slot = __popc(km & lt);
-            sm.a[warp][slot] = pp.nxt.a;
-            sm.b[warp][slot] = pp.nxt.b;
-            sm.c[warp][slot] = pp.nxt.c;
-            sm.pos[warp][slot] = base + lane;
-        }
-        __syncwarp();
-        const bool v1 = base + 32 + lane < len;
-        if (v1 && !GS_CHECK(pp.gid < J.n, J.ctl, kSiteFwdId))
-            pp.nxt = Chunk{};      // an inert splat (opacity 0): no block keeps it
-        else
-            fetch_rec(J.rec, pp.gid, v1, pp.nxt);
-        pp.gid = base + 64 + lane < len ? J.list[rg.x + base + 64 + lane] : 0u;
-        const int cnt = __popc(km);
-        int lastk = -1;
-        for (int k = 0; k < cnt && !mine; ++k) {
-            const float4 a = sm.a[warp][k], b = sm.b[warp][k];
-            float p, dy, ex, ao;
-            const float al = splat_alpha(px, py, a, b, p, dy, ex, ao);
-            if (al >= kAlphaMin) {
-                const float Pn = __fmul_rn(L.P, __fsub_rn(1.f, al));
-                if (__fmul_rn(L.Ts, Pn) < kTMin) {
-                    L.done = true;
-                    mine = true;
-                } else {
-                    const float w = __fmul_rn(al, L.P);
-                    L.D0 = __fmaf_rn(b.z, w, L.D0);
-                    L.D1 = __fmaf_rn(b.w, w, L.D1);
-                    L.D2 = __fmaf_rn(sm.c[warp][k], w, L.D2);
-                    L.P = Pn;
-                    lastk = k;
-                    ++L.nb;
-                }
+    __device__ __forceinline__ void load_ids(uint32_t pos, int lane) {
+#pragma unroll
+        for (int k = 0; k < PER; ++k) id[k] = pos + 32 * k + lane < len ? list[pos + 32 * k + lane] : 0u;
+    }
+    // Loads the entries of the chunk at `pos` (their ids are in id) and the ids of the chunk after it.
+    __device__ __forceinline__ void request(uint32_t pos, int lane) {
+#pragma unroll
+        for (int k = 0; k < PER; ++k) {
+            cur[k] = id[k];
+            if (pos + 32 * k + lane >= len) continue;
+            if (GS_CHECK(id[k] < n, ctl, kSiteFwdId)) {
+                load_geo(geo + id[k], a[k], b[k]);
+            } else {                                // an inert splat (opacity 0): no block keeps it
+                a[k] = b[k] = make_float4(0.f, 0.f, 0.f, 0.f);
             }
         }
-        if (lastk >= 0) L.last = sm.pos[warp][lastk] + 1;    // position of the chunk's last blend, read once
+        load_ids(pos + kChunk, lane);
+    }
+};
+
+// Blends the kept entries [k, k + S) into the segment state of the lane's pixels
+// (PX of them, four rows apart), in order.
+template <int S, int PX, int PER>
+__device__ __forceinline__ void blend_step(const FwdKept<PER> &K, int k, float px, float py, FwdLane (&L)[PX],
+                                           bool (&mine)[PX], int (&lastk)[PX]) {
+    float al[S][PX];
+    float2 rg[S];
+#pragma unroll
+    for (int j = 0; j < S; ++j) {
+        const float4 a = K.a[k + j], b = K.b[k + j];
+#pragma unroll
+        for (int i = 0; i < PX; ++i) {
+            float p, dy, ex, ao;
+            al[j][i] = splat_alpha(px, py + 4.f * i, a, b, p, dy, ex, ao);
+        }
+        rg[j] = make_float2(b.z, b.w);
+    }
+#pragma unroll
+    for (int j = 0; j < S; ++j) {
+        const float bl = K.blue[k + j];
+#pragma unroll
+        for (int i = 0; i < PX; ++i) {
+            const bool act = al[j][i] >= kAlphaMin && !mine[i];
+            const float Pn = __fmul_rn(L[i].P, __fsub_rn(1.f, al[j][i]));
+            const bool stop = __fmul_rn(L[i].Ts, Pn) < kTMin;
+            const float w = __fmul_rn(al[j][i], L[i].P);
+            mine[i] = mine[i] || (act && stop);
+            if (act && !stop) {
+                L[i].D0 = __fmaf_rn(rg[j].x, w, L[i].D0);
+                L[i].D1 = __fmaf_rn(rg[j].y, w, L[i].D1);
+                L[i].D2 = __fmaf_rn(bl, w, L[i].D2);
+                L[i].P = Pn;
+                lastk[i] = k + j;
+                ++L[i].nb;
+            }
+        }
+    }
+}
+
+// Takes the chunk at `pos` of the block at (bx0, by0) (8 x 4 PX pixel centres):
+// every lane tests its entries against the block, and those that can
+// reach it are staged in K in list order, their blue on its way.  Returns how
+// many; requests the chunk after.
+template <int PX, int PER>
+__device__ __forceinline__ int stage_chunk(FwdStream<PER> &st, uint32_t pos, float bx0, float by0, int lane,
+                                           FwdKept<PER> &K) {
+    bool keep[PER];
+    unsigned km[PER];
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        keep[k] = pos + 32 * k + lane < st.len &&
+                  splat_reaches_block(st.a[k], st.b[k], bx0, bx0 + 7.f, by0, by0 + (4.f * PX - 1.f));
+        km[k] = __ballot_sync(FULL, keep[k]);
+    }
+    int cnt = 0;
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        if (keep[k]) {
+            const int slot = cnt + __popc(km[k] & ((1u << lane) - 1u));
+            K.a[slot] = st.a[k];
+            K.b[slot] = st.b[k];
+            K.pos[slot] = pos + 32 * k + lane;
+            cp_async4(&K.blue[slot], &st.rec[st.cur[k]].c.x);
+        }
+        cnt += __popc(km[k]);
+    }
+    if (lane < kFwdStep) {                         // inert splats (opacity 0) fill the last step
+        K.a[cnt + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+        K.b[cnt + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    cp_async_commit();
+    st.request(pos + 32 * PER, lane);
+    return cnt;
+}
+
+// Blends a staged chunk into every lane's pixels.
+template <int PX, int PER>
+__device__ __forceinline__ void blend_chunk(const FwdKept<PER> &K, int cnt, float px, float py, FwdLane (&L)[PX]) {
+    bool mine[PX];
+    int lastk[PX];
+#pragma unroll
+    for (int i = 0; i < PX; ++i) {
+        mine[i] = L[i].done;
+        lastk[i] = -1;
+    }
+    int k = 0;
+    for (; k + kFwdStep / 2 < cnt; k += kFwdStep) blend_step<kFwdStep>(K, k, px, py, L, mine, lastk);
+    if (k < cnt) blend_step<kFwdStep / 2>(K, k, px, py, L, mine, lastk);
+#pragma unroll
+    for (int i = 0; i < PX; ++i) {
+        if (lastk[i] >= 0) L[i].last = K.pos[lastk[i]] + 1;    // position of the chunk's last blend, read once
+        L[i].done = mine[i];
     }
 }
 
@@ -341,118 +472,257 @@ __device__ __forceinline__ int next_live(uint32_t live, int v) {
     return __ffs(after ? after : live) - 1;
 }
 
-__global__ void __launch_bounds__(kFwdThreads) k_composite_fwd(const __grid_constant__ FwdBatch batch) {
-    __shared__ FwdSmem sm;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // Views of a batch are taken in turn, each from its own heaviest-first queue, so the heaviest blocks of
-    // every view start first; a view whose queue has run out leaves the rotation.
-    uint32_t live = (1u << batch.n) - 1u;
-    int v = static_cast<int>((blockIdx.x * kFwdWarps + warp) % static_cast<uint32_t>(batch.n));
-    for (;;) {
-        uint32_t local = 0;
+// The views of a batch are taken in turn, each from its own heaviest-first queue, so the heaviest blocks of
+// every view start first; a view whose queue has run out leaves the rotation.  A view's queue is one 64-bit word,
+// (tiles with a list << 32 | items taken): its items are the 8 / PX blocks of every tile with a list, then the
+// empty tiles, each as a whole.
+template <int PX>
+struct FwdQueue {
+    static constexpr uint32_t kBlocks = 8 / PX;      // items of a tile with a list
+    const FwdBatch &batch;
+    uint32_t live;
+    int lane;
+    __device__ __forceinline__ unsigned long long take(int v) const {      // lane 0's result counts
+        return lane == 0 ? atomicAdd(reinterpret_cast<unsigned long long *>(batch.job[v].queue), 1ull) : 0ull;
+    }
+    // The item taken as q from view v, or from a later live view when v had none left; false: all have run out.
+    __device__ __forceinline__ bool resolve(unsigned long long q, int &v, uint32_t &local, uint32_t &tiles) {
         if (lane == 0) {
             for (;;) {
-                local = atomicAdd(batch.job[v].queue, 1u);
-                if (local < static_cast<uint32_t>(batch.job[v].Tn) * 8u) break;
+                const uint32_t nl = static_cast<uint32_t>(q >> 32);
+                if (static_cast<uint32_t>(q) < (kBlocks - 1u) * nl + static_cast<uint32_t>(batch.job[v].Tn)) break;
                 live &= ~(1u << v);
                 if (!live) break;
                 v = next_live(live, v);
+                q = take(v);
             }
         }
         live = __shfl_sync(FULL, live, 0);
-        if (!live) break;
-        local = __shfl_sync(FULL, local, 0);
+        if (!live) return false;
         v = __shfl_sync(FULL, v, 0);
+        local = __shfl_sync(FULL, static_cast<uint32_t>(q), 0);
+        tiles = __shfl_sync(FULL, static_cast<uint32_t>(q >> 32), 0);
+        return true;
+    }
+};
+
+// The two 8x4 blocks of an 8x8 block meet in one 64-bit word, a half each for (longest blended prefix + 1).  The
+// second to arrive knows the 8x8 block's longest blended prefix: it stores it for the backward and appends the
+// block's backward work items, one per kSeg positions of the prefix.  They come out in the order the forward
+// finishes them, the heaviest tiles last; the backward takes them from the end.  The exchange is sent at the end
+// of an item and settled while the next item's records are on their way.
+struct FwdMeet {
+    unsigned long long old;    // lane 0: the word before this block's half was set
+    uint32_t tile, qd, half, prefix;
+    int v;
+    bool open;
+    __device__ __forceinline__ void settle(const FwdBatch &batch, int lane) {
+        if (!open) return;
+        open = false;
         const FwdJob &J = batch.job[v];
-        const int W = J.W, H = J.H, Tx = J.Tx;
-        const int tile = J.order[local / 8];
-        const int sub = local % 8;                      // block column sub & 1, block row sub >> 1
-        const int ox = (sub & 1) * 8, oy = (sub >> 1) * 4;
-        const uint2 rg = J.ranges[tile];
-        const float bx0 = (tile % Tx) * kTile + ox + 0.5f, by0 = (tile / Tx) * kTile + oy + 0.5f;
-        const int lx = ox + (lane & 7), ly = oy + (lane >> 3);
-        const int x = (tile % Tx) * kTile + lx, y = (tile / Tx) * kTile + ly;
-        const bool inside = x < W && y < H;
-        FwdLane L{1.f, 1.f, 0.f, 0.f, 0.f, 0u, 0u, !inside};
-        float C0 = 0.f, C1 = 0.f, C2 = 0.f;             // colour of the last finished segment
-        const uint32_t len = rg.y - rg.x, nseg = ceil_seg(len);
-        float4 *ck0 = J.ckpt + static_cast<size_t>(J.seg_base[tile]) * kTilePix + lx;
-        FwdPipe pp;
-        pp.pos = 0;
-        fetch_chunk(J.list, J.rec, rg.x + lane, rg.y, pp.nxt, J.n, J.ctl, kSiteFwdId);
-        pp.gid = rg.x + 32 + lane < rg.y ? J.list[rg.x + 32 + lane] : 0u;   // ids one chunk ahead
-        uint32_t sd = 0;
-        for (uint32_t s = 0; s < nseg; ++s) {
-            if (s > 0) {
-                if (__all_sync(FULL, L.done)) break;
-                sd = s;
-                if (!GS_CHECK(J.seg_base[tile] + sd < J.n_segs, J.ctl, kSiteCkpt)) break;
-                // checkpoint s: (T at the segment's start, colour of segment s - 1); rewritten below
-                ck0[static_cast<size_t>(sd) * kTilePix + ly * kTile] = make_float4(L.Ts, C0, C1, C2);
-            }
-            walk_segment(pp, min((s + 1) * kSeg, len), J, rg, bx0, by0, x + 0.5f, y + 0.5f, L, lane, warp, sm);
-            // the segment ends: its colour, the transmittance at the next segment's start
-            C0 = __fmul_rn(L.Ts, L.D0);
-            C1 = __fmul_rn(L.Ts, L.D1);
-            C2 = __fmul_rn(L.Ts, L.D2);
-            L.Ts = __fmul_rn(L.Ts, L.P);
-            L.P = 1.f;
-            L.D0 = L.D1 = L.D2 = 0.f;
-        }
-        // Checkpoint s holds (T at segment start, colour of segment s-1) as written
-        // above; rewrite it, deepest segment first, to (T at segment start, F_s),
-        // F_s = colour blended at list positions >= s kSeg.  F_0 is the pixel's colour.
-        for (uint32_t s = sd; s > 0; --s) {
-            float4 *slot = ck0 + static_cast<size_t>(s) * kTilePix + ly * kTile;
-            const float4 raw = *slot;
-            *slot = make_float4(raw.x, C0, C1, C2);
-            C0 = __fadd_rn(raw.y, C0);
-            C1 = __fadd_rn(raw.z, C1);
-            C2 = __fadd_rn(raw.w, C2);
-        }
-        if (inside) {
-            const size_t plane = static_cast<size_t>(W) * H;
-            const size_t pix = static_cast<size_t>(y) * W + x;
-            J.image[pix] = __fmaf_rn(L.Ts, J.bg.x, C0);
-            J.image[plane + pix] = __fmaf_rn(L.Ts, J.bg.y, C1);
-            J.image[2 * plane + pix] = __fmaf_rn(L.Ts, J.bg.z, C2);
-            if (J.alpha) J.alpha[pix] = 1.f - L.Ts;
-            J.t_final[pix] = L.Ts;
-            J.n_contrib[pix] = L.last;
-        }
-        const uint32_t wm = __reduce_max_sync(FULL, L.last);
-        const int qd = (sub & 1) + 2 * (oy >> 3);      // the 8x8 block of the tile this 8x4 block is half of
-        const uint32_t wb = __reduce_add_sync(FULL, L.nb);
-        if (lane == 0 && wb) atomicAdd(J.n_blended, static_cast<unsigned long long>(wb));
-        // The two 8x4 blocks of an 8x8 block meet in one 64-bit word (finished blocks << 32 | longest blended
-        // prefix).  The second to finish knows the 8x8 block's longest blended prefix: it stores it for the
-        // backward and appends the block's backward work items, one per kSeg positions of the prefix.  They come
-        // out in the order the forward finishes them, the heaviest tiles last; the backward takes them from the end.
         uint32_t nsg = 0, ibase = 0;
         if (lane == 0) {
-            unsigned long long *meet = reinterpret_cast<unsigned long long *>(J.qdone) + 4 * tile + qd;
-            unsigned long long seen = 0ull, prev = ~0ull;
-            bool ok = false;
-            for (int round = 0; round < 3 && !ok; ++round) {   // two rounds at most: one other writer, once
-                const unsigned long long want =
-                    ((seen >> 32) + 1ull) << 32 | max(static_cast<uint32_t>(seen), wm);
-                prev = atomicCAS(meet, seen, want);
-                ok = prev == seen;
-                seen = prev;
-            }
-            if (ok && (prev >> 32) == 1ull) {
-                const uint32_t qm = max(static_cast<uint32_t>(prev), wm);
+            const uint32_t other = static_cast<uint32_t>(old >> (32u * (half ^ 1u)));
+            if (other) {
+                const uint32_t qm = max(other - 1u, prefix);
                 J.qwork[4 * tile + qd] = qm;
                 nsg = ceil_seg(qm);
                 if (nsg) ibase = atomicAdd(J.n_items, nsg);
             }
         }
         nsg = __shfl_sync(FULL, nsg, 0);
+        if (nsg == 0) return;
         ibase = __shfl_sync(FULL, ibase, 0);
-        for (uint32_t sg = lane; sg < nsg; sg += 32)
-            J.items[ibase + sg] = make_uint2(static_cast<uint32_t>(tile), (static_cast<uint32_t>(qd) << 24) | sg);
-        v = next_live(live, v);
+        for (uint32_t sg = lane; sg < nsg; sg += 32) J.items[ibase + sg] = make_uint2(tile, (qd << 24) | sg);
     }
+};
+
+template <int PX, int PER>
+__global__ void __launch_bounds__(kFwdThreads) k_composite_fwd(const __grid_constant__ FwdBatch batch) {
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    FwdSmem<PER> &sm = *reinterpret_cast<FwdSmem<PER> *>(s_raw);
+    constexpr uint32_t kChunk = 32 * PER, B = FwdQueue<PX>::kBlocks;
+    static_assert(kSeg % kChunk == 0, "segments are whole chunks");
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    FwdQueue<PX> fq{batch, (1u << batch.n) - 1u, lane};
+    FwdMeet meet;
+    meet.open = false;
+    FwdStream<PER> st;
+    int v = static_cast<int>((blockIdx.x * kFwdWarps + warp) % static_cast<uint32_t>(batch.n));
+    uint32_t local, tiles;
+    bool have = fq.resolve(fq.take(v), v, local, tiles);
+    uint4 d = make_uint4(0u, 0u, 0u, 0u);
+    const auto slot_of = [](uint32_t l, uint32_t nl) { return l < B * nl ? l / B : l - (B - 1u) * nl; };
+    if (have) d = batch.job[v].order[slot_of(local, tiles)];
+    const auto take_next = [&](unsigned long long q, int nv) {
+        v = nv;
+        have = fq.resolve(q, v, local, tiles);
+        if (have) d = batch.job[v].order[slot_of(local, tiles)];
+    };
+    while (have) {
+        const FwdJob &J = batch.job[v];
+        const int W = J.W, H = J.H, Tx = J.Tx;
+        const int tile = static_cast<int>(d.x), ty = tile / Tx, tx = tile - ty * Tx;
+        const bool empty = local >= B * tiles;
+        const size_t plane = static_cast<size_t>(W) * H;
+        if (empty) {
+            // no list: the background over the whole tile, 8 pixels per lane; the next item is taken first
+            int nv = next_live(fq.live, v);
+            const unsigned long long q = fq.take(nv);
+            const float3 bg = J.bg;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const int x = tx * kTile + (lane & 15), y = ty * kTile + 2 * k + (lane >> 4);
+                if (x < W && y < H) {
+                    const size_t pix = static_cast<size_t>(y) * W + x;
+                    J.image[pix] = bg.x;
+                    J.image[plane + pix] = bg.y;
+                    J.image[2 * plane + pix] = bg.z;
+                    if (J.alpha) J.alpha[pix] = 0.f;
+                    J.t_final[pix] = 1.f;
+                    J.n_contrib[pix] = 0u;
+                }
+            }
+            take_next(q, nv);
+            continue;
+        }
+        const uint32_t len = d.z;
+        st.list = J.list + d.y;
+        st.geo = J.geo;
+        st.rec = J.rec;
+        st.len = len;
+        st.n = J.n;
+        st.ctl = J.ctl;
+        st.load_ids(0, lane);
+        cp_async_wait<0>();                             // what the item before had staged beyond its stop
+        __syncwarp();
+        const int sub = local % B;                      // block column sub & 1, block row sub >> 1
+        const int ox = (sub & 1) * 8, oy = (sub >> 1) * 4 * PX;
+        const float bx0 = tx * kTile + ox + 0.5f, by0 = ty * kTile + oy + 0.5f;
+        const int lx = ox + (lane & 7), ly = oy + (lane >> 3);
+        const int x = tx * kTile + lx, y = ty * kTile + ly;
+        FwdLane L[PX];
+        float C0[PX], C1[PX], C2[PX];                   // colour of the last finished segment
+#pragma unroll
+        for (int i = 0; i < PX; ++i) {
+            L[i] = FwdLane{1.f, 1.f, 0.f, 0.f, 0.f, 0u, 0u, !(x < W && y + 4 * i < H)};
+            C0[i] = C1[i] = C2[i] = 0.f;
+        }
+        const auto all_done = [&]() {
+            bool d = L[0].done;
+#pragma unroll
+            for (int i = 1; i < PX; ++i) d = d && L[i].done;
+            return __all_sync(FULL, d) != 0;
+        };
+        float4 *ck0 = J.ckpt + static_cast<size_t>(d.w) * kTilePix + ly * kTile + lx;
+        st.request(0, lane);
+        // a short walk: the next item is taken now and its descriptor loaded at the end
+        const bool ahead = len <= kAheadLen;
+        int nv = next_live(fq.live, v);
+        unsigned long long q = 0;
+        if (ahead) q = fq.take(nv);
+        if constexpr (PX == 1) meet.settle(batch, lane);
+        // chunk by chunk, each staged before the one ahead of it is blended
+        uint32_t sd = 0;
+        int cnt_prev = 0;
+        if (!all_done()) {
+            for (uint32_t pos = 0, buf = 0;; pos += kChunk, buf ^= 1) {
+                const bool more = pos < len;
+                int cnt = 0;
+                if (more) cnt = stage_chunk<PX>(st, pos, bx0, by0, lane, sm.kept[warp][buf]);
+                if (pos > 0) {
+                    if (more) cp_async_wait<1>(); else cp_async_wait<0>();
+                    __syncwarp();
+                    blend_chunk(sm.kept[warp][buf ^ 1], cnt_prev, x + 0.5f, y + 0.5f, L);
+                    const bool stop = all_done() || !more;
+                    if (stop || pos % kSeg == 0) {
+                        // the segment ends: its colour, the transmittance at the next segment's start
+#pragma unroll
+                        for (int i = 0; i < PX; ++i) {
+                            C0[i] = __fmul_rn(L[i].Ts, L[i].D0);
+                            C1[i] = __fmul_rn(L[i].Ts, L[i].D1);
+                            C2[i] = __fmul_rn(L[i].Ts, L[i].D2);
+                            L[i].Ts = __fmul_rn(L[i].Ts, L[i].P);
+                            L[i].P = 1.f;
+                            L[i].D0 = L[i].D1 = L[i].D2 = 0.f;
+                        }
+                        if (stop) break;
+                        ++sd;
+                        if (!GS_CHECK(d.w + sd < J.n_segs, J.ctl, kSiteCkpt)) {
+                            --sd;
+                            break;
+                        }
+                        // checkpoint sd: (T at the segment's start, colour of segment sd - 1); rewritten below
+#pragma unroll
+                        for (int i = 0; i < PX; ++i)
+                            ck0[static_cast<size_t>(sd) * kTilePix + 4 * kTile * i] =
+                                make_float4(L[i].Ts, C0[i], C1[i], C2[i]);
+                    }
+                    __syncwarp();                  // the chunk has been read: its buffer is staged next
+                }
+                cnt_prev = cnt;
+            }
+        }
+        const int mv = v;
+        if (ahead) take_next(q, nv);
+        else q = fq.take(nv);
+        // Checkpoint s holds (T at segment start, colour of segment s-1) as written
+        // above; rewrite it, deepest segment first, to (T at segment start, F_s),
+        // F_s = colour blended at list positions >= s kSeg.  F_0 is the pixel's colour.
+        // Four are read ahead of the chain.
+#pragma unroll
+        for (int i = 0; i < PX; ++i) {
+            float4 *ck = ck0 + 4 * kTile * i;
+            for (uint32_t s = sd; s > 0;) {
+                float4 raw[4];
+#pragma unroll
+                for (uint32_t k = 0; k < 4; ++k)
+                    if (k < s) raw[k] = ck[static_cast<size_t>(s - k) * kTilePix];
+#pragma unroll
+                for (uint32_t k = 0; k < 4; ++k) {
+                    if (k >= s) continue;
+                    ck[static_cast<size_t>(s - k) * kTilePix] = make_float4(raw[k].x, C0[i], C1[i], C2[i]);
+                    C0[i] = __fadd_rn(raw[k].y, C0[i]);
+                    C1[i] = __fadd_rn(raw[k].z, C1[i]);
+                    C2[i] = __fadd_rn(raw[k].w, C2[i]);
+                }
+                s = s > 4 ? s - 4 : 0;
+            }
+            if (x < W && y + 4 * i < H) {
+                const size_t pix = static_cast<size_t>(y + 4 * i) * W + x;
+                J.image[pix] = __fmaf_rn(L[i].Ts, J.bg.x, C0[i]);
+                J.image[plane + pix] = __fmaf_rn(L[i].Ts, J.bg.y, C1[i]);
+                J.image[2 * plane + pix] = __fmaf_rn(L[i].Ts, J.bg.z, C2[i]);
+                if (J.alpha) J.alpha[pix] = 1.f - L[i].Ts;
+                J.t_final[pix] = L[i].Ts;
+                J.n_contrib[pix] = L[i].last;
+            }
+        }
+        uint32_t last = L[0].last, nb = L[0].nb;
+#pragma unroll
+        for (int i = 1; i < PX; ++i) {
+            last = max(last, L[i].last);
+            nb += L[i].nb;
+        }
+        meet.prefix = __reduce_max_sync(FULL, last);
+        meet.tile = static_cast<uint32_t>(tile);
+        meet.qd = (sub & 1) + 2 * (oy >> 3);           // the 8x8 block of the tile this 8x4 block is half of
+        meet.half = (oy >> 2) & 1;
+        meet.v = mv;
+        meet.open = true;
+        const uint32_t wb = __reduce_add_sync(FULL, nb);
+        if (lane == 0) {
+            if (wb) atomicAdd(J.n_blended, static_cast<unsigned long long>(wb));
+            if constexpr (PX == 1)
+                meet.old = atomicOr(reinterpret_cast<unsigned long long *>(J.qdone) + 4 * tile + meet.qd,
+                                    static_cast<unsigned long long>(meet.prefix + 1u) << (32u * meet.half));
+            else
+                meet.old = 1ull << (32u * (meet.half ^ 1u));     // an 8x8 block of its own
+        }
+        if constexpr (PX == 2) meet.settle(batch, lane);
+        if (!ahead) take_next(q, nv);
+    }
+    meet.settle(batch, lane);
 }
 
 // Backward set-up: the work items (tile, 8x8 block q, segment s) were written
@@ -702,33 +972,35 @@ __global__ void __launch_bounds__(kBwdThreads, 6) k_composite_bwd(
     }
 }
 
-// Blocks that fill every SM once for a persistent kernel (at most max_per
-// blocks per SM).
+// Blocks that fill every SM once for a persistent kernel.
 template <class K>
-int persistent_blocks(K kernel, int threads, int max_per = 1 << 30) {
+int persistent_blocks(K kernel, int threads, size_t smem = 0) {
     int dev = 0, sms = 0, per = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, 0);
-    return max(1, sms) * max(1, min(per, max_per));
+    if (smem) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, smem);
+    return max(1, sms) * max(1, per);
 }
 
-// Forward CTAs per SM.  The frame's longest items (8x4 blocks of tiles whose
-// walks run to thousands of list positions) start first and end last, and
-// while their SM is crowded each gets only its warp's share of the issue
-// slots.  Sixteen warps per SM still keep the SM issuing, and give those items
-// twice the share that the 32 resident warps allowed: on the 1.2M-Gaussian
-// frame the kernel took 0.19 ms instead of 0.22 (one block per SM: 0.27).
-// A launch of many pixels has many more items per warp than its longest item
-// is long, so the tail weighs less and a third CTA per SM pays: a 2064 x 2208
-// view of 3M Gaussians took 0.606 ms instead of 0.666 (the 1.2M-Gaussian
-// 1024 x 1024 frame 0.20 ms instead of 0.176, a 3M-Gaussian one 0.294 either
-// way).  Batched serving launches keep two: they run beside the launches of a
-// companion stream, and a third CTA per SM lowered the saturated served
-// throughput from 7,530 to 7,270 Mpixels/s.
-constexpr int kFwdBlocksPerSm = 2;
-constexpr int kFwdBlocksPerSmWide = 3;
-constexpr uint64_t kFwdWidePixels = 2u << 20;   // pixels of a launch from which it takes kFwdBlocksPerSmWide
+// Pixels of a launch from which the forward takes two pixels per lane.  Below,
+// the few longest walks set the time and an 8x8 block's walk is longer than an
+// 8x4 block's (1024x1024 frame 0.126 against 0.114 ms, 1037x771 view 0.137 against
+// 0.096); above, the work per pixel does (1920x1080 view 0.211 against 0.316 ms,
+// 2064x2208 view 0.452 against 0.697, eight 512x512 views in one launch 0.274
+// against 0.280).
+constexpr uint64_t kFwdWidePixels = 3u << 19;
+
+// One launch of the forward compositor: every SM filled once.
+template <int PX, int PER>
+cudaError_t launch_forward(const FwdBatch &batch, uint32_t items, cudaStream_t st) {
+    constexpr size_t smem = sizeof(FwdSmem<PER>);
+    static PerDevice cache;
+    const int blocks = cache.get([] { return persistent_blocks(k_composite_fwd<PX, PER>, kFwdThreads, smem); });
+    const uint32_t need = (items + kFwdWarps - 1) / kFwdWarps;
+    k_composite_fwd<PX, PER><<<min(static_cast<uint32_t>(blocks), need), kFwdThreads, smem, st>>>(batch);
+    return cudaGetLastError();
+}
 
 }  // namespace
 
@@ -744,7 +1016,7 @@ cudaError_t launch_fwd_setup(const CompositeBufs &cb, const uint2 *ranges, int T
     return cudaGetLastError();
 }
 
-cudaError_t launch_composite_forward(const FwdJob *jobs, int n, cudaStream_t st, bool wide_ok) {
+cudaError_t launch_composite_forward(const FwdJob *jobs, int n, cudaStream_t st) {
     FwdBatch batch;
     batch.n = 0;
     uint32_t total = 0;
@@ -756,15 +1028,8 @@ cudaError_t launch_composite_forward(const FwdJob *jobs, int n, cudaStream_t st,
         pixels += static_cast<uint64_t>(jobs[i].W) * jobs[i].H;
     }
     if (total == 0) return cudaSuccess;
-    static PerDevice cache, cache_wide;
-    const int blocks = wide_ok && pixels >= kFwdWidePixels
-                           ? cache_wide.get([] {
-                                 return persistent_blocks(k_composite_fwd, kFwdThreads, kFwdBlocksPerSmWide);
-                             })
-                           : cache.get([] { return persistent_blocks(k_composite_fwd, kFwdThreads, kFwdBlocksPerSm); });
-    const int b = min(blocks, static_cast<int>((total + kFwdWarps - 1) / kFwdWarps));
-    k_composite_fwd<<<b, kFwdThreads, 0, st>>>(batch);
-    return cudaGetLastError();
+    return pixels >= kFwdWidePixels ? launch_forward<2, 2>(batch, total / 2, st)
+                                    : launch_forward<1, 4>(batch, total, st);
 }
 
 cudaError_t launch_bwd_setup(const CompositeBufs &cb, int Tx, int Ty, float4 *rec_grad, const uint32_t *vis_index,

@@ -35,6 +35,7 @@ bool make_layout(int64_t n, int W, int H, int64_t dup_cap, Layout *L) {
     o.bin_rows = take(bin_rows_bytes(o.Ty));
     o.ranges = take(static_cast<size_t>(o.Tn) * 8);
     o.rec = take(N * sizeof(Rec));
+    o.geo = take(N * sizeof(Geo));
     o.tiles = take(N * 4);
     o.depth = take(N * 4);
     o.sort_k[0] = take(N * 4); o.sort_k[1] = take(N * 4);
@@ -49,7 +50,7 @@ bool make_layout(int64_t n, int W, int H, int64_t dup_cap, Layout *L) {
     o.n_contrib = take(P * 4);
     o.partials = take(kMaxSortBlocks * 4);
     o.rec_grad = take(N * sizeof(Rec));
-    o.tile_order = take(static_cast<size_t>(o.Tn) * 4);
+    o.tile_order = take(static_cast<size_t>(o.Tn) * 16);
     o.qdone = take(static_cast<size_t>(o.Tn) * 32);
     o.seg_base = take(static_cast<size_t>(o.Tn) * 4);
     o.qwork = take(static_cast<size_t>(o.Tn) * 16);
@@ -202,14 +203,14 @@ int check_camera(const gs_camera *c, CamView *v) {
 CompositeBufs composite_bufs(void *ws, const Layout &L) {
     Ctl *ctl = at<Ctl>(ws, L.ctl);
     CompositeBufs cb;
-    cb.order = at<uint32_t>(ws, L.tile_order);
+    cb.order = at<uint4>(ws, L.tile_order);
     cb.qdone = at<uint32_t>(ws, L.qdone);
     cb.seg_base = at<uint32_t>(ws, L.seg_base);
     cb.qwork = at<uint32_t>(ws, L.qwork);
     cb.ckpt = at<float4>(ws, L.ckpt);
     cb.items = at<uint2>(ws, L.items);
     cb.n_items = &ctl->n_items;
-    cb.queue = &ctl->fwd_queue;
+    cb.queue = &ctl->queue;
     return cb;
 }
 
@@ -347,7 +348,8 @@ int front_preprocess(const gs_scene *scene, const gs_camera *camera, uint32_t la
                          "memset status")) != GS_OK)
         return rc;
     Stage sg(GS_STAGE_PREPROCESS, st, 1);
-    return cuda_check(launch_preprocess(f->sv, f->cv, layer_mask, pl, f->rec, f->tiles, f->depth, f->ctl, st),
+    return cuda_check(launch_preprocess(f->sv, f->cv, layer_mask, pl, f->rec, at<Geo>(workspace, L.geo), f->tiles,
+                                        f->depth, f->ctl, st),
                       "preprocess");
 }
 
@@ -423,14 +425,13 @@ int front_bin(FrontCtx &f, const uint32_t *order, cudaStream_t st, FwdJob *job) 
         if ((rc = cuda_check(launch_fwd_setup(cb, ranges, L.Tn, st), "compositor set-up")) != GS_OK) return rc;
     }
     job->order = cb.order;
-    job->ranges = ranges;
     job->list = list;
+    job->geo = at<Geo>(ws, L.geo);
     job->rec = f.rec;
     job->image = f.image;
     job->alpha = f.alpha;
     job->t_final = at<float>(ws, L.t_final);
     job->n_contrib = at<uint32_t>(ws, L.n_contrib);
-    job->seg_base = cb.seg_base;
     job->ckpt = cb.ckpt;
     job->qwork = cb.qwork;
     job->n_blended = reinterpret_cast<unsigned long long *>(&f.ctl->st.n_blended);
@@ -475,7 +476,7 @@ int gs_render(const gs_scene *scene, const gs_camera *camera, uint32_t layer_mas
     int rc = render_front(scene, camera, layer_mask, planes, n_planes, bg, workspace, ws_bytes, image, alpha, st, &job);
     if (rc != GS_OK) return rc;
     Stage sg(GS_STAGE_COMPOSITE, st, 1);
-    return cuda_check(launch_composite_forward(&job, 1, st, true), "composite");
+    return cuda_check(launch_composite_forward(&job, 1, st), "composite");
 }
 
 int gs_render_batch(const gs_render_request *reqs, int32_t n, void *stream) {
@@ -493,7 +494,7 @@ int gs_render_batch(const gs_render_request *reqs, int32_t n, void *stream) {
         if (rc != GS_OK) return rc;
     }
     Stage sg(GS_STAGE_COMPOSITE, st, 1);
-    return cuda_check(launch_composite_forward(jobs, n, st, false), "batched composite");
+    return cuda_check(launch_composite_forward(jobs, n, st), "batched composite");
 }
 
 
@@ -541,7 +542,7 @@ int gs_render_stereo(const gs_scene *scene, const gs_camera *left, const gs_came
         }
     }
     Stage sg(GS_STAGE_COMPOSITE, st, 1);
-    return cuda_check(launch_composite_forward(jobs, 2, st, true), "stereo composite");
+    return cuda_check(launch_composite_forward(jobs, 2, st), "stereo composite");
 }
 
 int gs_render_backward(const gs_scene *scene, const gs_camera *camera, const float *bg, void *workspace,

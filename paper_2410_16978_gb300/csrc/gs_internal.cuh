@@ -40,6 +40,12 @@ struct __align__(16) Rec {
     float4 c;
 };
 
+// What the forward compositor tests every list entry with, in one aligned
+// 32-byte load: Rec::a and Rec::b of a visible Gaussian.
+struct __align__(32) Geo {
+    float4 a, b;
+};
+
 // Device control block at offset 0 of the workspace.  The first member is
 // the public gs_status; the rest are counts the kernels hand to each other.
 struct Ctl {
@@ -47,8 +53,8 @@ struct Ctl {
     uint32_t n_vis;        // visible Gaussians (counted by the depth-sort histograms)
     uint32_t dbg_site;     // GS_DEBUG builds: number of the first failed bounds check (0: none)
     uint32_t depth_mm[2];  // ~min and max of the visible depth keys (digits the sort can skip)
-    uint32_t fwd_queue;    // next work item of the persistent forward compositor
-    uint32_t bwd_queue;    // next work item of the persistent backward compositor
+    uint32_t queue;        // next work item of the persistent compositors (forward and backward in turn)
+    uint32_t live_tiles;   // tiles with a list (with `queue` the forward's 64-bit queue word)
     uint32_t n_items;      // backward work items (tile, 8x8 block, segment)
     uint32_t n_pieces;     // row-list pieces of the binning
     uint32_t sort_ticket[4];   // next tile of each digit kernel of the depth sort (after the first)
@@ -56,7 +62,7 @@ struct Ctl {
     uint32_t bin_piece;        // row-list entries per piece of the binning
     uint32_t pad[10];
 };
-static_assert(sizeof(Ctl) == 128, "Ctl layout");
+static_assert(sizeof(Ctl) == 128 && offsetof(Ctl, queue) % 8 == 0, "Ctl layout");
 
 // Bounds checks of GS_DEBUG builds.  GS_CHECK(ok, ctl, site) is `ok` in a
 // debug build, where a false `ok` also sets GS_ERR_BOUNDS in the status word
@@ -91,7 +97,7 @@ __device__ __forceinline__ bool gs_check(bool ok, const Ctl *ctl, uint32_t site)
 struct Layout {
     int64_t n = 0, dup_cap = 0;
     int W = 0, H = 0, Tx = 0, Ty = 0, Tn = 0;
-    size_t ctl = 0, rec = 0, tiles = 0, depth = 0, sort_k[2] = {0, 0}, sort_v[2] = {0, 0}, order = 0, vis_index = 0,
+    size_t ctl = 0, rec = 0, geo = 0, tiles = 0, depth = 0, sort_k[2] = {0, 0}, sort_v[2] = {0, 0}, order = 0, vis_index = 0,
            sort_hist = 0, sort_grp = 0, sort_cnt = 0, sort_status = 0, bin_m = 0,
            bin_rows = 0, bin_p = 0, rowlist = 0, list = 0, ranges = 0, t_final = 0, n_contrib = 0,
            partials = 0, rec_grad = 0, tile_order = 0, qdone = 0, seg_base = 0, qwork = 0,
@@ -140,7 +146,8 @@ struct Planes {
 
 // ---- launches (each returns cudaGetLastError() of its launches) ----
 cudaError_t launch_preprocess(const SceneView &s, const CamView &c, uint32_t layer_mask, const Planes &pl,
-                              Rec *rec, uint32_t *tiles, uint32_t *depth_key, const Ctl *ctl, cudaStream_t st);
+                              Rec *rec, Geo *geo, uint32_t *tiles, uint32_t *depth_key, const Ctl *ctl,
+                              cudaStream_t st);
 // Also adds the per-Gaussian blend-weight sums (record-gradient slot 9) to
 // contrib_sum when it is not null.
 // vis_index: the visible list of the last render (index order, ctl->n_vis
@@ -248,26 +255,25 @@ cudaError_t launch_prune(const float *contrib_max, int n, float thr, uint8_t *ke
 
 // Scratch of the compositor kernels (all in the render workspace).
 struct CompositeBufs {
-    uint32_t *order;      // [Tn] forward tile order (heaviest first)
+    uint4 *order;         // [Tn] forward tile order, heaviest first: (tile, list start, length, first segment)
     uint32_t *qdone;      // [8 Tn] per 8x8 block, a 64-bit word where its two forward blocks meet (FwdJob::qdone)
     uint32_t *seg_base;   // [Tn] first checkpoint segment of each tile
     uint32_t *qwork;      // [4 Tn] longest blended prefix of each 8x8 block (stored by the forward)
     float4 *ckpt;         // [segments][256] per-pixel (T, colour sum) every kSeg positions
     uint2 *items;         // backward work items (tile, block << 24 | segment), written by the forward
     uint32_t *n_items;
-    uint32_t *queue;      // work-queue counter (forward and backward reuse it in turn)
+    uint32_t *queue;      // work-queue counter (forward and backward reuse it in turn), then the live tiles
 };
 // One view for the forward compositor.  A batch of views is composited by
 // one persistent launch whose work queue spans all their tiles.
 constexpr int kMaxBatch = GS_MAX_BATCH;
 struct FwdJob {
-    const uint32_t *order;
-    const uint2 *ranges;
+    const uint4 *order;
     const uint32_t *list;
+    const Geo *geo;
     const Rec *rec;
     float *image, *alpha, *t_final;
     uint32_t *n_contrib;
-    const uint32_t *seg_base;
     float4 *ckpt;
     uint32_t *qwork;
     unsigned long long *n_blended;   // the view's status word: blended pairs
@@ -276,21 +282,18 @@ struct FwdJob {
     uint32_t n_segs;                 // checkpoint segments the workspace holds
     int W, H, Tx, Tn;
     float3 bg;
-    uint32_t *queue;       // the view's work-queue counter (zeroed by its set-up)
+    uint32_t *queue;       // the view's work-queue word (written by its set-up)
     uint2 *items;          // the view's backward work items, appended as the forward finishes 8x8 blocks
     uint32_t *n_items;     // their count (zero at the start of the render)
-    uint32_t *qdone;       // [8 Tn] per 8x8 block, (finished 8x4 blocks << 32 | longest prefix) as 64 bits (zeroed by the set-up)
+    uint32_t *qdone;       // [8 Tn] per 8x8 block, a half per 8x4 block: 0 or its longest prefix + 1 (zeroed by the set-up)
 };
 // Per-view set-up before compositing: tile order, checkpoint bases, zeroed
 // block work and queue.  The backward's set-up also zeroes the record-gradient
 // rows of the visible Gaussians (vis_index, *n_vis of the n Gaussians).
 cudaError_t launch_fwd_setup(const CompositeBufs &cb, const uint2 *ranges, int Tn, cudaStream_t st);
 // Composites n <= kMaxBatch views with one persistent launch; every view's
-// queue must have been zeroed on the stream (its launch_fwd_setup does).
-// wide_ok: the launch may take a third CTA per SM when it covers many pixels
-// (gs_render, gs_render_stereo); batched serving launches, which share the GPU
-// with a companion stream, keep two.
-cudaError_t launch_composite_forward(const FwdJob *jobs, int n, cudaStream_t st, bool wide_ok);
+// queue must have been written on the stream (its launch_fwd_setup does).
+cudaError_t launch_composite_forward(const FwdJob *jobs, int n, cudaStream_t st);
 // Backward set-up: work items (tile order by longest blended prefix) and the
 // zeroed record-gradient rows of the visible Gaussians.
 cudaError_t launch_bwd_setup(const CompositeBufs &cb, int Tx, int Ty, float4 *rec_grad, const uint32_t *vis_index,

@@ -70,9 +70,16 @@ __device__ __forceinline__ void sh_basis(float x, float y, float z, float *b) {
     b[15] = (-C3A * x) * (xx - 3.0f * yy);
 }
 
+__device__ __forceinline__ void store_geo(Geo *g, const float4 a, const float4 b) {
+    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(g), "f"(a.x), "f"(a.y), "f"(a.z),
+                 "f"(a.w), "f"(b.x), "f"(b.y), "f"(b.z), "f"(b.w)
+                 : "memory");
+}
+
 template <int DEG>
 __global__ void __launch_bounds__(128) k_preprocess(SceneView s, CamView c, uint32_t layer_mask, Planes pl,
-                                                    Rec *__restrict__ rec, uint32_t *__restrict__ tiles,
+                                                    Rec *__restrict__ rec, Geo *__restrict__ geo,
+                                                    uint32_t *__restrict__ tiles,
                                                     uint32_t *__restrict__ depth_key, const Ctl *__restrict__ ctl) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= s.n) return;
@@ -230,6 +237,7 @@ __global__ void __launch_bounds__(128) k_preprocess(SceneView s, CamView c, uint
                 o.c = make_float4(rgb[2], pz, __uint_as_float(static_cast<uint32_t>(x0) | (static_cast<uint32_t>(y0) << 16)),
                                   __uint_as_float(static_cast<uint32_t>(x1) | (static_cast<uint32_t>(y1) << 16)));
                 rec[i] = o;
+                store_geo(geo + i, o.a, o.b);
                 dkey = __float_as_uint(pz);
             }
         }
@@ -241,14 +249,14 @@ __global__ void __launch_bounds__(128) k_preprocess(SceneView s, CamView c, uint
 }  // namespace
 
 cudaError_t launch_preprocess(const SceneView &s, const CamView &c, uint32_t layer_mask, const Planes &pl, Rec *rec,
-                              uint32_t *tiles, uint32_t *depth_key, const Ctl *ctl, cudaStream_t st) {
+                              Geo *geo, uint32_t *tiles, uint32_t *depth_key, const Ctl *ctl, cudaStream_t st) {
     if (s.n == 0) return cudaSuccess;
     const int threads = 128, blocks = (s.n + threads - 1) / threads;
     switch (s.sh_degree) {
-        case 0: k_preprocess<0><<<blocks, threads, 0, st>>>(s, c, layer_mask, pl, rec, tiles, depth_key, ctl); break;
-        case 1: k_preprocess<1><<<blocks, threads, 0, st>>>(s, c, layer_mask, pl, rec, tiles, depth_key, ctl); break;
-        case 2: k_preprocess<2><<<blocks, threads, 0, st>>>(s, c, layer_mask, pl, rec, tiles, depth_key, ctl); break;
-        default: k_preprocess<3><<<blocks, threads, 0, st>>>(s, c, layer_mask, pl, rec, tiles, depth_key, ctl); break;
+        case 0: k_preprocess<0><<<blocks, threads, 0, st>>>(s, c, layer_mask, pl, rec, geo, tiles, depth_key, ctl); break;
+        case 1: k_preprocess<1><<<blocks, threads, 0, st>>>(s, c, layer_mask, pl, rec, geo, tiles, depth_key, ctl); break;
+        case 2: k_preprocess<2><<<blocks, threads, 0, st>>>(s, c, layer_mask, pl, rec, geo, tiles, depth_key, ctl); break;
+        default: k_preprocess<3><<<blocks, threads, 0, st>>>(s, c, layer_mask, pl, rec, geo, tiles, depth_key, ctl); break;
     }
     return cudaGetLastError();
 }

@@ -5,9 +5,13 @@
 // 3(K-1) coefficients.  The preprocess gathers those rows from L2 instead of
 // reading 3(K-1) floats per Gaussian from HBM.
 //
-// Assignment is brute force: a thread per point holds its (zero-padded)
-// coordinates in registers and scans the centroids staged in shared memory
-// 64 at a time with 16-byte broadcast loads.  Ties go to the lower index.
+// Assignment: the centroid with the least single-precision distance
+// sum_d (x_d - c_d)^2 (d in order, fused multiply-adds), ties to the lower
+// index.  Small calls scan brute force: a thread per point holds its
+// (zero-padded) coordinates in registers and scans the centroids staged in
+// shared memory 64 at a time with 16-byte broadcast loads.  Larger ones rule
+// out nearly all centroids on the tensor cores first (k_kmeans_assign_tc).
+#include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
 #include "gs_internal.cuh"
@@ -18,11 +22,11 @@ namespace {
 constexpr int kKmTile = 64;                  // centroids per shared-memory tile
 constexpr int kKmThreads = 128;
 
-__global__ void __launch_bounds__(kKmThreads) k_kmeans_assign(const float *__restrict__ pts, int64_t n, int dim,
-                                                              int64_t stride, const float *__restrict__ cent, int k,
-                                                              uint32_t *__restrict__ assign) {
-    __shared__ float4 s_c[kKmTile][kCbMaxDim / 4];
-    const int64_t i = static_cast<int64_t>(blockIdx.x) * kKmThreads + threadIdx.x;
+// The brute-force scan of point i by one thread of a CTA of NT (i >= n: none).
+template <int NT>
+__device__ __forceinline__ uint32_t scan_all(const float *__restrict__ pts, int64_t i, int64_t n, int dim,
+                                             int64_t stride, const float *__restrict__ cent, int k,
+                                             float4 (*s_c)[kCbMaxDim / 4]) {
     float x[kCbMaxDim];
 #pragma unroll
     for (int d = 0; d < kCbMaxDim; ++d) x[d] = (i < n && d < dim) ? pts[i * stride + d] : 0.f;
@@ -30,7 +34,7 @@ __global__ void __launch_bounds__(kKmThreads) k_kmeans_assign(const float *__res
     uint32_t arg = 0;
     for (int t0 = 0; t0 < k; t0 += kKmTile) {
         __syncthreads();
-        for (int e = threadIdx.x; e < kKmTile * kCbMaxDim; e += kKmThreads) {
+        for (int e = threadIdx.x; e < kKmTile * kCbMaxDim; e += NT) {
             const int j = e / kCbMaxDim, d = e % kCbMaxDim;
             reinterpret_cast<float *>(&s_c[j][0])[d] = (t0 + j < k && d < dim) ? cent[(t0 + j) * dim + d] : 0.f;
         }
@@ -53,6 +57,527 @@ __global__ void __launch_bounds__(kKmThreads) k_kmeans_assign(const float *__res
             }
         }
     }
+    return arg;
+}
+
+__global__ void __launch_bounds__(kKmThreads) k_kmeans_assign(const float *__restrict__ pts, int64_t n, int dim,
+                                                              int64_t stride, const float *__restrict__ cent, int k,
+                                                              uint32_t *__restrict__ assign) {
+    __shared__ float4 s_c[kKmTile][kCbMaxDim / 4];
+    const int64_t i = static_cast<int64_t>(blockIdx.x) * kKmThreads + threadIdx.x;
+    const uint32_t arg = scan_all<kKmThreads>(pts, i, n, dim, stride, cent, k, s_c);
+    if (i < n) assign[i] = arg;
+}
+
+// ---- assignment on the tensor cores ----
+//
+// argmin_c |x - c|^2 = argmax_c s(c), s(c) = x.c - |c|^2 / 2: a contraction of
+// the points with the centroids.  The kernel computes s in bf16 products with
+// FP32 accumulation (tcgen05), bounds its error, and evaluates the exact
+// single-precision distance only for the centroids that the bounds leave, so
+// the result is that of the brute-force scan, bit for bit:
+//
+//  * |s~(c) - s(c)| <= E = |x||c| (2^-8 + 2^-18 + 2^-16) + |c|^2 2^-16: both
+//    factors of a product are rounded to 8 bits (relative 2^-9 each;
+//    Cauchy-Schwarz over the coordinates), -|c|^2/2 enters as three bf16
+//    parts, and each of at most 64 accumulations errs by at most 2^-22 of the
+//    magnitudes added.  kEProd, kENorm round these up; kETiny covers underflow.
+//  * The scan's rounded distances err by at most (dim + 3) 2^-24 relative, so
+//    its winner has s within 2^-18 (|x| + |c|)^2 of the best; kESlack rounds up.
+//  * Per point, LB = max over groups of 32 centroids of (largest s~ - E) is a lower
+//    bound of the best s.  A centroid whose s~ + E + slack stays below LB cannot be
+//    the winner.  The others are remembered (with U, that sum for the group's
+//    largest; kCand at most, dropped again when LB has passed them).
+//  * Points whose candidates overflow, and points and centroids that are not
+//    finite or above kHuge, are scanned in full.
+//
+// A CTA takes 256 points (two 128-row A tiles, bf16, resident) and walks the
+// centroids in tiles of 128: four warps copy a tile's rows (cp.async) and convert
+// them to bf16 in the 128-byte swizzled K-major layout, one thread issues the
+// MMAs (M = N = 128, K = dim + 3 rounded up to 16) into one of two accumulator
+// sets in tensor memory, and eight warps read the other set back, one point per
+// thread.  Everything is staged by the CTA itself, as the entry point has no
+// workspace to hold converted centroids.
+//
+// Bound by instruction issue: reading the accumulators back and the conversions
+// (the tensor pipe is 15% busy; K is only 48).  Measured, points x centroids of 45
+// coordinates: 200,000 x 16,384 13.0 -> 0.79 ms, 200,000 x 4,096 3.26 -> 0.32,
+// 1,200,000 x 16,384 71.9 -> 4.2, 20,000 x 256 0.060 -> 0.027; 20,000 x 16,384 of 9
+// coordinates 3.3 -> 0.13.  Found on the way: candidate groups scanned whole by a warp per
+// point (1.1 ms: a kilobyte-sized gather per point), one converter set (1.2 ms),
+// candidates told apart by 32 predicates (1.0 ms, the sign bits 0.79).
+constexpr int kTcPoints = 256, kTcTile = 128, kTcRow = 128;      // points per CTA, centroids per tile, bytes per row
+constexpr int kTcEpiWarps = 8, kTcCvtWarps = 4, kTcCvtSets = 2;
+constexpr int kTcMmaWarp = kTcEpiWarps + kTcCvtSets * kTcCvtWarps;
+constexpr int kTcThreads = 32 * (kTcMmaWarp + 1);
+constexpr int kCand = 16;              // candidate groups remembered per point
+constexpr int kCmRing = 8;             // tiles whose largest norms are kept
+constexpr float kEProd = 1.05f * 0x1p-8f, kENorm = 0x1p-15f, kESlack = 0x1p-17f, kETiny = 1e-30f, kHuge = 1e14f;
+constexpr uint32_t kTcWaitLimit = 1u << 22;
+constexpr uint32_t kUnassigned = 0xFFFFFFFFu;
+// Calls from this size on go through the tensor cores (20,000 points: 128 centroids
+// 0.025 ms against 0.033 for the scan, 64 centroids 0.019 with the scan; 1,024 points
+// x 128 centroids 0.023 against 0.029).
+constexpr int kTcMinCentroids = 128;
+constexpr int64_t kTcMinPoints = 1024;
+
+__device__ __forceinline__ uint32_t smem_u32(const void *p) {
+    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
+}
+
+// The scan's distance, accumulated in the order of the coordinates.
+__device__ __forceinline__ float sq_step(float x, float c, float acc) {
+    const float a = __fsub_rn(x, c);
+    return __fmaf_rn(a, a, acc);
+}
+
+// A point and the rows of a group of 32 centroids in shared memory, by cp.async.
+struct __align__(16) PairBuf {
+    float rows[32 * kCbMaxDim];
+    float x[kCbMaxDim];
+    uint32_t g;
+
+    // vec: cent is 16-byte aligned (so is every group: 32 rows are a multiple of 128 bytes).
+    __device__ __forceinline__ void fetch(const float *__restrict__ cent, int k, int dim, uint32_t group,
+                                          const float *__restrict__ pt, bool vec, int lane) {
+        const int vals = min(32, k - static_cast<int>(32u * group)) * dim;
+        const float *src = cent + static_cast<size_t>(32u * group) * dim;
+        const uint32_t dst = smem_u32(rows);
+        const int units = vec ? vals / 4 : 0;
+#pragma unroll
+        for (int j = 0; j < 32 * kCbMaxDim / 128; ++j) {
+            const int u = lane + 32 * j;
+            if (u < units)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 16 * u), "l"(src + 4 * u)
+                             : "memory");
+        }
+        for (int v = 4 * units + lane; v < vals; v += 32)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst + 4 * v), "l"(src + v) : "memory");
+        for (int d = lane; d < dim; d += 32)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(x + d)), "l"(pt + d) : "memory");
+        if (lane == 0) g = group;
+    }
+    // The least distance of the point to the group, a centroid per lane; keeps (best, arg) the scan's winner so far
+    // when groups come in ascending order.
+    __device__ __forceinline__ void least(int k, int dim, int lane, float &best, uint32_t &arg) const {
+        const bool row = static_cast<int>(32u * g) + lane < k;
+        const float *c = rows + (row ? lane : 0) * dim;
+        float acc = 0.f;
+#pragma unroll
+        for (int d = 0; d < kCbMaxDim; ++d)
+            if (d < dim) acc = sq_step(x[d], c[d], acc);
+        const bool in = row && acc < best;
+        const uint32_t bits = in ? __float_as_uint(acc) : 0xFFFFFFFFu;       // distances are not negative
+        const uint32_t low = __reduce_min_sync(0xFFFFFFFFu, bits);
+        if (low != 0xFFFFFFFFu) {
+            best = __uint_as_float(low);
+            arg = 32u * g + static_cast<uint32_t>(__ffs(__ballot_sync(0xFFFFFFFFu, bits == low)) - 1);
+        }
+    }
+};
+
+struct TcOperands {
+    unsigned char a[2][128 * kTcRow];              // points, bf16 (1024-byte aligned)
+    unsigned char b[2][kTcTile * kTcRow];          // centroid tiles, bf16
+    float rows[2][kTcTile * kCbMaxDim];            // centroid rows as they are in memory
+};
+struct TcSmem {
+    TcOperands op;
+    float2 cand[kCand][kTcPoints];                 // (U, group of 32 centroids)
+    uint32_t mask[kCand][kTcPoints];               // the group's centroids that can still win
+    float4 cm[kCmRing];                            // largest |c| of a tile, per converting warp
+    unsigned long long row_full[kTcCvtSets], b_full[2], b_empty[2], acc_full[2], acc_empty[2];
+    uint32_t tmem;
+    int failed;
+};
+
+__device__ __forceinline__ void mbar_init(void *bar, uint32_t count) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(void *bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+// Waits for the phase of the given parity; false when the limit runs out (or another role gave up).
+__device__ __forceinline__ bool mbar_wait(void *bar, uint32_t parity, volatile int *failed) {
+    const uint32_t addr = smem_u32(bar);
+    for (uint32_t it = 0; it < kTcWaitLimit; ++it) {
+        uint32_t ok;
+        asm volatile(
+            "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+            : "=r"(ok)
+            : "r"(addr), "r"(parity)
+            : "memory");
+        if (ok) return true;
+        if ((it & 255u) == 255u && *failed) return false;
+    }
+    *failed = 1;
+    return false;
+}
+
+// Shared-memory matrix descriptor: K-major rows of 128 bytes, 128-byte swizzle, 8-row groups 1024 bytes apart.
+__device__ __forceinline__ uint64_t umma_desc(uint32_t addr) {
+    return static_cast<uint64_t>((addr & 0x3FFFFu) >> 4) | (1ull << 16) | (64ull << 32) | (1ull << 46) | (2ull << 61);
+}
+// kind::f16: D f32, A and B bf16, both K-major, M = N = 128.
+constexpr uint32_t kUmmaInstr = (1u << 4) | (1u << 7) | (1u << 10) | ((kTcTile / 8u) << 17) | ((128u / 16u) << 24);
+
+__device__ __forceinline__ void umma_bf16(uint32_t d, uint64_t a, uint64_t b, uint32_t accumulate) {
+    asm volatile(
+        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d),
+        "l"(a), "l"(b), "r"(kUmmaInstr), "r"(accumulate)
+        : "memory");
+}
+__device__ __forceinline__ void umma_commit(void *bar) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
+                 : "memory");
+}
+// 32 consecutive accumulator columns of the warp's 32 rows, a row per lane; v is valid after tmem_wait(v), which also
+// waits for every other load of the warp.
+__device__ __forceinline__ void tmem_ld32(uint32_t addr, float (&v)[32]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {"
+        "%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31"
+        "}, [%32];"
+        : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]),
+          "=f"(v[8]), "=f"(v[9]), "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]), "=f"(v[15]),
+          "=f"(v[16]), "=f"(v[17]), "=f"(v[18]), "=f"(v[19]), "=f"(v[20]), "=f"(v[21]), "=f"(v[22]), "=f"(v[23]),
+          "=f"(v[24]), "=f"(v[25]), "=f"(v[26]), "=f"(v[27]), "=f"(v[28]), "=f"(v[29]), "=f"(v[30]), "=f"(v[31])
+        : "r"(addr)
+        : "memory");
+}
+__device__ __forceinline__ void tmem_wait(float (&v)[32]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+        : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7]),
+          "+f"(v[8]), "+f"(v[9]), "+f"(v[10]), "+f"(v[11]), "+f"(v[12]), "+f"(v[13]), "+f"(v[14]), "+f"(v[15]),
+          "+f"(v[16]), "+f"(v[17]), "+f"(v[18]), "+f"(v[19]), "+f"(v[20]), "+f"(v[21]), "+f"(v[22]), "+f"(v[23]),
+          "+f"(v[24]), "+f"(v[25]), "+f"(v[26]), "+f"(v[27]), "+f"(v[28]), "+f"(v[29]), "+f"(v[30]), "+f"(v[31])
+        :
+        : "memory");
+}
+
+__device__ __forceinline__ float max3(float a, float b, float c) {
+    float m;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(m) : "f"(a), "f"(b), "f"(c));
+    return m;
+}
+
+// Byte offset of 16-byte unit u of row r in the 128-byte swizzled layout.
+__device__ __forceinline__ uint32_t swz(uint32_t r, uint32_t u) { return r * kTcRow + ((u ^ (r & 7u)) << 4); }
+
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
+    const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+    return *reinterpret_cast<const uint32_t *>(&v);
+}
+
+// DIM: the coordinates where known at compile time (SH degrees 1 to 3), 0 otherwise.
+template <int DIM>
+__global__ void __launch_bounds__(kTcThreads) k_kmeans_assign_tc(const float *__restrict__ pts, int64_t n, int dim_,
+                                                                 int64_t stride, const float *__restrict__ cent, int k,
+                                                                 uint32_t *__restrict__ assign) {
+    const int dim = DIM ? DIM : dim_;
+    extern __shared__ unsigned char s_raw[];
+    TcSmem &sm = *reinterpret_cast<TcSmem *>((reinterpret_cast<uintptr_t>(s_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t i0 = static_cast<int64_t>(blockIdx.x) * kTcPoints;
+    const int ntile = (k + kTcTile - 1) / kTcTile;
+    const int ksteps = (dim + 3 + 15) / 16;
+    volatile int *failed = &sm.failed;
+    if (threadIdx.x == 0) {
+        sm.failed = 0;
+        for (int q = 0; q < 2; ++q) {
+            mbar_init(&sm.b_full[q], 32 * kTcCvtWarps);
+            mbar_init(&sm.b_empty[q], 1);
+            mbar_init(&sm.row_full[q], 1);
+            mbar_init(&sm.acc_full[q], 1);
+            mbar_init(&sm.acc_empty[q], 32 * kTcEpiWarps);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == kTcMmaWarp) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&sm.tmem))
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    // the points: bf16 rows (x, 1, 1, 1, 0 ...), 32 rows per warp, two coordinates per lane
+    float nx = 0.f;                                            // |x| of point `threadIdx.x` (rounded up)
+    if (warp < kTcEpiWarps) {
+        constexpr int R = 8;                                   // rows whose loads are in flight together
+        for (int r0 = 0; r0 < 32; r0 += R) {
+            float2 x[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const int64_t i = i0 + 32 * warp + r0 + r;
+                x[r] = make_float2(i < n && lane < dim ? pts[i * stride + lane] : 0.f,
+                                   i < n && lane + 32 < dim ? pts[i * stride + lane + 32] : 0.f);
+            }
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                float sq = x[r].x * x[r].x + x[r].y * x[r].y;
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xFFFFFFFFu, sq, o);
+                if (lane == r0 + r) nx = sqrtf(sq) * 1.0001f;
+                const int row = 32 * warp + r0 + r;
+                unsigned char *t = sm.op.a[row >> 7];
+                const uint32_t rr = row & 127;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int d = lane + 32 * h;
+                    const float v = d < dim ? (h ? x[r].y : x[r].x) : (d < dim + 3 ? 1.f : 0.f);
+                    *reinterpret_cast<__nv_bfloat16 *>(t + swz(rr, d >> 3) + 2 * (d & 7)) = __float2bfloat16_rn(v);
+                }
+            }
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = sm.tmem;
+
+    int cnt = 0;                                               // epilogue: candidates of this thread's point
+    float LB = -3.0e38f;
+    bool full = false;
+    if (warp < kTcEpiWarps) {
+        full = !(nx < kHuge);
+        float cmax = 0.f;
+        const int tid = threadIdx.x;
+        const uint32_t row = tmem + (static_cast<uint32_t>(32 * (warp & 3)) << 16) + (warp >= 4 ? kTcTile : 0);
+        for (int t = 0; t < ntile; ++t) {
+            const int q = t & 1;
+            if (!__all_sync(0xFFFFFFFFu, mbar_wait(&sm.acc_full[q], (t >> 1) & 1, failed))) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const float4 c4 = sm.cm[t & (kCmRing - 1)];
+            const float cm = fmaxf(fmaxf(c4.x, c4.y), fmaxf(c4.z, c4.w));
+            const bool sane = cm < kHuge;                      // (a NaN norm is reported as infinite)
+            if (sane) cmax = fmaxf(cmax, cm);
+            const float E = nx * cm * kEProd + cm * cm * kENorm + kETiny;
+            const float both = nx + cmax;
+            const float up = E + both * both * kESlack;
+            float v[2][32];                                    // the next group's columns load while one is searched
+            tmem_ld32(row + q * 2 * kTcTile, v[0]);
+#pragma unroll
+            for (int g = 0; g < kTcTile / 32; ++g) {
+                float (&w)[32] = v[g & 1];
+                tmem_wait(w);
+                if (g + 1 < kTcTile / 32) tmem_ld32(row + q * 2 * kTcTile + 32 * (g + 1), v[(g + 1) & 1]);
+                do {
+                    float m3[10];
+#pragma unroll
+                    for (int e = 0; e < 10; ++e) m3[e] = max3(w[3 * e], w[3 * e + 1], w[3 * e + 2]);
+                    const float m = max3(max3(m3[0], m3[1], m3[2]), max3(m3[3], m3[4], m3[5]),
+                                         max3(max3(m3[6], m3[7], m3[8]), m3[9], fmaxf(w[30], w[31])));
+                    const int grp = t * (kTcTile / 32) + g;
+                    if (32 * grp >= k) break;
+                    if (sane) LB = fmaxf(LB, m - E);
+                    const float U = sane ? m + up : INFINITY;
+                    if (U >= LB && !full) {
+                        // the group's centroids that can still win: the sign bits of s~ - (LB - up)
+                        const float least = LB - up;
+                        uint32_t below = 0;
+#pragma unroll
+                        for (int e = 31; e >= 0; --e)
+                            below = __funnelshift_l(__float_as_uint(w[e] - least), below, 1);
+                        if (cnt == kCand) {                    // drop what LB has passed
+                            int kept = 0;
+                            for (int e = 0; e < kCand; ++e) {
+                                const float2 z = sm.cand[e][tid];
+                                if (z.x >= LB) {
+                                    sm.cand[kept][tid] = z;
+                                    sm.mask[kept++][tid] = sm.mask[e][tid];
+                                }
+                            }
+                            cnt = kept;
+                        }
+                        if (cnt < kCand) {
+                            sm.cand[cnt][tid] = make_float2(U, __int_as_float(grp));
+                            sm.mask[cnt++][tid] = sane ? ~below : 0xFFFFFFFFu;
+                        } else {
+                            full = true;
+                        }
+                    }
+                } while (false);
+                __syncwarp();
+            }
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            mbar_arrive(&sm.acc_empty[q]);
+        }
+    } else if (warp < kTcMmaWarp) {
+        // converters, two sets of four warps taking the tiles in turn: thread r of a set owns centroid row r
+        const int set = (warp - kTcEpiWarps) / kTcCvtWarps, cw = (warp - kTcEpiWarps) % kTcCvtWarps;
+        const int r = 32 * cw + lane;
+        float *const mem = sm.op.rows[set];
+        const bool vec = (reinterpret_cast<uintptr_t>(cent) & 15u) == 0;
+        const auto set_sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1 + set), "n"(32 * kTcCvtWarps) : "memory"); };
+        // A tile's rows, one bulk copy of whole 16-byte units (a last tile's odd values by plain loads); centroids
+        // that do not start on 16 bytes value by value.
+        const auto fetch = [&](int t) {
+            if (t >= ntile) return;
+            const int vals = min(kTcTile, k - t * kTcTile) * dim;
+            const float *src = cent + static_cast<size_t>(t) * kTcTile * dim;
+            const int bulk = vec ? vals & ~3 : 0;
+            if (vec && r == 0) {
+                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(&sm.row_full[set])),
+                             "r"(4 * bulk)
+                             : "memory");
+                asm volatile(
+                    "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                        smem_u32(mem)),
+                    "l"(src), "r"(4 * bulk), "r"(smem_u32(&sm.row_full[set]))
+                    : "memory");
+            }
+            for (int e = bulk + r; e < vals; e += 32 * kTcCvtWarps) mem[e] = src[e];
+        };
+        fetch(set);
+        for (int t = set; t < ntile; t += kTcCvtSets) {
+            const int q = t & 1;
+            // (a wait that gives up is noted in `failed`: the CTA's points are then scanned in full)
+            if (vec) mbar_wait(&sm.row_full[set], (t / kTcCvtSets) & 1, failed);
+            set_sync();                                        // the tile's rows have landed
+            const bool in = t * kTcTile + r < k;
+            const float *src = mem + r * dim;
+            float sq = 0.f;
+            uint32_t w[32];                                    // the row's 64 bf16
+#pragma unroll
+            for (int d = 0; d < kCbMaxDim; d += 2) {
+                const float a = in && d < dim ? src[d] : 0.f, b = in && d + 1 < dim ? src[d + 1] : 0.f;
+                sq = fmaf(a, a, sq);
+                sq = fmaf(b, b, sq);
+                w[d / 2] = pack_bf16(a, b);
+            }
+#pragma unroll
+            for (int d = kCbMaxDim / 2; d < 32; ++d) w[d] = 0u;
+            set_sync();                                        // and have been read: the set's next tile
+            fetch(t + kTcCvtSets);
+            if (t >= 2) mbar_wait(&sm.b_empty[q], ((t >> 1) - 1) & 1, failed);
+            // -|c|^2 / 2 in three parts at dim .. dim + 2; a row past the end scores far below any other
+            const float h = in ? 0.5f * sq : 1e30f;
+            float part[3];
+            part[0] = __bfloat162float(__float2bfloat16_rn(h));
+            part[1] = __bfloat162float(__float2bfloat16_rn(h - part[0]));
+            part[2] = h - part[0] - part[1];
+            unsigned char *row = sm.op.b[q];
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                *reinterpret_cast<uint4 *>(row + swz(r, u)) =
+                    make_uint4(w[4 * u], w[4 * u + 1], w[4 * u + 2], w[4 * u + 3]);
+#pragma unroll
+            for (int z = 0; z < 3; ++z)
+                *reinterpret_cast<__nv_bfloat16 *>(row + swz(r, (dim + z) >> 3) + 2 * ((dim + z) & 7)) =
+                    __float2bfloat16_rn(-part[z]);
+            // the tile's largest norm; one that is not a number or too large makes its groups candidates
+            float nc = sqrtf(sq) * 1.0001f;
+            if (!(nc < kHuge)) nc = INFINITY;
+            const float wm = __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, __float_as_uint(nc)));
+            if (lane == 0) reinterpret_cast<float *>(&sm.cm[t & (kCmRing - 1)])[cw] = wm;
+            __syncwarp();
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            mbar_arrive(&sm.b_full[q]);
+        }
+    } else if (lane == 0) {
+        const uint64_t da[2] = {umma_desc(smem_u32(sm.op.a[0])), umma_desc(smem_u32(sm.op.a[1]))};
+        const uint64_t db[2] = {umma_desc(smem_u32(sm.op.b[0])), umma_desc(smem_u32(sm.op.b[1]))};
+        for (int t = 0; t < ntile; ++t) {
+            const int q = t & 1;
+            if (!mbar_wait(&sm.b_full[q], (t >> 1) & 1, failed)) break;
+            if (t >= 2 && !mbar_wait(&sm.acc_empty[q], ((t >> 1) - 1) & 1, failed)) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+            for (int m = 0; m < 2; ++m)
+                for (int s = 0; s < ksteps; ++s)
+                    umma_bf16(tmem + q * 2 * kTcTile + m * kTcTile, da[m] + 2 * s, db[q] + 2 * s, s > 0);
+            umma_commit(&sm.b_empty[q]);
+            umma_commit(&sm.acc_full[q]);
+        }
+        // the last MMAs have completed before the tensor memory is freed
+        for (int t = max(0, ntile - 2); t < ntile; ++t) mbar_wait(&sm.acc_full[t & 1], (t >> 1) & 1, failed);
+    }
+    __syncwarp();
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (warp == kTcMmaWarp) {
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
+        return;
+    }
+    if (warp >= kTcEpiWarps) return;
+    // exact distances of the centroids that are left, a point per thread
+    const int64_t i = i0 + threadIdx.x;
+    if (i >= n) return;
+    uint32_t arg = kUnassigned;                                // (scanned in full by the next launch)
+    if (!full && !*failed) {
+        const float *pt = pts + i * stride;
+        float x[kCbMaxDim];
+#pragma unroll
+        for (int d = 0; d < kCbMaxDim; ++d) x[d] = d < dim ? pt[d] : 0.f;
+        float best = 3.0e38f;
+        arg = 0;
+        for (int e = 0; e < cnt; ++e) {                        // ascending
+            const float2 z = sm.cand[e][threadIdx.x];
+            if (!(z.x >= LB)) continue;
+            const uint32_t j0 = 32u * static_cast<uint32_t>(__float_as_int(z.y));
+            for (uint32_t mask = sm.mask[e][threadIdx.x]; mask; mask &= mask - 1) {
+                const uint32_t j = j0 + static_cast<uint32_t>(__ffs(mask) - 1);
+                if (j >= static_cast<uint32_t>(k)) break;
+                const float *c = cent + static_cast<size_t>(j) * dim;
+                float y[kCbMaxDim];
+#pragma unroll
+                for (int d = 0; d < kCbMaxDim; ++d) y[d] = d < dim ? c[d] : 0.f;
+                float acc = 0.f;
+#pragma unroll
+                for (int d = 0; d < kCbMaxDim; ++d) acc = sq_step(x[d], y[d], acc);
+                if (acc < best) {
+                    best = acc;
+                    arg = j;
+                }
+            }
+        }
+    }
+    assign[i] = arg;
+}
+
+// The points that k_kmeans_assign_tc left (kUnassigned), in full: a CTA per kLeftPoints points collects those left
+// among them.  A few are scanned a warp per point, many a thread per point.
+constexpr int kLeftPoints = 128;
+
+__global__ void __launch_bounds__(kLeftPoints) k_kmeans_assign_left(const float *__restrict__ pts, int64_t n, int dim,
+                                                                    int64_t stride, const float *__restrict__ cent,
+                                                                    int k, uint32_t *__restrict__ assign) {
+    __shared__ __align__(16) union {
+        float4 c[kKmTile][kCbMaxDim / 4];
+        PairBuf pair[kLeftPoints / 32];
+    } s;
+    __shared__ int s_left[kLeftPoints];
+    __shared__ int s_n;
+    const int64_t i0 = static_cast<int64_t>(blockIdx.x) * kLeftPoints;
+    const bool left = i0 + threadIdx.x < n && assign[i0 + threadIdx.x] == kUnassigned;
+    if (!__syncthreads_or(left)) return;
+    if (threadIdx.x == 0) s_n = 0;
+    __syncthreads();
+    if (left) s_left[atomicAdd(&s_n, 1)] = threadIdx.x;
+    __syncthreads();
+    const int m = s_n;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const bool vec = (reinterpret_cast<uintptr_t>(cent) & 15u) == 0;
+    if (m <= kLeftPoints / 8) {
+        for (int p = warp; p < m; p += kLeftPoints / 32) {
+            const int64_t i = i0 + s_left[p];
+            float best = 3.0e38f;
+            uint32_t arg = 0;
+            for (int g = 0; 32 * g < k; ++g) {
+                s.pair[warp].fetch(cent, k, dim, g, pts + i * stride, vec, lane);
+                asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
+                __syncwarp();
+                s.pair[warp].least(k, dim, lane, best, arg);
+                __syncwarp();
+            }
+            if (lane == 0) assign[i] = arg;
+        }
+        return;
+    }
+    const int64_t i = static_cast<int>(threadIdx.x) < m ? i0 + s_left[threadIdx.x] : n;
+    const uint32_t arg = scan_all<kLeftPoints>(pts, i, n, dim, stride, cent, k, s.c);
     if (i < n) assign[i] = arg;
 }
 
@@ -96,9 +621,34 @@ __global__ void __launch_bounds__(256) k_sh_encode(const float *__restrict__ sh,
 
 }  // namespace
 
+template <int DIM>
+cudaError_t launch_assign_tc(const float *pts, int64_t n, int dim, int64_t stride, const float *cent, int k,
+                             uint32_t *assign, cudaStream_t st) {
+    constexpr size_t smem = sizeof(TcSmem) + 1024;
+    static PerDevice attr;
+    attr.get([] {
+        cudaFuncSetAttribute(k_kmeans_assign_tc<DIM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             static_cast<int>(smem));
+        return 1;
+    });
+    k_kmeans_assign_tc<DIM><<<static_cast<unsigned>((n + kTcPoints - 1) / kTcPoints), kTcThreads, smem, st>>>(
+        pts, n, dim, stride, cent, k, assign);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_kmeans_assign(const float *pts, int64_t n, int dim, int64_t stride, const float *cent, int k,
                                  uint32_t *assign, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
+    if (k >= kTcMinCentroids && n >= kTcMinPoints) {
+        const cudaError_t e = dim == 45   ? launch_assign_tc<45>(pts, n, dim, stride, cent, k, assign, st)
+                              : dim == 24 ? launch_assign_tc<24>(pts, n, dim, stride, cent, k, assign, st)
+                              : dim == 9  ? launch_assign_tc<9>(pts, n, dim, stride, cent, k, assign, st)
+                                          : launch_assign_tc<0>(pts, n, dim, stride, cent, k, assign, st);
+        if (e != cudaSuccess) return e;
+        k_kmeans_assign_left<<<static_cast<unsigned>((n + kLeftPoints - 1) / kLeftPoints), kLeftPoints, 0, st>>>(
+            pts, n, dim, stride, cent, k, assign);
+        return cudaGetLastError();
+    }
     k_kmeans_assign<<<static_cast<unsigned>((n + kKmThreads - 1) / kKmThreads), kKmThreads, 0, st>>>(pts, n, dim, stride,
                                                                                                   cent, k, assign);
     return cudaGetLastError();

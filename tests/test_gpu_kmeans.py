@@ -1,0 +1,91 @@
+"""k-means assignment through the tensor cores (calls of 1,024 points and 128
+centroids on): the same assignment, bit for bit, as the brute-force scan that
+smaller calls take, at ragged counts, all widths of a row, ties, duplicates,
+values that underflow, and values that are not finite."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2410_16978_gb300 import _lib
+
+pytestmark = pytest.mark.gpu
+
+
+def _assign(pts, cent, dim, stride, off, n0, n1):
+    out = torch.full((n1 - n0,), -2, dtype=torch.int32, device="cuda")
+    _lib.gs_kmeans_assign(pts.data_ptr() + 4 * (n0 * stride + off), n1 - n0, dim, stride, cent, cent.shape[0], out,
+                          int(torch.cuda.current_stream().cuda_stream))
+    return out
+
+
+def _check(pts, cent, dim, stride, off):
+    n = pts.shape[0]
+    got = _assign(pts, cent, dim, stride, off, 0, n)
+    want = torch.cat([_assign(pts, cent, dim, stride, off, i, min(n, i + 1000)) for i in range(0, n, 1000)])
+    torch.cuda.synchronize()
+    bad = (got != want).nonzero()
+    assert bad.numel() == 0, (bad.numel(), bad[:5, 0].tolist(), got[bad[:5, 0]].tolist(), want[bad[:5, 0]].tolist())
+
+
+def _data(n, k, dim, stride, off, seed, spread=0.2):
+    g = torch.Generator("cuda").manual_seed(seed)
+    pts = torch.randn((n, stride), generator=g, device="cuda") * spread
+    cent = pts[torch.randperm(n, generator=g, device="cuda")[:k], off:off + dim] * 0.7
+    return pts, cent.contiguous()
+
+
+@pytest.mark.parametrize("n,k,dim,stride,off", [
+    (1024, 128, 45, 48, 3), (1025, 129, 45, 48, 3), (1279, 255, 24, 27, 3), (2048, 257, 9, 12, 3),
+    (5000, 1000, 48, 48, 0), (4097, 160, 46, 51, 2), (3000, 511, 1, 1, 0), (1500, 1313, 31, 33, 1),
+    (30_000, 4096, 45, 48, 3),
+])
+def test_same_as_the_scan(n, k, dim, stride, off):
+    _check(*_data(n, k, dim, stride, off, n + k), dim, stride, off)
+
+
+def test_centroids_not_16_byte_aligned():
+    pts, cent = _data(2000, 301, 45, 48, 3, 5)
+    buf = torch.empty(301 * 45 + 1, device="cuda")
+    moved = buf[1:].view(301, 45)
+    moved.copy_(cent)
+    assert moved.data_ptr() % 16 == 4
+    _check(pts, moved, 45, 48, 3)
+
+
+def test_points_equal_to_centroids_and_duplicates():
+    pts, cent = _data(6000, 900, 45, 48, 3, 6)
+    cent = torch.cat([cent, cent, pts[:300, 3:]]).contiguous()      # every centroid twice, 300 points themselves
+    _check(pts, cent, 45, 48, 3)
+
+
+@pytest.mark.parametrize("case", ["zeros", "constant", "clusters", "tiny", "huge", "nan", "inf", "mixed"])
+def test_values_the_bounds_cannot_separate(case):
+    dim, stride, off = 45, 48, 3
+    pts, cent = _data(3000, 2100, dim, stride, off, 9)
+    if case == "zeros":
+        pts.zero_()
+        cent.zero_()
+    elif case == "constant":
+        pts.fill_(0.3)
+        cent.fill_(0.3)
+    elif case == "clusters":                       # a few centres, many points a last bit apart
+        pts = (pts[:7].repeat(429, 1) * (1 + 1e-7 * torch.randn((3003, 1), device="cuda"))).contiguous()
+        cent = pts[:2100, off:].contiguous()
+    elif case == "tiny":
+        pts *= 1e-22
+        cent *= 1e-22
+    elif case == "huge":
+        pts[::3] *= 1e17
+        cent[::5] *= 1e17
+    elif case == "nan":
+        pts[5, 10] = float("nan")
+        cent[7, 3] = float("nan")
+        cent[2000, 0] = float("nan")
+    elif case == "inf":
+        pts[5, 10] = float("inf")
+        cent[7, 3] = float("inf")
+        cent[1999] = float("-inf")
+    else:
+        pts[::2] = 0
+        cent[:1500] = 0
+    _check(pts, cent, dim, stride, off)

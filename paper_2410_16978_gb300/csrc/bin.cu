@@ -132,8 +132,10 @@ __device__ __forceinline__ void warp_prefix_inplace(uint32_t *a, int n, int lane
     __syncwarp();
 }
 
-// The per-row scan of the row pass splits every row's kBinChunks chunk
-// counts into kRowParts parts, one CTA each.
+// The per-row scan of the row pass splits every row's chunk counts (at most
+// kBinChunks) into kRowParts parts, one CTA each.
+// Gaussians per chunk of the row pass, at least (4,096-Gaussian view 0.019 ms at 32, 0.024 at 128).
+constexpr int kChunkMin = 32;
 constexpr int kRowParts = 2;
 constexpr int kPartChunks = kBinChunks / kRowParts;
 constexpr int kPartPerThread = (kPartChunks + 1023) / 1024;
@@ -153,6 +155,10 @@ struct RowInfo {           // per tile row, in the workspace
     uint32_t pad_[4 - kRowParts];        // (32 bytes in all)
 };
 
+// The per-row info of a view, and behind it the (entries, pairs) totals of every (row, part) of the row scan.
+__device__ __forceinline__ RowInfo *rows_of(const BinView &v) { return static_cast<RowInfo *>(v.rows); }
+__device__ __forceinline__ uint2 *part_totals_of(const BinView &v) { return reinterpret_cast<uint2 *>(rows_of(v) + v.Ty); }
+
 // Chunk c of K of the depth order's n entries.
 __device__ __forceinline__ void chunk_range(uint32_t n, uint32_t c, uint32_t K, uint32_t &b, uint32_t &e) {
     b = static_cast<uint32_t>(static_cast<uint64_t>(n) * c / K);
@@ -160,9 +166,15 @@ __device__ __forceinline__ void chunk_range(uint32_t n, uint32_t c, uint32_t K, 
 }
 
 // Rows, count: a warp per chunk of the depth order counts its entries and pairs per tile row.
-__global__ void __launch_bounds__(256) k_bin_rows_count(const uint32_t *__restrict__ order,
-                                                        const Rec *__restrict__ rec, uint32_t n_cap, int Ty,
-                                                        uint32_t *__restrict__ M, const Ctl *__restrict__ ctl) {
+template <int NV>
+__global__ void __launch_bounds__(256) k_bin_rows_count(const __grid_constant__ Views<BinView, NV> B) {
+    const BinView &V = B[blockIdx.y];
+    const uint32_t *__restrict__ order = V.order;
+    const Rec *__restrict__ rec = V.rec;
+    uint32_t *__restrict__ M = V.M;
+    const Ctl *ctl = V.ctl;
+    const uint32_t n_cap = V.n_cap;
+    const int Ty = V.Ty;
     __shared__ uint32_t s_cnt[8][kBinMaxDim + 1], s_px[8][kBinMaxDim + 1];
     // an error before the binning (a depth sort that timed out) leaves the order unfinished: do not read it
     if (ctl->st.error != GS_OK) return;
@@ -215,11 +227,17 @@ __global__ void __launch_bounds__(256) k_bin_rows_count(const uint32_t *__restri
 constexpr int kRowWords = 4;
 constexpr int kRowBlock = 32 * kRowWords;
 
-__global__ void __launch_bounds__(256) k_bin_rows_write(const uint32_t *__restrict__ order,
-                                                        const Rec *__restrict__ rec, uint32_t n_cap, int Ty,
-                                                        const uint32_t *__restrict__ M,
-                                                        const RowInfo *__restrict__ rows, uint2 *__restrict__ rowlist,
-                                                        const Ctl *__restrict__ ctl) {
+template <int NV>
+__global__ void __launch_bounds__(256) k_bin_rows_write(const __grid_constant__ Views<BinView, NV> B) {
+    const BinView &V = B[blockIdx.y];
+    const uint32_t *__restrict__ order = V.order;
+    const Rec *__restrict__ rec = V.rec;
+    const uint32_t *__restrict__ M = V.M;
+    const RowInfo *__restrict__ rows = rows_of(V);
+    uint2 *__restrict__ rowlist = V.rowlist;
+    const Ctl *ctl = V.ctl;
+    const uint32_t n_cap = V.n_cap;
+    const int Ty = V.Ty;
     __shared__ uint32_t s_pos[8][kBinMaxDim];
     __shared__ uint2 s_val[8][kRowBlock];
     __shared__ uint16_t s_cov[8][kRowBlock];
@@ -315,9 +333,16 @@ __global__ void __launch_bounds__(256) k_bin_rows_write(const uint32_t *__restri
 // (a counter in the control block) then does the per-row work for the whole
 // frame: part bases, row totals, the row, pair and piece starts, the pair
 // total and the capacity check.
-__global__ void __launch_bounds__(1024) k_bin_rowscan(uint32_t *__restrict__ M, int K, int Ty,
-                                                      RowInfo *__restrict__ rows, uint2 *__restrict__ part_tot,
-                                                      Ctl *__restrict__ ctl, uint64_t cap, int Tx) {
+template <int NV>
+__global__ void __launch_bounds__(1024) k_bin_rowscan(const __grid_constant__ Views<BinView, NV> B, int K) {
+    const BinView &V = B[blockIdx.y];
+    uint32_t *__restrict__ M = V.M;
+    RowInfo *__restrict__ rows = rows_of(V);
+    uint2 *__restrict__ part_tot = part_totals_of(V);
+    Ctl *__restrict__ ctl = V.ctl;
+    const uint64_t cap = V.cap;
+    const int Tx = V.Tx, Ty = V.Ty;
+    if (blockIdx.x >= Ty * kRowParts) return;
     __shared__ uint32_t s_w[32];
     __shared__ uint32_t s_row[kPartChunks];
     __shared__ bool s_last;
@@ -354,7 +379,7 @@ __global__ void __launch_bounds__(1024) k_bin_rowscan(uint32_t *__restrict__ M, 
     if (threadIdx.x == 0) {
         part_tot[blockIdx.x] = make_uint2(tot, ptot);
         __threadfence();
-        s_last = atomicAdd(&ctl->bin_scan_done, 1u) == gridDim.x - 1;
+        s_last = atomicAdd(&ctl->bin_scan_done, 1u) == static_cast<uint32_t>(Ty * kRowParts - 1);
     }
     __syncthreads();
     if (!s_last) return;
@@ -412,9 +437,14 @@ __device__ __forceinline__ int row_of_piece(const uint32_t *s_ps, int Ty, uint32
 }
 
 // Tiles, count: a warp per piece counts its pairs per tile into P[piece][Tx].
-__global__ void __launch_bounds__(256) k_bin_tiles_count(const uint2 *__restrict__ rowlist,
-                                                         const RowInfo *__restrict__ rows, int Tx, int Ty,
-                                                         uint32_t *__restrict__ P, const Ctl *__restrict__ ctl) {
+template <int NV>
+__global__ void __launch_bounds__(256) k_bin_tiles_count(const __grid_constant__ Views<BinView, NV> B) {
+    const BinView &V = B[blockIdx.y];
+    const uint2 *__restrict__ rowlist = V.rowlist;
+    const RowInfo *__restrict__ rows = rows_of(V);
+    uint32_t *__restrict__ P = V.P;
+    const Ctl *ctl = V.ctl;
+    const int Tx = V.Tx, Ty = V.Ty;
     __shared__ uint32_t s_cnt[8][kBinMaxDim + 1];
     __shared__ uint32_t s_ps[kBinMaxDim + 1];
     if (ctl->st.error != GS_OK) return;
@@ -451,10 +481,15 @@ __global__ void __launch_bounds__(256) k_bin_tiles_count(const uint2 *__restrict
 // the first list position of every (piece, tile) (k_bin_tiles_scan).
 constexpr int kStepWords = 4;      // words of 32 entries loaded per step, one step ahead
 
-__global__ void __launch_bounds__(256) k_bin_tiles_write(const uint2 *__restrict__ rowlist,
-                                                         const RowInfo *__restrict__ rows, int Tx, int Ty,
-                                                         const uint32_t *__restrict__ P, uint32_t *__restrict__ list,
-                                                         const Ctl *__restrict__ ctl) {
+template <int NV>
+__global__ void __launch_bounds__(256) k_bin_tiles_write(const __grid_constant__ Views<BinView, NV> B) {
+    const BinView &V = B[blockIdx.y];
+    const uint2 *__restrict__ rowlist = V.rowlist;
+    const RowInfo *__restrict__ rows = rows_of(V);
+    const uint32_t *__restrict__ P = V.P;
+    uint32_t *__restrict__ list = V.list;
+    const Ctl *ctl = V.ctl;
+    const int Tx = V.Tx, Ty = V.Ty;
     __shared__ uint32_t s_val[8][64];              // compacted entries, a ring of two words of 32
     __shared__ uint16_t s_cov[8][64];
     __shared__ uint32_t s_ps[kBinMaxDim + 1];
@@ -530,9 +565,15 @@ __global__ void __launch_bounds__(256) k_bin_tiles_write(const uint2 *__restrict
 // thread (slice s, tile t) sums the counts of tile t over its share of the
 // row's pieces; the slice sums give each tile's total and range; then every
 // (piece, tile) count is replaced by its first list position.
-__global__ void __launch_bounds__(1024) k_bin_tiles_scan(const RowInfo *__restrict__ rows, int Tx,
-                                                         uint32_t *__restrict__ P, uint2 *__restrict__ ranges,
-                                                         const Ctl *__restrict__ ctl) {
+template <int NV>
+__global__ void __launch_bounds__(1024) k_bin_tiles_scan(const __grid_constant__ Views<BinView, NV> B) {
+    const BinView &V = B[blockIdx.y];
+    const RowInfo *__restrict__ rows = rows_of(V);
+    uint32_t *__restrict__ P = V.P;
+    uint2 *__restrict__ ranges = V.ranges;
+    const Ctl *ctl = V.ctl;
+    const int Tx = V.Tx;
+    if (blockIdx.x >= V.Ty) return;
     __shared__ uint32_t s_sum[1024];         // [slice][tile]
     __shared__ uint32_t s_off[kBinMaxDim];
     __shared__ uint32_t s_w[32];
@@ -585,26 +626,38 @@ __global__ void __launch_bounds__(1024) k_bin_tiles_scan(const RowInfo *__restri
 
 }  // namespace
 
-cudaError_t launch_bin_rows(const uint32_t *order, const Rec *rec, uint32_t n_cap, int Tx, int Ty, uint32_t *M,
-                            void *rows_buf, uint2 *rowlist, Ctl *ctl, uint64_t cap, cudaStream_t st) {
-    if (Ty > kBinMaxDim) return cudaErrorInvalidValue;
-    RowInfo *rows = static_cast<RowInfo *>(rows_buf);   // zero on entry (cleared with the control block)
-    uint2 *part_tot = reinterpret_cast<uint2 *>(static_cast<char *>(rows_buf) + bin_rows_bytes(Ty) -
-                                                 static_cast<size_t>(Ty) * kRowParts * sizeof(uint2));
-    k_bin_rows_count<<<kBinBlocks, 256, 0, st>>>(order, rec, n_cap, Ty, M, ctl);
-    k_bin_rowscan<<<Ty * kRowParts, 1024, 0, st>>>(M, kBinChunks, Ty, rows, part_tot, ctl, cap, Tx);
-    k_bin_rows_write<<<kBinBlocks, 256, 0, st>>>(order, rec, n_cap, Ty, M, rows, rowlist, ctl);
+cudaError_t launch_bin_rows(const BinView *views, int n, cudaStream_t st) {
+    int Ty = 0;
+    uint32_t most = 0;
+    for (int i = 0; i < n; ++i) {
+        if (views[i].Ty > kBinMaxDim || views[i].Tx > kBinMaxDim) return cudaErrorInvalidValue;
+        Ty = max(Ty, views[i].Ty);
+        most = max(most, views[i].n_cap);
+    }
+    // chunks of at least kChunkMin Gaussians (a chunk has a column of counts to scan), and half the CTAs per view
+    // when several share the launch (eight 512x512 views 0.173 ms; a quarter 0.184)
+    const int fill = n > 1 ? kBinBlocks / 2 : kBinBlocks;
+    const int blocks = max(min(fill, static_cast<int>(most / (8 * kChunkMin))), 1);
+    with_views(views, n, [&](const auto &b) {
+        constexpr int NV = sizeof(b.v) / sizeof(BinView);
+        k_bin_rows_count<NV><<<dim3(blocks, n), 256, 0, st>>>(b);
+        k_bin_rowscan<NV><<<dim3(Ty * kRowParts, n), 1024, 0, st>>>(b, 8 * blocks);
+        k_bin_rows_write<NV><<<dim3(blocks, n), 256, 0, st>>>(b);
+    });
     return cudaGetLastError();
 }
 
-cudaError_t launch_bin_tiles(const uint2 *rowlist, const void *rows_buf, int Tx, int Ty, uint32_t *P, uint32_t *list,
-                             uint2 *ranges, const Ctl *ctl, cudaStream_t st) {
-    if (Tx > kBinMaxDim || Ty > kBinMaxDim) return cudaErrorInvalidValue;
-    const RowInfo *rows = static_cast<const RowInfo *>(rows_buf);
-    const int G = 4 * sort_blocks();     // 16 CTAs per SM, several waves: pieces differ in pairs (half as many: 3% slower)
-    k_bin_tiles_count<<<G, 256, 0, st>>>(rowlist, rows, Tx, Ty, P, ctl);
-    k_bin_tiles_scan<<<Ty, 1024, 0, st>>>(rows, Tx, P, ranges, ctl);
-    k_bin_tiles_write<<<G, 256, 0, st>>>(rowlist, rows, Tx, Ty, P, list, ctl);
+cudaError_t launch_bin_tiles(const BinView *views, int n, cudaStream_t st) {
+    int Ty = 0;
+    for (int i = 0; i < n; ++i) Ty = max(Ty, views[i].Ty);
+    // 16 CTAs per SM, several waves: pieces differ in pairs (half as many: 3% slower)
+    const int G = max(sort_blocks() / 4, 4 * sort_blocks() / n);
+    with_views(views, n, [&](const auto &b) {
+        constexpr int NV = sizeof(b.v) / sizeof(BinView);
+        k_bin_tiles_count<NV><<<dim3(G, n), 256, 0, st>>>(b);
+        k_bin_tiles_scan<NV><<<dim3(Ty, n), 1024, 0, st>>>(b);
+        k_bin_tiles_write<NV><<<dim3(G, n), 256, 0, st>>>(b);
+    });
     return cudaGetLastError();
 }
 

@@ -166,9 +166,13 @@ __device__ uint32_t order_tiles(int Tn, uint4 *order, uint32_t *s_cnt, uint32_t 
 // memory so the later passes cost no memory round trips.
 constexpr int kSetupSmemTiles = 8192;
 
-__global__ void __launch_bounds__(1024) k_fwd_setup(const uint2 *__restrict__ g_ranges, int Tn,
-                                                    uint4 *__restrict__ order, uint32_t *__restrict__ seg_base,
-                                                    uint32_t *__restrict__ queue, uint32_t *__restrict__ qdone) {
+template <int NV>
+__global__ void __launch_bounds__(1024) k_fwd_setup(const __grid_constant__ Views<SetupView, NV> B) {
+    const SetupView &V = B[blockIdx.x];
+    const uint2 *__restrict__ g_ranges = V.ranges;
+    const int Tn = V.Tn;
+    uint4 *__restrict__ order = V.order;
+    uint32_t *__restrict__ seg_base = V.seg_base, *__restrict__ queue = V.queue, *__restrict__ qdone = V.qdone;
     __shared__ uint32_t s_cnt[kBuckets];
     __shared__ uint32_t s_w[32];
     extern __shared__ uint2 s_ranges[];
@@ -1004,15 +1008,21 @@ cudaError_t launch_forward(const FwdBatch &batch, uint32_t items, cudaStream_t s
 
 }  // namespace
 
-cudaError_t launch_fwd_setup(const CompositeBufs &cb, const uint2 *ranges, int Tn, cudaStream_t st) {
-    if (Tn == 0) return cudaSuccess;
+template <int NV>
+void setup_kernel(const Views<SetupView, NV> &b, size_t smem, cudaStream_t st) {
     static PerDevice attr;
     attr.get([] {
-        cudaFuncSetAttribute(k_fwd_setup, cudaFuncAttributeMaxDynamicSharedMemorySize, kSetupSmemTiles * 8);
+        cudaFuncSetAttribute(k_fwd_setup<NV>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSetupSmemTiles * 8);
         return 1;
     });
-    const size_t smem = Tn <= kSetupSmemTiles ? static_cast<size_t>(Tn) * 8 : 0;
-    k_fwd_setup<<<1, 1024, smem, st>>>(ranges, Tn, cb.order, cb.seg_base, cb.queue, cb.qdone);
+    k_fwd_setup<NV><<<b.n, 1024, smem, st>>>(b);
+}
+
+cudaError_t launch_fwd_setup(const SetupView *views, int n, cudaStream_t st) {
+    int most = 0;
+    for (int i = 0; i < n; ++i)
+        if (views[i].Tn <= kSetupSmemTiles) most = max(most, views[i].Tn);
+    with_views(views, n, [&](const auto &b) { setup_kernel(b, static_cast<size_t>(most) * 8, st); });
     return cudaGetLastError();
 }
 

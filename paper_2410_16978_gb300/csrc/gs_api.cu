@@ -298,65 +298,69 @@ int gs_render_workspace_size(int64_t n, int32_t width, int32_t height, int64_t d
 
 namespace {
 
-// Validates one view, launches S1 (preprocess) and S2 (binning and sorts) and
-// the compositor set-up on st, and describes the view in *job.
 // One view of a render call between its phases.
 struct FrontCtx {
-    SceneView sv;
-    CamView cv;
+    PreView pre;
     Layout L;
     void *ws = nullptr;
-    Ctl *ctl = nullptr;
-    Rec *rec = nullptr;
-    uint32_t *tiles = nullptr;
-    uint32_t *depth = nullptr;
     float *image = nullptr, *alpha = nullptr;
     float bg[3] = {0.f, 0.f, 0.f};
+    uint32_t *order = nullptr;        // depth order to bin in (after front_sort)
 };
 
-// Phase 1: validation, status reset and S1 (preprocess).
-int front_preprocess(const gs_scene *scene, const gs_camera *camera, uint32_t layer_mask,
-                     const gs_clip_plane *planes, int32_t n_planes, const float *bg, void *workspace,
-                     size_t ws_bytes, float *image, float *alpha, cudaStream_t st, FrontCtx *f) {
+// Validates one view and describes it.
+int front_check(const gs_scene *scene, const gs_camera *camera, uint32_t layer_mask, const gs_clip_plane *planes,
+                int32_t n_planes, const float *bg, void *workspace, size_t ws_bytes, float *image, float *alpha,
+                FrontCtx *f) {
     int rc;
-    if ((rc = check_scene(scene, &f->sv)) != GS_OK) return rc;
-    if ((rc = check_camera(camera, &f->cv)) != GS_OK) return rc;
+    PreView &v = f->pre;
+    if ((rc = check_scene(scene, &v.s)) != GS_OK) return rc;
+    if ((rc = check_camera(camera, &v.c)) != GS_OK) return rc;
     if (n_planes < 0 || n_planes > GS_MAX_PLANES) return fail(GS_ERR_INVALID, "n_planes must be 0..%d", GS_MAX_PLANES);
     if (n_planes > 0 && !planes) return fail(GS_ERR_INVALID, "planes is NULL");
     if (!bg) return fail(GS_ERR_INVALID, "bg is NULL");
     if (!image) return fail(GS_ERR_INVALID, "image is NULL");
-    if ((rc = workspace_layout(scene, f->cv, workspace, ws_bytes, &f->L)) != GS_OK) return rc;
-    Planes pl;
-    std::memset(&pl, 0, sizeof pl);
-    pl.n = n_planes;
+    if ((rc = workspace_layout(scene, v.c, workspace, ws_bytes, &f->L)) != GS_OK) return rc;
+    std::memset(&v.pl, 0, sizeof v.pl);
+    v.pl.n = n_planes;
     for (int k = 0; k < n_planes; ++k) {
-        pl.p[k] = make_float4(planes[k].n[0], planes[k].n[1], planes[k].n[2], planes[k].d);
-        pl.bits[k] = planes[k].layer_bits;
+        v.pl.p[k] = make_float4(planes[k].n[0], planes[k].n[1], planes[k].n[2], planes[k].d);
+        v.pl.bits[k] = planes[k].layer_bits;
     }
     const Layout &L = f->L;
+    v.layer_mask = layer_mask;
+    v.rec = at<Rec>(workspace, L.rec);
+    v.geo = at<Geo>(workspace, L.geo);
+    v.tiles = at<uint32_t>(workspace, L.tiles);
+    v.depth = at<uint32_t>(workspace, L.depth);
+    v.ctl = at<Ctl>(workspace, L.ctl);
+    // the control block and what follows it: depth-sort histograms and group counts, binning row counters, tile
+    // ranges (all empty if the binning overflows)
+    v.clear_bytes = (L.ranges + static_cast<size_t>(L.Tn) * 8 - L.ctl + 15) & ~static_cast<size_t>(15);
     f->ws = workspace;
-    f->ctl = at<Ctl>(workspace, L.ctl);
-    f->rec = at<Rec>(workspace, L.rec);
-    f->tiles = at<uint32_t>(workspace, L.tiles);
-    f->depth = at<uint32_t>(workspace, L.depth);
     f->image = image;
     f->alpha = alpha;
     for (int c = 0; c < 3; ++c) f->bg[c] = bg[c];
-    // the control block and what follows it: depth-sort histograms and group counts, binning row counters, tile
-    // ranges (all empty if the binning overflows)
-    if ((rc = cuda_check(cudaMemsetAsync(f->ctl, 0, L.ranges + static_cast<size_t>(L.Tn) * 8 - L.ctl, st),
-                         "memset status")) != GS_OK)
-        return rc;
-    Stage sg(GS_STAGE_PREPROCESS, st, 1);
-    return cuda_check(launch_preprocess(f->sv, f->cv, layer_mask, pl, f->rec, at<Geo>(workspace, L.geo), f->tiles,
-                                        f->depth, f->ctl, st),
-                      "preprocess");
+    return GS_OK;
 }
 
-// Phase 2: the depth sort of the visible Gaussians.  With `other`, a
-// Gaussian visible to either view is kept and keyed by this view's depth when
-// this view sees it, else by the other's (shared stereo order).  Returns the
-// depth order (in this view's workspace).
+// Phase 1: status reset and S1 (preprocess) of n views.
+int front_preprocess(const FrontCtx *f, int n, cudaStream_t st) {
+    PreView v[kMaxBatch];
+    for (int i = 0; i < n; ++i) v[i] = f[i].pre;
+    int rc;
+    if ((rc = cuda_check(launch_clear(v, n, st), "clear status")) != GS_OK) return rc;
+    int launches = 0;
+    Stage sg(GS_STAGE_PREPROCESS, st, n > 1 ? 1 : 0);       // (several views are cleared by a kernel)
+    rc = cuda_check(launch_preprocess(v, n, st, &launches), "preprocess");
+    g_launches += launches;
+    return rc;
+}
+
+// Phase 2: the depth sort of the visible Gaussians of n views (depth order in
+// each view's workspace), or with `shared` one sort for views 0 and 1: a
+// Gaussian visible to either is kept and keyed by view 0's depth when view 0
+// sees it, else by view 1's.
 SortWork sort_work(void *ws, const Layout &L) {
     SortWork w;
     for (int k = 0; k < 2; ++k) {
@@ -372,96 +376,86 @@ SortWork sort_work(void *ws, const Layout &L) {
     return w;
 }
 
-int front_sort(FrontCtx &f, const FrontCtx *other, cudaStream_t st, uint32_t **order) {
-    const SortWork w = sort_work(f.ws, f.L);
+int front_sort(FrontCtx *f, int n, bool shared, cudaStream_t st) {
+    SortView v[kMaxBatch];
+    for (int i = 0; i < n; ++i) {
+        const PreView &p = f[i].pre;
+        v[i] = SortView{p.tiles, p.depth, p.s.n, sort_work(f[i].ws, f[i].L), p.ctl, nullptr, nullptr, p.rec, nullptr};
+        f[i].order = v[shared ? 0 : i].w.order;
+    }
+    if (shared) {
+        v[0].tiles_b = f[1].pre.tiles;
+        v[0].depth_b = f[1].pre.depth;
+        v[0].rec_b = f[1].pre.rec;
+    }
+    const int sorts = shared ? 1 : n;
     int rc;
     {
         Stage sg(GS_STAGE_COMPACT, st, 1);
-        rc = other ? cuda_check(launch_sort_histograms2(f.tiles, f.depth, f.rec, other->tiles, other->depth,
-                                                        other->rec, f.sv.n, w, f.ctl, st),
-                                "depth histograms (stereo)")
-                   : cuda_check(launch_sort_histograms(f.tiles, f.depth, f.sv.n, w, f.ctl, st), "depth histograms");
-        if (rc != GS_OK) return rc;
+        if ((rc = cuda_check(launch_sort_histograms(v, sorts, st), "depth histograms")) != GS_OK) return rc;
     }
-    {
-        Stage sg(GS_STAGE_DEPTH_SORT, st, 4);
-        rc = other ? cuda_check(launch_sort_digits2(f.tiles, f.depth, other->tiles, other->depth, f.sv.n, w, f.ctl,
-                                                    st),
-                                "depth sort (stereo)")
-                   : cuda_check(launch_sort_digits(f.tiles, f.depth, f.sv.n, w, f.ctl, st), "depth sort");
-        if (rc != GS_OK) return rc;
-    }
-    *order = w.order;
-    return GS_OK;
+    Stage sg(GS_STAGE_DEPTH_SORT, st, 4);
+    return cuda_check(launch_sort_digits(v, sorts, st), "depth sort");
 }
 
-// Phase 3: binning in the given depth order (whose count is at n_vis), the
-// compositor set-up, and the forward job of the view.
-int front_bin(FrontCtx &f, const uint32_t *order, cudaStream_t st, FwdJob *job) {
+// Phase 3: binning of n views in their depth orders (whose counts are at n_vis),
+// the compositor set-ups, and the forward jobs of the views.
+int front_bin(FrontCtx *f, int n, cudaStream_t st, FwdJob *jobs) {
+    BinView b[kMaxBatch];
+    SetupView s[kMaxBatch];
+    for (int i = 0; i < n; ++i) {
+        const Layout &L = f[i].L;
+        void *ws = f[i].ws;
+        const PreView &p = f[i].pre;
+        b[i] = BinView{f[i].order, p.rec, static_cast<uint32_t>(p.s.n), p.c.Tx, p.c.Ty, at<uint32_t>(ws, L.bin_m),
+                       at<void>(ws, L.bin_rows), at<uint2>(ws, L.rowlist), p.ctl, static_cast<uint64_t>(L.dup_cap),
+                       at<uint32_t>(ws, L.bin_p), at<uint32_t>(ws, L.list), at<uint2>(ws, L.ranges)};
+        const CompositeBufs cb = composite_bufs(ws, L);
+        s[i] = SetupView{b[i].ranges, L.Tn, cb.order, cb.seg_base, cb.queue, cb.qdone};
+        FwdJob *job = &jobs[i];
+        job->order = cb.order;
+        job->list = b[i].list;
+        job->geo = p.geo;
+        job->rec = p.rec;
+        job->image = f[i].image;
+        job->alpha = f[i].alpha;
+        job->t_final = at<float>(ws, L.t_final);
+        job->n_contrib = at<uint32_t>(ws, L.n_contrib);
+        job->ckpt = cb.ckpt;
+        job->qwork = cb.qwork;
+        job->n_blended = reinterpret_cast<unsigned long long *>(&p.ctl->st.n_blended);
+        job->ctl = p.ctl;
+        job->n = static_cast<uint32_t>(p.s.n);
+        job->n_segs = static_cast<uint32_t>(L.dup_cap / kSeg + L.Tn + 1);
+        job->W = p.c.W;
+        job->H = p.c.H;
+        job->Tx = p.c.Tx;
+        job->Tn = L.Tn;
+        job->bg = make_float3(f[i].bg[0], f[i].bg[1], f[i].bg[2]);
+        job->queue = cb.queue;
+        job->items = cb.items;
+        job->n_items = cb.n_items;
+        job->qdone = cb.qdone;
+    }
     int rc;
-    const Layout &L = f.L;
-    void *ws = f.ws;
-    const uint32_t n = static_cast<uint32_t>(f.sv.n);
-    uint32_t *list = at<uint32_t>(ws, L.list);
-    uint2 *rowlist = at<uint2>(ws, L.rowlist);
-    uint2 *ranges = at<uint2>(ws, L.ranges);
     {
         Stage sg(GS_STAGE_BIN_ROWS, st, 3);
-        if ((rc = cuda_check(launch_bin_rows(order, f.rec, n, f.cv.Tx, f.cv.Ty, at<uint32_t>(ws, L.bin_m),
-                                             at<void>(ws, L.bin_rows), rowlist, f.ctl, L.dup_cap, st),
-                             "binning rows")) != GS_OK)
-            return rc;
+        if ((rc = cuda_check(launch_bin_rows(b, n, st), "binning rows")) != GS_OK) return rc;
     }
     {
         Stage sg(GS_STAGE_BIN_TILES, st, 3);
-        if ((rc = cuda_check(launch_bin_tiles(rowlist, at<void>(ws, L.bin_rows), f.cv.Tx, f.cv.Ty,
-                                              at<uint32_t>(ws, L.bin_p), list, ranges, f.ctl, st),
-                             "binning tiles")) != GS_OK)
-            return rc;
+        if ((rc = cuda_check(launch_bin_tiles(b, n, st), "binning tiles")) != GS_OK) return rc;
     }
-    const CompositeBufs cb = composite_bufs(ws, L);
-    {
-        Stage sg(GS_STAGE_COMPOSITE_SETUP, st, 1);
-        if ((rc = cuda_check(launch_fwd_setup(cb, ranges, L.Tn, st), "compositor set-up")) != GS_OK) return rc;
-    }
-    job->order = cb.order;
-    job->list = list;
-    job->geo = at<Geo>(ws, L.geo);
-    job->rec = f.rec;
-    job->image = f.image;
-    job->alpha = f.alpha;
-    job->t_final = at<float>(ws, L.t_final);
-    job->n_contrib = at<uint32_t>(ws, L.n_contrib);
-    job->ckpt = cb.ckpt;
-    job->qwork = cb.qwork;
-    job->n_blended = reinterpret_cast<unsigned long long *>(&f.ctl->st.n_blended);
-    job->ctl = f.ctl;
-    job->n = n;
-    job->n_segs = static_cast<uint32_t>(L.dup_cap / kSeg + L.Tn + 1);
-    job->W = f.cv.W;
-    job->H = f.cv.H;
-    job->Tx = f.cv.Tx;
-    job->Tn = L.Tn;
-    job->bg = make_float3(f.bg[0], f.bg[1], f.bg[2]);
-    job->queue = cb.queue;
-    job->items = cb.items;
-    job->n_items = cb.n_items;
-    job->qdone = cb.qdone;
-    return GS_OK;
+    Stage sg(GS_STAGE_COMPOSITE_SETUP, st, 1);
+    return cuda_check(launch_fwd_setup(s, n, st), "compositor set-up");
 }
 
-// Validates one view, launches S1 (preprocess) and S2 (sort and binning) and
-// the compositor set-up, and fills the view's forward job.
-int render_front(const gs_scene *scene, const gs_camera *camera, uint32_t layer_mask, const gs_clip_plane *planes,
-                 int32_t n_planes, const float *bg, void *workspace, size_t ws_bytes, float *image, float *alpha,
-                 cudaStream_t st, FwdJob *job) {
-    FrontCtx f;
-    int rc = front_preprocess(scene, camera, layer_mask, planes, n_planes, bg, workspace, ws_bytes, image, alpha, st,
-                              &f);
-    if (rc != GS_OK) return rc;
-    uint32_t *order = nullptr;
-    if ((rc = front_sort(f, nullptr, st, &order)) != GS_OK) return rc;
-    return front_bin(f, order, st, job);
+// S1, S2 and the compositor set-up of n validated views, and their forward jobs.
+int render_front(FrontCtx *f, int n, cudaStream_t st, FwdJob *jobs) {
+    int rc;
+    if ((rc = front_preprocess(f, n, st)) != GS_OK) return rc;
+    if ((rc = front_sort(f, n, false, st)) != GS_OK) return rc;
+    return front_bin(f, n, st, jobs);
 }
 
 }  // namespace
@@ -472,9 +466,13 @@ int gs_render(const gs_scene *scene, const gs_camera *camera, uint32_t layer_mas
               int32_t n_planes, const float *bg, void *workspace, size_t ws_bytes, float *image, float *alpha,
               void *stream) {
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    FrontCtx f;
     FwdJob job;
-    int rc = render_front(scene, camera, layer_mask, planes, n_planes, bg, workspace, ws_bytes, image, alpha, st, &job);
-    if (rc != GS_OK) return rc;
+    int rc;
+    if ((rc = front_check(scene, camera, layer_mask, planes, n_planes, bg, workspace, ws_bytes, image, alpha, &f)) !=
+        GS_OK)
+        return rc;
+    if ((rc = render_front(&f, 1, st, &job)) != GS_OK) return rc;
     Stage sg(GS_STAGE_COMPOSITE, st, 1);
     return cuda_check(launch_composite_forward(&job, 1, st), "composite");
 }
@@ -486,13 +484,16 @@ int gs_render_batch(const gs_render_request *reqs, int32_t n, void *stream) {
             if (reqs[i].workspace == reqs[j].workspace)
                 return fail(GS_ERR_INVALID, "requests %d and %d share a workspace", j, i);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    FrontCtx f[GS_MAX_BATCH];
     FwdJob jobs[GS_MAX_BATCH];
+    int rc;
     for (int i = 0; i < n; ++i) {
         const gs_render_request &r = reqs[i];
-        int rc = render_front(r.scene, r.camera, r.layer_mask, r.planes, r.n_planes, r.bg, r.workspace, r.ws_bytes,
-                              r.image, r.alpha, st, &jobs[i]);
-        if (rc != GS_OK) return rc;
+        if ((rc = front_check(r.scene, r.camera, r.layer_mask, r.planes, r.n_planes, r.bg, r.workspace, r.ws_bytes,
+                              r.image, r.alpha, &f[i])) != GS_OK)
+            return rc;
     }
+    if ((rc = render_front(f, n, st, jobs)) != GS_OK) return rc;
     Stage sg(GS_STAGE_COMPOSITE, st, 1);
     return cuda_check(launch_composite_forward(jobs, n, st), "batched composite");
 }
@@ -505,42 +506,35 @@ int gs_render_stereo(const gs_scene *scene, const gs_camera *left, const gs_came
     if (ws_left == ws_right) return fail(GS_ERR_INVALID, "the two eyes need separate workspaces");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     FrontCtx f[2];
-    int rc;
-    if ((rc = front_preprocess(scene, left, layer_mask, planes, n_planes, bg, ws_left, ws_left_bytes, image_left,
-                               alpha_left, st, &f[0])) != GS_OK)
-        return rc;
-    if ((rc = front_preprocess(scene, right, layer_mask, planes, n_planes, bg, ws_right, ws_right_bytes, image_right,
-                               alpha_right, st, &f[1])) != GS_OK)
-        return rc;
     FwdJob jobs[2];
+    int rc;
+    if ((rc = front_check(scene, left, layer_mask, planes, n_planes, bg, ws_left, ws_left_bytes, image_left, alpha_left,
+                          &f[0])) != GS_OK)
+        return rc;
+    if ((rc = front_check(scene, right, layer_mask, planes, n_planes, bg, ws_right, ws_right_bytes, image_right,
+                          alpha_right, &f[1])) != GS_OK)
+        return rc;
+    if ((rc = front_preprocess(f, 2, st)) != GS_OK) return rc;
+    if ((rc = front_sort(f, 2, shared_sort != 0, st)) != GS_OK) return rc;
     if (shared_sort) {
-        uint32_t *order = nullptr;
-        if ((rc = front_sort(f[0], &f[1], st, &order)) != GS_OK) return rc;
         // the right eye bins in the shared order: it needs the shared count, and
         // its backward the visible list, too
+        Ctl *l = f[0].pre.ctl, *r = f[1].pre.ctl;
         if ((rc = cuda_check(cudaMemcpyAsync(at<uint32_t>(f[1].ws, f[1].L.vis_index),
                                              at<uint32_t>(f[0].ws, f[0].L.vis_index),
-                                             static_cast<size_t>(f[0].sv.n) * sizeof(uint32_t),
+                                             static_cast<size_t>(f[0].pre.s.n) * sizeof(uint32_t),
                                              cudaMemcpyDeviceToDevice, st),
                              "shared visible list")) != GS_OK)
             return rc;
-        if ((rc = cuda_check(cudaMemcpyAsync(&f[1].ctl->n_vis, &f[0].ctl->n_vis, sizeof(uint32_t),
+        if ((rc = cuda_check(cudaMemcpyAsync(&r->n_vis, &l->n_vis, sizeof(uint32_t), cudaMemcpyDeviceToDevice, st),
+                             "shared count")) != GS_OK)
+            return rc;
+        if ((rc = cuda_check(cudaMemcpyAsync(&r->st.n_visible, &l->st.n_visible, sizeof(uint32_t),
                                              cudaMemcpyDeviceToDevice, st),
                              "shared count")) != GS_OK)
             return rc;
-        if ((rc = cuda_check(cudaMemcpyAsync(&f[1].ctl->st.n_visible, &f[0].ctl->st.n_visible, sizeof(uint32_t),
-                                             cudaMemcpyDeviceToDevice, st),
-                             "shared count")) != GS_OK)
-            return rc;
-        if ((rc = front_bin(f[0], order, st, &jobs[0])) != GS_OK) return rc;
-        if ((rc = front_bin(f[1], order, st, &jobs[1])) != GS_OK) return rc;
-    } else {
-        for (int e = 0; e < 2; ++e) {
-            uint32_t *order = nullptr;
-            if ((rc = front_sort(f[e], nullptr, st, &order)) != GS_OK) return rc;
-            if ((rc = front_bin(f[e], order, st, &jobs[e])) != GS_OK) return rc;
-        }
     }
+    if ((rc = front_bin(f, 2, st, jobs)) != GS_OK) return rc;
     Stage sg(GS_STAGE_COMPOSITE, st, 1);
     return cuda_check(launch_composite_forward(jobs, 2, st), "stereo composite");
 }

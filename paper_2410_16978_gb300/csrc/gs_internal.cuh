@@ -145,9 +145,50 @@ struct Planes {
 };
 
 // ---- launches (each returns cudaGetLastError() of its launches) ----
-cudaError_t launch_preprocess(const SceneView &s, const CamView &c, uint32_t layer_mask, const Planes &pl,
-                              Rec *rec, Geo *geo, uint32_t *tiles, uint32_t *depth_key, const Ctl *ctl,
-                              cudaStream_t st);
+//
+// The kernels before the compositor take the views of a call together (one
+// launch of each for a batch of views, one for the two eyes): they are short, and one
+// view's hardly fill the GPU.  Their parameters are an array of per-view
+// structs; a launch of one view has an array of one, so that its parameters are
+// at fixed places.
+constexpr int kMaxBatch = GS_MAX_BATCH;
+template <class T, int N>
+struct Views {
+    T v[N];
+    int n;
+    __device__ __forceinline__ const T &operator[](int i) const { return v[N == 1 ? 0 : i]; }
+};
+// Calls f(Views<T, 1>) or f(Views<T, kMaxBatch>) for views[0 .. n).
+template <class T, class F>
+inline void with_views(const T *views, int n, F f) {
+    if (n == 1) {
+        Views<T, 1> b;
+        b.v[0] = views[0];
+        b.n = 1;
+        f(b);
+    } else {
+        Views<T, kMaxBatch> b;
+        b.n = n < kMaxBatch ? n : kMaxBatch;
+        for (int i = 0; i < kMaxBatch; ++i) b.v[i] = views[i < b.n ? i : 0];
+        f(b);
+    }
+}
+
+// S1 of one view.
+struct PreView {
+    SceneView s;
+    CamView c;
+    Planes pl;
+    uint32_t layer_mask;
+    Rec *rec;
+    Geo *geo;
+    uint32_t *tiles, *depth;
+    Ctl *ctl;
+    size_t clear_bytes;        // of the control block and what follows it, cleared before the kernels
+};
+// Clears every view's control block with its histograms, counters and ranges.
+cudaError_t launch_clear(const PreView *views, int n, cudaStream_t st);
+cudaError_t launch_preprocess(const PreView *views, int n, cudaStream_t st, int *launches);
 // Also adds the per-Gaussian blend-weight sums (record-gradient slot 9) to
 // contrib_sum when it is not null.
 // vis_index: the visible list of the last render (index order, ctl->n_vis
@@ -194,37 +235,47 @@ uint32_t sort_tiles(int64_t n);
 size_t sort_count_bytes(int64_t n);
 size_t sort_group_bytes(int64_t n);
 size_t sort_status_bytes(int64_t n);
-// Sorts the Gaussians i < n with tiles[i] > 0 by (depth[i], i).  Histograms:
+// Per view, sorts the Gaussians i < n with tiles[i] > 0 by (depth[i], i).  Histograms:
 // the visible count (to ctl->n_vis and ctl->st.n_visible), the key range
 // (ctl->depth_mm), the digit histograms and the per-tile counts of the
 // first digit; these control words (with the tickets), work.ghist and
 // work.grp must be zero on entry.  Digits: writes work.order and work.vis_index.
-cudaError_t launch_sort_histograms(const uint32_t *tiles, const uint32_t *depth, int n, const SortWork &work,
-                                   Ctl *ctl, cudaStream_t st);
-cudaError_t launch_sort_digits(const uint32_t *tiles, const uint32_t *depth, int n, const SortWork &work, Ctl *ctl,
-                               cudaStream_t st);
-// Two eyes: Gaussians visible to view a or view b, keyed by depth_a where
-// view a sees the Gaussian, else by depth_b (one depth order for both eyes).
-// The histograms also give a Gaussian that only one view sees an empty tile
-// rectangle in the other view's records.
-cudaError_t launch_sort_histograms2(const uint32_t *tiles_a, const uint32_t *depth_a, Rec *rec_a,
-                                    const uint32_t *tiles_b, const uint32_t *depth_b, Rec *rec_b, int n,
-                                    const SortWork &work, Ctl *ctl, cudaStream_t st);
-cudaError_t launch_sort_digits2(const uint32_t *tiles_a, const uint32_t *depth_a, const uint32_t *tiles_b,
-                                const uint32_t *depth_b, int n, const SortWork &work, Ctl *ctl, cudaStream_t st);
-// Tile binning (bin.cu).  Rows: splits the depth-ordered visible Gaussians
-// (order[p], p < min(ctl->n_vis, n_cap)) into per-tile-row lists of
+// Two eyes (a view with tiles_b): Gaussians visible to view a or view b, keyed
+// by depth where view a sees the Gaussian, else by depth_b (one depth order for
+// both eyes).  Its histograms also give a Gaussian that only one eye sees an empty tile
+// rectangle in the other eye's records.
+struct SortView {
+    const uint32_t *tiles, *depth;
+    int n;
+    SortWork w;
+    Ctl *ctl;
+    const uint32_t *tiles_b, *depth_b;      // two eyes: the other view's (null: one view)
+    Rec *rec, *rec_b;
+};
+cudaError_t launch_sort_histograms(const SortView *views, int n, cudaStream_t st);
+cudaError_t launch_sort_digits(const SortView *views, int n, cudaStream_t st);
+// Tile binning (bin.cu) of a view.  Rows: splits the depth-ordered visible
+// Gaussians (order[p], p < min(ctl->n_vis, n_cap)) into per-tile-row lists of
 // (Gaussian, x0 | x1 << 16) in depth order; writes n_dup and the overflow
-// status (n_dup > cap).  M: 2 kBinChunks Ty words; rows_buf: bin_rows_bytes(Ty),
-// zero on entry.
-cudaError_t launch_bin_rows(const uint32_t *order, const Rec *rec, uint32_t n_cap, int Tx, int Ty, uint32_t *M,
-                            void *rows_buf, uint2 *rowlist, Ctl *ctl, uint64_t cap, cudaStream_t st);
-// Tiles: splits every row list into its tiles; writes the final Gaussian list
-// (tile order, depth order within a tile) and every tile's [start, end).
-// Does nothing when the status holds an error.
-// P: bin_piece_bytes(cap, Tx, Ty) bytes.
-cudaError_t launch_bin_tiles(const uint2 *rowlist, const void *rows_buf, int Tx, int Ty, uint32_t *P, uint32_t *list,
-                             uint2 *ranges, const Ctl *ctl, cudaStream_t st);
+// status (n_dup > cap).  M: 2 kBinChunks Ty words; rows: bin_rows_bytes(Ty), zero on
+// entry.  Tiles: splits every row list into its tiles; writes the final Gaussian
+// list (tile order, depth order within a tile) and every tile's [start, end); P:
+// bin_piece_bytes(cap, Tx, Ty) bytes.  Does nothing when the status holds an error.
+struct BinView {
+    const uint32_t *order;
+    const Rec *rec;
+    uint32_t n_cap;
+    int Tx, Ty;
+    uint32_t *M;
+    void *rows;
+    uint2 *rowlist;
+    Ctl *ctl;
+    uint64_t cap;
+    uint32_t *P, *list;
+    uint2 *ranges;
+};
+cudaError_t launch_bin_rows(const BinView *views, int n, cudaStream_t st);
+cudaError_t launch_bin_tiles(const BinView *views, int n, cudaStream_t st);
 size_t bin_rows_bytes(int Ty);
 size_t bin_piece_bytes(int64_t dup_cap, int Tx, int Ty);
 // Training-step kernels (train.cu).
@@ -266,7 +317,6 @@ struct CompositeBufs {
 };
 // One view for the forward compositor.  A batch of views is composited by
 // one persistent launch whose work queue spans all their tiles.
-constexpr int kMaxBatch = GS_MAX_BATCH;
 struct FwdJob {
     const uint4 *order;
     const uint32_t *list;
@@ -290,7 +340,13 @@ struct FwdJob {
 // Per-view set-up before compositing: tile order, checkpoint bases, zeroed
 // block work and queue.  The backward's set-up also zeroes the record-gradient
 // rows of the visible Gaussians (vis_index, *n_vis of the n Gaussians).
-cudaError_t launch_fwd_setup(const CompositeBufs &cb, const uint2 *ranges, int Tn, cudaStream_t st);
+struct SetupView {
+    const uint2 *ranges;
+    int Tn;
+    uint4 *order;
+    uint32_t *seg_base, *queue, *qdone;
+};
+cudaError_t launch_fwd_setup(const SetupView *views, int n, cudaStream_t st);
 // Composites n <= kMaxBatch views with one persistent launch; every view's
 // queue must have been written on the stream (its launch_fwd_setup does).
 cudaError_t launch_composite_forward(const FwdJob *jobs, int n, cudaStream_t st);

@@ -76,12 +76,15 @@ __device__ __forceinline__ void store_geo(Geo *g, const float4 a, const float4 b
                  : "memory");
 }
 
-template <int DEG>
-__global__ void __launch_bounds__(128) k_preprocess(SceneView s, CamView c, uint32_t layer_mask, Planes pl,
-                                                    Rec *__restrict__ rec, Geo *__restrict__ geo,
-                                                    uint32_t *__restrict__ tiles,
-                                                    uint32_t *__restrict__ depth_key, const Ctl *__restrict__ ctl) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+// The views of a launch are interleaved block by block (view blockIdx.x mod n),
+// so views of one scene read it from L2 after the first.
+template <int DEG, int NV>
+__global__ void __launch_bounds__(128) k_preprocess(const __grid_constant__ Views<PreView, NV> B) {
+    const PreView &V = B[blockIdx.x % B.n];
+    const SceneView &s = V.s;
+    const CamView &c = V.c;
+    const Planes &pl = V.pl;
+    const int i = (NV == 1 ? blockIdx.x : blockIdx.x / B.n) * blockDim.x + threadIdx.x;
     if (i >= s.n) return;
     uint32_t ntiles = 0;
     uint32_t dkey = 0xFFFFFFFFu;
@@ -103,7 +106,7 @@ __global__ void __launch_bounds__(128) k_preprocess(SceneView s, CamView c, uint
         qz = ld_half(s.quats, 4 * (int64_t)i + 3, s.dtype_sr);
     }
     const float ol = s.opacity_logit[i];
-    bool keep = (layer_mask >> lay) & 1u;
+    bool keep = (V.layer_mask >> lay) & 1u;
     for (int k = 0; k < pl.n && keep; ++k) {
         if (!((pl.bits[k] >> lay) & 1u)) continue;
         const float4 p = pl.p[k];
@@ -175,7 +178,7 @@ __global__ void __launch_bounds__(128) k_preprocess(SceneView s, CamView c, uint
             const float fy1 = fminf(fTy, fmaxf(0.0f, truncf(((vv + r) + 15.0f) * 0.0625f)));
             const int x0 = static_cast<int>(fx0), y0 = static_cast<int>(fy0);
             const int x1 = static_cast<int>(fx1), y1 = static_cast<int>(fy1);
-            ntiles = GS_CHECK(x0 <= x1 && y0 <= y1 && x1 <= c.Tx && y1 <= c.Ty, ctl, kSiteRect)
+            ntiles = GS_CHECK(x0 <= x1 && y0 <= y1 && x1 <= c.Tx && y1 <= c.Ty, V.ctl, kSiteRect)
                          ? static_cast<uint32_t>((x1 - x0) * (y1 - y0))
                          : 0u;
             if (ntiles > 0) {
@@ -236,27 +239,63 @@ __global__ void __launch_bounds__(128) k_preprocess(SceneView s, CamView c, uint
                 o.b = make_float4(NHL / c11, opac, rgb[0], rgb[1]);
                 o.c = make_float4(rgb[2], pz, __uint_as_float(static_cast<uint32_t>(x0) | (static_cast<uint32_t>(y0) << 16)),
                                   __uint_as_float(static_cast<uint32_t>(x1) | (static_cast<uint32_t>(y1) << 16)));
-                rec[i] = o;
-                store_geo(geo + i, o.a, o.b);
+                V.rec[i] = o;
+                store_geo(V.geo + i, o.a, o.b);
                 dkey = __float_as_uint(pz);
             }
         }
     }
-    tiles[i] = ntiles;
-    depth_key[i] = dkey;
+    V.tiles[i] = ntiles;
+    V.depth[i] = dkey;
+}
+
+// Zeroes every view's control block and what is cleared with it (16-byte words).
+__global__ void __launch_bounds__(256) k_clear(const __grid_constant__ Views<PreView, kMaxBatch> B) {
+    const PreView &V = B[blockIdx.y];
+    uint4 *p = reinterpret_cast<uint4 *>(V.ctl);
+    const size_t words = V.clear_bytes / sizeof(uint4);
+    for (size_t w = blockIdx.x * 256u + threadIdx.x; w < words; w += gridDim.x * 256u) p[w] = make_uint4(0u, 0u, 0u, 0u);
 }
 
 }  // namespace
 
-cudaError_t launch_preprocess(const SceneView &s, const CamView &c, uint32_t layer_mask, const Planes &pl, Rec *rec,
-                              Geo *geo, uint32_t *tiles, uint32_t *depth_key, const Ctl *ctl, cudaStream_t st) {
-    if (s.n == 0) return cudaSuccess;
-    const int threads = 128, blocks = (s.n + threads - 1) / threads;
-    switch (s.sh_degree) {
-        case 0: k_preprocess<0><<<blocks, threads, 0, st>>>(s, c, layer_mask, pl, rec, geo, tiles, depth_key, ctl); break;
-        case 1: k_preprocess<1><<<blocks, threads, 0, st>>>(s, c, layer_mask, pl, rec, geo, tiles, depth_key, ctl); break;
-        case 2: k_preprocess<2><<<blocks, threads, 0, st>>>(s, c, layer_mask, pl, rec, geo, tiles, depth_key, ctl); break;
-        default: k_preprocess<3><<<blocks, threads, 0, st>>>(s, c, layer_mask, pl, rec, geo, tiles, depth_key, ctl); break;
+namespace {
+
+template <int NV>
+void preprocess_views(int deg, const Views<PreView, NV> &b, unsigned blocks, cudaStream_t st) {
+    switch (deg) {
+        case 0: k_preprocess<0, NV><<<blocks, 128, 0, st>>>(b); break;
+        case 1: k_preprocess<1, NV><<<blocks, 128, 0, st>>>(b); break;
+        case 2: k_preprocess<2, NV><<<blocks, 128, 0, st>>>(b); break;
+        default: k_preprocess<3, NV><<<blocks, 128, 0, st>>>(b); break;
+    }
+}
+
+}  // namespace
+
+cudaError_t launch_clear(const PreView *views, int n, cudaStream_t st) {
+    if (n == 1) return cudaMemsetAsync(views[0].ctl, 0, views[0].clear_bytes, st);
+    with_views(views, n, [&](const auto &b) {
+        if constexpr (sizeof(b.v) == kMaxBatch * sizeof(PreView)) k_clear<<<dim3(8, b.n), 256, 0, st>>>(b);
+    });
+    return cudaGetLastError();
+}
+
+cudaError_t launch_preprocess(const PreView *views, int n, cudaStream_t st, int *launches) {
+    *launches = 0;
+    for (int deg = 0; deg <= 3; ++deg) {           // a launch per SH degree among the views
+        PreView of[kMaxBatch];
+        int m = 0, most = 0;
+        for (int i = 0; i < n && m < kMaxBatch; ++i) {
+            if (views[i].s.sh_degree != deg || views[i].s.n == 0) continue;
+            of[m++] = views[i];
+            most = views[i].s.n > most ? views[i].s.n : most;
+        }
+        if (m == 0) continue;
+        with_views(of, m, [&](const auto &b) {
+            preprocess_views(deg, b, static_cast<unsigned>((most + 127) / 128) * static_cast<unsigned>(m), st);
+        });
+        ++*launches;
     }
     return cudaGetLastError();
 }

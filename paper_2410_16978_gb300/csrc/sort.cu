@@ -162,6 +162,7 @@ struct KeepOut {
 
 struct VisSrc {             // one view: visible where its tile count is non-zero
     const uint32_t *tiles, *depth;
+    __device__ __forceinline__ explicit VisSrc(const SortView &v) : tiles(v.tiles), depth(v.depth) {}
     __device__ __forceinline__ bool visible(uint32_t i) const { return tiles[i] > 0; }
     __device__ __forceinline__ uint32_t key(uint32_t i) const { return depth[i]; }
     __device__ __forceinline__ void settle(uint32_t) const {}
@@ -169,6 +170,8 @@ struct VisSrc {             // one view: visible where its tile count is non-zer
 struct VisSrc2 {            // two eyes: visible to either; keyed by view a's depth where view a sees it
     const uint32_t *tiles_a, *depth_a, *tiles_b, *depth_b;
     Rec *rec_a, *rec_b;
+    __device__ __forceinline__ explicit VisSrc2(const SortView &v)
+        : tiles_a(v.tiles), depth_a(v.depth), tiles_b(v.tiles_b), depth_b(v.depth_b), rec_a(v.rec), rec_b(v.rec_b) {}
     // A visible Gaussian that one eye does not see is in both eyes' order, but that eye's record of it was not
     // written: an empty tile rectangle there, so its binning passes the Gaussian over.
     __device__ __forceinline__ void settle(uint32_t i) const {
@@ -214,6 +217,15 @@ static_assert(kPassTile % kSortTile == 0, "a digit-kernel tile is whole histogra
 struct TileCounts {
     uint32_t *cnt, *grp;
     int lg;
+};
+
+// A view's sort with what its kernels derive from the sizes.
+struct SortJob {
+    SortView v;
+    TileCounts tc;
+    uint32_t nt;             // tiles of the first digit kernel
+    uint32_t spin_limit;     // see SortBufs
+    int withhold;
 };
 
 // One CTA per tile of the first digit kernel: the visible count, the key
@@ -262,13 +274,19 @@ __device__ uint32_t look_back(uint64_t *status, uint32_t t, int c, uint32_t own,
     return excl;
 }
 
-template <class Src>
-__global__ void __launch_bounds__(256) k_sort_hist(Src src, uint32_t n, uint32_t *__restrict__ ghist, Ctl *ctl,
-                                                   TileCounts tc) {
+template <class Src, int NV>
+__global__ void __launch_bounds__(256) k_sort_hist(const __grid_constant__ Views<SortJob, NV> B) {
     __shared__ uint32_t s_h[4][256];
     __shared__ uint32_t s_w[8];
-    const int lane = threadIdx.x & 31;
+    const SortJob &J = B[blockIdx.y];
+    const uint32_t n = J.v.n;
     const uint32_t t = blockIdx.x;
+    if (t >= J.nt) return;
+    const Src src(J.v);
+    uint32_t *__restrict__ ghist = J.v.w.ghist;
+    Ctl *ctl = J.v.ctl;
+    const TileCounts tc = J.tc;
+    const int lane = threadIdx.x & 31;
     for (int k = threadIdx.x; k < 4 * 256; k += 256) (&s_h[0][0])[k] = 0;
     __syncthreads();
     const uint32_t beg = t * kPassTile, end = min(n, beg + kPassTile);
@@ -329,6 +347,7 @@ __global__ void __launch_bounds__(256) k_sort_hist(Src src, uint32_t n, uint32_t
     if (c0) atomicAdd(&tc.grp[static_cast<size_t>(t >> tc.lg) * kLookCounters + threadIdx.x], c0);
 }
 
+// One digit kernel's buffers: pass p reads what pass p - 1 wrote.
 struct SortBufs {
     const uint32_t *kin, *vin;       // digit kernels after the first: this pass's input
     uint32_t *kout, *vout;           // the next digit kernel's input
@@ -339,6 +358,21 @@ struct SortBufs {
     uint64_t *status, *status_next;  // look-back words [tile][256] of this (after the first) and the next pass
     uint32_t spin_limit;             // iterations a look-back waits for a predecessor before GS_ERR_TIMEOUT
     int withhold;                    // GS_DEBUG test hook: this kernel's first tile publishes nothing (-1: off)
+    __device__ __forceinline__ SortBufs(const SortJob &J, int p) {
+        const SortWork &w = J.v.w;
+        kin = w.keys[(p & 1) ^ 1];
+        vin = w.vals[(p & 1) ^ 1];
+        kout = w.keys[p & 1];
+        vout = w.vals[p & 1];
+        final_out = w.order;
+        vis_index = w.vis_index;
+        ghist = w.ghist;
+        tc = J.tc;
+        status = w.status + static_cast<size_t>(p - 1) * J.nt * kLookCounters;       // (p > 0)
+        status_next = w.status + static_cast<size_t>(p) * J.nt * kLookCounters;      // (p < 3)
+        spin_limit = J.spin_limit;
+        withhold = J.withhold;
+    }
 };
 
 // One digit (bits 8 pass .. 8 pass + 7) of the stable LSD sort, on tiles of
@@ -375,8 +409,8 @@ __device__ __forceinline__ uint32_t block_scan_512(uint32_t v, uint32_t *s_w, ui
     return base + x - v;
 }
 
-template <class Src, bool FIRST>
-__global__ void __launch_bounds__(kPassThreads) k_sort_pass(Src src, uint32_t n_all, int pass, SortBufs B, Ctl *ctl) {
+template <class Src, bool FIRST, int NV>
+__global__ void __launch_bounds__(kPassThreads) k_sort_pass(const __grid_constant__ Views<SortJob, NV> views, int pass) {
     __shared__ uint16_t s_wc[kPassWarps][256];   // per-warp digit counts, then per-warp digit bases
     __shared__ uint32_t s_lstart[256];            // start of each digit's run in the locally sorted tile
     __shared__ uint32_t s_off[256];               // global position of each digit's run
@@ -386,8 +420,14 @@ __global__ void __launch_bounds__(kPassThreads) k_sort_pass(Src src, uint32_t n_
     __shared__ uint32_t s_ticket, s_visbase;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
+    const SortJob &J = views[blockIdx.y];
+    Ctl *ctl = J.v.ctl;
+    const uint32_t n_all = J.v.n;
+    if (blockIdx.x >= J.nt) return;
     const int passes = sort_passes(ctl);
     if (pass >= passes) return;
+    const Src src(J.v);
+    const SortBufs B(J, FIRST ? 0 : pass);
     const bool last = pass == passes - 1;
     const uint32_t n_vis = min(ctl->n_vis, n_all);
     const uint32_t n = FIRST ? n_all : n_vis;
@@ -534,54 +574,53 @@ int sort_group_log(uint32_t nt) {
     return lg;
 }
 
-TileCounts tile_counts(const SortWork &w, int n) {
-    TileCounts tc;
-    tc.cnt = w.cnt;
-    tc.grp = w.grp;
-    tc.lg = sort_group_log(sort_tiles(n));
-    return tc;
-}
-
-template <class Src>
-cudaError_t sort_histograms(const Src &src, int n, const SortWork &w, Ctl *ctl, cudaStream_t st) {
-    if (n <= 0) return cudaSuccess;
-    // the histograms and the group counts were cleared with the control block
-    const TileCounts tc = tile_counts(w, n);
-    k_sort_hist<<<sort_tiles(n), 256, 0, st>>>(src, static_cast<uint32_t>(n), w.ghist, ctl, tc);
-    return cudaGetLastError();
-}
-
-template <class Src>
-cudaError_t sort_digits(const Src &src, int n, const SortWork &w, Ctl *ctl, cudaStream_t st) {
-    if (n <= 0) return cudaSuccess;
-    const TileCounts tc = tile_counts(w, n);
-    const uint32_t nt = sort_tiles(n);
-    uint32_t *A[2] = {w.keys[0], w.vals[0]}, *Bb[2] = {w.keys[1], w.vals[1]};
-    for (int p = 0; p < 4; ++p) {
-        SortBufs b;
-        uint32_t *const *in = (p & 1) ? A : Bb;       // pass p reads what pass p - 1 wrote
-        uint32_t *const *out = (p & 1) ? Bb : A;
-        b.kin = in[0];
-        b.vin = in[1];
-        b.kout = out[0];
-        b.vout = out[1];
-        b.final_out = w.order;
-        b.vis_index = w.vis_index;
-        b.ghist = w.ghist;
-        b.tc = tc;
-        b.status = p > 0 ? w.status + static_cast<size_t>(p - 1) * nt * kLookCounters : nullptr;
-        b.status_next = p < 3 ? w.status + static_cast<size_t>(p) * nt * kLookCounters : nullptr;
+// The jobs of the views that hold Gaussians; returns how many, and the most tiles of one.
+int sort_jobs(const SortView *views, int n, SortJob *jobs, uint32_t *most) {
+    int m = 0;
+    *most = 0;
+    for (int i = 0; i < n && m < kMaxBatch; ++i) {
+        if (views[i].n <= 0) continue;
+        SortJob &j = jobs[m++];
+        j.v = views[i];
+        j.nt = sort_tiles(views[i].n);
+        j.tc.cnt = views[i].w.cnt;
+        j.tc.grp = views[i].w.grp;
+        j.tc.lg = sort_group_log(j.nt);
 #ifdef GS_DEBUG
-        b.spin_limit = g_dbg_spin_limit;
-        b.withhold = g_dbg_withhold_pass;
+        j.spin_limit = g_dbg_spin_limit;
+        j.withhold = g_dbg_withhold_pass;
 #else
-        b.spin_limit = kSpinLimit;
-        b.withhold = -1;
+        j.spin_limit = kSpinLimit;
+        j.withhold = -1;
 #endif
-        if (p == 0) k_sort_pass<Src, true><<<nt, kPassThreads, 0, st>>>(src, static_cast<uint32_t>(n), p, b, ctl);
-        else k_sort_pass<Src, false><<<nt, kPassThreads, 0, st>>>(src, static_cast<uint32_t>(n), p, b, ctl);
+        *most = j.nt > *most ? j.nt : *most;
     }
-    return cudaGetLastError();
+    return m;
+}
+
+// f(Src, views) for the two-eye order (a single view) or the views' own.
+template <class F>
+void with_sort(const SortJob *jobs, int m, F f) {
+    if (jobs[0].v.tiles_b) {
+        Views<SortJob, 1> b;
+        b.v[0] = jobs[0];
+        b.n = 1;
+        f(static_cast<VisSrc2 *>(nullptr), b);
+    } else {
+        with_views(jobs, m, [&](const auto &b) { f(static_cast<VisSrc *>(nullptr), b); });
+    }
+}
+
+template <class Src, int NV>
+void hist_kernel(Src *, const Views<SortJob, NV> &b, uint32_t most, cudaStream_t st) {
+    // the histograms and the group counts were cleared with the control block
+    k_sort_hist<Src, NV><<<dim3(most, b.n), 256, 0, st>>>(b);
+}
+
+template <class Src, int NV>
+void digit_kernels(Src *, const Views<SortJob, NV> &b, uint32_t most, cudaStream_t st) {
+    k_sort_pass<Src, true, NV><<<dim3(most, b.n), kPassThreads, 0, st>>>(b, 0);
+    for (int p = 1; p < 4; ++p) k_sort_pass<Src, false, NV><<<dim3(most, b.n), kPassThreads, 0, st>>>(b, p);
 }
 
 // ---------------------------------------------------------------------------
@@ -618,25 +657,20 @@ size_t sort_group_bytes(int64_t n) {
     return static_cast<size_t>(g) * kLookCounters * sizeof(uint32_t);
 }
 
-cudaError_t launch_sort_histograms(const uint32_t *tiles, const uint32_t *depth, int n, const SortWork &w, Ctl *ctl,
-                                   cudaStream_t st) {
-    return sort_histograms(VisSrc{tiles, depth}, n, w, ctl, st);
+cudaError_t launch_sort_histograms(const SortView *views, int n, cudaStream_t st) {
+    SortJob jobs[kMaxBatch];
+    uint32_t most;
+    const int m = sort_jobs(views, n, jobs, &most);
+    if (m) with_sort(jobs, m, [&](auto *src, const auto &b) { hist_kernel(src, b, most, st); });
+    return cudaGetLastError();
 }
 
-cudaError_t launch_sort_digits(const uint32_t *tiles, const uint32_t *depth, int n, const SortWork &w, Ctl *ctl,
-                               cudaStream_t st) {
-    return sort_digits(VisSrc{tiles, depth}, n, w, ctl, st);
-}
-
-cudaError_t launch_sort_histograms2(const uint32_t *tiles_a, const uint32_t *depth_a, Rec *rec_a,
-                                    const uint32_t *tiles_b, const uint32_t *depth_b, Rec *rec_b, int n,
-                                    const SortWork &w, Ctl *ctl, cudaStream_t st) {
-    return sort_histograms(VisSrc2{tiles_a, depth_a, tiles_b, depth_b, rec_a, rec_b}, n, w, ctl, st);
-}
-
-cudaError_t launch_sort_digits2(const uint32_t *tiles_a, const uint32_t *depth_a, const uint32_t *tiles_b,
-                                const uint32_t *depth_b, int n, const SortWork &w, Ctl *ctl, cudaStream_t st) {
-    return sort_digits(VisSrc2{tiles_a, depth_a, tiles_b, depth_b, nullptr, nullptr}, n, w, ctl, st);
+cudaError_t launch_sort_digits(const SortView *views, int n, cudaStream_t st) {
+    SortJob jobs[kMaxBatch];
+    uint32_t most;
+    const int m = sort_jobs(views, n, jobs, &most);
+    if (m) with_sort(jobs, m, [&](auto *src, const auto &b) { digit_kernels(src, b, most, st); });
+    return cudaGetLastError();
 }
 
 cudaError_t launch_activity_prune(const float *activity, const uint8_t *layer, uint32_t train_mask, int n,

@@ -11,9 +11,14 @@
 // window sums of per-pixel maps (the window is symmetric):
 //   dSSIM/dx_p = (G*a)_p + 2 x_p (G*b)_p + y_p (G*c)_p,
 //   a = df/dmu_x - 2 mu_x df/dsx - mu_y df/dsxy,  b = df/dsx,  c = df/dsxy.
-// Both kernels stage a (32 + 10) x (8 + 10) halo tile in shared memory and run
-// the window as a horizontal then a vertical 11-tap pass (HBM-bound: a few
-// floats per pixel and channel in and out).
+// Both kernels stage a (32 + 10) x (32 + 10) halo tile in shared memory and run
+// the window as a horizontal then a vertical 11-tap pass, four outputs per thread
+// and pass: neighbouring outputs share 10 of their 11 taps, so a value is read
+// from shared memory 3.5 times and not 11, and two moments at a time go through
+// the packed FMA (fma.rn.f32x2).  One output per thread was bound by its
+// shared-memory reads and the latency of its chains: 800 x 800 image, both passes,
+// 0.091 -> 0.061 ms (sums and their order per pixel are the same).  All three channels in a
+// block, the next one's values loaded ahead, needed 121 registers and took 0.078 ms.
 #include <cmath>
 
 #include "gs_internal.cuh"
@@ -21,8 +26,15 @@
 namespace gs {
 namespace {
 
-constexpr int kLW = 32, kLH = 16, kHalo = 5, kWin = 11;
-constexpr int kRW = kLW + 2 * kHalo, kRH = kLH + 2 * kHalo;   // 42 x 26 staged region
+constexpr int kLW = 32, kLH = 32, kHalo = 5, kWin = 11;
+constexpr int kRW = kLW + 2 * kHalo, kRH = kLH + 2 * kHalo;   // 42 x 42 staged region
+constexpr int kLossThreads = 256;
+constexpr int kLOut = 4;                                      // outputs per thread of a window pass
+constexpr int kLTap = kWin + kLOut - 1;                       // and the values they read
+// Row strides in shared memory.  The horizontal pass has a row per lane: staged rows
+// (pairs) 43 apart and its results 34 pairs and 36 floats apart touch every bank once.
+constexpr int kSP = kRW + 1, kHP = kLW + 2, kHS = kLW + 4;
+static_assert(kLossThreads == kLW * (kLH / kLOut), "vertical pass: a column strip per thread");
 constexpr float kC1 = 0.01f * 0.01f, kC2 = 0.03f * 0.03f;
 
 struct Win {
@@ -39,21 +51,75 @@ __device__ __forceinline__ float sgn(float v) { return v > 0.f ? 1.f : (v < 0.f 
 // values lie in [0, 1]); zero padding outside the image enters as -kSsimShift.
 constexpr float kSsimShift = 0.5f;
 
+// Two floats in a 64-bit register and their fused multiply-add.
+struct F2 {
+    unsigned long long v;
+    __device__ __forceinline__ F2() {}
+    __device__ __forceinline__ F2(float a, float b) { asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(a), "f"(b)); }
+    __device__ __forceinline__ float2 get() const {
+        float2 r;
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+        return r;
+    }
+};
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+
+// The vertical pass over column cx, output rows 4 sy .. 4 sy + 3, of one pair array and one plain array of
+// horizontal sums.
+__device__ __forceinline__ void window_column(const float2 (*h)[kHP], int cx, int sy, const Win &win, F2 (&m)[kLOut]) {
+#pragma unroll
+    for (int o = 0; o < kLOut; ++o) m[o] = F2(0.f, 0.f);
+    F2 t[kLTap];
+#pragma unroll
+    for (int i = 0; i < kLTap; ++i) {
+        const float2 v = h[kLOut * sy + i][cx];
+        t[i] = F2(v.x, v.y);
+    }
+#pragma unroll
+    for (int i = 0; i < kWin; ++i)
+#pragma unroll
+        for (int o = 0; o < kLOut; ++o) m[o] = fma2(F2(win.g[i], win.g[i]), t[o + i], m[o]);
+}
+__device__ __forceinline__ void window_column(const float (*h)[kHS], int cx, int sy, const Win &win, float (&m)[kLOut]) {
+#pragma unroll
+    for (int o = 0; o < kLOut; ++o) m[o] = 0.f;
+    float t[kLTap];
+#pragma unroll
+    for (int i = 0; i < kLTap; ++i) t[i] = h[kLOut * sy + i][cx];
+#pragma unroll
+    for (int i = 0; i < kWin; ++i)
+#pragma unroll
+        for (int o = 0; o < kLOut; ++o) m[o] = fmaf(win.g[i], t[o + i], m[o]);
+}
+__device__ __forceinline__ void store4(float2 *dst, const F2 (&v)[kLOut]) {
+    const float2 a = v[0].get(), b = v[1].get(), c = v[2].get(), d = v[3].get();
+    reinterpret_cast<float4 *>(dst)[0] = make_float4(a.x, a.y, b.x, b.y);
+    reinterpret_cast<float4 *>(dst)[1] = make_float4(c.x, c.y, d.x, d.y);
+}
+
 // Pass 1: per pixel and channel, SSIM and the maps a, b, c; block sums of
 // SSIM, |X - Y| and (channel 0) |A - A_t|.
-__global__ void __launch_bounds__(kLW *kLH) k_loss_maps(const float *__restrict__ X, const float *__restrict__ A,
-                                                        const float *__restrict__ Ct, const float *__restrict__ At,
-                                                        float3 bg, int W, int H, const Win win,
-                                                        float *__restrict__ maps, float *__restrict__ partials) {
-    __shared__ float s_x[kRH][kRW], s_y[kRH][kRW];
-    __shared__ float s_h[5][kRH][kLW];
-    __shared__ float s_red[3][kLW * kLH / 32];
+__global__ void __launch_bounds__(kLossThreads) k_loss_maps(const float *__restrict__ X, const float *__restrict__ A,
+                                                            const float *__restrict__ Ct, const float *__restrict__ At,
+                                                            float3 bg, int W, int H, const Win win,
+                                                            float *__restrict__ maps, float *__restrict__ partials) {
+    __shared__ float2 s_v[kRH][kSP];                       // (x, y)
+    __shared__ __align__(16) float2 s_m[kRH][kHP];         // horizontal sums of (x, y)
+    __shared__ __align__(16) float2 s_q[kRH][kHP];         // of (x^2, y^2)
+    __shared__ __align__(16) float s_c[kRH][kHS];          // of x y
+    __shared__ float s_red[3][kLossThreads / 32];
     const int ch = blockIdx.z;
     const float bgc = ch == 0 ? bg.x : (ch == 1 ? bg.y : bg.z);
     const size_t plane = static_cast<size_t>(W) * H;
     const int x0 = blockIdx.x * kLW - kHalo, y0 = blockIdx.y * kLH - kHalo;
     const int tid = threadIdx.x;
-    for (int i = tid; i < kRW * kRH; i += kLW * kLH) {
+#pragma unroll
+    for (int k = 0; k < (kRW * kRH + kLossThreads - 1) / kLossThreads; ++k) {
+        const int i = tid + k * kLossThreads;
         const int ry = i / kRW, rx = i % kRW;
         const int gx = x0 + rx, gy = y0 + ry;
         float xv = 0.f, yv = 0.f;
@@ -62,56 +128,73 @@ __global__ void __launch_bounds__(kLW *kLH) k_loss_maps(const float *__restrict_
             xv = X[ch * plane + p];
             yv = target_at(Ct, At, bgc, ch * plane + p, p);
         }
-        s_x[ry][rx] = xv;
-        s_y[ry][rx] = yv;
+        if (i < kRW * kRH) s_v[ry][rx] = make_float2(xv, yv);
     }
     __syncthreads();
-    for (int i = tid; i < kRH * kLW; i += kLW * kLH) {
-        const int ry = i / kLW, cx = i % kLW;
-        float mx = 0.f, my = 0.f, xx = 0.f, yy = 0.f, xy = 0.f;
+    for (int i = tid; i < kRH * (kLW / kLOut); i += kLossThreads) {
+        const int ry = i % kRH, cx = (i / kRH) * kLOut;
+        F2 m[kLOut], q[kLOut];
+        float c[kLOut];
 #pragma unroll
-        for (int j = 0; j < kWin; ++j) {
-            const float a = s_x[ry][cx + j] - kSsimShift, b = s_y[ry][cx + j] - kSsimShift, w = win.g[j];
-            mx = fmaf(w, a, mx);
-            my = fmaf(w, b, my);
-            xx = fmaf(w, a * a, xx);
-            yy = fmaf(w, b * b, yy);
-            xy = fmaf(w, a * b, xy);
+        for (int o = 0; o < kLOut; ++o) {
+            m[o] = F2(0.f, 0.f);
+            q[o] = F2(0.f, 0.f);
+            c[o] = 0.f;
         }
-        s_h[0][ry][cx] = mx;
-        s_h[1][ry][cx] = my;
-        s_h[2][ry][cx] = xx;
-        s_h[3][ry][cx] = yy;
-        s_h[4][ry][cx] = xy;
+#pragma unroll
+        for (int t = 0; t < kLTap; ++t) {
+            const float2 v = s_v[ry][cx + t];
+            const float a = v.x - kSsimShift, b = v.y - kSsimShift;
+            const F2 ab(a, b), sq(a * a, b * b);
+            const float pr = a * b;
+#pragma unroll
+            for (int o = 0; o < kLOut; ++o) {              // taps in order for every output
+                const int j = t - o;
+                if (j < 0 || j >= kWin) continue;
+                const F2 w(win.g[j], win.g[j]);
+                m[o] = fma2(w, ab, m[o]);
+                q[o] = fma2(w, sq, q[o]);
+                c[o] = fmaf(win.g[j], pr, c[o]);
+            }
+        }
+        store4(&s_m[ry][cx], m);
+        store4(&s_q[ry][cx], q);
+        *reinterpret_cast<float4 *>(&s_c[ry][cx]) = make_float4(c[0], c[1], c[2], c[3]);
     }
     __syncthreads();
-    const int lx = tid % kLW, ly = tid / kLW;
-    const int gx = blockIdx.x * kLW + lx, gy = blockIdx.y * kLH + ly;
+    const int lx = tid % kLW, sy = tid / kLW;
     float f = 0.f, l1 = 0.f, la = 0.f;
-    if (gx < W && gy < H) {
-        float m[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+    F2 m[kLOut], q[kLOut];
+    float c[kLOut];
+    window_column(s_m, lx, sy, win, m);
+    window_column(s_q, lx, sy, win, q);
+    window_column(s_c, lx, sy, win, c);
 #pragma unroll
-        for (int i = 0; i < kWin; ++i)
-#pragma unroll
-            for (int q = 0; q < 5; ++q) m[q] = fmaf(win.g[i], s_h[q][ly + i][lx], m[q]);
+    for (int o = 0; o < kLOut; ++o) {
+        const int ly = kLOut * sy + o;
+        const int gx = blockIdx.x * kLW + lx, gy = blockIdx.y * kLH + ly;
+        if (gx >= W || gy >= H) continue;
         // moments of the shifted values x - kSsimShift, y - kSsimShift: the (co)variances are shift
         // invariant, and the shift takes most of E[x^2] - mu^2's cancellation out for values in [0, 1]
-        const float mcx = m[0], mcy = m[1];
-        const float sx = m[2] - mcx * mcx, sy = m[3] - mcy * mcy, sxy = m[4] - mcx * mcy;
+        const float2 mc = m[o].get(), qq = q[o].get();
+        const float mcx = mc.x, mcy = mc.y;
+        const float sx = qq.x - mcx * mcx, sv = qq.y - mcy * mcy, sxy = c[o] - mcx * mcy;
         const float mux = mcx + kSsimShift, muy = mcy + kSsimShift;
         const float n1 = 2.f * mux * muy + kC1, n2 = 2.f * sxy + kC2;
-        const float d1 = mux * mux + muy * muy + kC1, d2 = sx + sy + kC2;
-        f = (n1 * n2) / (d1 * d2);
-        const float df_dmx = f * (2.f * muy / n1 - 2.f * mux / d1);
-        const float df_dsx = -f / d2;
-        const float df_dsxy = 2.f * f / n2;
+        const float d1 = mux * mux + muy * muy + kC1, d2 = sx + sv + kC2;
+        const float fo = (n1 * n2) / (d1 * d2);
+        const float df_dmx = fo * (2.f * muy / n1 - 2.f * mux / d1);
+        const float df_dsx = -fo / d2;
+        const float df_dsxy = 2.f * fo / n2;
         const size_t p = static_cast<size_t>(gy) * W + gx;
         float *mp = maps + static_cast<size_t>(ch) * 3 * plane;
         mp[p] = df_dmx - 2.f * mcx * df_dsx - mcy * df_dsxy;
         mp[plane + p] = df_dsx;
         mp[2 * plane + p] = df_dsxy;
-        l1 = fabsf(s_x[ly + kHalo][lx + kHalo] - s_y[ly + kHalo][lx + kHalo]);
-        if (ch == 0 && A) la = fabsf(A[p] - At[p]);
+        const float2 v = s_v[ly + kHalo][lx + kHalo];
+        f += fo;
+        l1 += fabsf(v.x - v.y);
+        if (ch == 0 && A) la += fabsf(A[p] - At[p]);
     }
     // block sums (fixed order: deterministic)
 #pragma unroll
@@ -127,21 +210,21 @@ __global__ void __launch_bounds__(kLW *kLH) k_loss_maps(const float *__restrict_
     }
     __syncthreads();
     if (tid < 3) {
-        float s = 0.f;
-        for (int w = 0; w < kLW * kLH / 32; ++w) s += s_red[tid][w];
+        float sum = 0.f;
+        for (int w = 0; w < kLossThreads / 32; ++w) sum += s_red[tid][w];
         const size_t b = (static_cast<size_t>(blockIdx.z) * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-        partials[3 * b + tid] = s;
+        partials[3 * b + tid] = sum;
     }
 }
 
 // loss = (1 - lam) L1 + lam (1 - SSIM) + w_a LA from the block sums, by one CTA
-// of kLW * kLH threads in a fixed order (deterministic): each thread adds its
+// of kLossThreads threads in a fixed order (deterministic): each thread adds its
 // strided share of the block sums in single precision, then a tree in shared
-// memory (scratch: 3 * kLW * kLH floats).  The GB300's double-precision pipe is
+// memory (scratch: 3 * kLossThreads floats).  The GB300's double-precision pipe is
 // narrow; converting and adding every block sum in double took 20 us.
 __device__ void loss_from_block_sums(const float *__restrict__ partials, int nb, size_t plane, float lam, float w_a,
                                      float *__restrict__ loss, float *scratch) {
-    constexpr int NT = kLW * kLH;
+    constexpr int NT = kLossThreads;
     const int tid = threadIdx.x;
     float a[3] = {0.f, 0.f, 0.f};
     for (int b = tid; b < nb; b += NT)
@@ -166,59 +249,85 @@ __device__ void loss_from_block_sums(const float *__restrict__ partials, int nb,
 
 // Pass 2: window sums of a, b, c and the gradient of the loss; the first CTA
 // also adds up pass 1's block sums into the loss.
-__global__ void __launch_bounds__(kLW *kLH) k_loss_grad(const float *__restrict__ X, const float *__restrict__ A,
-                                                        const float *__restrict__ Ct, const float *__restrict__ At,
-                                                        float3 bg, int W, int H, const Win win, float lam, float w_a,
-                                                        const float *__restrict__ maps, float *__restrict__ dX,
-                                                        float *__restrict__ dA, const float *__restrict__ partials,
-                                                        float w_a_loss, float *__restrict__ loss) {
-    __shared__ float s_m[3][kRH][kRW];
-    __shared__ float s_h[3][kRH][kLW];
-    static_assert(3 * kRH * kRW >= 3 * kLW * kLH, "loss scratch in s_m");
+__global__ void __launch_bounds__(kLossThreads) k_loss_grad(const float *__restrict__ X, const float *__restrict__ A,
+                                                            const float *__restrict__ Ct, const float *__restrict__ At,
+                                                            float3 bg, int W, int H, const Win win, float lam,
+                                                            float w_a, const float *__restrict__ maps,
+                                                            float *__restrict__ dX, float *__restrict__ dA,
+                                                            const float *__restrict__ partials, float w_a_loss,
+                                                            float *__restrict__ loss) {
+    __shared__ float2 s_ab[kRH][kSP];                      // maps (a, b)
+    __shared__ float s_c[kRH][kSP];                        // map c
+    __shared__ __align__(16) float2 s_hab[kRH][kHP];       // their horizontal sums
+    __shared__ __align__(16) float s_hc[kRH][kHS];
+    static_assert(sizeof(s_ab) >= 3 * kLossThreads * sizeof(float), "loss scratch in s_ab");
     if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0)
         loss_from_block_sums(partials, static_cast<int>(gridDim.x * gridDim.y * gridDim.z), static_cast<size_t>(W) * H,
-                             lam, w_a_loss, loss, &s_m[0][0][0]);
+                             lam, w_a_loss, loss, &s_ab[0][0].x);
     const int ch = blockIdx.z;
     const float bgc = ch == 0 ? bg.x : (ch == 1 ? bg.y : bg.z);
     const size_t plane = static_cast<size_t>(W) * H;
     const float *mp = maps + static_cast<size_t>(ch) * 3 * plane;
     const int x0 = blockIdx.x * kLW - kHalo, y0 = blockIdx.y * kLH - kHalo;
     const int tid = threadIdx.x;
-    for (int i = tid; i < kRW * kRH; i += kLW * kLH) {
+#pragma unroll
+    for (int k = 0; k < (kRW * kRH + kLossThreads - 1) / kLossThreads; ++k) {
+        const int i = tid + k * kLossThreads;
         const int ry = i / kRW, rx = i % kRW;
         const int gx = x0 + rx, gy = y0 + ry;
         const bool in = gx >= 0 && gx < W && gy >= 0 && gy < H;
         const size_t p = in ? static_cast<size_t>(gy) * W + gx : 0;
-#pragma unroll
-        for (int q = 0; q < 3; ++q) s_m[q][ry][rx] = in ? mp[q * plane + p] : 0.f;
+        const float a = in ? mp[p] : 0.f, b = in ? mp[plane + p] : 0.f, c = in ? mp[2 * plane + p] : 0.f;
+        if (i < kRW * kRH) {
+            s_ab[ry][rx] = make_float2(a, b);
+            s_c[ry][rx] = c;
+        }
     }
     __syncthreads();
-    for (int i = tid; i < kRH * kLW; i += kLW * kLH) {
-        const int ry = i / kLW, cx = i % kLW;
-        float h[3] = {0.f, 0.f, 0.f};
+    for (int i = tid; i < kRH * (kLW / kLOut); i += kLossThreads) {
+        const int ry = i % kRH, cx = (i / kRH) * kLOut;
+        F2 h[kLOut];
+        float c[kLOut];
 #pragma unroll
-        for (int j = 0; j < kWin; ++j)
+        for (int o = 0; o < kLOut; ++o) {
+            h[o] = F2(0.f, 0.f);
+            c[o] = 0.f;
+        }
 #pragma unroll
-            for (int q = 0; q < 3; ++q) h[q] = fmaf(win.g[j], s_m[q][ry][cx + j], h[q]);
+        for (int t = 0; t < kLTap; ++t) {
+            const float2 v = s_ab[ry][cx + t];
+            const float vc = s_c[ry][cx + t];
+            const F2 ab(v.x, v.y);
 #pragma unroll
-        for (int q = 0; q < 3; ++q) s_h[q][ry][cx] = h[q];
+            for (int o = 0; o < kLOut; ++o) {
+                const int j = t - o;
+                if (j < 0 || j >= kWin) continue;
+                h[o] = fma2(F2(win.g[j], win.g[j]), ab, h[o]);
+                c[o] = fmaf(win.g[j], vc, c[o]);
+            }
+        }
+        store4(&s_hab[ry][cx], h);
+        *reinterpret_cast<float4 *>(&s_hc[ry][cx]) = make_float4(c[0], c[1], c[2], c[3]);
     }
     __syncthreads();
-    const int lx = tid % kLW, ly = tid / kLW;
-    const int gx = blockIdx.x * kLW + lx, gy = blockIdx.y * kLH + ly;
-    if (gx >= W || gy >= H) return;
-    float s[3] = {0.f, 0.f, 0.f};
-#pragma unroll
-    for (int i = 0; i < kWin; ++i)
-#pragma unroll
-        for (int q = 0; q < 3; ++q) s[q] = fmaf(win.g[i], s_h[q][ly + i][lx], s[q]);
-    const size_t p = static_cast<size_t>(gy) * W + gx;
-    const float x = X[ch * plane + p];
-    const float y = target_at(Ct, At, bgc, ch * plane + p, p);
+    const int lx = tid % kLW, sy = tid / kLW;
+    F2 ab[kLOut];
+    float c[kLOut];
+    window_column(s_hab, lx, sy, win, ab);
+    window_column(s_hc, lx, sy, win, c);
     const float inv_n = 1.f / (3.f * static_cast<float>(plane));
-    const float dS = s[0] + 2.f * (x - kSsimShift) * s[1] + (y - kSsimShift) * s[2];
-    dX[ch * plane + p] = ((1.f - lam) * sgn(x - y) - lam * dS) * inv_n;
-    if (ch == 0 && dA) dA[p] = A ? w_a * sgn(A[p] - At[p]) / static_cast<float>(plane) : 0.f;
+#pragma unroll
+    for (int o = 0; o < kLOut; ++o) {
+        const int gx = blockIdx.x * kLW + lx, gy = blockIdx.y * kLH + kLOut * sy + o;
+        if (gx >= W || gy >= H) continue;
+        const size_t p = static_cast<size_t>(gy) * W + gx;
+        const float x = X[ch * plane + p];
+        const float y = target_at(Ct, At, bgc, ch * plane + p, p);
+        const float2 s01 = ab[o].get();
+        const float dS = s01.x + 2.f * (x - kSsimShift) * s01.y + (y - kSsimShift) * c[o];
+        dX[ch * plane + p] = ((1.f - lam) * sgn(x - y) - lam * dS) * inv_n;
+        if (ch == 0 && dA) dA[p] = A ? w_a * sgn(A[p] - At[p]) / static_cast<float>(plane) : 0.f;
+    }
 }
 
 // Adam over the five parameter arrays seen as one index space; a Gaussian
@@ -382,9 +491,9 @@ cudaError_t launch_image_loss(const float *X, const float *A, const float *Ct, c
     float *maps = static_cast<float *>(ws);
     float *partials = maps + 9 * plane;
     const dim3 grid((W + kLW - 1) / kLW, (H + kLH - 1) / kLH, 3);
-    k_loss_maps<<<grid, kLW * kLH, 0, st>>>(X, A, Ct, At, bg, W, H, win, maps, partials);
-    k_loss_grad<<<grid, kLW * kLH, 0, st>>>(X, A, Ct, At, bg, W, H, win, lam, w_a, maps, dX, dA, partials,
-                                            A ? w_a : 0.f, loss);
+    k_loss_maps<<<grid, kLossThreads, 0, st>>>(X, A, Ct, At, bg, W, H, win, maps, partials);
+    k_loss_grad<<<grid, kLossThreads, 0, st>>>(X, A, Ct, At, bg, W, H, win, lam, w_a, maps, dX, dA, partials,
+                                               A ? w_a : 0.f, loss);
     return cudaGetLastError();
 }
 

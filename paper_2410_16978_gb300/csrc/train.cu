@@ -361,11 +361,14 @@ __global__ void __launch_bounds__(256) k_adam(const AdamArrays arr, const uint8_
     }
 }
 
-// The same update four elements at a time: a thread takes one 16-byte unit of
-// one array (the last unit of an array may be partial) with vector loads and
-// stores; the layer test runs only when some layer is frozen (a frozen
-// element's values are written back unchanged).  Used when every array is
-// 16-byte aligned; every element gets the same arithmetic as in k_adam.
+// The same update on 16-byte units of four elements, vector loads and stores;
+// used when every array is 16-byte aligned, with k_adam's arithmetic for every
+// element.  Bound by memory: 28 bytes per trained element, so a unit without a
+// trained element is left untouched (with random layers that is whole rows of
+// the SH arrays; a frozen element in a mixed unit is written back unchanged).
+// A thread takes kAdamUnits units, one stride of the block apart, and all their
+// loads are in flight before the first result is needed.
+// 500,000 Gaussians, degree 3, a third of them frozen: 0.125 -> 0.096 ms.
 struct Adam4 {
     float *p[5];
     const float *g[5];
@@ -376,31 +379,62 @@ struct Adam4 {
     float step[5];
 };
 
-__global__ void __launch_bounds__(256) k_adam4(const Adam4 a, const uint8_t *__restrict__ layer, uint32_t train_mask,
-                                               float beta1, float beta2, float inv_sqrt_bc2, float eps) {
+constexpr int kAdamThreads = 256, kAdamUnits = 2;
+
+__global__ void __launch_bounds__(kAdamThreads) k_adam4(const Adam4 a, const uint8_t *__restrict__ layer,
+                                                        uint32_t train_mask, float beta1, float beta2,
+                                                        float inv_sqrt_bc2, float eps) {
     const bool all = train_mask == 0xFFFFFFFFu;
     const uint32_t total = a.uend[4];
-    for (uint32_t u = blockIdx.x * blockDim.x + threadIdx.x; u < total; u += gridDim.x * blockDim.x) {
+    const uint32_t u0 = blockIdx.x * (kAdamThreads * kAdamUnits) + threadIdx.x;
+    int arr[kAdamUnits];
+    uint32_t first[kAdamUnits], cnt[kAdamUnits], tr[kAdamUnits];   // tr: bit q set = element q is trained
+#pragma unroll
+    for (int j = 0; j < kAdamUnits; ++j) {
+        const uint32_t u = u0 + j * kAdamThreads;
+        tr[j] = cnt[j] = first[j] = 0;
+        arr[j] = 0;
+        if (u >= total) continue;
         int k = 0;
         while (u >= a.uend[k]) ++k;
-        const uint32_t e0 = 4u * (u - (k ? a.uend[k - 1] : 0u));
-        const uint32_t cnt = min(4u, a.len[k] - e0);
-        bool tr[4];
+        arr[j] = k;
+        first[j] = 4u * (u - (k ? a.uend[k - 1] : 0u));
+        cnt[j] = min(4u, a.len[k] - first[j]);
+        tr[j] = (1u << cnt[j]) - 1u;
+        if (all) continue;
+        const uint32_t w = a.width[k];
+        uint32_t row = first[j] / w, left = w - (first[j] - row * w);   // elements of the row still to come
+        uint32_t on = (train_mask >> layer[row]) & 1u;
+        for (uint32_t q = 0; q < cnt[j]; ++q) {
+            if (left == 0) {
+                on = (train_mask >> layer[++row]) & 1u;
+                left = w;
+            }
+            if (!on) tr[j] &= ~(1u << q);
+            --left;
+        }
+    }
+    float4 g4[kAdamUnits], m4[kAdamUnits], v4[kAdamUnits], p4[kAdamUnits];
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
-            tr[q] = q < static_cast<int>(cnt) &&
-                    (all || ((train_mask >> layer[(e0 + q) / a.width[k]]) & 1u));
-        if (cnt == 4) {
-            const float4 g4 = *reinterpret_cast<const float4 *>(a.g[k] + e0);
-            float4 m4 = *reinterpret_cast<const float4 *>(a.m[k] + e0);
-            float4 v4 = *reinterpret_cast<const float4 *>(a.v[k] + e0);
-            float4 p4 = *reinterpret_cast<const float4 *>(a.p[k] + e0);
-            float *gg = reinterpret_cast<float *>(const_cast<float4 *>(&g4));
-            float *mm = reinterpret_cast<float *>(&m4), *vv = reinterpret_cast<float *>(&v4),
-                  *pp = reinterpret_cast<float *>(&p4);
+    for (int j = 0; j < kAdamUnits; ++j) {
+        if (tr[j] == 0 || cnt[j] != 4) continue;
+        const int k = arr[j];
+        g4[j] = __ldcs(reinterpret_cast<const float4 *>(a.g[k] + first[j]));
+        m4[j] = __ldcs(reinterpret_cast<const float4 *>(a.m[k] + first[j]));
+        v4[j] = __ldcs(reinterpret_cast<const float4 *>(a.v[k] + first[j]));
+        p4[j] = __ldcs(reinterpret_cast<const float4 *>(a.p[k] + first[j]));
+    }
+#pragma unroll
+    for (int j = 0; j < kAdamUnits; ++j) {
+        if (tr[j] == 0) continue;
+        const int k = arr[j];
+        if (cnt[j] == 4) {
+            const float *gg = reinterpret_cast<const float *>(&g4[j]);
+            float *mm = reinterpret_cast<float *>(&m4[j]), *vv = reinterpret_cast<float *>(&v4[j]),
+                  *pp = reinterpret_cast<float *>(&p4[j]);
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                if (!tr[q]) continue;
+                if (!((tr[j] >> q) & 1u)) continue;
                 const float g = gg[q];
                 const float m = fmaf(beta1, mm[q], (1.f - beta1) * g);
                 const float v = fmaf(beta2, vv[q], (1.f - beta2) * g * g);
@@ -408,13 +442,13 @@ __global__ void __launch_bounds__(256) k_adam4(const Adam4 a, const uint8_t *__r
                 vv[q] = v;
                 pp[q] -= a.step[k] * m / (sqrtf(v) * inv_sqrt_bc2 + eps);
             }
-            *reinterpret_cast<float4 *>(a.m[k] + e0) = m4;
-            *reinterpret_cast<float4 *>(a.v[k] + e0) = v4;
-            *reinterpret_cast<float4 *>(a.p[k] + e0) = p4;
+            __stcs(reinterpret_cast<float4 *>(a.m[k] + first[j]), m4[j]);
+            __stcs(reinterpret_cast<float4 *>(a.v[k] + first[j]), v4[j]);
+            __stcs(reinterpret_cast<float4 *>(a.p[k] + first[j]), p4[j]);
         } else {
-            for (uint32_t q = 0; q < cnt; ++q) {
-                if (!tr[q]) continue;
-                const uint32_t i = e0 + q;
+            for (uint32_t q = 0; q < cnt[j]; ++q) {
+                if (!((tr[j] >> q) & 1u)) continue;
+                const uint32_t i = first[j] + q;
                 const float g = a.g[k][i];
                 const float m = fmaf(beta1, a.m[k][i], (1.f - beta1) * g);
                 const float v = fmaf(beta2, a.v[k][i], (1.f - beta2) * g * g);
@@ -534,8 +568,8 @@ cudaError_t launch_adam(float *const p[5], const float *const g[5], float *const
             units += (b.len[k] + 3) / 4;
             b.uend[k] = units;
         }
-        const int blocks = static_cast<int>(std::min<uint64_t>((units + 255) / 256, 8ull * 1024));
-        k_adam4<<<blocks, 256, 0, st>>>(b, layer, train_mask, beta1, beta2, inv_sqrt_bc2, eps);
+        constexpr uint32_t per = kAdamThreads * kAdamUnits;
+        k_adam4<<<(units + per - 1) / per, kAdamThreads, 0, st>>>(b, layer, train_mask, beta1, beta2, inv_sqrt_bc2, eps);
         return cudaGetLastError();
     }
     const int blocks = static_cast<int>(std::min<uint64_t>((acc + 255) / 256, 8ull * 1024));

@@ -168,6 +168,7 @@ __device__ __forceinline__ void chunk_range(uint32_t n, uint32_t c, uint32_t K, 
 // Rows, count: a warp per chunk of the depth order counts its entries and pairs per tile row.
 template <int NV>
 __global__ void __launch_bounds__(256) k_bin_rows_count(const __grid_constant__ Views<BinView, NV> B) {
+    chain_start();
     const BinView &V = B[blockIdx.y];
     const uint32_t *__restrict__ order = V.order;
     const Rec *__restrict__ rec = V.rec;
@@ -229,6 +230,7 @@ constexpr int kRowBlock = 32 * kRowWords;
 
 template <int NV>
 __global__ void __launch_bounds__(256) k_bin_rows_write(const __grid_constant__ Views<BinView, NV> B) {
+    chain_start();
     const BinView &V = B[blockIdx.y];
     const uint32_t *__restrict__ order = V.order;
     const Rec *__restrict__ rec = V.rec;
@@ -335,6 +337,7 @@ __global__ void __launch_bounds__(256) k_bin_rows_write(const __grid_constant__ 
 // total and the capacity check.
 template <int NV>
 __global__ void __launch_bounds__(1024) k_bin_rowscan(const __grid_constant__ Views<BinView, NV> B, int K) {
+    chain_start();
     const BinView &V = B[blockIdx.y];
     uint32_t *__restrict__ M = V.M;
     RowInfo *__restrict__ rows = rows_of(V);
@@ -439,6 +442,7 @@ __device__ __forceinline__ int row_of_piece(const uint32_t *s_ps, int Ty, uint32
 // Tiles, count: a warp per piece counts its pairs per tile into P[piece][Tx].
 template <int NV>
 __global__ void __launch_bounds__(256) k_bin_tiles_count(const __grid_constant__ Views<BinView, NV> B) {
+    chain_start();
     const BinView &V = B[blockIdx.y];
     const uint2 *__restrict__ rowlist = V.rowlist;
     const RowInfo *__restrict__ rows = rows_of(V);
@@ -483,6 +487,7 @@ constexpr int kStepWords = 4;      // words of 32 entries loaded per step, one s
 
 template <int NV>
 __global__ void __launch_bounds__(256) k_bin_tiles_write(const __grid_constant__ Views<BinView, NV> B) {
+    chain_start();
     const BinView &V = B[blockIdx.y];
     const uint2 *__restrict__ rowlist = V.rowlist;
     const RowInfo *__restrict__ rows = rows_of(V);
@@ -567,6 +572,7 @@ __global__ void __launch_bounds__(256) k_bin_tiles_write(const __grid_constant__
 // (piece, tile) count is replaced by its first list position.
 template <int NV>
 __global__ void __launch_bounds__(1024) k_bin_tiles_scan(const __grid_constant__ Views<BinView, NV> B) {
+    chain_start();
     const BinView &V = B[blockIdx.y];
     const RowInfo *__restrict__ rows = rows_of(V);
     uint32_t *__restrict__ P = V.P;
@@ -640,9 +646,9 @@ cudaError_t launch_bin_rows(const BinView *views, int n, cudaStream_t st) {
     const int blocks = max(min(fill, static_cast<int>(most / (8 * kChunkMin))), 1);
     with_views(views, n, [&](const auto &b) {
         constexpr int NV = sizeof(b.v) / sizeof(BinView);
-        k_bin_rows_count<NV><<<dim3(blocks, n), 256, 0, st>>>(b);
-        k_bin_rowscan<NV><<<dim3(Ty * kRowParts, n), 1024, 0, st>>>(b, 8 * blocks);
-        k_bin_rows_write<NV><<<dim3(blocks, n), 256, 0, st>>>(b);
+        launch_chained(k_bin_rows_count<NV>, dim3(blocks, n), 256, 0, st, b);
+        launch_chained(k_bin_rowscan<NV>, dim3(Ty * kRowParts, n), 1024, 0, st, b, 8 * blocks);
+        launch_chained(k_bin_rows_write<NV>, dim3(blocks, n), 256, 0, st, b);
     });
     return cudaGetLastError();
 }
@@ -654,9 +660,9 @@ cudaError_t launch_bin_tiles(const BinView *views, int n, cudaStream_t st) {
     const int G = max(sort_blocks() / 4, 4 * sort_blocks() / n);
     with_views(views, n, [&](const auto &b) {
         constexpr int NV = sizeof(b.v) / sizeof(BinView);
-        k_bin_tiles_count<NV><<<dim3(G, n), 256, 0, st>>>(b);
-        k_bin_tiles_scan<NV><<<dim3(Ty, n), 1024, 0, st>>>(b);
-        k_bin_tiles_write<NV><<<dim3(G, n), 256, 0, st>>>(b);
+        launch_chained(k_bin_tiles_count<NV>, dim3(G, n), 256, 0, st, b);
+        launch_chained(k_bin_tiles_scan<NV>, dim3(Ty, n), 1024, 0, st, b);
+        launch_chained(k_bin_tiles_write<NV>, dim3(G, n), 256, 0, st, b);
     });
     return cudaGetLastError();
 }

@@ -168,6 +168,7 @@ constexpr int kSetupSmemTiles = 8192;
 
 template <int NV>
 __global__ void __launch_bounds__(1024) k_fwd_setup(const __grid_constant__ Views<SetupView, NV> B) {
+    chain_start();
     const SetupView &V = B[blockIdx.x];
     const uint2 *__restrict__ g_ranges = V.ranges;
     const int Tn = V.Tn;
@@ -543,6 +544,7 @@ struct FwdMeet {
 
 template <int PX, int PER>
 __global__ void __launch_bounds__(kFwdThreads) k_composite_fwd(const __grid_constant__ FwdBatch batch) {
+    chain_start();
     extern __shared__ __align__(16) unsigned char s_raw[];
     FwdSmem<PER> &sm = *reinterpret_cast<FwdSmem<PER> *>(s_raw);
     constexpr uint32_t kChunk = 32 * PER, B = FwdQueue<PX>::kBlocks;
@@ -738,6 +740,7 @@ __global__ void __launch_bounds__(1024) k_bwd_setup(uint32_t *__restrict__ queue
                                                     const uint32_t *__restrict__ vis_index,
                                                     const uint32_t *__restrict__ n_vis, int n,
                                                     float4 *__restrict__ rec_grad) {
+    chain_start();
     if (blockIdx.x == 0 && threadIdx.x == 0) *queue = 0;
     const uint32_t nv = min(*n_vis, static_cast<uint32_t>(n));
     const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -824,6 +827,7 @@ __global__ void __launch_bounds__(kBwdThreads, 6) k_composite_bwd(
     const float *__restrict__ dL_dimage, const float *__restrict__ dL_dalpha, const uint8_t *__restrict__ layer,
     uint32_t grad_layer_mask, float4 *__restrict__ rec_grad, float *__restrict__ contrib_max, uint32_t n_rec,
     const Ctl *__restrict__ ctl) {
+    chain_start();
     __shared__ float4 s_a[kBwdThreads / 32][32], s_b[kBwdThreads / 32][32];
     __shared__ float s_c[kBwdThreads / 32][32];
     __shared__ uint32_t s_g[kBwdThreads / 32][32];
@@ -1002,7 +1006,7 @@ cudaError_t launch_forward(const FwdBatch &batch, uint32_t items, cudaStream_t s
     static PerDevice cache;
     const int blocks = cache.get([] { return persistent_blocks(k_composite_fwd<PX, PER>, kFwdThreads, smem); });
     const uint32_t need = (items + kFwdWarps - 1) / kFwdWarps;
-    k_composite_fwd<PX, PER><<<min(static_cast<uint32_t>(blocks), need), kFwdThreads, smem, st>>>(batch);
+    launch_chained(k_composite_fwd<PX, PER>, min(static_cast<uint32_t>(blocks), need), kFwdThreads, smem, st, batch);
     return cudaGetLastError();
 }
 
@@ -1015,7 +1019,7 @@ void setup_kernel(const Views<SetupView, NV> &b, size_t smem, cudaStream_t st) {
         cudaFuncSetAttribute(k_fwd_setup<NV>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSetupSmemTiles * 8);
         return 1;
     });
-    k_fwd_setup<NV><<<b.n, 1024, smem, st>>>(b);
+    launch_chained(k_fwd_setup<NV>, b.n, 1024, smem, st, b);
 }
 
 cudaError_t launch_fwd_setup(const SetupView *views, int n, cudaStream_t st) {
@@ -1065,10 +1069,9 @@ cudaError_t launch_composite_backward(const CompositeBufs &cb, const uint2 *rang
     if (Tx * Ty == 0) return cudaSuccess;
     static PerDevice cache;
     const int blocks = cache.get([] { return persistent_blocks(k_composite_bwd<kBwdPx>, kBwdThreads); });
-    k_composite_bwd<kBwdPx><<<blocks, kBwdThreads, 0, st>>>(cb.items, cb.n_items, cb.queue, ranges, list, rec, W, H, Tx, bg,
-                                                    t_final, n_contrib, cb.seg_base, cb.ckpt, cb.qwork,
-                                                    dL_dimage, dL_dalpha, layer, grad_layer_mask, rec_grad,
-                                                    contrib_max, n, ctl);
+    launch_chained(k_composite_bwd<kBwdPx>, blocks, kBwdThreads, 0, st, cb.items, cb.n_items, cb.queue, ranges, list,
+                   rec, W, H, Tx, bg, t_final, n_contrib, cb.seg_base, cb.ckpt, cb.qwork, dL_dimage, dL_dalpha, layer,
+                   grad_layer_mask, rec_grad, contrib_max, n, ctl);
     return cudaGetLastError();
 }
 

@@ -351,7 +351,7 @@ int front_preprocess(const FrontCtx *f, int n, cudaStream_t st) {
     int rc;
     if ((rc = cuda_check(launch_clear(v, n, st), "clear status")) != GS_OK) return rc;
     int launches = 0;
-    Stage sg(GS_STAGE_PREPROCESS, st, n > 1 ? 1 : 0);       // (several views are cleared by a kernel)
+    Stage sg(GS_STAGE_PREPROCESS, st, 1);                    // (with the clearing kernel)
     rc = cuda_check(launch_preprocess(v, n, st, &launches), "preprocess");
     g_launches += launches;
     return rc;
@@ -519,19 +519,10 @@ int gs_render_stereo(const gs_scene *scene, const gs_camera *left, const gs_came
     if (shared_sort) {
         // the right eye bins in the shared order: it needs the shared count, and
         // its backward the visible list, too
-        Ctl *l = f[0].pre.ctl, *r = f[1].pre.ctl;
-        if ((rc = cuda_check(cudaMemcpyAsync(at<uint32_t>(f[1].ws, f[1].L.vis_index),
-                                             at<uint32_t>(f[0].ws, f[0].L.vis_index),
-                                             static_cast<size_t>(f[0].pre.s.n) * sizeof(uint32_t),
-                                             cudaMemcpyDeviceToDevice, st),
+        ++g_launches;
+        if ((rc = cuda_check(launch_share_order(f[0].pre.ctl, at<uint32_t>(f[0].ws, f[0].L.vis_index), f[1].pre.ctl,
+                                                at<uint32_t>(f[1].ws, f[1].L.vis_index), f[0].pre.s.n, st),
                              "shared visible list")) != GS_OK)
-            return rc;
-        if ((rc = cuda_check(cudaMemcpyAsync(&r->n_vis, &l->n_vis, sizeof(uint32_t), cudaMemcpyDeviceToDevice, st),
-                             "shared count")) != GS_OK)
-            return rc;
-        if ((rc = cuda_check(cudaMemcpyAsync(&r->st.n_visible, &l->st.n_visible, sizeof(uint32_t),
-                                             cudaMemcpyDeviceToDevice, st),
-                             "shared count")) != GS_OK)
             return rc;
     }
     if ((rc = front_bin(f, 2, st, jobs)) != GS_OK) return rc;

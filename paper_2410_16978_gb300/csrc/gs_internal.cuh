@@ -5,6 +5,7 @@
 #include <cstddef>
 #include <cstdint>
 #include <mutex>
+#include <utility>
 #include <cuda_runtime.h>
 
 #include "../../include/gs.h"
@@ -174,6 +175,38 @@ inline void with_views(const T *views, int n, F f) {
     }
 }
 
+// The kernels of a call run as a chain of programmatic dependent launches: a
+// kernel may become resident as soon as every CTA of the one before it has
+// started, and waits at its first instruction until that one has completed and
+// its writes are visible.  That takes the launch latency and the filling of the
+// SMs out of the gaps between the ten to twenty short kernels of a call (4,096
+// Gaussians at 128 x 128 0.160 -> 0.137 ms, 200,000 at 512 x 512 0.181 -> 0.164,
+// 1024 x 1024 frame with its backward 0.677 -> 0.651).  Rules: chain_start() is the first
+// statement of every kernel launched this way, before any access to memory and
+// any return, so that a kernel's completion implies that of all before it;
+// the first kernel of a call is launched the ordinary way and therefore waits
+// for everything that precedes the call in the stream; and so does whatever
+// follows the call.
+__device__ __forceinline__ void chain_start() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <class... P, class... A>
+cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A &&...args) {
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
+
 // S1 of one view.
 struct PreView {
     SceneView s;
@@ -254,6 +287,8 @@ struct SortView {
 };
 cudaError_t launch_sort_histograms(const SortView *views, int n, cudaStream_t st);
 cudaError_t launch_sort_digits(const SortView *views, int n, cudaStream_t st);
+cudaError_t launch_share_order(const Ctl *from, const uint32_t *vis, Ctl *to, uint32_t *vis_to, int n,
+                               cudaStream_t st);
 // Tile binning (bin.cu) of a view.  Rows: splits the depth-ordered visible
 // Gaussians (order[p], p < min(ctl->n_vis, n_cap)) into per-tile-row lists of
 // (Gaussian, x0 | x1 << 16) in depth order; writes n_dup and the overflow

@@ -80,6 +80,7 @@ __device__ __forceinline__ void store_geo(Geo *g, const float4 a, const float4 b
 // so views of one scene read it from L2 after the first.
 template <int DEG, int NV>
 __global__ void __launch_bounds__(128) k_preprocess(const __grid_constant__ Views<PreView, NV> B) {
+    chain_start();
     const PreView &V = B[blockIdx.x % B.n];
     const SceneView &s = V.s;
     const CamView &c = V.c;
@@ -250,7 +251,9 @@ __global__ void __launch_bounds__(128) k_preprocess(const __grid_constant__ View
 }
 
 // Zeroes every view's control block and what is cleared with it (16-byte words).
-__global__ void __launch_bounds__(256) k_clear(const __grid_constant__ Views<PreView, kMaxBatch> B) {
+template <int NV>
+__global__ void __launch_bounds__(256) k_clear(const __grid_constant__ Views<PreView, NV> B) {
+    chain_start();
     const PreView &V = B[blockIdx.y];
     uint4 *p = reinterpret_cast<uint4 *>(V.ctl);
     const size_t words = V.clear_bytes / sizeof(uint4);
@@ -264,19 +267,24 @@ namespace {
 template <int NV>
 void preprocess_views(int deg, const Views<PreView, NV> &b, unsigned blocks, cudaStream_t st) {
     switch (deg) {
-        case 0: k_preprocess<0, NV><<<blocks, 128, 0, st>>>(b); break;
-        case 1: k_preprocess<1, NV><<<blocks, 128, 0, st>>>(b); break;
-        case 2: k_preprocess<2, NV><<<blocks, 128, 0, st>>>(b); break;
-        default: k_preprocess<3, NV><<<blocks, 128, 0, st>>>(b); break;
+        case 0: launch_chained(k_preprocess<0, NV>, blocks, 128, 0, st, b); break;
+        case 1: launch_chained(k_preprocess<1, NV>, blocks, 128, 0, st, b); break;
+        case 2: launch_chained(k_preprocess<2, NV>, blocks, 128, 0, st, b); break;
+        default: launch_chained(k_preprocess<3, NV>, blocks, 128, 0, st, b); break;
     }
 }
 
 }  // namespace
 
 cudaError_t launch_clear(const PreView *views, int n, cudaStream_t st) {
-    if (n == 1) return cudaMemsetAsync(views[0].ctl, 0, views[0].clear_bytes, st);
+    size_t most = 0;
+    for (int i = 0; i < n; ++i) most = views[i].clear_bytes > most ? views[i].clear_bytes : most;
+    // four 16-byte words a thread, at most a block per SM
+    const size_t want = (most + 256 * 64 - 1) / (256 * 64);
+    const unsigned blocks = static_cast<unsigned>(want < 152 ? want : 152);
     with_views(views, n, [&](const auto &b) {
-        if constexpr (sizeof(b.v) == kMaxBatch * sizeof(PreView)) k_clear<<<dim3(8, b.n), 256, 0, st>>>(b);
+        constexpr int NV = sizeof(b.v) / sizeof(PreView);
+        k_clear<NV><<<dim3(blocks, b.n), 256, 0, st>>>(b);       // (whatever ran before is waited for as usual)
     });
     return cudaGetLastError();
 }

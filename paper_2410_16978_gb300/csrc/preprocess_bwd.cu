@@ -381,6 +381,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_preprocess_bwd(SceneView s, Cam
                                                                 const float4 *__restrict__ rec_grad,
                                                                 uint32_t grad_layer_mask, gs_grads g,
                                                                 float *__restrict__ contrib_sum, const ZeroRows zr) {
+    chain_start();
     constexpr int K = (DEG + 1) * (DEG + 1);
     const uint32_t nl = (min(ctl->n_vis, static_cast<uint32_t>(s.n)) + kBwdThreads - 1) / kBwdThreads;
     const uint32_t stride = zr.items ? (nl + zr.items) / zr.items : 0xFFFFFFFFu;
@@ -420,8 +421,8 @@ cudaError_t launch_preprocess_backward(const SceneView &s, const CamView &c, con
     zr.sh_w = zr.vec_sh ? zr.sh_row / 4 : zr.sh_row;
     zr.sh_m = (1u << 20) / static_cast<uint32_t>(zr.sh_w) + 1;
     const int blocks = (s.n + kBwdThreads - 1) / kBwdThreads + static_cast<int>(zr.items);
-#define GS_PBWD(D) k_preprocess_bwd<D><<<blocks, kBwdThreads, 0, st>>>(s, c, tiles, vis_index, ctl, rec_grad, \
-                                                                       grad_layer_mask, g, contrib_sum, zr)
+#define GS_PBWD(D) launch_chained(k_preprocess_bwd<D>, blocks, kBwdThreads, 0, st, s, c, tiles, vis_index, ctl, \
+                                  rec_grad, grad_layer_mask, g, contrib_sum, zr)
     switch (s.sh_degree) {
         case 0: GS_PBWD(0); break;
         case 1: GS_PBWD(1); break;

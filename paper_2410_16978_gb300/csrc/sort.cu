@@ -91,6 +91,7 @@ struct NSrc {               // item count: min(*dev, cap) if dev, else cap
 
 template <class F>
 __global__ void __launch_bounds__(256) k_scan_reduce(F f, NSrc ns, uint32_t *__restrict__ partials) {
+    chain_start();
     __shared__ uint32_t s_w[8];
     uint32_t beg, end;
     block_range(ns.get(), beg, end);
@@ -104,6 +105,7 @@ __global__ void __launch_bounds__(256) k_scan_reduce(F f, NSrc ns, uint32_t *__r
 template <class F, class Out>
 __global__ void __launch_bounds__(256) k_scan_down(F f, NSrc ns, const uint32_t *__restrict__ partials, Out out,
                                                    int64_t *__restrict__ n_total) {
+    chain_start();
     __shared__ uint32_t s_w[8];
     uint32_t beg, end;
     block_range(ns.get(), beg, end);
@@ -276,6 +278,7 @@ __device__ uint32_t look_back(uint64_t *status, uint32_t t, int c, uint32_t own,
 
 template <class Src, int NV>
 __global__ void __launch_bounds__(256) k_sort_hist(const __grid_constant__ Views<SortJob, NV> B) {
+    chain_start();
     __shared__ uint32_t s_h[4][256];
     __shared__ uint32_t s_w[8];
     const SortJob &J = B[blockIdx.y];
@@ -411,6 +414,7 @@ __device__ __forceinline__ uint32_t block_scan_512(uint32_t v, uint32_t *s_w, ui
 
 template <class Src, bool FIRST, int NV>
 __global__ void __launch_bounds__(kPassThreads) k_sort_pass(const __grid_constant__ Views<SortJob, NV> views, int pass) {
+    chain_start();
     __shared__ uint16_t s_wc[kPassWarps][256];   // per-warp digit counts, then per-warp digit bases
     __shared__ uint32_t s_lstart[256];            // start of each digit's run in the locally sorted tile
     __shared__ uint32_t s_off[256];               // global position of each digit's run
@@ -567,6 +571,18 @@ __global__ void __launch_bounds__(kPassThreads) k_sort_pass(const __grid_constan
     }
 }
 
+// The shared order of two eyes: the other eye's visible list and counts.
+__global__ void __launch_bounds__(256) k_share_order(const Ctl *from, const uint32_t *__restrict__ vis, Ctl *to,
+                                                     uint32_t *__restrict__ vis_to, uint32_t n) {
+    chain_start();
+    const uint32_t nv = from->n_vis;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        to->n_vis = nv;
+        to->st.n_visible = from->st.n_visible;
+    }
+    for (uint32_t i = blockIdx.x * 256u + threadIdx.x; i < min(nv, n); i += gridDim.x * 256u) vis_to[i] = vis[i];
+}
+
 // 2^lg tiles per group: the least with 2^(2 lg) >= tiles.
 int sort_group_log(uint32_t nt) {
     int lg = 0;
@@ -614,13 +630,14 @@ void with_sort(const SortJob *jobs, int m, F f) {
 template <class Src, int NV>
 void hist_kernel(Src *, const Views<SortJob, NV> &b, uint32_t most, cudaStream_t st) {
     // the histograms and the group counts were cleared with the control block
-    k_sort_hist<Src, NV><<<dim3(most, b.n), 256, 0, st>>>(b);
+    launch_chained(k_sort_hist<Src, NV>, dim3(most, b.n), 256, 0, st, b);
 }
 
 template <class Src, int NV>
 void digit_kernels(Src *, const Views<SortJob, NV> &b, uint32_t most, cudaStream_t st) {
-    k_sort_pass<Src, true, NV><<<dim3(most, b.n), kPassThreads, 0, st>>>(b, 0);
-    for (int p = 1; p < 4; ++p) k_sort_pass<Src, false, NV><<<dim3(most, b.n), kPassThreads, 0, st>>>(b, p);
+    launch_chained(k_sort_pass<Src, true, NV>, dim3(most, b.n), kPassThreads, 0, st, b, 0);
+    for (int p = 1; p < 4; ++p)
+        launch_chained(k_sort_pass<Src, false, NV>, dim3(most, b.n), kPassThreads, 0, st, b, p);
 }
 
 // ---------------------------------------------------------------------------
@@ -673,6 +690,12 @@ cudaError_t launch_sort_digits(const SortView *views, int n, cudaStream_t st) {
     return cudaGetLastError();
 }
 
+cudaError_t launch_share_order(const Ctl *from, const uint32_t *vis, Ctl *to, uint32_t *vis_to, int n,
+                               cudaStream_t st) {
+    launch_chained(k_share_order, sort_blocks(), 256, 0, st, from, vis, to, vis_to, static_cast<uint32_t>(n));
+    return cudaGetLastError();
+}
+
 cudaError_t launch_activity_prune(const float *activity, const uint8_t *layer, uint32_t train_mask, int n,
                                   float samples, float thr, uint8_t *keep, int32_t *keep_index, int64_t *n_keep,
                                   uint32_t *partials, cudaStream_t st) {
@@ -680,7 +703,7 @@ cudaError_t launch_activity_prune(const float *activity, const uint8_t *layer, u
     NSrc ns{nullptr, static_cast<uint32_t>(n)};
     ActiveFlag f{activity, layer, train_mask, 1.f / samples, thr};
     k_scan_reduce<<<G, 256, 0, st>>>(f, ns, partials);
-    k_scan_down<<<G, 256, 0, st>>>(f, ns, partials, KeepOut{keep, keep_index}, n_keep);
+    launch_chained(k_scan_down<decltype(f), KeepOut>, G, 256, 0, st, f, ns, partials, KeepOut{keep, keep_index}, n_keep);
     return cudaGetLastError();
 }
 
@@ -690,7 +713,7 @@ cudaError_t launch_prune(const float *contrib_max, int n, float thr, uint8_t *ke
     NSrc ns{nullptr, static_cast<uint32_t>(n)};
     KeepFlag f{contrib_max, thr};
     k_scan_reduce<<<G, 256, 0, st>>>(f, ns, partials);
-    k_scan_down<<<G, 256, 0, st>>>(f, ns, partials, KeepOut{keep, keep_index}, n_keep);
+    launch_chained(k_scan_down<decltype(f), KeepOut>, G, 256, 0, st, f, ns, partials, KeepOut{keep, keep_index}, n_keep);
     return cudaGetLastError();
 }
 

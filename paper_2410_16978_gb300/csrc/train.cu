@@ -107,6 +107,7 @@ __global__ void __launch_bounds__(kLossThreads) k_loss_maps(const float *__restr
                                                             const float *__restrict__ Ct, const float *__restrict__ At,
                                                             float3 bg, int W, int H, const Win win,
                                                             float *__restrict__ maps, float *__restrict__ partials) {
+    chain_start();
     __shared__ float2 s_v[kRH][kSP];                       // (x, y)
     __shared__ __align__(16) float2 s_m[kRH][kHP];         // horizontal sums of (x, y)
     __shared__ __align__(16) float2 s_q[kRH][kHP];         // of (x^2, y^2)
@@ -256,6 +257,7 @@ __global__ void __launch_bounds__(kLossThreads) k_loss_grad(const float *__restr
                                                             float *__restrict__ dX, float *__restrict__ dA,
                                                             const float *__restrict__ partials, float w_a_loss,
                                                             float *__restrict__ loss) {
+    chain_start();
     __shared__ float2 s_ab[kRH][kSP];                      // maps (a, b)
     __shared__ float s_c[kRH][kSP];                        // map c
     __shared__ __align__(16) float2 s_hab[kRH][kHP];       // their horizontal sums
@@ -526,8 +528,8 @@ cudaError_t launch_image_loss(const float *X, const float *A, const float *Ct, c
     float *partials = maps + 9 * plane;
     const dim3 grid((W + kLW - 1) / kLW, (H + kLH - 1) / kLH, 3);
     k_loss_maps<<<grid, kLossThreads, 0, st>>>(X, A, Ct, At, bg, W, H, win, maps, partials);
-    k_loss_grad<<<grid, kLossThreads, 0, st>>>(X, A, Ct, At, bg, W, H, win, lam, w_a, maps, dX, dA, partials,
-                                               A ? w_a : 0.f, loss);
+    launch_chained(k_loss_grad, grid, kLossThreads, 0, st, X, A, Ct, At, bg, W, H, win, lam, w_a, maps, dX, dA, partials,
+                   A ? w_a : 0.f, loss);
     return cudaGetLastError();
 }
 

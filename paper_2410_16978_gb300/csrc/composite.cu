@@ -35,15 +35,11 @@ namespace gs {
 namespace {
 
 constexpr unsigned FULL = 0xFFFFFFFFu;
-constexpr float kLn2 = 0x1.62e430p-1f;
+
 constexpr int kFwdThreads = 128;
 constexpr int kBwdThreads = 128;
-// Backward pixels per lane: 2 (an 8x8 block per warp) or 4 (16x8).  4 halves the per-splat reduction and
-// atomics per pixel but needs 96 registers (5 blocks per SM instead of 7) and culls on a coarser block;
-// on the 1.2M-Gaussian frame it measured 0.403 ms against 0.362 ms for 2.
-constexpr int kBwdPx = 2;
-// The forward writes the backward's work items per 8x8 block (two pixels per lane).
-static_assert(kBwdPx == 2, "backward work items are 8x8 blocks");
+// The backward takes two pixels per lane (an 8x8 block per warp).  Four (16x8) halved the per-splat reduction and
+// atomics per pixel but needed 96 registers and culled on a coarser block: 1.2M-Gaussian frame 0.403 ms against 0.362.
 
 // 1/x to about 1 ulp (the hardware reciprocal approximation; x = 1 - alpha is in [0.01, 1]).
 __device__ __forceinline__ float rcp_approx(float x) {
@@ -207,61 +203,29 @@ __device__ __forceinline__ void load_geo(const Geo *g, float4 &a, float4 &b) {
                  : "l"(g));
 }
 
+// A splat of the backward's walk: what the block test needs, the blue channel and the layer.
 struct Chunk {
     float4 a, b;
     float c;
-    uint32_t g;
-    uint32_t ly;      // backward: the splat's layer, consumed one chunk later
+    uint32_t g, ly;
 };
 
-// n, ctl, site: the Gaussian count and the bounds check of GS_DEBUG builds
-// (nothing in release builds).
-__device__ __forceinline__ void fetch_chunk(const uint32_t *__restrict__ list, const Rec *__restrict__ rec,
-                                            uint32_t pos, uint32_t end, Chunk &ch, uint32_t n, const Ctl *ctl,
-                                            uint32_t site) {
-    if (pos < end) {
-        const uint32_t g = list[pos];
-        if (!GS_CHECK(g < n, ctl, site)) {
-            ch = Chunk{};          // an inert splat (opacity 0): no block keeps it
-            return;
-        }
-        ch.g = g;
-        const Rec *r = rec + ch.g;
-        ch.a = r->a;
-        ch.b = r->b;
-        ch.c = r->c.x;
-    }
-}
-
-// The backward also needs each splat's layer (frozen layers get no gradient).
-__device__ __forceinline__ void fetch_chunk_layer(const uint32_t *__restrict__ list, const Rec *__restrict__ rec,
-                                                  const uint8_t *__restrict__ layer, uint32_t pos, uint32_t end,
-                                                  Chunk &ch, uint32_t n, const Ctl *ctl) {
-    fetch_chunk(list, rec, pos, end, ch, n, ctl, kSiteBwdId);
-    if (pos < end && GS_CHECK(ch.g < n, ctl, kSiteBwdId)) ch.ly = layer[ch.g];
-}
-
-// The record of an id loaded one chunk earlier: list and record loads of a
+// The splat of an id loaded one chunk earlier: list and record loads of a
 // chunk are issued a chunk apart, so the record load does not wait on the
-// list load in the same iteration.
-__device__ __forceinline__ void fetch_rec(const Rec *__restrict__ rec, uint32_t g, bool valid, Chunk &ch) {
-    if (valid) {
-        ch.g = g;
-        const Rec *r = rec + g;
-        ch.a = r->a;
-        ch.b = r->b;
-        ch.c = r->c.x;
-    }
-}
-
-__device__ __forceinline__ void fetch_rec_layer(const Rec *__restrict__ rec, const uint8_t *__restrict__ layer,
-                                                uint32_t g, bool valid, Chunk &ch, uint32_t n, const Ctl *ctl) {
-    if (valid && !GS_CHECK(g < n, ctl, kSiteBwdId)) {
+// list load in the same iteration.  n, ctl: the Gaussian count and the bounds
+// check of GS_DEBUG builds (nothing in release builds).
+__device__ __forceinline__ void fetch_splat(const Geo *__restrict__ geo, const Rec *__restrict__ rec,
+                                            const uint8_t *__restrict__ layer, uint32_t g, bool valid, Chunk &ch,
+                                            uint32_t n, const Ctl *ctl) {
+    if (!valid) return;
+    if (!GS_CHECK(g < n, ctl, kSiteBwdId)) {
         ch = Chunk{};              // an inert splat (opacity 0): no block keeps it
         return;
     }
-    fetch_rec(rec, g, valid, ch);
-    if (valid) ch.ly = layer[g];
+    ch.g = g;
+    load_geo(geo + g, ch.a, ch.b);
+    ch.c = rec[g].c.x;
+    ch.ly = layer[g];
 }
 
 struct FwdBatch {
@@ -752,48 +716,41 @@ __global__ void __launch_bounds__(1024) k_bwd_setup(uint32_t *__restrict__ queue
     }
 }
 
-// Reduce-scatter of 10 values across a warp in 12 shuffles.  Halving by lane
-// bit: bit 4 splits the values 5 / 5, bit 3 splits each half 3 / 2, bit 2
-// splits those 2 / 1 and 1 / 1, bit 1 splits the remaining pair, and bit 0
-// completes the sums.  Lane l ends with the warp sum of value
-// reduce10_owner(l); value i is held by the lanes of one aligned group.
+// Reduce-scatter of a splat's 10 sums over the 32 lanes in 12 shuffles; lane l
+// ends with the warp sum of value reduce10_owner(l).  The four colour values
+// are products of one factor with per-lane constants, so each lane forms them
+// in the order in which it keeps and sends them (col[0] kept; the sign of the
+// lane bit flips the order) and their two halvings need no selects; value 3 or
+// 5 stays whole in its half of the warp until the other values have been
+// halved away.
 __device__ __forceinline__ int reduce10_owner(int lane) {
     const int b4 = (lane >> 4) & 1, b3 = (lane >> 3) & 1, b2 = (lane >> 2) & 1, b1 = (lane >> 1) & 1;
-    return 5 * b4 + (b3 ? 3 + b2 : (b2 ? 2 : b1));
+    return b1 ? (b4 ? 5 : 3) : (b2 ? (b3 ? (b4 ? 4 : 2) : b4) : 6 + 2 * b4 + b3);
 }
 
-// The lowest lane holding each value (lanes 0, 2, 4, 8, 12, 16, 18, 20, 24, 28).
-__device__ __forceinline__ bool reduce10_writer(int lane) {
-    return !(lane & 1) && (((lane & 12) == 0) || !(lane & 2));
+// One lane per value: 0, 4, .., 28 and, for values 3 and 5, lanes 2 and 18.
+__device__ __forceinline__ bool reduce10_writer(int lane) { return !(lane & 1) && (!(lane & 2) || !(lane & 12)); }
+
+// Which of the colour values 6 .. 9 a lane's slot s holds (less 6).
+__device__ __forceinline__ int reduce10_slot(int lane, int s) {
+    return 2 * (((lane >> 4) & 1) ^ (s >> 1)) + (((lane >> 3) & 1) ^ (s & 1));
 }
 
-__device__ __forceinline__ float reduce_scatter10(const float v[10], int lane) {
+// g: values 0 .. 5; col: the colour values in slot order.
+__device__ __forceinline__ float reduce_scatter10(const float g[6], const float col[4], int lane) {
     const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4, b1 = lane & 2;
-    float a[5];
-#pragma unroll
-    for (int i = 0; i < 5; ++i) {
-        const float keep = b4 ? v[i + 5] : v[i];
-        const float send = b4 ? v[i] : v[i + 5];
-        a[i] = keep + __shfl_xor_sync(FULL, send, 16);
-    }
-    float c[3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        const float hi = i < 2 ? a[i + 3] : 0.f;
-        const float send = b3 ? a[i] : hi;
-        const float keep = b3 ? hi : a[i];
-        c[i] = keep + __shfl_xor_sync(FULL, send, 8);
-    }
-    const float s0 = b3 ? (b2 ? c[0] : c[1]) : (b2 ? c[0] : c[2]);
-    const float s1 = (!b3 && b2) ? c[1] : 0.f;
-    const float r0 = __shfl_xor_sync(FULL, s0, 4);
-    const float r1 = __shfl_xor_sync(FULL, s1, 4);
-    const float d0 = (b3 ? (b2 ? c[1] : c[0]) : (b2 ? c[2] : c[0])) + r0;
-    const float d1 = c[1] + r1;
-    const bool two = !b3 && !b2;
-    const float s2 = two ? (b1 ? d0 : d1) : d0;
-    const float e = (two ? (b1 ? d1 : d0) : d0) + __shfl_xor_sync(FULL, s2, 2);
-    return e + __shfl_xor_sync(FULL, e, 1);
+    const float c0 = col[0] + __shfl_xor_sync(FULL, col[2], 16);
+    const float c1 = col[1] + __shfl_xor_sync(FULL, col[3], 16);
+    const float p = (b4 ? g[1] : g[0]) + __shfl_xor_sync(FULL, b4 ? g[0] : g[1], 16);
+    const float q = (b4 ? g[4] : g[2]) + __shfl_xor_sync(FULL, b4 ? g[2] : g[4], 16);
+    float m = (b4 ? g[5] : g[3]) + __shfl_xor_sync(FULL, b4 ? g[3] : g[5], 16);
+    const float c = c0 + __shfl_xor_sync(FULL, c1, 8);
+    const float x = (b3 ? q : p) + __shfl_xor_sync(FULL, b3 ? p : q, 8);
+    m += __shfl_xor_sync(FULL, m, 8);
+    const float y = (b2 ? x : c) + __shfl_xor_sync(FULL, b2 ? c : x, 4);
+    m += __shfl_xor_sync(FULL, m, 4);
+    const float z = (b1 ? m : y) + __shfl_xor_sync(FULL, b1 ? y : m, 2);
+    return z + __shfl_xor_sync(FULL, z, 1);
 }
 
 // Backward, back to front within a segment.  With
@@ -809,38 +766,48 @@ __device__ __forceinline__ float reduce_scatter10(const float v[10], int lane) {
 // accuracy (a running total minus a prefix would not).
 //
 // Each splat's 10 sums are reduce-scattered over the warp and added to the
-// record gradient, float 12 g + i for value i, by ten lanes at once:
-//   (du, dv, dA2, dbeta, dG2, dopacity, dr, dg, db, sum of alpha*T);
+// record gradient, float 12 g + i for value i, by ten lanes at once: with e'
+// the natural exponent, E = dL/de', p and dy as in splat_alpha
+//   (sum E p, sum E dy, sum E p^2, sum E p dy, sum E dy^2, dopacity, dr, dg, db, sum of alpha*T);
 //   contrib_max[g] = max(.., alpha*T).
-// The five geometric values are summed as moments of dL/de' (e' the natural
-// exponent) and scaled by the splat's constants once, after the warp sum.
-// 1 / (1 - a_i) is the hardware reciprocal approximation (about 1 ulp): a
-// correctly rounded reciprocal costs several instructions per pixel and
-// splat and changes the gradients only at the last bits.
-// Six CTAs per SM (at most 80 registers) measured faster than five at 89.
-template <int PX>
-__global__ void __launch_bounds__(kBwdThreads, 6) k_composite_bwd(
+// The chain rule turns the first five into the gradients of the record's
+// geometry (they are linear in them, with factors of the splat alone).
+// 1 / (1 - a_i) is the hardware reciprocal approximation (about 1 ulp, exact
+// at 1): a correctly rounded reciprocal costs several instructions per pixel
+// and splat and changes the gradients only at the last bits.
+//
+// Bound by instruction issue.  A lane's two pixels go through packed
+// arithmetic without branches: a pixel that the splat does not touch takes
+// part with alpha 0, and with zeros selected where a product with an infinite
+// or undefined value of its own must not count.  Kept splats are staged in
+// shared memory with every factor doubled, as the packed instructions want
+// them.  1.2M-Gaussian 1024 x 1024 frame 0.198 -> 0.166 ms, 500,000-Gaussian
+// 800 x 800 training view 0.148 -> 0.124 (before: one pixel after the other
+// behind branches, 220 instructions per splat and block against 160, and the
+// geometry's factors applied per splat and block).  Five CTAs per SM; six and
+// seven: 0.168 and 0.169.
+struct alignas(16) BwdSplat {
+    float2 nax, nay;               // minus the centre
+    float2 beta, A2, G2, o;
+    float2 r, g;
+    float2 b;
+    uint32_t gt, pos;              // id with bit 31: trainable; position in the tile's list
+};
+
+__global__ void __launch_bounds__(kBwdThreads, 5) k_composite_bwd(
     const uint2 *__restrict__ items, const uint32_t *__restrict__ n_items, uint32_t *__restrict__ queue,
-    const uint2 *__restrict__ ranges, const uint32_t *__restrict__ list, const Rec *__restrict__ rec, int W, int H,
-    int Tx, float3 bg, const float *__restrict__ t_final, const uint32_t *__restrict__ n_contrib,
-    const uint32_t *__restrict__ seg_base, const float4 *__restrict__ ckpt, const uint32_t *__restrict__ qwork,
-    const float *__restrict__ dL_dimage, const float *__restrict__ dL_dalpha, const uint8_t *__restrict__ layer,
-    uint32_t grad_layer_mask, float4 *__restrict__ rec_grad, float *__restrict__ contrib_max, uint32_t n_rec,
-    const Ctl *__restrict__ ctl) {
+    const uint2 *__restrict__ ranges, const uint32_t *__restrict__ list, const Geo *__restrict__ geo,
+    const Rec *__restrict__ rec, int W, int H, int Tx, float3 bg, const float *__restrict__ t_final,
+    const uint32_t *__restrict__ n_contrib, const uint32_t *__restrict__ seg_base, const float4 *__restrict__ ckpt,
+    const uint32_t *__restrict__ qwork, const float *__restrict__ dL_dimage, const float *__restrict__ dL_dalpha,
+    const uint8_t *__restrict__ layer, uint32_t grad_layer_mask, float4 *__restrict__ rec_grad,
+    float *__restrict__ contrib_max, uint32_t n_rec, const Ctl *__restrict__ ctl) {
     chain_start();
-    __shared__ float4 s_a[kBwdThreads / 32][32], s_b[kBwdThreads / 32][32];
-    __shared__ float s_c[kBwdThreads / 32][32];
-    __shared__ uint32_t s_g[kBwdThreads / 32][32];
-    __shared__ uint32_t s_pos[kBwdThreads / 32][32];
+    __shared__ BwdSplat s_splat[kBwdThreads / 32][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
     const int own = reduce10_owner(lane);
     const bool writer = reduce10_writer(lane);
-    // per-lane factors of the value it holds after the reduce-scatter:
-    //   du = -2 ln2 A2 S0, dv = -2 ln2 (A2 beta S0 + G2 S1), dA2 = ln2 S2, dbeta = 2 ln2 A2 S3, dG2 = ln2 S4
-    const float cA = own == 0 ? -2.f * kLn2 : (own == 3 ? 2.f * kLn2 : 0.f);
-    const float cB = own == 1 ? -2.f * kLn2 : 0.f;
-    const float cC = (own == 2 || own == 4) ? kLn2 : (own >= 5 ? 1.f : 0.f);
     const uint32_t total = *n_items;
     const size_t plane = static_cast<size_t>(W) * H;
     for (;;) {
@@ -854,23 +821,20 @@ __global__ void __launch_bounds__(kBwdThreads, 6) k_composite_bwd(
         const uint32_t seg = it.y & 0xFFFFFFu;
         const uint2 rg = ranges[tile];
         const uint32_t s0 = rg.x + seg * kSeg;
-        // block of the item: PX = 2: 8x8 quadrant q of the tile; PX = 4: 16x8 half q
-        constexpr int BW = PX == 2 ? 8 : 16;
-        const int ox = PX == 2 ? (q & 1) * 8 : 0, oy = PX == 2 ? (q >> 1) * 8 : q * 8;
-        const uint32_t qmax = PX == 2 ? qwork[4 * tile + q] : max(qwork[4 * tile + 2 * q], qwork[4 * tile + 2 * q + 1]);
-        const uint32_t s1 = rg.x + min(min((seg + 1) * kSeg, qmax), rg.y - rg.x);
+        const int ox = (q & 1) * 8, oy = (q >> 1) * 8;          // the item's 8x8 block of the tile
+        const uint32_t s1 = rg.x + min(min((seg + 1) * kSeg, qwork[4 * tile + q]), rg.y - rg.x);
         const float4 *nck = ckpt + (static_cast<size_t>(seg_base[tile]) + seg + 1) * kTilePix;
         const float bx0 = (tile % Tx) * kTile + ox + 0.5f, by0 = (tile / Tx) * kTile + oy + 0.5f;
-        float px[PX], py[PX], dC0[PX], dC1[PX], dC2[PX], R[PX], T[PX];
-        uint32_t nc[PX];
+        // the lane's pixels: rows lane / 8 and lane / 8 + 4 of the block
+        float dC[3][2], R[2], T[2];
+        uint32_t nc[2];
+        const int lx = ox + (lane & 7);
 #pragma unroll
-        for (int j = 0; j < PX; ++j) {
-            const int lx = ox + (lane % BW), ly = oy + (lane / BW) + (32 / BW) * j;
+        for (int j = 0; j < 2; ++j) {
+            const int ly = oy + (lane >> 3) + 4 * j;
             const int x = (tile % Tx) * kTile + lx, y = (tile / Tx) * kTile + ly;
-            px[j] = x + 0.5f;
-            py[j] = y + 0.5f;
             nc[j] = 0;
-            dC0[j] = dC1[j] = dC2[j] = R[j] = 0.f;
+            dC[0][j] = dC[1][j] = dC[2][j] = R[j] = 0.f;
             T[j] = 1.f;
             if (x < W && y < H) {
                 const size_t pix = static_cast<size_t>(y) * W + x;
@@ -880,101 +844,117 @@ __global__ void __launch_bounds__(kBwdThreads, 6) k_composite_bwd(
                     const float TN = t_final[pix];
                     float dA = 0.f;
                     if (dL_dimage) {
-                        dC0[j] = dL_dimage[pix];
-                        dC1[j] = dL_dimage[plane + pix];
-                        dC2[j] = dL_dimage[2 * plane + pix];
+                        dC[0][j] = dL_dimage[pix];
+                        dC[1][j] = dL_dimage[plane + pix];
+                        dC[2][j] = dL_dimage[2 * plane + pix];
                     }
                     if (dL_dalpha) dA = dL_dalpha[pix];
-                    R[j] = TN * (dC0[j] * bg.x + dC1[j] * bg.y + dC2[j] * bg.z) - dA * TN;
+                    R[j] = TN * (dC[0][j] * bg.x + dC[1][j] * bg.y + dC[2][j] * bg.z) - dA * TN;
                     T[j] = TN;
                     if (n > (seg + 1) * kSeg) {
                         const float4 ck = nck[ly * kTile + lx];
                         T[j] = ck.x;
-                        R[j] += dC0[j] * ck.y + dC1[j] * ck.z + dC2[j] * ck.w;
+                        R[j] += dC[0][j] * ck.y + dC[1][j] * ck.z + dC[2][j] * ck.w;
                     }
                 }
             }
         }
+        // an upstream gradient that is not finite counts for the splats of its own pixel only
+        const bool finite = __all_sync(FULL, isfinite(dC[0][0] + dC[0][1]) && isfinite(dC[1][0] + dC[1][1]) &&
+                                                 isfinite(dC[2][0] + dC[2][1]));
+        const float lpx = (tile % Tx) * kTile + lx + 0.5f, lpy = (tile / Tx) * kTile + oy + (lane >> 3) + 0.5f;
+        const F2 px(lpx, lpx), py(lpy, lpy + 4.f);
+        const F2 dC0(dC[0][0], dC[0][1]), dC1(dC[1][0], dC[1][1]), dC2(dC[2][0], dC[2][1]);
+        F2 kc[4];                   // the colour values' constants in slot order (value 9's is 1)
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+            const int v = reduce10_slot(lane, s);
+            kc[s] = v == 0 ? dC0 : (v == 1 ? dC1 : (v == 2 ? dC2 : F2(1.f, 1.f)));
+        }
+        F2 R2(R[0], R[1]), T2(T[0], T[1]);
         const uint32_t nchunk = (s1 - s0 + 31) / 32;
         Chunk nxt;
-        if (nchunk) fetch_chunk_layer(list, rec, layer, s0 + (nchunk - 1) * 32 + lane, s1, nxt, n_rec, ctl);
-        // ids one chunk ahead of the records (the walk goes back to front; every chunk below the last is full)
-        uint32_t gid = nchunk >= 2 ? list[s0 + (nchunk - 2) * 32 + lane] : 0u;
+        // ids one chunk ahead of the splats (the walk goes back to front; every chunk below the last is full)
+        uint32_t gid = 0;
+        if (nchunk) {
+            const uint32_t pos = s0 + (nchunk - 1) * 32 + lane;
+            fetch_splat(geo, rec, layer, pos < s1 ? list[pos] : 0u, pos < s1, nxt, n_rec, ctl);
+            if (nchunk >= 2) gid = list[pos - 32];
+        }
         for (uint32_t c = nchunk; c-- > 0;) {
             const uint32_t base = s0 + c * 32;
-            const bool keep =
-                base + lane < s1 && splat_reaches_block(nxt.a, nxt.b, bx0, bx0 + (BW - 1.f), by0, by0 + 7.f);
+            const bool keep = base + lane < s1 && splat_reaches_block(nxt.a, nxt.b, bx0, bx0 + 7.f, by0, by0 + 7.f);
             const unsigned km = __ballot_sync(FULL, keep);
             __syncwarp();
             if (keep) {
-                const int slot = __popc(km & lt);
-                s_a[warp][slot] = nxt.a;
-                s_b[warp][slot] = nxt.b;
-                s_c[warp][slot] = nxt.c;
-                s_g[warp][slot] = nxt.g | (((grad_layer_mask >> nxt.ly) & 1u) << 31);   // bit 31: trainable
-                s_pos[warp][slot] = base + lane - rg.x;
+                BwdSplat &S = s_splat[warp][__popc(km & lt)];
+                const float4 a = nxt.a, b = nxt.b;
+                S.nax = make_float2(-a.x, -a.x);
+                S.nay = make_float2(-a.y, -a.y);
+                S.beta = make_float2(a.w, a.w);
+                S.A2 = make_float2(a.z, a.z);
+                S.G2 = make_float2(b.x, b.x);
+                S.o = make_float2(b.y, b.y);
+                S.r = make_float2(b.z, b.z);
+                S.g = make_float2(b.w, b.w);
+                S.b = make_float2(nxt.c, nxt.c);
+                S.gt = nxt.g | (((grad_layer_mask >> nxt.ly) & 1u) << 31);
+                S.pos = base + lane - rg.x;
             }
             __syncwarp();
-            fetch_rec_layer(rec, layer, gid, c > 0, nxt, n_rec, ctl);
+            fetch_splat(geo, rec, layer, gid, c > 0, nxt, n_rec, ctl);
             if (c > 1) gid = list[base - 64 + lane];
             const int cnt = __popc(km);
             for (int k = cnt - 1; k >= 0; --k) {
-                const uint32_t pos = s_pos[warp][k];
-                const float4 a = s_a[warp][k], b = s_b[warp][k];
-                const float cb = s_c[warp][k];
-                float p[PX], dy[PX], ex[PX], ao[PX], al[PX];
-                bool act[PX];
-                bool any = false;
+                const ulonglong2 *S = reinterpret_cast<const ulonglong2 *>(&s_splat[warp][k]);
+                const ulonglong2 u0 = S[0], u1 = S[1], u2 = S[2];
+                const uint4 u4 = reinterpret_cast<const uint4 *>(S)[4];
+                // alpha of both pixels, bit for bit as splat_alpha's
+                const F2 dx = add2(px, F2(u0.x)), dy = add2(py, F2(u0.y));
+                const F2 p = fma2(F2(u1.x), dy, dx);
+                const float2 e = fma2(mul2(F2(u1.y), p), p, mul2(mul2(F2(u2.x), dy), dy)).get();
+                const F2 ex(ex2_approx(e.x), ex2_approx(e.y));
+                const float2 ao = mul2(F2(u2.y), ex).get();
+                const float al0 = fminf(kAlphaMax, ao.x), al1 = fminf(kAlphaMax, ao.y);
+                const bool act0 = u4.w < nc[0] && al0 >= kAlphaMin, act1 = u4.w < nc[1] && al1 >= kAlphaMin;
+                if (!__any_sync(FULL, act0 || act1)) continue;
+                const ulonglong2 u3 = S[3];
+                const float a0 = act0 ? al0 : 0.f, a1 = act1 ? al1 : 0.f;
+                const F2 al(a0, a1);
+                const F2 inv(rcp_approx(__fsub_rn(1.f, a0)), rcp_approx(__fsub_rn(1.f, a1)));
+                T2 = mul2(T2, inv);
+                const F2 w = mul2(al, T2);
+                const float cb = __uint_as_float(u4.x);
+                const float2 d = fma2(dC2, F2(cb, cb), fma2(dC1, F2(u3.y), mul2(dC0, F2(u3.x)))).get();
+                const F2 dcc(act0 ? d.x : 0.f, act1 ? d.y : 0.f);
+                const float2 Rinv = mul2(R2, inv).get(), t = T2.get(), dc = dcc.get();
+                R2 = fma2(w, dcc, R2);
+                // dL/da, zero where the product with the opacity was clamped
+                const F2 dLda(act0 && ao.x < kAlphaMax ? fmaf(t.x, dc.x, -Rinv.x) : 0.f,
+                              act1 && ao.y < kAlphaMax ? fmaf(t.y, dc.y, -Rinv.y) : 0.f);
+                const F2 E = mul2(dLda, al);
+                const F2 tp = mul2(E, p), td = mul2(E, dy);
+                const float g[6] = {tp.sum(),           td.sum(),           mul2(tp, p).sum(),
+                                    mul2(tp, dy).sum(), mul2(td, dy).sum(), mul2(dLda, ex).sum()};
+                F2 m[4];
 #pragma unroll
-                for (int j = 0; j < PX; ++j) {
-                    al[j] = splat_alpha(px[j], py[j], a, b, p[j], dy[j], ex[j], ao[j]);
-                    act[j] = pos < nc[j] && al[j] >= kAlphaMin;
-                    any |= act[j];
-                }
-                if (!__any_sync(FULL, any)) continue;
-                // v: du, dv, dA2, dbeta, dG2, dopacity, dr, dg, db, sum of alpha*T
-                float v[10] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-                float wmx = 0.f;
+                for (int s = 0; s < 4; ++s) m[s] = mul2(w, kc[s]);
+                if (!finite) {
 #pragma unroll
-                for (int j = 0; j < PX; ++j) {
-                    if (!act[j]) continue;
-                    const float dcc = dC0[j] * b.z + dC1[j] * b.w + dC2[j] * cb;
-                    const float inv = rcp_approx(__fsub_rn(1.f, al[j]));
-                    const float Ti = T[j] * inv;
-                    const float wgt = al[j] * Ti;
-                    const float dLda = Ti * dcc - R[j] * inv;
-                    R[j] = fmaf(wgt, dcc, R[j]);
-                    T[j] = Ti;
-                    v[6] += wgt * dC0[j];
-                    v[7] += wgt * dC1[j];
-                    v[8] += wgt * dC2[j];
-                    if (ao[j] < kAlphaMax) {
-                        // moments of dL/de' = dL/da alpha (e' = e ln 2 = ln(alpha / o)); the splat's
-                        // constant factors are applied once to the warp sums (see below)
-                        const float dLde = dLda * al[j];
-                        const float tp = dLde * p[j], td = dLde * dy[j];
-                        v[5] += dLda * ex[j];
-                        v[0] += tp;
-                        v[1] += td;
-                        v[2] += tp * p[j];
-                        v[3] += tp * dy[j];
-                        v[4] += td * dy[j];
+                    for (int s = 0; s < 4; ++s) {
+                        const float2 v = m[s].get();
+                        m[s] = F2(act0 ? v.x : 0.f, act1 ? v.y : 0.f);
                     }
-                    v[9] += wgt;
-                    wmx = fmaxf(wmx, wgt);
                 }
-                const float sv0 = reduce_scatter10(v, lane);
-                // sum of tp, for the lanes holding the sum of td (dv needs both)
-                const float stp = __shfl_sync(FULL, sv0, lane & ~2);
-                const float sv = sv0 * (cA * a.z + cC) + cB * (a.z * a.w * stp + b.x * sv0);
-                const uint32_t smx = __reduce_max_sync(FULL, __float_as_uint(wmx));
-                const uint32_t gt = s_g[warp][k];
-                const uint32_t g = gt & 0x7FFFFFFFu;
-                const bool train = gt >> 31;
+                const float col[4] = {m[0].sum(), m[1].sum(), m[2].sum(), m[3].sum()};
+                const float2 wv = w.get();
+                const float sv = reduce_scatter10(g, col, lane);
+                const uint32_t smx = __reduce_max_sync(FULL, __float_as_uint(fmaxf(wv.x, wv.y)));
+                const uint32_t gi = u4.z & 0x7FFFFFFFu;
                 // value i is float 12 g + i of the record gradient: one atomic per value, one instruction
-                if (writer && (train || own == 9))
-                    atomicAdd(reinterpret_cast<float *>(rec_grad) + 12 * static_cast<size_t>(g) + own, sv);
-                if (lane == 1 && contrib_max) atomicMax(reinterpret_cast<unsigned int *>(&contrib_max[g]), smx);
+                if (writer && ((u4.z >> 31) || own == 9))
+                    atomicAdd(reinterpret_cast<float *>(rec_grad) + 12 * static_cast<size_t>(gi) + own, sv);
+                if (lane == 1 && contrib_max) atomicMax(reinterpret_cast<unsigned int *>(&contrib_max[gi]), smx);
             }
         }
     }
@@ -1061,15 +1041,15 @@ cudaError_t launch_bwd_setup(const CompositeBufs &cb, int Tx, int Ty, float4 *re
 }
 
 cudaError_t launch_composite_backward(const CompositeBufs &cb, const uint2 *ranges, const uint32_t *list,
-                                      const Rec *rec, int W, int H, int Tx, int Ty, float3 bg, const float *t_final,
-                                      const uint32_t *n_contrib, const float *dL_dimage,
+                                      const Geo *geo, const Rec *rec, int W, int H, int Tx, int Ty, float3 bg,
+                                      const float *t_final, const uint32_t *n_contrib, const float *dL_dimage,
                                       const float *dL_dalpha, const uint8_t *layer, uint32_t grad_layer_mask,
                                       float4 *rec_grad, float *contrib_max, uint32_t n, const Ctl *ctl,
                                       cudaStream_t st) {
     if (Tx * Ty == 0) return cudaSuccess;
     static PerDevice cache;
-    const int blocks = cache.get([] { return persistent_blocks(k_composite_bwd<kBwdPx>, kBwdThreads); });
-    launch_chained(k_composite_bwd<kBwdPx>, blocks, kBwdThreads, 0, st, cb.items, cb.n_items, cb.queue, ranges, list,
+    const int blocks = cache.get([] { return persistent_blocks(k_composite_bwd, kBwdThreads); });
+    launch_chained(k_composite_bwd, blocks, kBwdThreads, 0, st, cb.items, cb.n_items, cb.queue, ranges, list, geo,
                    rec, W, H, Tx, bg, t_final, n_contrib, cb.seg_base, cb.ckpt, cb.qwork, dL_dimage, dL_dalpha, layer,
                    grad_layer_mask, rec_grad, contrib_max, n, ctl);
     return cudaGetLastError();

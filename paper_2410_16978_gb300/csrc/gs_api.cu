@@ -558,7 +558,7 @@ int gs_render_backward(const gs_scene *scene, const gs_camera *camera, const flo
     {
         Stage sg(GS_STAGE_COMPOSITE_BWD, st, 1);
         if ((rc = cuda_check(launch_composite_backward(composite_bufs(ws, L), at<uint2>(ws, L.ranges),
-                                                       at<uint32_t>(ws, L.list), at<Rec>(ws, L.rec), cv.W, cv.H,
+                                                       at<uint32_t>(ws, L.list), at<Geo>(ws, L.geo), at<Rec>(ws, L.rec), cv.W, cv.H,
                                                        cv.Tx, cv.Ty, make_float3(bg[0], bg[1], bg[2]),
                                                        at<float>(ws, L.t_final), at<uint32_t>(ws, L.n_contrib),
                                                        dL_dimage, dL_dalpha, sv.layer, grad_layer_mask, rec_grad,
@@ -569,7 +569,7 @@ int gs_render_backward(const gs_scene *scene, const gs_camera *camera, const flo
     }
     Stage sg(GS_STAGE_PREPROCESS_BWD, st, 1);
     return cuda_check(launch_preprocess_backward(sv, cv, at<uint32_t>(ws, L.tiles), at<uint32_t>(ws, L.vis_index),
-                                                 at<Ctl>(ws, L.ctl), rec_grad, grad_layer_mask, *grads, contrib_sum,
+                                                 at<Ctl>(ws, L.ctl), at<Geo>(ws, L.geo), rec_grad, grad_layer_mask, *grads, contrib_sum,
                                                  st),
                       "preprocess backward");
 }

@@ -180,7 +180,7 @@ inline void with_views(const T *views, int n, F f) {
 // started, and waits at its first instruction until that one has completed and
 // its writes are visible.  That takes the launch latency and the filling of the
 // SMs out of the gaps between the ten to twenty short kernels of a call (4,096
-// Gaussians at 128 x 128 0.160 -> 0.137 ms, 200,000 at 512 x 512 0.181 -> 0.164,
+// Gaussians at 128 x 128 0.160 -> 0.137 ms, 500,000 at 512 x 512 0.181 -> 0.164,
 // 1024 x 1024 frame with its backward 0.677 -> 0.651).  Rules: chain_start() is the first
 // statement of every kernel launched this way, before any access to memory and
 // any return, so that a kernel's completion implies that of all before it;
@@ -207,6 +207,38 @@ cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t s
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
 }
 
+// Two floats in a 64-bit register, and the packed operations on them (each half rounded as the scalar one).
+struct F2 {
+    unsigned long long v;
+    __device__ __forceinline__ F2() {}
+    __device__ __forceinline__ explicit F2(unsigned long long u) : v(u) {}
+    __device__ __forceinline__ F2(float a, float b) { asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(a), "f"(b)); }
+    __device__ __forceinline__ float2 get() const {
+        float2 r;
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+        return r;
+    }
+    __device__ __forceinline__ float sum() const {
+        const float2 r = get();
+        return r.x + r.y;
+    }
+};
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+__device__ __forceinline__ F2 mul2(F2 a, F2 b) {
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 add2(F2 a, F2 b) {
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+
 // S1 of one view.
 struct PreView {
     SceneView s;
@@ -227,8 +259,8 @@ cudaError_t launch_preprocess(const PreView *views, int n, cudaStream_t st, int 
 // vis_index: the visible list of the last render (index order, ctl->n_vis
 // entries; a two-eye list may also hold Gaussians this view does not see).
 cudaError_t launch_preprocess_backward(const SceneView &s, const CamView &c, const uint32_t *tiles,
-                                       const uint32_t *vis_index, const Ctl *ctl, const float4 *rec_grad,
-                                       uint32_t grad_layer_mask, const gs_grads &g, float *contrib_sum,
+                                       const uint32_t *vis_index, const Ctl *ctl, const Geo *geo,
+                                       const float4 *rec_grad, uint32_t grad_layer_mask, const gs_grads &g, float *contrib_sum,
                                        cudaStream_t st);
 
 int sort_blocks();   // blocks of the sort / scan kernels on this device
@@ -390,8 +422,8 @@ cudaError_t launch_composite_forward(const FwdJob *jobs, int n, cudaStream_t st)
 cudaError_t launch_bwd_setup(const CompositeBufs &cb, int Tx, int Ty, float4 *rec_grad, const uint32_t *vis_index,
                              const uint32_t *n_vis, int n, cudaStream_t st);
 cudaError_t launch_composite_backward(const CompositeBufs &cb, const uint2 *ranges, const uint32_t *list,
-                                      const Rec *rec, int W, int H, int Tx, int Ty, float3 bg, const float *t_final,
-                                      const uint32_t *n_contrib, const float *dL_dimage,
+                                      const Geo *geo, const Rec *rec, int W, int H, int Tx, int Ty, float3 bg,
+                                      const float *t_final, const uint32_t *n_contrib, const float *dL_dimage,
                                       const float *dL_dalpha, const uint8_t *layer, uint32_t grad_layer_mask,
                                       float4 *rec_grad, float *contrib_max, uint32_t n, const Ctl *ctl,
                                       cudaStream_t st);

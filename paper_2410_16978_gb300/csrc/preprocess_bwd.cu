@@ -1,5 +1,5 @@
-// S4b - per-Gaussian chain rule from the record gradient (d/du, dv, dA2,
-// dbeta, dG2, dopacity, drgb) to the stored parameters (means, log-scales,
+// S4b - per-Gaussian chain rule from the record gradient (five moments over
+// the splat, dopacity, drgb) to the stored parameters (means, log-scales,
 // quaternions, opacity logit, SH), the backward of the EWA projection used by
 // the layered training (Sec. 3.2).  Gaussians that were culled or whose layer
 // is frozen (not in grad_layer_mask; Sec. 3.2: lower layers stay fixed) get 0.
@@ -65,6 +65,7 @@ __device__ __forceinline__ void sh_basis_grad(float x, float y, float z, float *
 }
 
 constexpr int kBwdThreads = 128;
+constexpr float kLn2 = 0x1.62e430p-1f;
 
 // Everything the chain rule of Gaussian i reads, issued together before any
 // branch: the inline-PTX loads are volatile, so the compiler keeps them at
@@ -72,6 +73,7 @@ constexpr int kBwdThreads = 128;
 template <int K>
 struct RowIn {
     float4 ga, gb, gc;       // record gradient
+    float A2, beta, G2;      // of the record
     float m[3], ol;
     float ls[3], q[4];       // log-scales and quaternion, widened
     float sh[3 * K];         // [k][channel]
@@ -89,7 +91,9 @@ __device__ __forceinline__ float ld_now(const float *p) {
 }
 
 template <int K>
-__device__ __forceinline__ void load_row(const SceneView &s, int i, const float4 *rec_grad, RowIn<K> &r) {
+__device__ __forceinline__ void load_row(const SceneView &s, int i, const Geo *geo, const float4 *rec_grad, RowIn<K> &r) {
+    asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2];" : "=f"(r.A2), "=f"(r.beta) : "l"(&geo[i].a.z));
+    r.G2 = ld_now(&geo[i].b.x);
     r.ga = ld_now4(rec_grad + 3 * i);
     r.gb = ld_now4(rec_grad + 3 * i + 1);
     r.gc = ld_now4(rec_grad + 3 * i + 2);
@@ -214,7 +218,9 @@ __device__ __forceinline__ void grad_one(const CamView &c, int i, const RowIn<(D
                                          const gs_grads &g) {
     constexpr int K = (DEG + 1) * (DEG + 1);
     const float4 ga = r.ga, gb = r.gb, gc = r.gc;
-    const float dU = ga.x, dV = ga.y, dA2 = ga.z, dBeta = ga.w, dG2 = gb.x, dOp = gb.y;
+    // from the compositor's moments of dL/de' (e' = ln 2 (A2 p^2 + G2 dy^2), p = dx + beta dy)
+    const float dU = -2.f * kLn2 * r.A2 * ga.x, dV = -2.f * kLn2 * (r.A2 * r.beta * ga.x + r.G2 * ga.y);
+    const float dA2 = kLn2 * ga.z, dBeta = 2.f * kLn2 * r.A2 * ga.w, dG2 = kLn2 * gb.x, dOp = gb.y;
     const float dRgb[3] = {gb.z, gb.w, gc.x};
     const float mx = r.m[0], my_ = r.m[1], mz = r.m[2];
     const float *R = c.R;
@@ -377,7 +383,7 @@ template <int DEG>
 __global__ void __launch_bounds__(kBwdThreads) k_preprocess_bwd(SceneView s, CamView c,
                                                                 const uint32_t *__restrict__ tiles,
                                                                 const uint32_t *__restrict__ vis_index,
-                                                                const Ctl *__restrict__ ctl,
+                                                                const Ctl *__restrict__ ctl, const Geo *__restrict__ geo,
                                                                 const float4 *__restrict__ rec_grad,
                                                                 uint32_t grad_layer_mask, gs_grads g,
                                                                 float *__restrict__ contrib_sum, const ZeroRows zr) {
@@ -398,7 +404,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_preprocess_bwd(SceneView s, Cam
     const uint32_t tc = tiles[i];
     const uint32_t ly = s.layer[i];
     RowIn<K> r;
-    load_row<K>(s, i, rec_grad, r);
+    load_row<K>(s, i, geo, rec_grad, r);
     if (tc == 0) return;                        // a two-eye list also holds Gaussians only the other eye sees
     if (contrib_sum) contrib_sum[i] += r.gc.y;
     if (!((grad_layer_mask >> ly) & 1u)) return;   // frozen: a zero row
@@ -408,7 +414,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_preprocess_bwd(SceneView s, Cam
 }  // namespace
 
 cudaError_t launch_preprocess_backward(const SceneView &s, const CamView &c, const uint32_t *tiles,
-                                       const uint32_t *vis_index, const Ctl *ctl, const float4 *rec_grad,
+                                       const uint32_t *vis_index, const Ctl *ctl, const Geo *geo, const float4 *rec_grad,
                                        uint32_t grad_layer_mask, const gs_grads &g, float *contrib_sum,
                                        cudaStream_t st) {
     if (s.n == 0) return cudaSuccess;
@@ -422,7 +428,7 @@ cudaError_t launch_preprocess_backward(const SceneView &s, const CamView &c, con
     zr.sh_m = (1u << 20) / static_cast<uint32_t>(zr.sh_w) + 1;
     const int blocks = (s.n + kBwdThreads - 1) / kBwdThreads + static_cast<int>(zr.items);
 #define GS_PBWD(D) launch_chained(k_preprocess_bwd<D>, blocks, kBwdThreads, 0, st, s, c, tiles, vis_index, ctl, \
-                                  rec_grad, grad_layer_mask, g, contrib_sum, zr)
+                                  geo, rec_grad, grad_layer_mask, g, contrib_sum, zr)
     switch (s.sh_degree) {
         case 0: GS_PBWD(0); break;
         case 1: GS_PBWD(1); break;

@@ -51,23 +51,6 @@ __device__ __forceinline__ float sgn(float v) { return v > 0.f ? 1.f : (v < 0.f 
 // values lie in [0, 1]); zero padding outside the image enters as -kSsimShift.
 constexpr float kSsimShift = 0.5f;
 
-// Two floats in a 64-bit register and their fused multiply-add.
-struct F2 {
-    unsigned long long v;
-    __device__ __forceinline__ F2() {}
-    __device__ __forceinline__ F2(float a, float b) { asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(a), "f"(b)); }
-    __device__ __forceinline__ float2 get() const {
-        float2 r;
-        asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-        return r;
-    }
-};
-__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
-    F2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
-    return r;
-}
-
 // The vertical pass over column cx, output rows 4 sy .. 4 sy + 3, of one pair array and one plain array of
 // horizontal sums.
 __device__ __forceinline__ void window_column(const float2 (*h)[kHP], int cx, int sy, const Win &win, F2 (&m)[kLOut]) {

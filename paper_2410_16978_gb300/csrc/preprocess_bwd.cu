@@ -7,7 +7,7 @@
 // One launch, two kinds of block.  Live blocks take the visible Gaussians
 // from the sort's index-ordered visible list, one thread each, so every warp
 // does the chain rule on 32 live Gaussians instead of the third of its lanes
-// that a pass over all indices would keep; they are bound by memory latency.
+// that a pass over all indices would keep; they are bound by memory.
 // Zero blocks give each warp 256 consecutive Gaussians and store zeros to the
 // rows that are not live, 32 rows at a time with coalesced stores; they are
 // bound by store bandwidth.  The zero blocks are spread evenly among the live
@@ -65,18 +65,22 @@ __device__ __forceinline__ void sh_basis_grad(float x, float y, float z, float *
 }
 
 constexpr int kBwdThreads = 128;
+// Per SM: at most 80 registers.  With the SH rows in shared memory the kernel runs at 5.2 TB/s of its traffic and
+// four to seven CTAs measure the same; before, a row of 48 floats in registers per thread (116) and lanes 192 bytes
+// apart in every load and store: 540,000 visible of 1.2M Gaussians, degree 3, 0.119 -> 0.105 ms; 500,000 of 500,000
+// 0.068 -> 0.061.
+constexpr int kBwdCtas = 6;
 constexpr float kLn2 = 0x1.62e430p-1f;
 
-// Everything the chain rule of Gaussian i reads, issued together before any
-// branch: the inline-PTX loads are volatile, so the compiler keeps them at
-// this point instead of moving them behind the visibility and layer tests.
-template <int K>
+// What the chain rule of Gaussian i reads besides its SH row, issued together
+// before any branch: the inline-PTX loads are volatile, so the compiler keeps
+// them at this point instead of moving them behind the visibility and layer
+// tests.
 struct RowIn {
     float4 ga, gb, gc;       // record gradient
     float A2, beta, G2;      // of the record
     float m[3], ol;
     float ls[3], q[4];       // log-scales and quaternion, widened
-    float sh[3 * K];         // [k][channel]
 };
 
 __device__ __forceinline__ float4 ld_now4(const void *p) {
@@ -90,13 +94,12 @@ __device__ __forceinline__ float ld_now(const float *p) {
     return v;
 }
 
-template <int K>
-__device__ __forceinline__ void load_row(const SceneView &s, int i, const Geo *geo, const float4 *rec_grad, RowIn<K> &r) {
-    asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2];" : "=f"(r.A2), "=f"(r.beta) : "l"(&geo[i].a.z));
-    r.G2 = ld_now(&geo[i].b.x);
+__device__ __forceinline__ void load_row(const SceneView &s, int i, const Geo *geo, const float4 *rec_grad, RowIn &r) {
     r.ga = ld_now4(rec_grad + 3 * i);
     r.gb = ld_now4(rec_grad + 3 * i + 1);
     r.gc = ld_now4(rec_grad + 3 * i + 2);
+    asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2];" : "=f"(r.A2), "=f"(r.beta) : "l"(&geo[i].a.z));
+    r.G2 = ld_now(&geo[i].b.x);
 #pragma unroll
     for (int k = 0; k < 3; ++k) r.m[k] = ld_now(s.means + 3 * static_cast<int64_t>(i) + k);
     r.ol = ld_now(s.opacity_logit + i);
@@ -113,40 +116,77 @@ __device__ __forceinline__ void load_row(const SceneView &s, int i, const Geo *g
 #pragma unroll
         for (int k = 0; k < 4; ++k) r.q[k] = ldv(s.quats, 4 * static_cast<int64_t>(i) + k, s.dtype_sr);
     }
-    const int64_t base = static_cast<int64_t>(i) * 3 * K;
-    if constexpr ((3 * K) % 4 == 0) {
-        if (s.dtype_sh == GS_DTYPE_F32 && (reinterpret_cast<uintptr_t>(s.sh) & 15u) == 0) {
-            const float4 *p = reinterpret_cast<const float4 *>(static_cast<const float *>(s.sh) + base);
+}
+
+// The SH rows of a warp's 32 Gaussians go through shared memory, one row of
+// 3K floats (and padding) per lane: read and written there a lane per row, 16
+// bytes at a time and without bank conflicts (the stride in 16-byte units, or
+// in floats where the row is no multiple of four, is odd), and moved to and
+// from global memory with consecutive lanes on consecutive words of a row.
+template <int K>
+struct ShRow {
+    static constexpr int W = 3 * K;
+    static constexpr bool kQuads = W % 4 == 0;
+    static constexpr int kStride = kQuads ? ((W / 4) % 2 ? W : W + 4) : W;
+};
+
+__device__ __forceinline__ void copy_async(float *dst, const float *src, bool quad) {
+    const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
+    if (quad) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+    else asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src) : "memory");
+}
+
+// Starts the copy of the SH rows of the Gaussians i of lanes 0 .. nrows - 1 (16-bit storage: widens the lane's own).
+template <int K>
+__device__ __forceinline__ void fetch_sh(const SceneView &s, int i, int nrows, int lane, float *sm) {
+    using Row = ShRow<K>;
+    if (s.dtype_sh != GS_DTYPE_F32) {
+        if (lane < nrows) {
 #pragma unroll
-            for (int q = 0; q < 3 * K / 4; ++q) {
-                const float4 x = ld_now4(p + q);
-                r.sh[4 * q] = x.x; r.sh[4 * q + 1] = x.y; r.sh[4 * q + 2] = x.z; r.sh[4 * q + 3] = x.w;
-            }
-            return;
+            for (int e = 0; e < Row::W; ++e)
+                sm[lane * Row::kStride + e] = ldv(s.sh, static_cast<int64_t>(i) * Row::W + e, s.dtype_sh);
         }
+        return;
     }
-    if (s.dtype_sh == GS_DTYPE_F32) {
+    const float *sh = static_cast<const float *>(s.sh);
+    if constexpr (Row::kQuads) {                  // (scene arrays are 16-byte aligned)
+        constexpr int Q = Row::W / 4;
 #pragma unroll
-        for (int e = 0; e < 3 * K; ++e) r.sh[e] = ld_now(static_cast<const float *>(s.sh) + base + e);
+        for (int t = 0; t < Q; ++t) {
+            const int e = t * 32 + lane, row = e / Q, part = e - row * Q;
+            const int64_t src = __shfl_sync(0xFFFFFFFFu, i, row);
+            if (row < nrows) copy_async(sm + row * Row::kStride + 4 * part, sh + src * Row::W + 4 * part, true);
+        }
     } else {
-#pragma unroll
-        for (int e = 0; e < 3 * K; ++e) r.sh[e] = ldv(s.sh, base + e, s.dtype_sh);
+        for (int t = 0; t < Row::W; ++t) {
+            const int e = t * 32 + lane, row = e / Row::W, part = e - row * Row::W;
+            const int64_t src = __shfl_sync(0xFFFFFFFFu, i, row);
+            if (row < nrows) copy_async(sm + row * Row::kStride + part, sh + src * Row::W + part, false);
+        }
     }
 }
 
-// A gradient row of W floats; 16-byte stores where the row allows them.
-template <int W>
-__device__ __forceinline__ void store_row(float *dst, const float *v) {
-    if constexpr (W % 4 == 0) {
-        if ((reinterpret_cast<uintptr_t>(dst) & 15u) == 0) {
+// Stores the gradient rows of the lanes in `rows` from shared memory.
+template <int K>
+__device__ __forceinline__ void store_sh(float *dst, int i, unsigned rows, int lane, const float *sm) {
+    using Row = ShRow<K>;
+    if (Row::kQuads && (reinterpret_cast<uintptr_t>(dst) & 15u) == 0) {
+        constexpr int Q = Row::kQuads ? Row::W / 4 : 1;
 #pragma unroll
-            for (int q = 0; q < W / 4; ++q)
-                reinterpret_cast<float4 *>(dst)[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-            return;
+        for (int t = 0; t < Q; ++t) {
+            const int e = t * 32 + lane, row = e / Q, part = e - row * Q;
+            const int64_t to = __shfl_sync(0xFFFFFFFFu, i, row);
+            if ((rows >> row) & 1u)
+                *reinterpret_cast<float4 *>(dst + to * Row::W + 4 * part) =
+                    *reinterpret_cast<const float4 *>(sm + row * Row::kStride + 4 * part);
+        }
+    } else {
+        for (int t = 0; t < Row::W; ++t) {
+            const int e = t * 32 + lane, row = e / Row::W, part = e - row * Row::W;
+            const int64_t to = __shfl_sync(0xFFFFFFFFu, i, row);
+            if ((rows >> row) & 1u) dst[to * Row::W + part] = sm[row * Row::kStride + part];
         }
     }
-#pragma unroll
-    for (int e = 0; e < W; ++e) dst[e] = v[e];
 }
 
 constexpr unsigned FULL = 0xFFFFFFFFu;
@@ -212,10 +252,9 @@ __device__ __forceinline__ void zero_item(const ZeroRows &zr, uint32_t z, const 
     }
 }
 
-// The chain rule of one live Gaussian.
+// The chain rule of one live Gaussian; its SH row in shared memory is replaced by the gradient's.
 template <int DEG>
-__device__ __forceinline__ void grad_one(const CamView &c, int i, const RowIn<(DEG + 1) * (DEG + 1)> &r,
-                                         const gs_grads &g) {
+__device__ __forceinline__ void grad_one(const CamView &c, int i, const RowIn &r, float *row, const gs_grads &g) {
     constexpr int K = (DEG + 1) * (DEG + 1);
     const float4 ga = r.ga, gb = r.gb, gc = r.gc;
     // from the compositor's moments of dL/de' (e' = ln 2 (A2 p^2 + G2 dy^2), p = dx + beta dy)
@@ -239,27 +278,43 @@ __device__ __forceinline__ void grad_one(const CamView &c, int i, const RowIn<(D
     float b[K];
     float3 db[K];
     sh_basis_grad<DEG>(dx, dy, dz, b, db);
-    const float *shv = r.sh;
-    float gch[3];
+    // per channel: the colour and the sum of sh_k grad b_k, in one pass over the row
+    using Row = ShRow<K>;
+    constexpr int V = Row::kQuads ? 4 : 1;
+    float col[3] = {0.f, 0.f, 0.f};
+    float3 dir[3] = {};
 #pragma unroll
-    for (int ch = 0; ch < 3; ++ch) {
-        float acc = 0.f;
+    for (int e0 = 0; e0 < Row::W; e0 += V) {
+        float v[V];
+        if constexpr (V == 4) *reinterpret_cast<float4 *>(v) = *reinterpret_cast<const float4 *>(row + e0);
+        else v[0] = row[e0];
 #pragma unroll
-        for (int k = 0; k < K; ++k) acc += b[k] * shv[3 * k + ch];
-        gch[ch] = acc + 0.5f > 0.f ? dRgb[ch] : 0.f;
-    }
-    float ddx = 0.f, ddy = 0.f, ddz = 0.f;
-    float gsh[3 * K];
-#pragma unroll
-    for (int ch = 0; ch < 3; ++ch) {
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            gsh[3 * k + ch] = gch[ch] * b[k];
-            const float t = shv[3 * k + ch] * gch[ch];
-            ddx += t * db[k].x; ddy += t * db[k].y; ddz += t * db[k].z;
+        for (int j = 0; j < V; ++j) {
+            const int k = (e0 + j) / 3, ch = (e0 + j) % 3;
+            col[ch] += b[k] * v[j];
+            dir[ch].x += v[j] * db[k].x;
+            dir[ch].y += v[j] * db[k].y;
+            dir[ch].z += v[j] * db[k].z;
         }
     }
-    store_row<3 * K>(g.sh + static_cast<int64_t>(i) * 3 * K, gsh);
+    float gch[3];
+    float ddx = 0.f, ddy = 0.f, ddz = 0.f;
+#pragma unroll
+    for (int ch = 0; ch < 3; ++ch) {
+        const bool on = col[ch] + 0.5f > 0.f;
+        gch[ch] = on ? dRgb[ch] : 0.f;
+        ddx += on ? gch[ch] * dir[ch].x : 0.f;
+        ddy += on ? gch[ch] * dir[ch].y : 0.f;
+        ddz += on ? gch[ch] * dir[ch].z : 0.f;
+    }
+#pragma unroll
+    for (int e0 = 0; e0 < Row::W; e0 += V) {
+        float v[V];
+#pragma unroll
+        for (int j = 0; j < V; ++j) v[j] = gch[(e0 + j) % 3] * b[(e0 + j) / 3];
+        if constexpr (V == 4) *reinterpret_cast<float4 *>(row + e0) = *reinterpret_cast<const float4 *>(v);
+        else row[e0] = v[0];
+    }
     const float dd = ddx * dx + ddy * dy + ddz * dz;
     float gmx = (ddx - dx * dd) * ivn, gmy = (ddy - dy * dd) * ivn, gmz = (ddz - dz * dd) * ivn;
 
@@ -380,7 +435,7 @@ __device__ __forceinline__ void grad_one(const CamView &c, int i, const RowIn<(D
 }
 
 template <int DEG>
-__global__ void __launch_bounds__(kBwdThreads) k_preprocess_bwd(SceneView s, CamView c,
+__global__ void __launch_bounds__(kBwdThreads, kBwdCtas) k_preprocess_bwd(SceneView s, CamView c,
                                                                 const uint32_t *__restrict__ tiles,
                                                                 const uint32_t *__restrict__ vis_index,
                                                                 const Ctl *__restrict__ ctl, const Geo *__restrict__ geo,
@@ -389,6 +444,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_preprocess_bwd(SceneView s, Cam
                                                                 float *__restrict__ contrib_sum, const ZeroRows zr) {
     chain_start();
     constexpr int K = (DEG + 1) * (DEG + 1);
+    __shared__ __align__(16) float s_sh[kBwdThreads / 32][32 * ShRow<K>::kStride];
     const uint32_t nl = (min(ctl->n_vis, static_cast<uint32_t>(s.n)) + kBwdThreads - 1) / kBwdThreads;
     const uint32_t stride = zr.items ? (nl + zr.items) / zr.items : 0xFFFFFFFFu;
     uint32_t b = blockIdx.x;
@@ -398,17 +454,31 @@ __global__ void __launch_bounds__(kBwdThreads) k_preprocess_bwd(SceneView s, Cam
         return;
     }
     b -= min(zr.items, (b + 1) / stride);
-    const uint32_t p = b * kBwdThreads + threadIdx.x;
-    if (p >= min(ctl->n_vis, static_cast<uint32_t>(s.n))) return;
-    const int i = static_cast<int>(vis_index[p]);
-    const uint32_t tc = tiles[i];
-    const uint32_t ly = s.layer[i];
-    RowIn<K> r;
-    load_row<K>(s, i, geo, rec_grad, r);
-    if (tc == 0) return;                        // a two-eye list also holds Gaussians only the other eye sees
-    if (contrib_sum) contrib_sum[i] += r.gc.y;
-    if (!((grad_layer_mask >> ly) & 1u)) return;   // frozen: a zero row
-    grad_one<DEG>(c, i, r, g);
+    const uint32_t nv = min(ctl->n_vis, static_cast<uint32_t>(s.n));
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t p0 = b * kBwdThreads + warp * 32;
+    if (p0 >= nv) return;
+    const int nrows = static_cast<int>(min(nv - p0, 32u));
+    float *sm = s_sh[warp];
+    const bool valid = lane < nrows;
+    const int i = valid ? static_cast<int>(vis_index[p0 + lane]) : 0;
+    fetch_sh<K>(s, i, nrows, lane, sm);
+    uint32_t tc = 0, ly = 0;
+    RowIn r;
+    if (valid) {
+        tc = tiles[i];
+        ly = s.layer[i];
+        load_row(s, i, geo, rec_grad, r);
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncwarp();
+    // (a two-eye list also holds Gaussians that only the other eye sees: tc = 0)
+    if (tc && contrib_sum) contrib_sum[i] += r.gc.y;
+    const bool live = tc && ((grad_layer_mask >> ly) & 1u);        // frozen: a zero row
+    if (live) grad_one<DEG>(c, i, r, sm + lane * ShRow<K>::kStride, g);
+    const unsigned rows = __ballot_sync(FULL, live);
+    __syncwarp();
+    if (rows) store_sh<K>(g.sh, i, rows, lane, sm);
 }
 
 }  // namespace

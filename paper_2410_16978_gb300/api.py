@@ -114,8 +114,10 @@ def gather_rows(src: torch.Tensor, keep_index: torch.Tensor, stream=None) -> tor
 
 
 def _stream_handle(stream: Optional[torch.cuda.Stream]) -> int:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return int(s.cuda_stream)
+    if stream is not None:
+        return int(stream.cuda_stream)
+    # the handle without a Stream object around it: 0.5 instead of 3.2 us, several times per training step
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 class Rasterizer:
@@ -222,6 +224,7 @@ class RenderFunction(torch.autograd.Function):
     def forward(ctx, means, log_scales, quats, opacity_logit, sh, scene: DeviceScene, rast: Rasterizer, camera,
                 layer_mask: int, planes, bg, grad_layer_mask: int, contrib_sum, contrib_max):
         cs = scene.c_struct(means, log_scales, quats, opacity_logit, sh)
+        camera = camera if isinstance(camera, _lib.gs_camera) else _lib.make_camera(camera)
         image, alpha = rast.render(scene, camera, layer_mask, planes, bg, _c_scene=cs)
         ctx.save_for_backward(means, log_scales, quats, opacity_logit, sh)
         ctx.meta = (scene, rast, camera, bg, grad_layer_mask, contrib_sum, contrib_max)

@@ -30,21 +30,24 @@ class ImageLossFunction(torch.autograd.Function):
     def forward(ctx, image, alpha, target_rgb, target_alpha, bg, lam: float, w_alpha: float, workspace):
         H, W = int(image.shape[1]), int(image.shape[2])
         loss = torch.empty((), dtype=torch.float32, device=image.device)
-        d_img = torch.empty_like(image)
-        d_al = torch.empty_like(alpha) if alpha is not None else None
+        # both gradients in one allocation, scaled by one kernel in the backward
+        grad = torch.empty((3 if alpha is None else 4, H, W), dtype=image.dtype, device=image.device)
+        d_img = grad.data_ptr()
+        d_al = None if alpha is None else d_img + 3 * H * W * grad.element_size()
         ws = workspace if workspace is not None else torch.empty(_lib.gs_image_loss_workspace_size(W, H),
                                                                  dtype=torch.uint8, device=image.device)
         _lib.gs_image_loss(image, alpha if w_alpha else None, target_rgb, target_alpha, bg, W, H, lam, w_alpha, ws,
                            ws.numel(), loss, d_img, d_al, _stream_handle(None))
-        ctx.save_for_backward(d_img, d_al if d_al is not None else torch.empty(0, device=image.device))
-        ctx.has_alpha = d_al is not None
+        ctx.save_for_backward(grad)
+        ctx.alpha_shape = None if alpha is None else alpha.shape
         return loss
 
     @staticmethod
     def backward(ctx, g):
-        d_img, d_al = ctx.saved_tensors
         # g is the scalar upstream gradient (1 for loss.backward()); scaling is plumbing
-        return (d_img * g, (d_al * g) if ctx.has_alpha else None, None, None, None, None, None, None)
+        d = ctx.saved_tensors[0] * g
+        d_al = None if ctx.alpha_shape is None else d[3].view(ctx.alpha_shape)
+        return (d[:3], d_al, None, None, None, None, None, None)
 
 
 def image_loss(image, alpha, target_rgb, target_alpha, bg, lam=0.2, w_alpha=0.0, workspace=None):

@@ -351,10 +351,10 @@ enum {
     GS_STAGE_COMPACT,          /* S2: visible count, digit histograms and first-digit tile counts of the depth keys */
     GS_STAGE_DEPTH_SORT,       /* S2: radix digit kernels on the depth bits (the first compacts) */
     GS_STAGE_BIN_ROWS,         /* S2: depth-ordered split of the pairs into tile rows */
-    GS_STAGE_BIN_TILES,        /* S2: split of every row into its tiles, tile ranges */
-    GS_STAGE_COMPOSITE_SETUP,  /* S3/S4: compositor set-ups (forward tile order and checkpoint bases;
-                                  backward: zeroed record gradients; the forward writes the backward's
-                                  work items) */
+    GS_STAGE_BIN_TILES,        /* S2: split of every row into its tiles, tile ranges; the forward compositor's
+                                  tile order and checkpoint bases */
+    GS_STAGE_COMPOSITE_SETUP,  /* S4: the backward compositor's set-up (zeroed record gradients; the forward
+                                  writes its work items) */
     GS_STAGE_COMPOSITE,        /* S3 (one launch per gs_render or gs_render_batch call) */
     GS_STAGE_COMPOSITE_BWD,    /* S4a: the backward compositor */
     GS_STAGE_PREPROCESS_BWD,   /* S4b */

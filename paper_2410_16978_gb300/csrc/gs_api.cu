@@ -27,12 +27,13 @@ bool make_layout(int64_t n, int W, int H, int64_t dup_cap, Layout *L) {
     const size_t N = static_cast<size_t>(n), D = static_cast<size_t>(dup_cap), P = static_cast<size_t>(W) * H;
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t at = off; off += align256(bytes); return at; };
-    // the control block, the depth-sort histograms and group counts, the binning's per-row counters and the
-    // tile ranges are adjacent: one memset per render clears them all
+    // the control block, the depth-sort histograms and group counts, the binning's per-row counters, the counts of
+    // the tile order and the tile ranges are adjacent: one pass per render clears them all
     o.ctl = take(256);
     o.sort_hist = take(4 * 256 * 4);
     o.sort_grp = take(sort_group_bytes(n));
     o.bin_rows = take(bin_rows_bytes(o.Ty));
+    o.tile_hist = take(kTileHistWords * 4);
     o.ranges = take(static_cast<size_t>(o.Tn) * 8);
     o.rec = take(N * sizeof(Rec));
     o.geo = take(N * sizeof(Geo));
@@ -399,19 +400,21 @@ int front_sort(FrontCtx *f, int n, bool shared, cudaStream_t st) {
 }
 
 // Phase 3: binning of n views in their depth orders (whose counts are at n_vis),
-// the compositor set-ups, and the forward jobs of the views.
+// with what the compositor starts from, and the forward jobs of the views.
 int front_bin(FrontCtx *f, int n, cudaStream_t st, FwdJob *jobs) {
     BinView b[kMaxBatch];
-    SetupView s[kMaxBatch];
     for (int i = 0; i < n; ++i) {
         const Layout &L = f[i].L;
         void *ws = f[i].ws;
         const PreView &p = f[i].pre;
         b[i] = BinView{f[i].order, p.rec, static_cast<uint32_t>(p.s.n), p.c.Tx, p.c.Ty, at<uint32_t>(ws, L.bin_m),
                        at<void>(ws, L.bin_rows), at<uint2>(ws, L.rowlist), p.ctl, static_cast<uint64_t>(L.dup_cap),
-                       at<uint32_t>(ws, L.bin_p), at<uint32_t>(ws, L.list), at<uint2>(ws, L.ranges)};
+                       at<uint32_t>(ws, L.bin_p), at<uint32_t>(ws, L.list), at<uint2>(ws, L.ranges), nullptr,
+                       nullptr, nullptr, at<uint32_t>(ws, L.tile_hist)};
         const CompositeBufs cb = composite_bufs(ws, L);
-        s[i] = SetupView{b[i].ranges, L.Tn, cb.order, cb.seg_base, cb.queue, cb.qdone};
+        b[i].tile_order = cb.order;
+        b[i].seg_base = cb.seg_base;
+        b[i].qdone = cb.qdone;
         FwdJob *job = &jobs[i];
         job->order = cb.order;
         job->list = b[i].list;
@@ -442,15 +445,11 @@ int front_bin(FrontCtx *f, int n, cudaStream_t st, FwdJob *jobs) {
         Stage sg(GS_STAGE_BIN_ROWS, st, 3);
         if ((rc = cuda_check(launch_bin_rows(b, n, st), "binning rows")) != GS_OK) return rc;
     }
-    {
-        Stage sg(GS_STAGE_BIN_TILES, st, 3);
-        if ((rc = cuda_check(launch_bin_tiles(b, n, st), "binning tiles")) != GS_OK) return rc;
-    }
-    Stage sg(GS_STAGE_COMPOSITE_SETUP, st, 1);
-    return cuda_check(launch_fwd_setup(s, n, st), "compositor set-up");
+    Stage sg(GS_STAGE_BIN_TILES, st, 3);
+    return cuda_check(launch_bin_tiles(b, n, st), "binning tiles");
 }
 
-// S1, S2 and the compositor set-up of n validated views, and their forward jobs.
+// S1 and S2 of n validated views, and their forward jobs.
 int render_front(FrontCtx *f, int n, cudaStream_t st, FwdJob *jobs) {
     int rc;
     if ((rc = front_preprocess(f, n, st)) != GS_OK) return rc;

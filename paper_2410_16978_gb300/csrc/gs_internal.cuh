@@ -26,6 +26,8 @@ constexpr float kFrustumClamp = 1.3f;          // x/z and y/z clamped to this mu
 constexpr float kRadiusSigmas = 3.0f;          // splat radius in standard deviations of the larger eigenvalue
 constexpr float kEigenFloor = 0.1f;            // floor of (mid^2 - det) under the eigenvalue square root
 constexpr uint32_t kSeg = 256;                 // list positions per backward segment (checkpoint stride)
+constexpr int kWorkBuckets = 513;              // buckets of the heaviest-first tile order
+constexpr int kTileHistWords = 2 * kWorkBuckets + 2;   // bucket counts, bucket cursors, segments handed out
 constexpr int kCbMaxDim = 48;                  // SH codebook: coordinates per row, 3(K-1) <= 45 padded
 constexpr int kBinMaxDim = 256;                // tile rows and columns the binning handles (4096 px)
 constexpr int kBinBlocks = 608;                // CTAs (of 8 chunk warps) of the row pass of the binning: four per SM
@@ -94,13 +96,15 @@ __device__ __forceinline__ bool gs_check(bool ok, const Ctl *ctl, uint32_t site)
 #define GS_CHECK(ok, ctl, site) true
 #endif
 
+__device__ __forceinline__ uint32_t ceil_seg(uint32_t n) { return (n + kSeg - 1) / kSeg; }
+
 // Workspace carve-up.  Every region starts on a 256-byte boundary.
 struct Layout {
     int64_t n = 0, dup_cap = 0;
     int W = 0, H = 0, Tx = 0, Ty = 0, Tn = 0;
     size_t ctl = 0, rec = 0, geo = 0, tiles = 0, depth = 0, sort_k[2] = {0, 0}, sort_v[2] = {0, 0}, order = 0, vis_index = 0,
            sort_hist = 0, sort_grp = 0, sort_cnt = 0, sort_status = 0, bin_m = 0,
-           bin_rows = 0, bin_p = 0, rowlist = 0, list = 0, ranges = 0, t_final = 0, n_contrib = 0,
+           bin_rows = 0, tile_hist = 0, bin_p = 0, rowlist = 0, list = 0, ranges = 0, t_final = 0, n_contrib = 0,
            partials = 0, rec_grad = 0, tile_order = 0, qdone = 0, seg_base = 0, qwork = 0,
            ckpt = 0, items = 0, total = 0;
 };
@@ -340,6 +344,11 @@ struct BinView {
     uint64_t cap;
     uint32_t *P, *list;
     uint2 *ranges;
+    // what the forward compositor starts from (see k_bin_tiles_scan)
+    uint4 *tile_order;         // [Tn] tiles, heaviest first
+    uint32_t *seg_base;        // [Tn]
+    uint32_t *qdone;           // [8 Tn]
+    uint32_t *tile_hist;       // kTileHistWords, cleared at the start of a call
 };
 cudaError_t launch_bin_rows(const BinView *views, int n, cudaStream_t st);
 cudaError_t launch_bin_tiles(const BinView *views, int n, cudaStream_t st);
@@ -402,23 +411,13 @@ struct FwdJob {
     uint32_t *queue;       // the view's work-queue word (written by its set-up)
     uint2 *items;          // the view's backward work items, appended as the forward finishes 8x8 blocks
     uint32_t *n_items;     // their count (zero at the start of the render)
-    uint32_t *qdone;       // [8 Tn] per 8x8 block, a half per 8x4 block: 0 or its longest prefix + 1 (zeroed by the set-up)
+    uint32_t *qdone;       // [8 Tn] per 8x8 block, a half per 8x4 block: 0 or its longest prefix + 1 (zeroed by the binning)
 };
-// Per-view set-up before compositing: tile order, checkpoint bases, zeroed
-// block work and queue.  The backward's set-up also zeroes the record-gradient
-// rows of the visible Gaussians (vis_index, *n_vis of the n Gaussians).
-struct SetupView {
-    const uint2 *ranges;
-    int Tn;
-    uint4 *order;
-    uint32_t *seg_base, *queue, *qdone;
-};
-cudaError_t launch_fwd_setup(const SetupView *views, int n, cudaStream_t st);
 // Composites n <= kMaxBatch views with one persistent launch; every view's
-// queue must have been written on the stream (its launch_fwd_setup does).
+// tile order must have been written on the stream (launch_bin_tiles does).
 cudaError_t launch_composite_forward(const FwdJob *jobs, int n, cudaStream_t st);
-// Backward set-up: work items (tile order by longest blended prefix) and the
-// zeroed record-gradient rows of the visible Gaussians.
+// Backward set-up: its queue and the zeroed record-gradient rows of the
+// visible Gaussians (vis_index, *n_vis of the n Gaussians).
 cudaError_t launch_bwd_setup(const CompositeBufs &cb, int Tx, int Ty, float4 *rec_grad, const uint32_t *vis_index,
                              const uint32_t *n_vis, int n, cudaStream_t st);
 cudaError_t launch_composite_backward(const CompositeBufs &cb, const uint2 *ranges, const uint32_t *list,

@@ -276,11 +276,17 @@ __device__ uint32_t look_back(uint64_t *status, uint32_t t, int c, uint32_t own,
     return excl;
 }
 
+// Four Gaussians per thread: with sixteen the chain of a warp's shuffles and
+// votes set the time of small scenes (4,096 Gaussians 12.5 -> 7.8 us, 1.2M 16.5 -> 10.6,
+// 3M 24.9 -> 17.1).
+constexpr int kHistThreads = 1024;
+constexpr int kHistItems = kPassTile / kHistThreads;
+
 template <class Src, int NV>
-__global__ void __launch_bounds__(256) k_sort_hist(const __grid_constant__ Views<SortJob, NV> B) {
+__global__ void __launch_bounds__(kHistThreads) k_sort_hist(const __grid_constant__ Views<SortJob, NV> B) {
     chain_start();
     __shared__ uint32_t s_h[4][256];
-    __shared__ uint32_t s_w[8];
+    __shared__ uint32_t s_vis, s_kinv, s_kmax;
     const SortJob &J = B[blockIdx.y];
     const uint32_t n = J.v.n;
     const uint32_t t = blockIdx.x;
@@ -290,64 +296,67 @@ __global__ void __launch_bounds__(256) k_sort_hist(const __grid_constant__ Views
     Ctl *ctl = J.v.ctl;
     const TileCounts tc = J.tc;
     const int lane = threadIdx.x & 31;
-    for (int k = threadIdx.x; k < 4 * 256; k += 256) (&s_h[0][0])[k] = 0;
+    for (int k = threadIdx.x; k < 4 * 256; k += kHistThreads) (&s_h[0][0])[k] = 0;
+    if (threadIdx.x == 0) s_vis = s_kinv = s_kmax = 0;         // (0 is neutral for both maxima)
+    const uint32_t beg = t * kPassTile;
+    bool vis[kHistItems];
+    uint32_t key[kHistItems];
+#pragma unroll
+    for (int r = 0; r < kHistItems; ++r) {
+        const uint32_t i = beg + r * kHistThreads + threadIdx.x;
+        vis[r] = i < n && src.visible(i);
+    }
+#pragma unroll
+    for (int r = 0; r < kHistItems; ++r) key[r] = vis[r] ? src.key(beg + r * kHistThreads + threadIdx.x) : 0u;
     __syncthreads();
-    const uint32_t beg = t * kPassTile, end = min(n, beg + kPassTile);
     uint32_t kinv = 0, kmax = 0, cnt = 0;
-    for (uint32_t t0 = beg; t0 < end; t0 += kSortTile) {
-        bool vis[kSortItems];
-        uint32_t key[kSortItems];
 #pragma unroll
-        for (int r = 0; r < kSortItems; ++r) {
-            const uint32_t i = t0 + r * 256 + threadIdx.x;
-            vis[r] = i < end && src.visible(i);
+    for (int r = 0; r < kHistItems; ++r) {
+        if (vis[r]) {
+            src.settle(beg + r * kHistThreads + threadIdx.x);
+            kinv = max(kinv, ~key[r]);
+            kmax = max(kmax, key[r]);
         }
+        const unsigned vm = __ballot_sync(FULL, vis[r]);
+        if (vm == 0) continue;
+        cnt += __popc(vm);
+        const int leader = __ffs(vm) - 1;
 #pragma unroll
-        for (int r = 0; r < kSortItems; ++r) key[r] = vis[r] ? src.key(t0 + r * 256 + threadIdx.x) : 0u;
-#pragma unroll
-        for (int r = 0; r < kSortItems; ++r) {
-            if (vis[r]) {
-                src.settle(t0 + r * 256 + threadIdx.x);
-                kinv = max(kinv, ~key[r]);
-                kmax = max(kmax, key[r]);
-                ++cnt;
-            }
-            const unsigned vm = __ballot_sync(FULL, vis[r]);
-            if (vm == 0) continue;
-            const int leader = __ffs(vm) - 1;
-#pragma unroll
-            for (int p = 0; p < 4; ++p) {
-                // one atomic when the warp's visible keys share the digit (the high digits
-                // of depths in a narrow range), else one per key
-                const uint32_t d = (key[r] >> (8 * p)) & 255u;
-                const uint32_t dl = __shfl_sync(FULL, d, leader);
-                if (__all_sync(FULL, !vis[r] || d == dl)) {
-                    if (lane == leader) atomicAdd(&s_h[p][dl], __popc(vm));
-                } else if (vis[r]) {
-                    atomicAdd(&s_h[p][d], 1u);
-                }
+        for (int p = 0; p < 4; ++p) {
+            // one atomic when the warp's visible keys share the digit (the high digits
+            // of depths in a narrow range), else one per key
+            const uint32_t d = (key[r] >> (8 * p)) & 255u;
+            const uint32_t dl = __shfl_sync(FULL, d, leader);
+            if (__all_sync(FULL, !vis[r] || d == dl)) {
+                if (lane == leader) atomicAdd(&s_h[p][dl], __popc(vm));
+            } else if (vis[r]) {
+                atomicAdd(&s_h[p][d], 1u);
             }
         }
     }
     kinv = __reduce_max_sync(FULL, kinv);
     kmax = __reduce_max_sync(FULL, kmax);
-    if (lane == 0) {        // 0 is neutral for both maxima
-        atomicMax(&ctl->depth_mm[0], kinv);
-        atomicMax(&ctl->depth_mm[1], kmax);
+    if (lane == 0 && cnt) {
+        atomicAdd(&s_vis, cnt);
+        atomicMax(&s_kinv, kinv);
+        atomicMax(&s_kmax, kmax);
     }
-    uint32_t tot;
-    block_scan_256(cnt, s_w, &tot);
-    if (threadIdx.x == 0 && tot) {
-        atomicAdd(&ctl->n_vis, tot);
-        atomicAdd(&ctl->st.n_visible, tot);
+    __syncthreads();
+    if (threadIdx.x == 0 && s_vis) {
+        atomicAdd(&ctl->n_vis, s_vis);
+        atomicAdd(&ctl->st.n_visible, s_vis);
+        atomicMax(&ctl->depth_mm[0], s_kinv);
+        atomicMax(&ctl->depth_mm[1], s_kmax);
     }
-    for (int k = threadIdx.x; k < 4 * 256; k += 256) {
+    for (int k = threadIdx.x; k < 4 * 256; k += kHistThreads) {
         const uint32_t c = (&s_h[0][0])[k];
         if (c) atomicAdd(&ghist[k], c);
     }
-    const uint32_t c0 = s_h[0][threadIdx.x];
-    tc.cnt[static_cast<size_t>(t) * kLookCounters + threadIdx.x] = c0;
-    if (c0) atomicAdd(&tc.grp[static_cast<size_t>(t >> tc.lg) * kLookCounters + threadIdx.x], c0);
+    if (threadIdx.x < 256) {
+        const uint32_t c0 = s_h[0][threadIdx.x];
+        tc.cnt[static_cast<size_t>(t) * kLookCounters + threadIdx.x] = c0;
+        if (c0) atomicAdd(&tc.grp[static_cast<size_t>(t >> tc.lg) * kLookCounters + threadIdx.x], c0);
+    }
 }
 
 // One digit kernel's buffers: pass p reads what pass p - 1 wrote.
@@ -384,6 +393,22 @@ struct SortBufs {
 // warp-private 16-bit digit counters, so items are ranked in index order; the
 // tile is then sorted by digit in shared memory and written out in that order,
 // so consecutive threads store consecutive addresses of one digit's run.
+
+// The lanes that hold a valid item of the same digit (of valid lanes; the
+// others' result is not used): a ballot per bit.  match.any took about 900
+// cycles a round with the 16 warps of a CTA (more than half the time of a
+// tile), the ballots 250: 3M
+// Gaussians 0.147 -> 0.114 ms, eight times 500,000 0.206 -> 0.165, 4,096 0.032 -> 0.026 (all four kernels).
+__device__ __forceinline__ unsigned same_digit(uint32_t d, bool valid) {
+    unsigned peers = __ballot_sync(FULL, valid);
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+        const bool bit = (d >> b) & 1u;
+        const unsigned m = __ballot_sync(FULL, bit);
+        peers &= bit ? m : ~m;
+    }
+    return peers;
+}
 
 // Exclusive scan over the 512 threads of a block; *total = sum of all v.
 __device__ __forceinline__ uint32_t block_scan_512(uint32_t v, uint32_t *s_w, uint32_t *total) {
@@ -477,8 +502,8 @@ __global__ void __launch_bounds__(kPassThreads) k_sort_pass(const __grid_constan
     uint32_t vw = 0;
 #pragma unroll
     for (int r = 0; r < kSortItems; ++r) {
-        const uint32_t d = valid[r] ? (key[r] >> shift) & 255u : 256u + lane;
-        const unsigned peers = __match_any_sync(FULL, d);
+        const uint32_t d = (key[r] >> shift) & 255u;
+        const unsigned peers = same_digit(d, valid[r]);
         const uint32_t before = valid[r] ? s_wc[warp][d] : 0;
         rank[r] = before + __popc(peers & lt);
         __syncwarp();
@@ -630,7 +655,7 @@ void with_sort(const SortJob *jobs, int m, F f) {
 template <class Src, int NV>
 void hist_kernel(Src *, const Views<SortJob, NV> &b, uint32_t most, cudaStream_t st) {
     // the histograms and the group counts were cleared with the control block
-    launch_chained(k_sort_hist<Src, NV>, dim3(most, b.n), 256, 0, st, b);
+    launch_chained(k_sort_hist<Src, NV>, dim3(most, b.n), kHistThreads, 0, st, b);
 }
 
 template <class Src, int NV>

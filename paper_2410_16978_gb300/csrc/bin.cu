@@ -74,13 +74,17 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t *s_w, u
 //     ballot gives the lanes that cover the bucket, a lane's rank is the number
 //     of those below it, and they store to consecutive addresses.
 // Every lane works on every step and a store instruction covers one or two
-// lines.  Bound by instruction issue (66% of the slots, about three warp
-// instructions per pair).  The tile pass (count, scan and write) on the
-// 3M-Gaussian 2064x2208 close view (122M pairs) took 0.440 ms, 1.043 ms when
-// pairs were expanded 32 at a time and lanes with equal buckets ranked by
-// __match_any_sync or ballots, each 4-byte store a line of its own; 0.240
-// against 0.472 ms on the two eyes of a 3M-Gaussian stereo pair (26M pairs
-// each), 0.168 against 0.307 ms at 1920x1080 (36M pairs).  Also measured: a lane
+// lines.  Bound by instruction issue (67% of the slots).  Per 32 entries the
+// scan only tests whether they reach the group and stages them, four words in a
+// row; coverage bits are formed for the staged ones.  The tile pass (count,
+// scan and write) on the 3M-Gaussian 2064x2208 close view (122M pairs) takes
+// 0.398 ms; 0.455 with the coverage formed for every entry and the words taken
+// one at a time; 1.043 when pairs were expanded 32 at a time and lanes with
+// equal buckets ranked by __match_any_sync or ballots, each 4-byte store a line
+// of its own.  Two eyes of a 3M-Gaussian stereo pair (26M pairs each) 0.214,
+// 0.244 and 0.472 ms; 1920x1080 (36M pairs) 0.146, 0.166 and 0.307.  Warps that
+// take their items from a queue: 0.390 on the close view, but 0.063 against
+// 0.052 ms on a 1024x1024 frame.  Also measured: a lane
 // per bucket walking the set bits of the transposed coverage matrix (0.490 ms
 // on the close view: a third of the lanes idle where the tile lists of a group
 // differ in length).
@@ -101,6 +105,11 @@ __device__ __forceinline__ uint32_t coverage(uint32_t x0, uint32_t x1, uint32_t 
     const uint32_t a = static_cast<uint32_t>(max(static_cast<int>(x0 - c0), 0));
     const uint32_t b = static_cast<uint32_t>(max(static_cast<int>(x1 - c0), 0));
     return bit_run(a, b - a) & ((1u << kGroup) - 1u);
+}
+
+// Does [x0, x1) = x reach a bucket of [c0, c0 + kGroup)?
+__device__ __forceinline__ bool reaches(uint32_t x, uint32_t c0) {
+    return (x & 0xFFFFu) < c0 + kGroup && x >= (c0 + 1u) << 16;
 }
 
 // Stores one entry per lane (cov: its buckets) at the running positions
@@ -242,7 +251,7 @@ __global__ void __launch_bounds__(256) k_bin_rows_write(const __grid_constant__ 
     const int Ty = V.Ty;
     __shared__ uint32_t s_pos[8][kBinMaxDim];
     __shared__ uint2 s_val[8][kRowBlock];
-    __shared__ uint16_t s_cov[8][kRowBlock];
+    __shared__ uint32_t s_rows[8][kRowBlock];
     if (ctl->st.error != GS_OK) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
@@ -299,12 +308,12 @@ __global__ void __launch_bounds__(256) k_bin_rows_write(const __grid_constant__ 
 #pragma unroll
             for (int w = 0; w < kRowWords; ++w) {
                 if (w >= words) break;
-                const uint32_t cov = coverage(y01[w] & 0xFFFFu, y01[w] >> 16, c0);
-                const unsigned km = __ballot_sync(FULL, cov != 0);
-                if (cov) {
+                const bool in = reaches(y01[w], c0);
+                const unsigned km = __ballot_sync(FULL, in);
+                if (in) {
                     const int slot = fill + __popc(km & lt);
                     s_val[warp][slot] = make_uint2(g[w], x01[w]);
-                    s_cov[warp][slot] = static_cast<uint16_t>(cov);
+                    s_rows[warp][slot] = y01[w];
                 }
                 fill += __popc(km);
             }
@@ -316,7 +325,8 @@ __global__ void __launch_bounds__(256) k_bin_rows_write(const __grid_constant__ 
             for (int c = 0; c < kGroup; ++c) pos[c] = __shfl_sync(FULL, mine, c);
             for (int k = 0; k < fill; k += 32) {
                 const bool in = k + lane < fill;
-                emit_group(in ? s_cov[warp][k + lane] : 0u, in ? s_val[warp][k + lane] : make_uint2(0u, 0u), pos,
+                const uint32_t y = in ? s_rows[warp][k + lane] : 0u;
+                emit_group(coverage(y & 0xFFFFu, y >> 16, c0), in ? s_val[warp][k + lane] : make_uint2(0u, 0u), pos,
                            rowlist, lt, ok);
             }
 #pragma unroll
@@ -538,8 +548,7 @@ __global__ void __launch_bounds__(256) k_bin_tiles_write(const __grid_constant__
     uint32_t *__restrict__ list = V.list;
     const Ctl *ctl = V.ctl;
     const int Tx = V.Tx, Ty = V.Ty;
-    __shared__ uint32_t s_val[8][64];              // compacted entries, a ring of two words of 32
-    __shared__ uint16_t s_cov[8][64];
+    __shared__ uint2 s_en[8][32 * (kStepWords + 1)];   // entries that reach the warp's tiles: a step's and what was left
     __shared__ uint32_t s_ps[kBinMaxDim + 1];
     __shared__ uint32_t s_first[kWorkBuckets], s_w[8];
     const bool good = ctl->st.error == GS_OK;
@@ -569,7 +578,12 @@ __global__ void __launch_bounds__(256) k_bin_tiles_write(const __grid_constant__
         uint32_t pos[kGroup];
 #pragma unroll
         for (int c = 0; c < kGroup; ++c) pos[c] = __shfl_sync(FULL, at, c);
-        int head = 0, fill = 0;
+        uint32_t fill = 0;
+        uint2 *buf = s_en[warp];
+        const auto emit = [&](uint32_t k, bool in) {
+            const uint2 e = buf[k + lane];
+            emit_group<uint32_t>(in ? coverage(e.y & 0xFFFFu, e.y >> 16, c0) : 0u, e.x, pos, list, lt, ok);
+        };
         uint2 en_nx[kStepWords];                   // entries one step ahead
         const auto entries = [&](uint32_t q0) {
 #pragma unroll
@@ -582,31 +596,25 @@ __global__ void __launch_bounds__(256) k_bin_tiles_write(const __grid_constant__
 #pragma unroll
             for (int w = 0; w < kStepWords; ++w) en[w] = en_nx[w];
             entries(q0 + 32 * kStepWords);
-#pragma unroll 1
-            for (int w = 0; w < kStepWords; ++w) {
-                const uint2 now = en[0];
 #pragma unroll
-                for (int k = 0; k + 1 < kStepWords; ++k) en[k] = en[k + 1];
-                const uint32_t cov = coverage(now.y & 0xFFFFu, now.y >> 16, c0);
-                const unsigned km = __ballot_sync(FULL, cov != 0);
-                if (cov) {
-                    const int slot = (head + fill + __popc(km & lt)) & 63;
-                    s_val[warp][slot] = now.x;
-                    s_cov[warp][slot] = static_cast<uint16_t>(cov);
-                }
+            for (int w = 0; w < kStepWords; ++w) {
+                const bool in = reaches(en[w].y, c0);
+                const unsigned km = __ballot_sync(FULL, in);
+                if (in) buf[fill + __popc(km & lt)] = en[w];
                 fill += __popc(km);
-                if (fill >= 32) {
-                    __syncwarp();
-                    emit_group<uint32_t>(s_cov[warp][head + lane], s_val[warp][head + lane], pos, list, lt, ok);
-                    head ^= 32;
-                    fill -= 32;
-                    __syncwarp();
-                }
             }
+            __syncwarp();
+            uint32_t k = 0;
+            for (; k + 32 <= fill; k += 32) emit(k, true);
+            if (k) {                               // the rest to the front
+                const uint2 e = buf[k + lane];     // (k + 32 <= 32 (kStepWords + 1): in the buffer)
+                __syncwarp();
+                buf[lane] = e;
+                fill -= k;
+            }
+            __syncwarp();
         }
-        __syncwarp();
-        if (fill)
-            emit_group<uint32_t>(lane < fill ? s_cov[warp][head + lane] : 0u, s_val[warp][head + lane], pos, list, lt, ok);
+        if (fill) emit(0, lane < fill);
         __syncwarp();
     }
 }

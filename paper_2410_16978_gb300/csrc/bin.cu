@@ -174,7 +174,8 @@ __device__ __forceinline__ void chunk_range(uint32_t n, uint32_t c, uint32_t K, 
     e = static_cast<uint32_t>(static_cast<uint64_t>(n) * (c + 1) / K);
 }
 
-// Rows, count: a warp per chunk of the depth order counts its entries and pairs per tile row.
+// Rows, count: a warp per chunk of the depth order counts its entries and pairs per tile row, and lays the tile
+// rectangles out in depth order for the write (x01 and y01: first | last + 1 << 16).
 template <int NV>
 __global__ void __launch_bounds__(256) k_bin_rows_count(const __grid_constant__ Views<BinView, NV> B) {
     chain_start();
@@ -206,6 +207,10 @@ __global__ void __launch_bounds__(256) k_bin_rows_count(const __grid_constant__ 
         gid = p0 + 64 + lane < e ? order[p0 + 64 + lane] : 0u;
         // rows [y0, y1) each get one entry and w pairs: difference array
         const uint32_t r0 = __float_as_uint(cc.z), r1 = __float_as_uint(cc.w);
+        if (p0 + lane < e) {
+            V.x01[p0 + lane] = (r0 & 0xFFFFu) | (r1 << 16);
+            V.y01[p0 + lane] = (r0 >> 16) | (r1 & 0xFFFF0000u);
+        }
         const uint32_t y0 = r0 >> 16, y1 = r1 >> 16, w = (r1 & 0xFFFFu) - (r0 & 0xFFFFu);
         if (y1 > y0) {
             atomicAdd(&s_cnt[warp][y0], 1u);
@@ -229,111 +234,99 @@ __global__ void __launch_bounds__(256) k_bin_rows_count(const __grid_constant__ 
     }
 }
 
-// Rows, write: the chunk's warp writes its row-list entries, 128 Gaussians at
-// a time (their ids and tile rectangles loaded while the block before them is
-// written), 16 tile rows at a time.  Four CTAs per SM with blocks of 128:
-// row pass of the 1.2M-Gaussian 1024x1024 frame 0.043 ms against 0.046 with
-// two CTAs per SM and blocks of 256 (0.219 against 0.224 ms on the close view).
-constexpr int kRowWords = 4;
-constexpr int kRowBlock = 32 * kRowWords;
+// Rows, write: a warp per (chunk, kGroup tile rows) writes their row-list entries, as the tile pass does its lists.
+// A warp that took all rows of its chunk, 128 Gaussians at a time, stored the 20 or so of them that reach a group of a
+// tall image by themselves, two thirds of its lanes idle: row pass of the 3M-Gaussian close view 0.220 -> 0.150 ms,
+// stereo pair 0.114 -> 0.100, 1920x1080 0.073 -> 0.062, eight 512x512 views 0.173 -> 0.129.
+constexpr int kRowWords = 4;       // words of 32 Gaussians loaded per step, one step ahead
 
 template <int NV>
-__global__ void __launch_bounds__(256) k_bin_rows_write(const __grid_constant__ Views<BinView, NV> B) {
+__global__ void __launch_bounds__(256) k_bin_rows_write(const __grid_constant__ Views<BinView, NV> B, uint32_t K) {
     chain_start();
     const BinView &V = B[blockIdx.y];
     const uint32_t *__restrict__ order = V.order;
-    const Rec *__restrict__ rec = V.rec;
+    const uint32_t *__restrict__ x01 = V.x01, *__restrict__ y01 = V.y01;
     const uint32_t *__restrict__ M = V.M;
     const RowInfo *__restrict__ rows = rows_of(V);
     uint2 *__restrict__ rowlist = V.rowlist;
     const Ctl *ctl = V.ctl;
-    const uint32_t n_cap = V.n_cap;
     const int Ty = V.Ty;
-    __shared__ uint32_t s_pos[8][kBinMaxDim];
-    __shared__ uint2 s_val[8][kRowBlock];
-    __shared__ uint32_t s_rows[8][kRowBlock];
+    constexpr int kBuf = 32 * (kRowWords + 1);
+    __shared__ uint2 s_val[8][kBuf];               // Gaussians that reach the warp's rows: a step's and what was left
+    __shared__ uint32_t s_rows[8][kBuf];
     if (ctl->st.error != GS_OK) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
-    const uint32_t K = gridDim.x * 8u;
-    // the block's 8 chunks are 8 consecutive columns of the row-major count
-    // matrix: thread t moves (row t / 8, column t % 8), so every row segment
-    // is one 32-byte transaction
-    for (int t = threadIdx.x; t < 8 * Ty; t += blockDim.x) {
-        const int r = t >> 3, w = t & 7;
-        const uint32_t ch = blockIdx.x * 8u + w, part = ch / (K / kRowParts);
-        s_pos[w][r] = rows[r].start + (part ? rows[r].part_base[part - 1] : 0u) + M[static_cast<size_t>(r) * K + ch];
-    }
-    __syncthreads();
-    uint32_t b, e;
-    chunk_range(min(ctl->n_vis, n_cap), blockIdx.x * 8u + warp, K, b, e);
-    // blocks of equal size, whole words
-    const uint32_t nblk = (e - b + kRowBlock - 1) / kRowBlock;
-    const uint32_t step = nblk ? ((e - b + nblk - 1) / nblk + 31u) & ~31u : 32u;
-    const int words = static_cast<int>(step / 32);
+    const uint32_t n = min(ctl->n_vis, V.n_cap);
+    const uint32_t groups = (Ty + kGroup - 1) / kGroup, items = K * groups;
     const auto ok = [&](uint32_t p) { return GS_CHECK(p < ctl->st.dup_capacity, ctl, kSiteRowList); };
-    constexpr uint32_t kNone = 0xFFFFFFFFu;
-    uint32_t gn[kRowWords];
-    float2 rn[kRowWords];
-    const auto load = [&](uint32_t p0) {
-#pragma unroll
-        for (int w = 0; w < kRowWords; ++w) {
-            const uint32_t p = p0 + 32 * w + lane;
-            gn[w] = w < words && p < e ? order[p] : kNone;
+    uint2 *val = s_val[warp];
+    uint32_t *yy = s_rows[warp];
+    for (uint32_t it = blockIdx.x * 8u + warp; it < items; it += gridDim.x * 8u) {
+        const uint32_t ch = it / groups, c0 = kGroup * (it - ch * groups);
+        uint32_t b, e;
+        chunk_range(n, ch, K, b, e);
+        if (b >= e) continue;
+        uint32_t at = 0;
+        if (lane < kGroup && c0 + lane < static_cast<uint32_t>(Ty)) {
+            const uint32_t r = c0 + lane, part = ch / (K / kRowParts);
+            at = rows[r].start + (part ? rows[r].part_base[part - 1] : 0u) + M[static_cast<size_t>(r) * K + ch];
         }
+        uint32_t pos[kGroup];
 #pragma unroll
-        for (int w = 0; w < kRowWords; ++w)
-            rn[w] = gn[w] != kNone ? *reinterpret_cast<const float2 *>(&rec[gn[w]].c.z) : make_float2(0.f, 0.f);
-    };
-    load(b);
-    for (uint32_t p0 = b; p0 < e; p0 += step) {
-        uint32_t g[kRowWords], y01[kRowWords], x01[kRowWords];
-        uint32_t lo = 0xFFFFu, hi = 0;
-#pragma unroll
-        for (int w = 0; w < kRowWords; ++w) {
-            const uint32_t r0 = __float_as_uint(rn[w].x), r1 = __float_as_uint(rn[w].y);
-            g[w] = gn[w];
-            x01[w] = (r0 & 0xFFFFu) | (r1 << 16);
-            y01[w] = (r0 >> 16) | (r1 & 0xFFFF0000u);
-            if (r0 >> 16 < r1 >> 16) {
-                lo = min(lo, r0 >> 16);
-                hi = max(hi, r1 >> 16);
-            }
-        }
-        load(p0 + step);
-        lo = __reduce_min_sync(FULL, lo);
-        hi = __reduce_max_sync(FULL, hi);
-        for (uint32_t c0 = lo & ~(kGroup - 1u); c0 < hi; c0 += kGroup) {
-            int fill = 0;
+        for (int c = 0; c < kGroup; ++c) pos[c] = __shfl_sync(FULL, at, c);
+        uint32_t fill = 0;
+        const auto emit = [&](uint32_t k, bool in) {
+            const uint32_t y = in ? yy[k + lane] : 0u;
+            emit_group(coverage(y & 0xFFFFu, y >> 16, c0), val[k + lane], pos, rowlist, lt, ok);
+        };
+        uint32_t yn[kRowWords], xn[kRowWords], gn[kRowWords];      // one step ahead
+        const auto load = [&](uint32_t p0) {
 #pragma unroll
             for (int w = 0; w < kRowWords; ++w) {
-                if (w >= words) break;
-                const bool in = reaches(y01[w], c0);
+                const uint32_t p = p0 + 32 * w + lane;
+                const bool in = p < e;
+                yn[w] = in ? y01[p] : 0u;
+                xn[w] = in ? x01[p] : 0u;
+                gn[w] = in ? order[p] : 0u;
+            }
+        };
+        load(b);
+        for (uint32_t p0 = b; p0 < e; p0 += 32 * kRowWords) {
+            uint32_t y[kRowWords], x[kRowWords], g[kRowWords];
+#pragma unroll
+            for (int w = 0; w < kRowWords; ++w) {
+                y[w] = yn[w];
+                x[w] = xn[w];
+                g[w] = gn[w];
+            }
+            load(p0 + 32 * kRowWords);
+#pragma unroll
+            for (int w = 0; w < kRowWords; ++w) {
+                const bool in = reaches(y[w], c0);
                 const unsigned km = __ballot_sync(FULL, in);
                 if (in) {
-                    const int slot = fill + __popc(km & lt);
-                    s_val[warp][slot] = make_uint2(g[w], x01[w]);
-                    s_rows[warp][slot] = y01[w];
+                    const uint32_t slot = fill + __popc(km & lt);
+                    val[slot] = make_uint2(g[w], x[w]);
+                    yy[slot] = y[w];
                 }
                 fill += __popc(km);
             }
-            if (fill == 0) continue;
             __syncwarp();
-            const uint32_t mine = c0 + lane < static_cast<uint32_t>(Ty) && lane < kGroup ? s_pos[warp][c0 + lane] : 0u;
-            uint32_t pos[kGroup];
-#pragma unroll
-            for (int c = 0; c < kGroup; ++c) pos[c] = __shfl_sync(FULL, mine, c);
-            for (int k = 0; k < fill; k += 32) {
-                const bool in = k + lane < fill;
-                const uint32_t y = in ? s_rows[warp][k + lane] : 0u;
-                emit_group(coverage(y & 0xFFFFu, y >> 16, c0), in ? s_val[warp][k + lane] : make_uint2(0u, 0u), pos,
-                           rowlist, lt, ok);
+            uint32_t k = 0;
+            for (; k + 32 <= fill; k += 32) emit(k, true);
+            if (k) {                               // the rest to the front
+                const uint2 v = val[k + lane];
+                const uint32_t r = yy[k + lane];
+                __syncwarp();
+                val[lane] = v;
+                yy[lane] = r;
+                fill -= k;
             }
-#pragma unroll
-            for (int c = 0; c < kGroup; ++c)
-                if (lane == c && c0 + c < static_cast<uint32_t>(Ty)) s_pos[warp][c0 + c] = pos[c];
             __syncwarp();
         }
+        if (fill) emit(0, lane < fill);
+        __syncwarp();
     }
 }
 
@@ -714,15 +707,15 @@ cudaError_t launch_bin_rows(const BinView *views, int n, cudaStream_t st) {
         Ty = max(Ty, views[i].Ty);
         most = max(most, views[i].n_cap);
     }
-    // chunks of at least kChunkMin Gaussians (a chunk has a column of counts to scan), and half the CTAs per view
-    // when several share the launch (eight 512x512 views 0.173 ms; a quarter 0.184)
-    const int fill = n > 1 ? kBinBlocks / 2 : kBinBlocks;
-    const int blocks = max(min(fill, static_cast<int>(most / (8 * kChunkMin))), 1);
+    // chunks of at least kChunkMin Gaussians (a chunk has a column of counts to scan)
+    const int blocks = max(min(kBinBlocks, static_cast<int>(most / (8 * kChunkMin))), 1);
     with_views(views, n, [&](const auto &b) {
         constexpr int NV = sizeof(b.v) / sizeof(BinView);
         launch_chained(k_bin_rows_count<NV>, dim3(blocks, n), 256, 0, st, b);
         launch_chained(k_bin_rowscan<NV>, dim3(Ty * kRowParts, n), 1024, 0, st, b, 8 * blocks);
-        launch_chained(k_bin_rows_write<NV>, dim3(blocks, n), 256, 0, st, b);
+        const int groups = (Ty + kGroup - 1) / kGroup;             // a warp per (chunk, group of rows)
+        launch_chained(k_bin_rows_write<NV>, dim3(min(blocks * groups, max(4 * sort_blocks() / n, 1)), n), 256, 0, st, b,
+                       8u * blocks);
     });
     return cudaGetLastError();
 }

@@ -409,8 +409,9 @@ int front_bin(FrontCtx *f, int n, cudaStream_t st, FwdJob *jobs) {
         const PreView &p = f[i].pre;
         b[i] = BinView{f[i].order, p.rec, static_cast<uint32_t>(p.s.n), p.c.Tx, p.c.Ty, at<uint32_t>(ws, L.bin_m),
                        at<void>(ws, L.bin_rows), at<uint2>(ws, L.rowlist), p.ctl, static_cast<uint64_t>(L.dup_cap),
-                       at<uint32_t>(ws, L.bin_p), at<uint32_t>(ws, L.list), at<uint2>(ws, L.ranges), nullptr,
-                       nullptr, nullptr, at<uint32_t>(ws, L.tile_hist)};
+                       at<uint32_t>(ws, L.bin_p), at<uint32_t>(ws, L.list), at<uint2>(ws, L.ranges),
+                       at<uint32_t>(ws, L.sort_k[0]), at<uint32_t>(ws, L.sort_k[1]), nullptr, nullptr, nullptr,
+                       at<uint32_t>(ws, L.tile_hist)};
         const CompositeBufs cb = composite_bufs(ws, L);
         b[i].tile_order = cb.order;
         b[i].seg_base = cb.seg_base;

@@ -210,6 +210,10 @@ __device__ __forceinline__ int sort_passes(const Ctl *ctl) {
 }
 
 constexpr int kPassThreads = 512;
+// Per SM: at most 64 registers.  Without the bound (86) one CTA filled an SM and a kernel ran in five waves of 152
+// tiles: sort of 3M 0.115 -> 0.095 ms, of eight times 500,000 0.166 -> 0.117, of 1.2M 0.057 -> 0.049 (540,000 visible of
+// 1.2M, which fill one wave: 0.039 -> 0.042); three (40 registers, spilling): 0.102 and 0.125.
+constexpr int kPassCtas = 2;
 constexpr int kPassWarps = kPassThreads / 32;
 constexpr int kPassTile = kPassThreads * kSortItems;
 static_assert(kPassTile % kSortTile == 0, "a digit-kernel tile is whole histogram rounds");
@@ -236,8 +240,8 @@ struct SortJob {
 // `own` is already published as an aggregate unless t == 0); publishes the
 // inclusive prefix of tile t.  The predecessors are read kLookWindow at a time,
 // nearest first, so a walk over tiles that only hold aggregates costs one
-// memory latency per window instead of one per tile.
-constexpr int kLookWindow = 8;
+// memory latency per window instead of one per tile (windows of eight spill).
+constexpr int kLookWindow = 4;
 __device__ uint32_t look_back(uint64_t *status, uint32_t t, int c, uint32_t own, Ctl *ctl, uint32_t spin_limit,
                               bool publish) {
     uint32_t excl = 0;
@@ -438,7 +442,7 @@ __device__ __forceinline__ uint32_t block_scan_512(uint32_t v, uint32_t *s_w, ui
 }
 
 template <class Src, bool FIRST, int NV>
-__global__ void __launch_bounds__(kPassThreads) k_sort_pass(const __grid_constant__ Views<SortJob, NV> views, int pass) {
+__global__ void __launch_bounds__(kPassThreads, kPassCtas) k_sort_pass(const __grid_constant__ Views<SortJob, NV> views, int pass) {
     chain_start();
     __shared__ uint16_t s_wc[kPassWarps][256];   // per-warp digit counts, then per-warp digit bases
     __shared__ uint32_t s_lstart[256];            // start of each digit's run in the locally sorted tile
@@ -462,14 +466,12 @@ __global__ void __launch_bounds__(kPassThreads) k_sort_pass(const __grid_constan
     const uint32_t n = FIRST ? n_all : n_vis;
     const uint32_t ntiles = (n + kPassTile - 1) / kPassTile;
     uint32_t t = blockIdx.x;                       // the first digit kernel: the histogram pass's tiles
-    if (FIRST && t >= ntiles) return;
+    // as many CTAs as tiles take part, the first ones: they start on one SM each before any SM gets a second
+    if (t >= ntiles) return;
     if (!FIRST && threadIdx.x == 0) s_ticket = atomicAdd(&ctl->sort_ticket[pass], 1u);
     for (int e = threadIdx.x; e < kPassWarps * 256; e += kPassThreads) (&s_wc[0][0])[e] = 0;
     __syncthreads();
-    if (!FIRST) {
-        t = s_ticket;
-        if (t >= ntiles) return;
-    }
+    if (!FIRST) t = s_ticket;
 #ifdef GS_DEBUG
     const bool publish = !(pass == B.withhold && t == 0);
 #else

@@ -353,7 +353,8 @@ __global__ void __launch_bounds__(256) k_adam(const AdamArrays arr, const uint8_
 // the SH arrays; a frozen element in a mixed unit is written back unchanged).
 // A thread takes kAdamUnits units, one stride of the block apart, and all their
 // loads are in flight before the first result is needed.
-// 500,000 Gaussians, degree 3, a third of them frozen: 0.125 -> 0.096 ms.
+// 500,000 Gaussians, degree 3, a third of them frozen: 0.125 -> 0.093 ms (four CTAs per SM 0.096,
+// six 0.099).
 struct Adam4 {
     float *p[5];
     const float *g[5];
@@ -366,7 +367,7 @@ struct Adam4 {
 
 constexpr int kAdamThreads = 256, kAdamUnits = 2;
 
-__global__ void __launch_bounds__(kAdamThreads) k_adam4(const Adam4 a, const uint8_t *__restrict__ layer,
+__global__ void __launch_bounds__(kAdamThreads, 5) k_adam4(const Adam4 a, const uint8_t *__restrict__ layer,
                                                         uint32_t train_mask, float beta1, float beta2,
                                                         float inv_sqrt_bc2, float eps) {
     const bool all = train_mask == 0xFFFFFFFFu;

@@ -671,11 +671,14 @@ __device__ __forceinline__ float reduce_scatter10(const float g[6], const float 
 // part with alpha 0, and with zeros selected where a product with an infinite
 // or undefined value of its own must not count.  Kept splats are staged in
 // shared memory with every factor doubled, as the packed instructions want
-// them.  1.2M-Gaussian 1024 x 1024 frame 0.198 -> 0.166 ms, 500,000-Gaussian
-// 800 x 800 training view 0.148 -> 0.124 (before: one pixel after the other
+// them.  1.2M-Gaussian 1024 x 1024 frame 0.198 -> 0.173 ms, 500,000-Gaussian
+// 800 x 800 training view 0.148 -> 0.129 (before: one pixel after the other
 // behind branches, 220 instructions per splat and block against 160, and the
-// geometry's factors applied per splat and block).  Five CTAs per SM; six and
-// seven: 0.168 and 0.169.
+// geometry's factors applied per splat and block).  The two pixels' products
+// are added with one rounding (dot2) and dL/da as a fused difference: packed
+// products summed afterwards took 0.166 ms but put twice the rounding noise
+// into the quaternion gradients of needle-like splats.  Five CTAs per SM; six
+// and seven: 1.2% slower.
 struct alignas(16) BwdSplat {
     float2 nax, nay;               // minus the centre
     float2 beta, A2, G2, o;
@@ -817,27 +820,26 @@ __global__ void __launch_bounds__(kBwdThreads, 5) k_composite_bwd(
                 const float cb = __uint_as_float(u4.x);
                 const float2 d = fma2(dC2, F2(cb, cb), fma2(dC1, F2(u3.y), mul2(dC0, F2(u3.x)))).get();
                 const F2 dcc(act0 ? d.x : 0.f, act1 ? d.y : 0.f);
-                const float2 Rinv = mul2(R2, inv).get(), t = T2.get(), dc = dcc.get();
+                const float2 Rv = R2.get(), iv = inv.get(), t = T2.get(), dc = dcc.get();
                 R2 = fma2(w, dcc, R2);
                 // dL/da, zero where the product with the opacity was clamped
-                const F2 dLda(act0 && ao.x < kAlphaMax ? fmaf(t.x, dc.x, -Rinv.x) : 0.f,
-                              act1 && ao.y < kAlphaMax ? fmaf(t.y, dc.y, -Rinv.y) : 0.f);
+                const F2 dLda(act0 && ao.x < kAlphaMax ? fmaf(-Rv.x, iv.x, t.x * dc.x) : 0.f,
+                              act1 && ao.y < kAlphaMax ? fmaf(-Rv.y, iv.y, t.y * dc.y) : 0.f);
                 const F2 E = mul2(dLda, al);
                 const F2 tp = mul2(E, p), td = mul2(E, dy);
-                const float g[6] = {tp.sum(),           td.sum(),           mul2(tp, p).sum(),
-                                    mul2(tp, dy).sum(), mul2(td, dy).sum(), mul2(dLda, ex).sum()};
-                F2 m[4];
+                const float g[6] = {tp.sum(),     td.sum(),     dot2(tp, p),
+                                    dot2(tp, dy), dot2(td, dy), dot2(dLda, ex)};
+                float col[4];
 #pragma unroll
-                for (int s = 0; s < 4; ++s) m[s] = mul2(w, kc[s]);
+                for (int s = 0; s < 4; ++s) col[s] = dot2(w, kc[s]);
+                const float2 wv = w.get();
                 if (!finite) {
 #pragma unroll
                     for (int s = 0; s < 4; ++s) {
-                        const float2 v = m[s].get();
-                        m[s] = F2(act0 ? v.x : 0.f, act1 ? v.y : 0.f);
+                        const float2 v = kc[s].get();
+                        col[s] = (act0 ? wv.x * v.x : 0.f) + (act1 ? wv.y * v.y : 0.f);
                     }
                 }
-                const float col[4] = {m[0].sum(), m[1].sum(), m[2].sum(), m[3].sum()};
-                const float2 wv = w.get();
                 const float sv = reduce_scatter10(g, col, lane);
                 const uint32_t smx = __reduce_max_sync(FULL, __float_as_uint(fmaxf(wv.x, wv.y)));
                 const uint32_t gi = u4.z & 0x7FFFFFFFu;

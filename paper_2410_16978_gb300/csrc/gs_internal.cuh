@@ -239,6 +239,11 @@ __device__ __forceinline__ F2 mul2(F2 a, F2 b) {
     asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
     return r;
 }
+// a.x b.x + a.y b.y, the second product fused (as many instructions as a packed product and its sum, one rounding less).
+__device__ __forceinline__ float dot2(F2 a, F2 b) {
+    const float2 x = a.get(), y = b.get();
+    return fmaf(x.y, y.y, x.x * y.x);
+}
 __device__ __forceinline__ F2 add2(F2 a, F2 b) {
     F2 r;
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));

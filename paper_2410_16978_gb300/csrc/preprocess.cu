@@ -88,19 +88,17 @@ __device__ __forceinline__ void store_geo(Geo *g, const float4 a, const float4 b
                  : "memory");
 }
 
-// The views of a launch are interleaved block by block (view blockIdx.x mod n),
-// so views of one scene read it from L2 after the first.
-template <int DEG, int NV>
+// Several views of one launch: with ONE they show the same scene and a thread
+// takes its Gaussian through all of them, so what does not depend on the view
+// (exponentials, rotation, covariance, opacity) is computed once; otherwise
+// the views are interleaved block by block (view blockIdx.x mod n).
+template <int DEG, int NV, bool ONE>
 __global__ void __launch_bounds__(128) k_preprocess(const __grid_constant__ Views<PreView, NV> B) {
     chain_start();
-    const PreView &V = B[blockIdx.x % B.n];
-    const SceneView &s = V.s;
-    const CamView &c = V.c;
-    const Planes &pl = V.pl;
-    const int i = (NV == 1 ? blockIdx.x : blockIdx.x / B.n) * blockDim.x + threadIdx.x;
+    const int view = ONE ? 0 : blockIdx.x % B.n;
+    const SceneView &s = B[view].s;
+    const int i = (NV == 1 || ONE ? blockIdx.x : blockIdx.x / B.n) * blockDim.x + threadIdx.x;
     if (i >= s.n) return;
-    uint32_t ntiles = 0;
-    uint32_t dkey = 0xFFFFFFFFu;
     const int lay = s.layer[i];
     const float mx = s.means[3 * i], my = s.means[3 * i + 1], mz = s.means[3 * i + 2];
     // the other per-Gaussian inputs but SH, loaded with these before the culling tests so that one memory
@@ -118,17 +116,30 @@ __global__ void __launch_bounds__(128) k_preprocess(const __grid_constant__ View
         qw = q[0]; qx = q[1]; qy = q[2]; qz = q[3];
     }
     const float ol = s.opacity_logit[i];
-    bool keep = (V.layer_mask >> lay) & 1u;
-    for (int k = 0; k < pl.n && keep; ++k) {
-        if (!((pl.bits[k] >> lay) & 1u)) continue;
-        const float4 p = pl.p[k];
-        const float dist = ((p.x * mx + p.y * my) + p.z * mz) + p.w;
-        if (dist < 0.0f) keep = false;
+    // not masked, not clipped and in front of the view's near plane
+    const auto kept = [&](const PreView &V) {
+        const Planes &pl = V.pl;
+        const float *R = V.c.R;
+        bool keep = (V.layer_mask >> lay) & 1u;
+        for (int k = 0; k < pl.n && keep; ++k) {
+            if (!((pl.bits[k] >> lay) & 1u)) continue;
+            const float4 p = pl.p[k];
+            const float dist = ((p.x * mx + p.y * my) + p.z * mz) + p.w;
+            if (dist < 0.0f) keep = false;
+        }
+        const float pz = ((R[6] * mx + R[7] * my) + R[8] * mz) + V.c.t[2];
+        return keep && pz > V.c.znear;
+    };
+    bool some;                                     // kept in the view, or for several: on in one of them
+    if constexpr (ONE) {
+        uint32_t layers = 0;
+        for (int v = 0; v < B.n; ++v) layers |= B[v].layer_mask;
+        some = (layers >> lay) & 1u;
+    } else {
+        some = kept(B[view]);
     }
-    const float *R = c.R;
-    const float pz = ((R[6] * mx + R[7] * my) + R[8] * mz) + c.t[2];
-    if (keep && !(pz > c.znear)) keep = false;
-    if (keep) {
+    float S00 = 0.f, S01 = 0.f, S02 = 0.f, S11 = 0.f, S12 = 0.f, S22 = 0.f, opac = 0.f;
+    if (some) {
         // the SH row (read only if the splat turns out visible) is brought into L2 while the projection runs
         if (s.dtype_sh != GS_DTYPE_SH_CODEBOOK) {
             constexpr int K = (DEG + 1) * (DEG + 1);
@@ -137,8 +148,6 @@ __global__ void __launch_bounds__(128) k_preprocess(const __grid_constant__ View
             asm volatile("prefetch.global.L2 [%0];" ::"l"(row));                  // first and last byte of the
             asm volatile("prefetch.global.L2 [%0];" ::"l"(row + bytes - 1));      // row: its one or two lines
         }
-        const float px = ((R[0] * mx + R[1] * my) + R[2] * mz) + c.t[0];
-        const float py = ((R[3] * mx + R[4] * my) + R[5] * mz) + c.t[1];
         const float s0 = exp_cw(ls0);
         const float s1 = exp_cw(ls1);
         const float s2 = exp_cw(ls2);
@@ -151,130 +160,146 @@ __global__ void __launch_bounds__(128) k_preprocess(const __grid_constant__ View
         const float m00 = r00 * s0, m01 = r01 * s1, m02 = r02 * s2;
         const float m10 = r10 * s0, m11 = r11 * s1, m12 = r12 * s2;
         const float m20 = r20 * s0, m21 = r21 * s1, m22 = r22 * s2;
-        const float S00 = (m00 * m00 + m01 * m01) + m02 * m02;
-        const float S01 = (m00 * m10 + m01 * m11) + m02 * m12;
-        const float S02 = (m00 * m20 + m01 * m21) + m02 * m22;
-        const float S11 = (m10 * m10 + m11 * m11) + m12 * m12;
-        const float S12 = (m10 * m20 + m11 * m21) + m12 * m22;
-        const float S22 = (m20 * m20 + m21 * m21) + m22 * m22;
-
-        const float limx = kFrustumClamp * ((0.5f * static_cast<float>(c.W)) / c.fx);
-        const float limy = kFrustumClamp * ((0.5f * static_cast<float>(c.H)) / c.fy);
-        const float izx = px / pz, izy = py / pz;
-        const float cxz = fminf(limx, fmaxf(-limx, izx));
-        const float cyz = fminf(limy, fmaxf(-limy, izy));
-        const float j00 = c.fx / pz, j02 = -(c.fx * cxz) / pz;
-        const float j11 = c.fy / pz, j12 = -(c.fy * cyz) / pz;
-        const float t00 = j00 * R[0] + j02 * R[6], t01 = j00 * R[1] + j02 * R[7], t02 = j00 * R[2] + j02 * R[8];
-        const float t10 = j11 * R[3] + j12 * R[6], t11 = j11 * R[4] + j12 * R[7], t12 = j11 * R[5] + j12 * R[8];
-        const float u00 = (t00 * S00 + t01 * S01) + t02 * S02;
-        const float u01 = (t00 * S01 + t01 * S11) + t02 * S12;
-        const float u02 = (t00 * S02 + t01 * S12) + t02 * S22;
-        const float u10 = (t10 * S00 + t11 * S01) + t12 * S02;
-        const float u11 = (t10 * S01 + t11 * S11) + t12 * S12;
-        const float u12 = (t10 * S02 + t11 * S12) + t12 * S22;
-        const float c00 = ((u00 * t00 + u01 * t01) + u02 * t02) + kDilation;
-        const float c01 = (u00 * t10 + u01 * t11) + u02 * t12;
-        const float c11 = ((u10 * t10 + u11 * t11) + u12 * t12) + kDilation;
-        const float det = c00 * c11 - c01 * c01;
-        if (det > 0.0f) {
-            const float mid = 0.5f * (c00 + c11);
-            const float disc = fmaxf(kEigenFloor, mid * mid - det);
-            const float lam = mid + sqrtf(disc);
-            const float r = ceilf(kRadiusSigmas * sqrtf(lam));
-            const float uu = c.fx * izx + c.cx, vv = c.fy * izy + c.cy;
-            const float fTx = static_cast<float>(c.Tx), fTy = static_cast<float>(c.Ty);
-            const float fx0 = fminf(fTx, fmaxf(0.0f, truncf((uu - r) * 0.0625f)));
-            const float fy0 = fminf(fTy, fmaxf(0.0f, truncf((vv - r) * 0.0625f)));
-            const float fx1 = fminf(fTx, fmaxf(0.0f, truncf(((uu + r) + 15.0f) * 0.0625f)));
-            const float fy1 = fminf(fTy, fmaxf(0.0f, truncf(((vv + r) + 15.0f) * 0.0625f)));
-            const int x0 = static_cast<int>(fx0), y0 = static_cast<int>(fy0);
-            const int x1 = static_cast<int>(fx1), y1 = static_cast<int>(fy1);
-            ntiles = GS_CHECK(x0 <= x1 && y0 <= y1 && x1 <= c.Tx && y1 <= c.Ty, V.ctl, kSiteRect)
-                         ? static_cast<uint32_t>((x1 - x0) * (y1 - y0))
-                         : 0u;
-            if (ntiles > 0) {
-                // view-dependent colour
-                const float campos0 = -((R[0] * c.t[0] + R[3] * c.t[1]) + R[6] * c.t[2]);
-                const float campos1 = -((R[1] * c.t[0] + R[4] * c.t[1]) + R[7] * c.t[2]);
-                const float campos2 = -((R[2] * c.t[0] + R[5] * c.t[1]) + R[8] * c.t[2]);
-                const float dx = mx - campos0, dy = my - campos1, dz = mz - campos2;
-                const float dn = sqrtf((dx * dx + dy * dy) + dz * dz);
-                constexpr int K = (DEG + 1) * (DEG + 1);
-                float b[K];
-                sh_basis<DEG>(dx / dn, dy / dn, dz / dn, b);
-                const int64_t base = static_cast<int64_t>(i) * K * 3;
-                float shv[3 * K];
-                if (s.dtype_sh == GS_DTYPE_SH_CODEBOOK) {
-                    // DC per Gaussian; coefficients k >= 1 from the FP16 table row (16-byte loads from L2)
-                    const float *dcp = static_cast<const float *>(s.sh) + static_cast<int64_t>(i) * 3;
-                    shv[0] = dcp[0]; shv[1] = dcp[1]; shv[2] = dcp[2];
-                    constexpr int ROW = cb_row_halves(K);
-                    const uint4 *row = reinterpret_cast<const uint4 *>(static_cast<const __half *>(s.sh_table) +
-                                                                       static_cast<int64_t>(s.sh_index[i]) * ROW);
+        S00 = (m00 * m00 + m01 * m01) + m02 * m02;
+        S01 = (m00 * m10 + m01 * m11) + m02 * m12;
+        S02 = (m00 * m20 + m01 * m21) + m02 * m22;
+        S11 = (m10 * m10 + m11 * m11) + m12 * m12;
+        S12 = (m10 * m20 + m11 * m21) + m12 * m22;
+        S22 = (m20 * m20 + m21 * m21) + m22 * m22;
+        opac = 1.0f / (1.0f + exp_cw(-ol));
+    }
+    const auto project = [&](const PreView &V) {
+        const CamView &c = V.c;
+        uint32_t ntiles = 0;
+        uint32_t dkey = 0xFFFFFFFFu;
+        const float *R = c.R;
+        const float pz = ((R[6] * mx + R[7] * my) + R[8] * mz) + c.t[2];
+        if (ONE ? kept(V) : some) {
+            const float px = ((R[0] * mx + R[1] * my) + R[2] * mz) + c.t[0];
+            const float py = ((R[3] * mx + R[4] * my) + R[5] * mz) + c.t[1];
+            const float limx = kFrustumClamp * ((0.5f * static_cast<float>(c.W)) / c.fx);
+            const float limy = kFrustumClamp * ((0.5f * static_cast<float>(c.H)) / c.fy);
+            const float izx = px / pz, izy = py / pz;
+            const float cxz = fminf(limx, fmaxf(-limx, izx));
+            const float cyz = fminf(limy, fmaxf(-limy, izy));
+            const float j00 = c.fx / pz, j02 = -(c.fx * cxz) / pz;
+            const float j11 = c.fy / pz, j12 = -(c.fy * cyz) / pz;
+            const float t00 = j00 * R[0] + j02 * R[6], t01 = j00 * R[1] + j02 * R[7], t02 = j00 * R[2] + j02 * R[8];
+            const float t10 = j11 * R[3] + j12 * R[6], t11 = j11 * R[4] + j12 * R[7], t12 = j11 * R[5] + j12 * R[8];
+            const float u00 = (t00 * S00 + t01 * S01) + t02 * S02;
+            const float u01 = (t00 * S01 + t01 * S11) + t02 * S12;
+            const float u02 = (t00 * S02 + t01 * S12) + t02 * S22;
+            const float u10 = (t10 * S00 + t11 * S01) + t12 * S02;
+            const float u11 = (t10 * S01 + t11 * S11) + t12 * S12;
+            const float u12 = (t10 * S02 + t11 * S12) + t12 * S22;
+            const float c00 = ((u00 * t00 + u01 * t01) + u02 * t02) + kDilation;
+            const float c01 = (u00 * t10 + u01 * t11) + u02 * t12;
+            const float c11 = ((u10 * t10 + u11 * t11) + u12 * t12) + kDilation;
+            const float det = c00 * c11 - c01 * c01;
+            if (det > 0.0f) {
+                const float mid = 0.5f * (c00 + c11);
+                const float disc = fmaxf(kEigenFloor, mid * mid - det);
+                const float lam = mid + sqrtf(disc);
+                const float r = ceilf(kRadiusSigmas * sqrtf(lam));
+                const float uu = c.fx * izx + c.cx, vv = c.fy * izy + c.cy;
+                const float fTx = static_cast<float>(c.Tx), fTy = static_cast<float>(c.Ty);
+                const float fx0 = fminf(fTx, fmaxf(0.0f, truncf((uu - r) * 0.0625f)));
+                const float fy0 = fminf(fTy, fmaxf(0.0f, truncf((vv - r) * 0.0625f)));
+                const float fx1 = fminf(fTx, fmaxf(0.0f, truncf(((uu + r) + 15.0f) * 0.0625f)));
+                const float fy1 = fminf(fTy, fmaxf(0.0f, truncf(((vv + r) + 15.0f) * 0.0625f)));
+                const int x0 = static_cast<int>(fx0), y0 = static_cast<int>(fy0);
+                const int x1 = static_cast<int>(fx1), y1 = static_cast<int>(fy1);
+                ntiles = GS_CHECK(x0 <= x1 && y0 <= y1 && x1 <= c.Tx && y1 <= c.Ty, V.ctl, kSiteRect)
+                             ? static_cast<uint32_t>((x1 - x0) * (y1 - y0))
+                             : 0u;
+                if (ntiles > 0) {
+                    // view-dependent colour
+                    const float campos0 = -((R[0] * c.t[0] + R[3] * c.t[1]) + R[6] * c.t[2]);
+                    const float campos1 = -((R[1] * c.t[0] + R[4] * c.t[1]) + R[7] * c.t[2]);
+                    const float campos2 = -((R[2] * c.t[0] + R[5] * c.t[1]) + R[8] * c.t[2]);
+                    const float dx = mx - campos0, dy = my - campos1, dz = mz - campos2;
+                    const float dn = sqrtf((dx * dx + dy * dy) + dz * dz);
+                    constexpr int K = (DEG + 1) * (DEG + 1);
+                    float b[K];
+                    sh_basis<DEG>(dx / dn, dy / dn, dz / dn, b);
+                    const int64_t base = static_cast<int64_t>(i) * K * 3;
+                    float shv[3 * K];
+                    if (s.dtype_sh == GS_DTYPE_SH_CODEBOOK) {
+                        // DC per Gaussian; coefficients k >= 1 from the FP16 table row (16-byte loads from L2)
+                        const float *dcp = static_cast<const float *>(s.sh) + static_cast<int64_t>(i) * 3;
+                        shv[0] = dcp[0]; shv[1] = dcp[1]; shv[2] = dcp[2];
+                        constexpr int ROW = cb_row_halves(K);
+                        const uint4 *row = reinterpret_cast<const uint4 *>(static_cast<const __half *>(s.sh_table) +
+                                                                           static_cast<int64_t>(s.sh_index[i]) * ROW);
 #pragma unroll
-                    for (int q = 0; q < ROW / 8; ++q) {
-                        const uint4 v = row[q];
-                        const __half2 *h = reinterpret_cast<const __half2 *>(&v);
+                        for (int q = 0; q < ROW / 8; ++q) {
+                            const uint4 v = row[q];
+                            const __half2 *h = reinterpret_cast<const __half2 *>(&v);
 #pragma unroll
-                        for (int r = 0; r < 4; ++r) {
-                            const float2 f = __half22float2(h[r]);
-                            const int d0 = 8 * q + 2 * r;
-                            if (d0 < 3 * (K - 1)) shv[3 + d0] = f.x;
-                            if (d0 + 1 < 3 * (K - 1)) shv[3 + d0 + 1] = f.y;
+                            for (int r = 0; r < 4; ++r) {
+                                const float2 f = __half22float2(h[r]);
+                                const int d0 = 8 * q + 2 * r;
+                                if (d0 < 3 * (K - 1)) shv[3 + d0] = f.x;
+                                if (d0 + 1 < 3 * (K - 1)) shv[3 + d0 + 1] = f.y;
+                            }
                         }
-                    }
-                } else if (s.dtype_sh == GS_DTYPE_F32 && (3 * K) % 4 == 0) {
-                    // 16-byte loads of this Gaussian's coefficients (its row starts 16-byte aligned)
-                    const float4 *src = reinterpret_cast<const float4 *>(static_cast<const float *>(s.sh) + base);
+                    } else if (s.dtype_sh == GS_DTYPE_F32 && (3 * K) % 4 == 0) {
+                        // 16-byte loads of this Gaussian's coefficients (its row starts 16-byte aligned)
+                        const float4 *src = reinterpret_cast<const float4 *>(static_cast<const float *>(s.sh) + base);
 #pragma unroll
-                    for (int k = 0; k < 3 * K / 4; ++k) {
-                        const float4 v = src[k];
-                        shv[4 * k] = v.x; shv[4 * k + 1] = v.y; shv[4 * k + 2] = v.z; shv[4 * k + 3] = v.w;
-                    }
-                } else if (s.dtype_sh != GS_DTYPE_F32 && (3 * K) % 4 == 0) {
-                    // 16-bit storage: rows of 96 bytes in 16-byte loads, of 24 in 8-byte ones (one coefficient at a
-                    // time: 1.5M Gaussians 0.076 ms against 0.062)
-                    const uint16_t *src = static_cast<const uint16_t *>(s.sh) + base;
-                    if constexpr ((3 * K) % 8 == 0) {
+                        for (int k = 0; k < 3 * K / 4; ++k) {
+                            const float4 v = src[k];
+                            shv[4 * k] = v.x; shv[4 * k + 1] = v.y; shv[4 * k + 2] = v.z; shv[4 * k + 3] = v.w;
+                        }
+                    } else if (s.dtype_sh != GS_DTYPE_F32 && (3 * K) % 4 == 0) {
+                        // 16-bit storage: rows of 96 bytes in 16-byte loads, of 24 in 8-byte ones (one coefficient at a
+                        // time: 1.5M Gaussians 0.076 ms against 0.062)
+                        const uint16_t *src = static_cast<const uint16_t *>(s.sh) + base;
+                        if constexpr ((3 * K) % 8 == 0) {
 #pragma unroll
-                        for (int k = 0; k < 3 * K / 8; ++k) {
-                            const uint4 v = reinterpret_cast<const uint4 *>(src)[k];
-                            widen4(make_uint2(v.x, v.y), s.dtype_sh, shv + 8 * k);
-                            widen4(make_uint2(v.z, v.w), s.dtype_sh, shv + 8 * k + 4);
+                            for (int k = 0; k < 3 * K / 8; ++k) {
+                                const uint4 v = reinterpret_cast<const uint4 *>(src)[k];
+                                widen4(make_uint2(v.x, v.y), s.dtype_sh, shv + 8 * k);
+                                widen4(make_uint2(v.z, v.w), s.dtype_sh, shv + 8 * k + 4);
+                            }
+                        } else {
+#pragma unroll
+                            for (int k = 0; k < 3 * K / 4; ++k)
+                                widen4(reinterpret_cast<const uint2 *>(src)[k], s.dtype_sh, shv + 4 * k);
                         }
                     } else {
 #pragma unroll
-                        for (int k = 0; k < 3 * K / 4; ++k)
-                            widen4(reinterpret_cast<const uint2 *>(src)[k], s.dtype_sh, shv + 4 * k);
+                        for (int k = 0; k < 3 * K; ++k) shv[k] = ld_half(s.sh, base + k, s.dtype_sh);
                     }
-                } else {
+                    float rgb[3];
 #pragma unroll
-                    for (int k = 0; k < 3 * K; ++k) shv[k] = ld_half(s.sh, base + k, s.dtype_sh);
+                    for (int ch = 0; ch < 3; ++ch) {
+                        float acc = b[0] * shv[ch];
+#pragma unroll
+                        for (int k = 1; k < K; ++k) acc = acc + b[k] * shv[3 * k + ch];
+                        rgb[ch] = fmaxf(acc + 0.5f, 0.0f);
+                    }
+                    const float NHL = -0x1.715476p-1f;   // -log2(e)/2
+                    Rec o;
+                    o.a = make_float4(uu, vv, (c11 / det) * NHL, -(c01 / c11));
+                    o.b = make_float4(NHL / c11, opac, rgb[0], rgb[1]);
+                    o.c = make_float4(rgb[2], pz, __uint_as_float(static_cast<uint32_t>(x0) | (static_cast<uint32_t>(y0) << 16)),
+                                      __uint_as_float(static_cast<uint32_t>(x1) | (static_cast<uint32_t>(y1) << 16)));
+                    V.rec[i] = o;
+                    store_geo(V.geo + i, o.a, o.b);
+                    dkey = __float_as_uint(pz);
                 }
-                float rgb[3];
-#pragma unroll
-                for (int ch = 0; ch < 3; ++ch) {
-                    float acc = b[0] * shv[ch];
-#pragma unroll
-                    for (int k = 1; k < K; ++k) acc = acc + b[k] * shv[3 * k + ch];
-                    rgb[ch] = fmaxf(acc + 0.5f, 0.0f);
-                }
-                const float NHL = -0x1.715476p-1f;   // -log2(e)/2
-                Rec o;
-                o.a = make_float4(uu, vv, (c11 / det) * NHL, -(c01 / c11));
-                const float opac = 1.0f / (1.0f + exp_cw(-ol));
-                o.b = make_float4(NHL / c11, opac, rgb[0], rgb[1]);
-                o.c = make_float4(rgb[2], pz, __uint_as_float(static_cast<uint32_t>(x0) | (static_cast<uint32_t>(y0) << 16)),
-                                  __uint_as_float(static_cast<uint32_t>(x1) | (static_cast<uint32_t>(y1) << 16)));
-                V.rec[i] = o;
-                store_geo(V.geo + i, o.a, o.b);
-                dkey = __float_as_uint(pz);
             }
         }
+        V.tiles[i] = ntiles;
+        V.depth[i] = dkey;
+    };
+    if constexpr (ONE) {
+#pragma unroll 1
+        for (int v = 0; v < B.n; ++v) project(B[v]);
+    } else {
+        project(B[view]);
     }
-    V.tiles[i] = ntiles;
-    V.depth[i] = dkey;
 }
 
 // Zeroes every view's control block and what is cleared with it (16-byte words).
@@ -291,13 +316,13 @@ __global__ void __launch_bounds__(256) k_clear(const __grid_constant__ Views<Pre
 
 namespace {
 
-template <int NV>
+template <int NV, bool ONE>
 void preprocess_views(int deg, const Views<PreView, NV> &b, unsigned blocks, cudaStream_t st) {
     switch (deg) {
-        case 0: launch_chained(k_preprocess<0, NV>, blocks, 128, 0, st, b); break;
-        case 1: launch_chained(k_preprocess<1, NV>, blocks, 128, 0, st, b); break;
-        case 2: launch_chained(k_preprocess<2, NV>, blocks, 128, 0, st, b); break;
-        default: launch_chained(k_preprocess<3, NV>, blocks, 128, 0, st, b); break;
+        case 0: launch_chained(k_preprocess<0, NV, ONE>, blocks, 128, 0, st, b); break;
+        case 1: launch_chained(k_preprocess<1, NV, ONE>, blocks, 128, 0, st, b); break;
+        case 2: launch_chained(k_preprocess<2, NV, ONE>, blocks, 128, 0, st, b); break;
+        default: launch_chained(k_preprocess<3, NV, ONE>, blocks, 128, 0, st, b); break;
     }
 }
 
@@ -316,6 +341,19 @@ cudaError_t launch_clear(const PreView *views, int n, cudaStream_t st) {
     return cudaGetLastError();
 }
 
+// Gaussians times views from which views of one scene are taken together; below, the blocks of one view leave SMs
+// idle.  Degree 3, two views of 131,072 Gaussians 22.6 against 20.6 us view by view, of 262,144 34.0 against 34.8;
+// eight views of 32,000 23.0 against 20.5, of 65,000 31.6 against 33.4, of 262,144 88.5 against 110.7, of 500,000
+// 155 against 199; the two eyes of the 3M-Gaussian stereo pair 120 against 131.
+constexpr int64_t kSharedMin = 1 << 19;
+
+bool same_scene(const SceneView &a, const SceneView &b) {
+    return a.means == b.means && a.log_scales == b.log_scales && a.quats == b.quats &&
+           a.opacity_logit == b.opacity_logit && a.sh == b.sh && a.layer == b.layer && a.sh_index == b.sh_index &&
+           a.sh_table == b.sh_table && a.sh_table_rows == b.sh_table_rows && a.n == b.n &&
+           a.sh_degree == b.sh_degree && a.dtype_sh == b.dtype_sh && a.dtype_sr == b.dtype_sr;
+}
+
 cudaError_t launch_preprocess(const PreView *views, int n, cudaStream_t st, int *launches) {
     *launches = 0;
     for (int deg = 0; deg <= 3; ++deg) {           // a launch per SH degree among the views
@@ -327,8 +365,13 @@ cudaError_t launch_preprocess(const PreView *views, int n, cudaStream_t st, int 
             most = views[i].s.n > most ? views[i].s.n : most;
         }
         if (m == 0) continue;
+        bool one = m > 1 && static_cast<int64_t>(most) * m >= kSharedMin;
+        for (int i = 1; i < m; ++i) one = one && same_scene(of[0].s, of[i].s);
+        const unsigned blocks = static_cast<unsigned>((most + 127) / 128);
         with_views(of, m, [&](const auto &b) {
-            preprocess_views(deg, b, static_cast<unsigned>((most + 127) / 128) * static_cast<unsigned>(m), st);
+            constexpr int NV = sizeof(b.v) / sizeof(PreView);
+            if (one) preprocess_views<NV, NV != 1>(deg, b, blocks, st);
+            else preprocess_views<NV, false>(deg, b, blocks * static_cast<unsigned>(m), st);
         });
         ++*launches;
     }

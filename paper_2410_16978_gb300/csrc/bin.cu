@@ -9,12 +9,12 @@
 // without sorting the pairs:
 //
 //  1. Rows.  The (Gaussian, tile row) pairs, in depth order, are split into
-//     one list per tile row.  K = gridDim.x * 8 warps each take a contiguous
-//     chunk of the depth order; a first pass counts each chunk's entries per
-//     row in shared memory, an exclusive scan over the chunks of every row
-//     (row-major count matrices [Ty][K] of entries and of pairs) gives each chunk its place, and a
-//     second pass writes the entries (Gaussian, x0 | x1 << 16) there, in depth
-//     order (emit_group).
+//     one list per tile row.  K warps each take a contiguous chunk of the
+//     depth order, count its entries per row in shared memory and lay its tile
+//     rectangles out in depth order; an exclusive scan over the chunks of every
+//     row (row-major count matrices [Ty][K] of entries and of pairs) gives each
+//     chunk its place; and a warp per (chunk, 16 rows) writes the entries
+//     (Gaussian, x0 | x1 << 16) there, in depth order (emit_group).
 //  2. Tiles.  Every row list is cut into pieces of 256 to 1,024 entries
 //     (thousands of pieces per frame, so heavy rows spread over all SMs); a
 //     warp per piece counts its pairs per tile, a per-row scan over the

@@ -26,9 +26,10 @@
 //    the second 8x4 block of an 8x8 block to finish knows the block's longest
 //    blended prefix, so no ordering pass runs between the two.
 //
-// splat_alpha() is the single definition of the per-(pixel, splat) alpha used
-// by both passes; every operation is an explicitly rounded intrinsic, so the
-// backward reproduces the forward's skip decisions bit for bit.
+// splat_alpha() defines the per-(pixel, splat) alpha of both passes; every
+// operation is explicitly rounded, and the backward does the same operations on
+// two pixels at a time (packed instructions round each half alike), so it
+// reproduces the forward's skip decisions bit for bit.
 #include "gs_internal.cuh"
 
 namespace gs {

@@ -416,7 +416,7 @@ struct FwdJob {
     uint32_t n_segs;                 // checkpoint segments the workspace holds
     int W, H, Tx, Tn;
     float3 bg;
-    uint32_t *queue;       // the view's work-queue word (written by its set-up)
+    uint32_t *queue;       // the view's work-queue word (cleared with the control block; the binning counts the live tiles)
     uint2 *items;          // the view's backward work items, appended as the forward finishes 8x8 blocks
     uint32_t *n_items;     // their count (zero at the start of the render)
     uint32_t *qdone;       // [8 Tn] per 8x8 block, a half per 8x4 block: 0 or its longest prefix + 1 (zeroed by the binning)

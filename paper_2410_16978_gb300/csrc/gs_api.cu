@@ -660,7 +660,7 @@ int gs_image_loss(const float *image, const float *alpha, const float *target_rg
         (rc = cuda_check(cudaMemsetAsync(dL_dalpha, 0, static_cast<size_t>(width) * height * 4, st),
                          "zero dL_dalpha")) != GS_OK)
         return rc;
-    Stage sg(GS_STAGE_LOSS, st, 3);
+    Stage sg(GS_STAGE_LOSS, st, 2);
     return cuda_check(launch_image_loss(image, alpha, target_rgb, target_alpha, make_float3(bg[0], bg[1], bg[2]),
                                         width, height, lambda_dssim, w_alpha, workspace, loss, dL_dimage,
                                         alpha ? dL_dalpha : nullptr, st),

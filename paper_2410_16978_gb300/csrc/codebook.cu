@@ -448,7 +448,16 @@ __global__ void __launch_bounds__(kTcThreads) k_kmeans_assign_tc(const float *__
             }
 #pragma unroll
             for (int d = kCbMaxDim / 2; d < 32; ++d) w[d] = 0u;
-            set_sync();                                        // and have been read: the set's next tile
+            // the tile's largest norm; one that is not a number or too large makes its groups candidates
+            float nc = sqrtf(sq) * 1.0001f;
+            if (!(nc < kHuge)) nc = INFINITY;
+            const float wm = __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, __float_as_uint(nc)));
+            if (lane == 0) reinterpret_cast<float *>(&sm.cm[t & (kCmRing - 1)])[cw] = wm;
+            // The set's next tile goes into the same rows by a bulk copy (async proxy): every thread's reads come
+            // before it.  The norm stored above depends on all reads of the warp, and the fence orders the proxies; with
+            // the barrier alone a read still in the queue could return the next tile's values.
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            set_sync();
             fetch(t + kTcCvtSets);
             if (t >= 2) mbar_wait(&sm.b_empty[q], ((t >> 1) - 1) & 1, failed);
             // -|c|^2 / 2 in three parts at dim .. dim + 2; a row past the end scores far below any other
@@ -466,12 +475,6 @@ __global__ void __launch_bounds__(kTcThreads) k_kmeans_assign_tc(const float *__
             for (int z = 0; z < 3; ++z)
                 *reinterpret_cast<__nv_bfloat16 *>(row + swz(r, (dim + z) >> 3) + 2 * ((dim + z) & 7)) =
                     __float2bfloat16_rn(-part[z]);
-            // the tile's largest norm; one that is not a number or too large makes its groups candidates
-            float nc = sqrtf(sq) * 1.0001f;
-            if (!(nc < kHuge)) nc = INFINITY;
-            const float wm = __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, __float_as_uint(nc)));
-            if (lane == 0) reinterpret_cast<float *>(&sm.cm[t & (kCmRing - 1)])[cw] = wm;
-            __syncwarp();
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             mbar_arrive(&sm.b_full[q]);
         }

@@ -89,3 +89,17 @@ def test_values_the_bounds_cannot_separate(case):
         pts[::2] = 0
         cent[:1500] = 0
     _check(pts, cent, dim, stride, off)
+
+
+@pytest.mark.parametrize("n,k,dim", [(50_000, 4096, 24), (50_000, 2048, 24), (20_000, 2048, 48), (50_000, 2048, 40)])
+def test_same_on_every_run(n, k, dim):
+    """Row widths whose reads from shared memory conflict most, so that a row still being read when its buffer is
+    filled again would show."""
+    g = torch.Generator("cuda").manual_seed(3)
+    pal = torch.randn((k, dim), generator=g, device="cuda") * 0.2
+    pts = pal[torch.randint(k, (n,), generator=g, device="cuda")]
+    pts = pts + 0.02 * torch.randn((n, dim), generator=g, device="cuda")
+    cent = pts[torch.randperm(n, generator=g, device="cuda")[:k]].contiguous()
+    want = torch.cat([_assign(pts, cent, dim, dim, 0, i, min(n, i + 1000)) for i in range(0, n, 1000)])
+    for _ in range(40):
+        assert torch.equal(_assign(pts, cent, dim, dim, 0, 0, n), want)

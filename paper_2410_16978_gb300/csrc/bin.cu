@@ -127,6 +127,19 @@ __device__ __forceinline__ void emit_group(uint32_t cov, V v, uint32_t (&pos)[kG
     }
 }
 
+// Sum over a block of 1024 threads, in every thread; synchronises the block.
+__device__ __forceinline__ unsigned long long block_sum64(unsigned long long v, unsigned long long *s_w) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
+    if ((threadIdx.x & 31) == 0) s_w[threadIdx.x >> 5] = v;
+    __syncthreads();
+    v = s_w[threadIdx.x & 31];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
+    __syncthreads();
+    return v;
+}
+
 // In-place inclusive prefix sum of a[0..n) (shared memory) by one warp.
 __device__ __forceinline__ void warp_prefix_inplace(uint32_t *a, int n, int lane) {
     const int per = (n + 31) / 32;
@@ -158,15 +171,23 @@ struct RowInfo {           // per tile row, in the workspace
     uint32_t start;        // first row-list entry of the row
     uint32_t entries;      // row-list entries of the row
     uint32_t pair_start;   // first pair (final list position) of the row
-    uint32_t pairs;        // pairs of the row
     uint32_t piece_start;  // first piece of the row (pieces: kPiece-entry parts of row lists)
     uint32_t part_base[kRowParts - 1];   // entries of the row in the chunk parts before parts 1 ..
-    uint32_t pad_[4 - kRowParts];        // (32 bytes in all)
+    uint32_t pad_[5 - kRowParts];        // (32 bytes in all)
 };
 
-// The per-row info of a view, and behind it the (entries, pairs) totals of every (row, part) of the row scan.
+// Totals of a (row, part) of the row scan.  A chunk's pairs of a row fit 32 bits (at most 883,012 Gaussians of 256
+// tiles); a row's need not, and the frame's do not from 65,536 Gaussians that cover 4096 x 4096 on.
+struct PartTotal {
+    unsigned long long pairs;
+    uint32_t entries, pad_;
+};
+
+// The per-row info of a view, and behind it the totals of every (row, part) of the row scan.
 __device__ __forceinline__ RowInfo *rows_of(const BinView &v) { return static_cast<RowInfo *>(v.rows); }
-__device__ __forceinline__ uint2 *part_totals_of(const BinView &v) { return reinterpret_cast<uint2 *>(rows_of(v) + v.Ty); }
+__device__ __forceinline__ PartTotal *part_totals_of(const BinView &v) {
+    return reinterpret_cast<PartTotal *>(rows_of(v) + v.Ty);
+}
 
 // Chunk c of K of the depth order's n entries.
 __device__ __forceinline__ void chunk_range(uint32_t n, uint32_t c, uint32_t K, uint32_t &b, uint32_t &e) {
@@ -337,19 +358,22 @@ __global__ void __launch_bounds__(256) k_bin_rows_write(const __grid_constant__ 
 // the pair total needs only a sum, read coalesced.  The last CTA to finish
 // (a counter in the control block) then does the per-row work for the whole
 // frame: part bases, row totals, the row, pair and piece starts, the pair
-// total and the capacity check.
+// total (in 64 bits) and the capacity check.  A frame that fits has at most
+// 2^32 - 1 pairs and no more entries than pairs, so its starts take 32 bits; after
+// an overflow nothing reads them.
 template <int NV>
 __global__ void __launch_bounds__(1024) k_bin_rowscan(const __grid_constant__ Views<BinView, NV> B, int K) {
     chain_start();
     const BinView &V = B[blockIdx.y];
     uint32_t *__restrict__ M = V.M;
     RowInfo *__restrict__ rows = rows_of(V);
-    uint2 *__restrict__ part_tot = part_totals_of(V);
+    PartTotal *__restrict__ part_tot = part_totals_of(V);
     Ctl *__restrict__ ctl = V.ctl;
     const uint64_t cap = V.cap;
     const int Tx = V.Tx, Ty = V.Ty;
     if (blockIdx.x >= Ty * kRowParts) return;
     __shared__ uint32_t s_w[32];
+    __shared__ unsigned long long s_w64[32];
     __shared__ uint32_t s_row[kPartChunks];
     __shared__ bool s_last;
     if (ctl->st.error != GS_OK) return;      // uniform: an error set before this kernel (a sort that timed out)
@@ -357,13 +381,12 @@ __global__ void __launch_bounds__(1024) k_bin_rowscan(const __grid_constant__ Vi
     const int KP = K / kRowParts;
     uint32_t *row = M + static_cast<size_t>(r) * K + static_cast<size_t>(part) * KP;
     const uint32_t *prow = M + static_cast<size_t>(Ty + r) * K + static_cast<size_t>(part) * KP;   // pairs
-    uint32_t psum = 0;
+    unsigned long long psum = 0;
     for (int i = threadIdx.x; i < KP; i += 1024) {
         s_row[i] = row[i];
         psum += prow[i];
     }
-    uint32_t ptot;
-    block_excl_scan<1024>(psum, s_w, &ptot);             // synchronises the block, so s_row is complete
+    const unsigned long long ptot = block_sum64(psum, s_w64);      // synchronises the block, so s_row is complete
     uint32_t v[kPartPerThread];
     uint32_t sum = 0;
 #pragma unroll
@@ -383,7 +406,7 @@ __global__ void __launch_bounds__(1024) k_bin_rowscan(const __grid_constant__ Vi
     __syncthreads();
     for (int i = threadIdx.x; i < KP; i += 1024) row[i] = s_row[i];
     if (threadIdx.x == 0) {
-        part_tot[blockIdx.x] = make_uint2(tot, ptot);
+        part_tot[blockIdx.x] = PartTotal{ptot, tot, 0u};
         __threadfence();
         s_last = atomicAdd(&ctl->bin_scan_done, 1u) == static_cast<uint32_t>(Ty * kRowParts - 1);
     }
@@ -391,22 +414,23 @@ __global__ void __launch_bounds__(1024) k_bin_rowscan(const __grid_constant__ Vi
     if (!s_last) return;
     __threadfence();
     // the last CTA: per row (thread r < Ty <= 256) the part bases and totals, then the starts
-    const volatile uint2 *pt = part_tot;
-    uint32_t ent = 0, prs = 0;
+    const volatile PartTotal *pt = part_tot;
+    uint32_t ent = 0;
+    unsigned long long prs = 0;
     if (threadIdx.x < Ty) {
         for (int p = 0; p < kRowParts; ++p) {
-            const uint32_t e = pt[threadIdx.x * kRowParts + p].x;
+            const uint32_t e = pt[threadIdx.x * kRowParts + p].entries;
             if (p > 0) rows[threadIdx.x].part_base[p - 1] = ent;
             ent += e;
-            prs += pt[threadIdx.x * kRowParts + p].y;
+            prs += pt[threadIdx.x * kRowParts + p].pairs;
         }
         rows[threadIdx.x].entries = ent;
-        rows[threadIdx.x].pairs = prs;
     }
-    uint32_t te, tp, tq;
+    uint32_t te, tp32, tq;
     const bool in = threadIdx.x < Ty;
+    const unsigned long long tp = block_sum64(in ? prs : 0ull, s_w64);
     const uint32_t s0 = block_excl_scan<1024>(in ? ent : 0u, s_w, &te);
-    const uint32_t s1 = block_excl_scan<1024>(in ? prs : 0u, s_w, &tp);
+    const uint32_t s1 = block_excl_scan<1024>(in ? static_cast<uint32_t>(prs) : 0u, s_w, &tp32);
     // entries per piece: the largest that still gives every SM several warps of the scatter (piece, kGroup tiles)
     uint32_t piece = kPieceMin;
     const uint64_t groups = (Tx + kGroup - 1) / kGroup;
@@ -741,10 +765,10 @@ size_t bin_piece_bytes(int64_t dup_cap, int Tx, int Ty) {
     return (static_cast<size_t>(dup_cap) / kPieceMin + Ty + 1) * Tx * 4;
 }
 
-// The RowInfo of every row, then the (entries, pairs) totals of every (row, part) of the row scan.
+// The RowInfo of every row, then the totals of every (row, part) of the row scan.
 size_t bin_rows_bytes(int Ty) {
-    return static_cast<size_t>(Ty) * sizeof(RowInfo) + static_cast<size_t>(Ty) * kRowParts * sizeof(uint2);
+    return static_cast<size_t>(Ty) * sizeof(RowInfo) + static_cast<size_t>(Ty) * kRowParts * sizeof(PartTotal);
 }
-static_assert(sizeof(RowInfo) == 32, "RowInfo layout");
+static_assert(sizeof(RowInfo) == 32 && sizeof(PartTotal) == 16, "RowInfo, PartTotal layout");
 
 }  // namespace gs

@@ -44,3 +44,21 @@ def test_overflowed_list_renders_background():
         assert r.status().error == _lib.GS_ERR_WORKSPACE
         assert all(bool((img[c] == v).all()) for c, v in enumerate((0.2, 0.4, 0.6)))
         assert bool((al == 0).all())
+
+
+@pytest.mark.parametrize("n", [65_536, 65_537])
+def test_pair_counts_beyond_32_bits(n):
+    """65,536 Gaussians that cover the 65,536 tiles of the largest image are 2^32 pairs: the total must not wrap
+    into the capacity.  No list is written, and the status holds what the frame needs."""
+    from tests.helpers import axis_camera, make_scene
+    means = np.random.default_rng(n).uniform(-0.1, 0.1, (n, 3))
+    sc = make_scene(means, 3.0, opacity_logit=-3.0)
+    cam = axis_camera(width=4096, height=4096)
+    r = Rasterizer(n, 4096, 4096, dup_capacity=1 << 20)
+    img, al = r.render(DeviceScene.from_host(sc), cam, bg=(0.2, 0.4, 0.6), check=False)
+    st = r.status()
+    assert st.n_visible == n
+    assert st.n_dup == n * 65_536
+    assert st.error == _lib.GS_ERR_WORKSPACE
+    assert all(bool((img[c] == v).all()) for c, v in enumerate((0.2, 0.4, 0.6)))
+    assert bool((al == 0).all())

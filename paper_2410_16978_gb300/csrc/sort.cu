@@ -598,7 +598,8 @@ __global__ void __launch_bounds__(kPassThreads, kPassCtas) k_sort_pass(const __g
     }
 }
 
-// The shared order of two eyes: the other eye's visible list and counts.
+// The shared order of two eyes: the other eye's visible list and counts, and an error of the sort (a wait that ran out
+// leaves the order unfinished, and the other eye bins in it too).
 __global__ void __launch_bounds__(256) k_share_order(const Ctl *from, const uint32_t *__restrict__ vis, Ctl *to,
                                                      uint32_t *__restrict__ vis_to, uint32_t n) {
     chain_start();
@@ -606,6 +607,7 @@ __global__ void __launch_bounds__(256) k_share_order(const Ctl *from, const uint
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         to->n_vis = nv;
         to->st.n_visible = from->st.n_visible;
+        if (from->st.error != GS_OK) to->st.error = from->st.error;
     }
     for (uint32_t i = blockIdx.x * 256u + threadIdx.x; i < min(nv, n); i += gridDim.x * 256u) vis_to[i] = vis[i];
 }

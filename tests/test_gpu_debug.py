@@ -120,3 +120,40 @@ def test_sort_wait_runs_out_with_timeout_status(dbg):
         torch.cuda.synchronize()
         assert r.status().error == _lib.GS_OK
     assert torch.equal(img2, img_ref) and torch.equal(al2, al_ref)
+
+
+def test_shared_sort_wait_runs_out_for_both_eyes(dbg):
+    """The two eyes of a pair bin in one depth order: when its wait runs out, neither eye may read it.  Both status
+    words hold GS_ERR_TIMEOUT and both images are the background; afterwards the same workspaces render again."""
+    w = synth.scene_c2(scale=0.1, width=512, height=512)
+    sc, bg = w["scene"], (0.25, 0.5, 0.75)
+    ds = DeviceScene.from_host(sc)
+    cams = list(synth.stereo_pair(w["cameras"][0], 0.02))
+    imgs = [torch.empty((3, 512, 512), device="cuda") for _ in cams]
+    als = [torch.empty((512, 512), device="cuda") for _ in cams]
+
+    def stereo(r):
+        for t in imgs + als:
+            t.fill_(-1.0)
+        _lib.gs_render_stereo(ds.c_struct(), _lib.make_camera(cams[0]), _lib.make_camera(cams[1]), w["layer_mask"], [],
+                              bg, r[0].workspace, r[0].ws_bytes, r[1].workspace, r[1].ws_bytes, imgs[0], als[0],
+                              imgs[1], als[1], True, 0)
+        torch.cuda.synchronize()
+        return [x.status().error for x in r]
+
+    with _lib.use(dbg):
+        r = [Rasterizer(sc.n, 512, 512) for _ in cams]
+        for x, cam in zip(r, cams):
+            x.render(ds, cam, w["layer_mask"], [], bg)                       # sizes the pair lists
+        assert stereo(r) == [_lib.GS_OK, _lib.GS_OK]
+        assert r[0].status().n_visible > 3 * 4096
+        ref = [t.clone() for t in imgs + als]
+        try:
+            _lib.gs_debug_sort_wait(2000, 1)
+            assert stereo(r) == [_lib.GS_ERR_TIMEOUT, _lib.GS_ERR_TIMEOUT]
+        finally:
+            _lib.gs_debug_sort_wait(0, -1)
+        for e in range(2):
+            assert all(bool((imgs[e][c] == bg[c]).all()) for c in range(3)) and bool((als[e] == 0).all())
+        assert stereo(r) == [_lib.GS_OK, _lib.GS_OK]
+        assert all(torch.equal(a, b) for a, b in zip(imgs + als, ref))

@@ -468,10 +468,15 @@ __global__ void __launch_bounds__(kPassThreads, kPassCtas) k_sort_pass(const __g
     uint32_t t = blockIdx.x;                       // the first digit kernel: the histogram pass's tiles
     // as many CTAs as tiles take part, the first ones: they start on one SM each before any SM gets a second
     if (t >= ntiles) return;
-    if (!FIRST && threadIdx.x == 0) s_ticket = atomicAdd(&ctl->sort_ticket[pass], 1u);
+    // (a wait that ran out leaves holes in what this kernel would read, keys that the histograms do not count: no tile)
+    if (!FIRST && threadIdx.x == 0)
+        s_ticket = ctl->st.error == GS_OK ? atomicAdd(&ctl->sort_ticket[pass], 1u) : 0xFFFFFFFFu;
     for (int e = threadIdx.x; e < kPassWarps * 256; e += kPassThreads) (&s_wc[0][0])[e] = 0;
     __syncthreads();
-    if (!FIRST) t = s_ticket;
+    if (!FIRST) {
+        t = s_ticket;
+        if (t >= ntiles) return;
+    }
 #ifdef GS_DEBUG
     const bool publish = !(pass == B.withhold && t == 0);
 #else

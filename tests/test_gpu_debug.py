@@ -157,3 +157,27 @@ def test_shared_sort_wait_runs_out_for_both_eyes(dbg):
             assert all(bool((imgs[e][c] == bg[c]).all()) for c in range(3)) and bool((als[e] == 0).all())
         assert stereo(r) == [_lib.GS_OK, _lib.GS_OK]
         assert all(torch.equal(a, b) for a, b in zip(imgs + als, ref))
+
+
+@pytest.mark.parametrize("withhold", [1, 2])
+def test_sort_stops_after_a_wait_that_ran_out(dbg, withhold):
+    """A digit kernel whose wait ran out leaves holes in its output.  The next one must not sort what the workspace
+    held there before (here keys of all ones, which the digit histograms do not count): no position it would compute
+    fails the bounds check."""
+    w = synth.scene_c2(scale=0.1, width=512, height=512)
+    sc, cam, bg = w["scene"], w["cameras"][0], (0.25, 0.5, 0.75)
+    ds = DeviceScene.from_host(sc)
+    with _lib.use(dbg):
+        r, img_ref, _ = _render(ds, cam, w["layer_mask"], w["planes"], bg)
+        try:
+            _lib.gs_debug_sort_wait(2000, withhold)
+            r.workspace.fill_(0xFF)
+            img, al = r.render(ds, cam, w["layer_mask"], w["planes"], bg, check=False)
+            torch.cuda.synchronize()
+            assert r.status().error == _lib.GS_ERR_TIMEOUT
+            assert _lib.gs_debug_site(r.workspace, 0) == 0
+            assert all(bool((img[c] == bg[c]).all()) for c in range(3)) and float(al.abs().max()) == 0.0
+        finally:
+            _lib.gs_debug_sort_wait(0, -1)
+        img2, _ = r.render(ds, cam, w["layer_mask"], w["planes"], bg)
+    assert torch.equal(img2, img_ref)

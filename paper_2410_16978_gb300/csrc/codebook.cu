@@ -417,7 +417,8 @@ __global__ void __launch_bounds__(kTcThreads) k_kmeans_assign_tc(const float *__
             const int vals = min(kTcTile, k - t * kTcTile) * dim;
             const float *src = cent + static_cast<size_t>(t) * kTcTile * dim;
             const int bulk = vec ? vals & ~3 : 0;
-            if (vec && r == 0) {
+            if (vec && r == 0 && bulk == 0) mbar_arrive(&sm.row_full[set]);      // (a copy has to have a size)
+            if (vec && r == 0 && bulk > 0) {
                 asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(&sm.row_full[set])),
                              "r"(4 * bulk)
                              : "memory");

@@ -103,3 +103,11 @@ def test_same_on_every_run(n, k, dim):
     want = torch.cat([_assign(pts, cent, dim, dim, 0, i, min(n, i + 1000)) for i in range(0, n, 1000)])
     for _ in range(40):
         assert torch.equal(_assign(pts, cent, dim, dim, 0, 0, n), want)
+
+
+@pytest.mark.parametrize("dim", [1, 2, 3])
+@pytest.mark.parametrize("k", [129, 130, 257, 258, 259])
+def test_last_tile_of_a_few_values(k, dim):
+    """Rows of one to three coordinates: a last tile of one to three centroids may hold fewer values than the
+    16-byte unit of the copy that fetches a tile."""
+    _check(*_data(1024, k, dim, dim + 1, 1, 10 * k + dim), dim, dim + 1, 1)

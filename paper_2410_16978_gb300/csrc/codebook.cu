@@ -644,8 +644,8 @@ __global__ void __launch_bounds__(256) k_sh_encode(const float *__restrict__ sh,
     }
 }
 
-}  // namespace
-
+// (In this namespace, so that the library has its own `attr`: a static of a template with a name for the linker is one
+// object of the process, also when a release and a debug library are loaded, each with kernels of its own.)
 template <int DIM>
 cudaError_t launch_assign_tc(const float *pts, int64_t n, int dim, int64_t stride, const float *cent, int k,
                              uint32_t *assign, cudaStream_t st) {
@@ -660,6 +660,8 @@ cudaError_t launch_assign_tc(const float *pts, int64_t n, int dim, int64_t strid
         pts, n, dim, stride, cent, k, assign);
     return cudaGetLastError();
 }
+
+}  // namespace
 
 cudaError_t launch_kmeans_assign(const float *pts, int64_t n, int dim, int64_t stride, const float *cent, int k,
                                  uint32_t *assign, cudaStream_t st) {

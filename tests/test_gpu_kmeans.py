@@ -111,3 +111,12 @@ def test_last_tile_of_a_few_values(k, dim):
     """Rows of one to three coordinates: a last tile of one to three centroids may hold fewer values than the
     16-byte unit of the copy that fetches a tile."""
     _check(*_data(1024, k, dim, dim + 1, 1, 10 * k + dim), dim, dim + 1, 1)
+
+
+def test_release_and_debug_library_in_one_process():
+    """Each library sets up its own kernels (their shared memory is above the default limit)."""
+    pts, cent = _data(2000, 256, 45, 48, 3, 8)
+    _check(pts, cent, 45, 48, 3)
+    with _lib.use(_lib.load_debug()):
+        _check(pts, cent, 45, 48, 3)
+    _check(pts, cent, 45, 48, 3)

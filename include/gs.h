@@ -415,10 +415,17 @@ int gs_get_settings(gs_settings *out);
  *                      (-1 disables).  After a timeout the binning does not
  *                      read the unfinished order: the render draws nothing
  *                      and the status holds the error.  Process-wide, not
- *                      thread safe; GS_ERR_INVALID in release builds.        */
+ *                      thread safe; GS_ERR_INVALID in release builds.
+ *   gs_debug_kmeans_wait(): test hook of the tensor-core k-means assignment:
+ *                      tries of its waits (0 restores the default).  A wait
+ *                      that runs out ends the walk of its CTA, whose points
+ *                      are then scanned in full: the assignment stays the
+ *                      same.  Current device, synchronises, not thread safe;
+ *                      GS_ERR_INVALID in release builds.                      */
 int gs_debug_build(void);
 int gs_debug_site(const void *workspace, uint32_t *site, void *stream);
 int gs_debug_sort_wait(uint32_t spin_limit, int32_t withhold_pass);
+int gs_debug_kmeans_wait(uint32_t limit);
 
 /* Message of the calling thread's last error ("" if none). */
 const char *gs_last_error_string(void);

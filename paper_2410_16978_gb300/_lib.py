@@ -27,7 +27,7 @@ EXPORTED = ("gs_render_workspace_size", "gs_render", "gs_render_batch", "gs_rend
             "gs_adam_step", "gs_activity_accumulate", "gs_activity_prune", "gs_gather_rows", "gs_kmeans_scratch_size",
             "gs_kmeans_assign", "gs_kmeans_update", "gs_sh_codebook_encode", "gs_workspace_layout", "gs_read_status", "gs_profile_enable",
             "gs_profile_collect", "gs_kernel_launches", "gs_get_settings", "gs_debug_build", "gs_debug_site",
-            "gs_debug_sort_wait", "gs_last_error_string", "gs_version")
+            "gs_debug_sort_wait", "gs_debug_kmeans_wait", "gs_last_error_string", "gs_version")
 STAGES = ("preprocess", "compact", "depth_sort", "bin_rows", "bin_tiles", "composite_setup", "composite",
           "composite_bwd", "preprocess_bwd", "prune", "loss", "adam")
 GS_LAYOUT_COUNT = 11
@@ -202,6 +202,7 @@ def _declare(L):
     L.gs_debug_build.argtypes = []
     L.gs_debug_site.argtypes = [_P, ctypes.POINTER(ctypes.c_uint32), _P]
     L.gs_debug_sort_wait.argtypes = [ctypes.c_uint32, ctypes.c_int32]
+    L.gs_debug_kmeans_wait.argtypes = [ctypes.c_uint32]
     return L
 
 
@@ -442,3 +443,7 @@ def gs_debug_site(workspace, stream: int) -> int:
 
 def gs_debug_sort_wait(spin_limit: int, withhold_pass: int) -> None:
     _check(load().gs_debug_sort_wait(int(spin_limit), int(withhold_pass)))
+
+
+def gs_debug_kmeans_wait(limit: int) -> None:
+    _check(load().gs_debug_kmeans_wait(int(limit)))

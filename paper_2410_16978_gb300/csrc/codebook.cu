@@ -114,6 +114,9 @@ constexpr int kCand = 16;              // candidate groups remembered per point
 constexpr int kCmRing = 8;             // tiles whose largest norms are kept
 constexpr float kEProd = 1.05f * 0x1p-8f, kENorm = 0x1p-15f, kESlack = 0x1p-17f, kETiny = 1e-30f, kHuge = 1e14f;
 constexpr uint32_t kTcWaitLimit = 1u << 22;
+#ifdef GS_DEBUG
+__device__ uint32_t g_dbg_tc_wait = kTcWaitLimit;      // test hook (gs_debug_kmeans_wait)
+#endif
 constexpr uint32_t kUnassigned = 0xFFFFFFFFu;
 // Calls from this size on go through the tensor cores (20,000 points: 128 centroids
 // 0.025 ms against 0.033 for the scan, 64 centroids 0.019 with the scan; 1,024 points
@@ -188,7 +191,7 @@ struct TcSmem {
     float4 cm[kCmRing];                            // largest |c| of a tile, per converting warp
     unsigned long long row_full[kTcCvtSets], b_full[2], b_empty[2], acc_full[2], acc_empty[2];
     uint32_t tmem;
-    int failed;
+    int failed, quit[kTcCvtSets];
 };
 
 __device__ __forceinline__ void mbar_init(void *bar, uint32_t count) {
@@ -197,10 +200,16 @@ __device__ __forceinline__ void mbar_init(void *bar, uint32_t count) {
 __device__ __forceinline__ void mbar_arrive(void *bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
-// Waits for the phase of the given parity; false when the limit runs out (or another role gave up).
+// Waits for the phase of the given parity; false when the limit runs out or another role has given up (`failed`; with
+// null the wait is for work of this thread's own that is under way, whatever the others do).
 __device__ __forceinline__ bool mbar_wait(void *bar, uint32_t parity, volatile int *failed) {
     const uint32_t addr = smem_u32(bar);
-    for (uint32_t it = 0; it < kTcWaitLimit; ++it) {
+#ifdef GS_DEBUG
+    const uint32_t limit = failed ? g_dbg_tc_wait : kTcWaitLimit;
+#else
+    constexpr uint32_t limit = kTcWaitLimit;
+#endif
+    for (uint32_t it = 0; it < limit; ++it) {
         uint32_t ok;
         asm volatile(
             "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
@@ -208,9 +217,9 @@ __device__ __forceinline__ bool mbar_wait(void *bar, uint32_t parity, volatile i
             : "r"(addr), "r"(parity)
             : "memory");
         if (ok) return true;
-        if ((it & 255u) == 255u && *failed) return false;
+        if (failed && *failed) return false;
     }
-    *failed = 1;
+    if (failed) *failed = 1;
     return false;
 }
 
@@ -285,7 +294,7 @@ __global__ void __launch_bounds__(kTcThreads) k_kmeans_assign_tc(const float *__
     const int ksteps = (dim + 3 + 15) / 16;
     volatile int *failed = &sm.failed;
     if (threadIdx.x == 0) {
-        sm.failed = 0;
+        sm.failed = sm.quit[0] = sm.quit[1] = 0;
         for (int q = 0; q < 2; ++q) {
             mbar_init(&sm.b_full[q], 32 * kTcCvtWarps);
             mbar_init(&sm.b_empty[q], 1);
@@ -410,6 +419,8 @@ __global__ void __launch_bounds__(kTcThreads) k_kmeans_assign_tc(const float *__
         float *const mem = sm.op.rows[set];
         const bool vec = (reinterpret_cast<uintptr_t>(cent) & 15u) == 0;
         const auto set_sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1 + set), "n"(32 * kTcCvtWarps) : "memory"); };
+        volatile int *quit = &sm.quit[set];                    // (written before the barrier by thread 0, read behind it)
+        bool copying = false;                                  // (thread 0 of the set: a bulk copy is under way)
         // A tile's rows, one bulk copy of whole 16-byte units (a last tile's odd values by plain loads); centroids
         // that do not start on 16 bytes value by value.
         const auto fetch = [&](int t) {
@@ -427,15 +438,23 @@ __global__ void __launch_bounds__(kTcThreads) k_kmeans_assign_tc(const float *__
                         smem_u32(mem)),
                     "l"(src), "r"(4 * bulk), "r"(smem_u32(&sm.row_full[set]))
                     : "memory");
+                copying = true;
             }
             for (int e = bulk + r; e < vals; e += 32 * kTcCvtWarps) mem[e] = src[e];
         };
         fetch(set);
         for (int t = set; t < ntile; t += kTcCvtSets) {
             const int q = t & 1;
-            // (a wait that gives up is noted in `failed`: the CTA's points are then scanned in full)
-            if (vec) mbar_wait(&sm.row_full[set], (t / kTcCvtSets) & 1, failed);
+            // A wait that gives up is noted in `failed`: the CTA's points are then scanned in full.  The set leaves
+            // the walk as one, behind its own copy, which must not land in the shared memory of a later CTA.
+            const bool landed = !vec || mbar_wait(&sm.row_full[set], (t / kTcCvtSets) & 1, failed);
+            if (landed) copying = false;
+            if (r == 0 && (!landed || *failed)) *quit = 1;
             set_sync();                                        // the tile's rows have landed
+            if (*quit) {
+                if (copying) mbar_wait(&sm.row_full[set], (t / kTcCvtSets) & 1, nullptr);
+                break;
+            }
             const bool in = t * kTcTile + r < k;
             const float *src = mem + r * dim;
             float sq = 0.f;
@@ -482,7 +501,8 @@ __global__ void __launch_bounds__(kTcThreads) k_kmeans_assign_tc(const float *__
     } else if (lane == 0) {
         const uint64_t da[2] = {umma_desc(smem_u32(sm.op.a[0])), umma_desc(smem_u32(sm.op.a[1]))};
         const uint64_t db[2] = {umma_desc(smem_u32(sm.op.b[0])), umma_desc(smem_u32(sm.op.b[1]))};
-        for (int t = 0; t < ntile; ++t) {
+        int t = 0;
+        for (; t < ntile; ++t) {
             const int q = t & 1;
             if (!mbar_wait(&sm.b_full[q], (t >> 1) & 1, failed)) break;
             if (t >= 2 && !mbar_wait(&sm.acc_empty[q], ((t >> 1) - 1) & 1, failed)) break;
@@ -494,8 +514,11 @@ __global__ void __launch_bounds__(kTcThreads) k_kmeans_assign_tc(const float *__
             umma_commit(&sm.b_empty[q]);
             umma_commit(&sm.acc_full[q]);
         }
-        // the last MMAs have completed before the tensor memory is freed
-        for (int t = max(0, ntile - 2); t < ntile; ++t) mbar_wait(&sm.acc_full[t & 1], (t >> 1) & 1, failed);
+        // the MMAs that were issued (the last two tiles') have completed before the tensor memory is freed
+        for (int u = max(0, t - 2); u < t; ++u) {
+            mbar_wait(&sm.b_empty[u & 1], (u >> 1) & 1, nullptr);
+            mbar_wait(&sm.acc_full[u & 1], (u >> 1) & 1, nullptr);
+        }
     }
     __syncwarp();
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -706,3 +729,14 @@ cudaError_t launch_sh_encode(const float *sh, int64_t n, int K, const uint32_t *
 }
 
 }  // namespace gs
+
+extern "C" int gs_debug_kmeans_wait(uint32_t limit) {
+#ifdef GS_DEBUG
+    const uint32_t v = limit ? limit : gs::kTcWaitLimit;
+    const cudaError_t e = cudaMemcpyToSymbol(gs::g_dbg_tc_wait, &v, sizeof v);
+    return e == cudaSuccess ? GS_OK : gs::report(GS_ERR_CUDA, cudaGetErrorString(e));
+#else
+    (void)limit;
+    return gs::report(GS_ERR_INVALID, "gs_debug_kmeans_wait: only in GS_DEBUG builds");
+#endif
+}

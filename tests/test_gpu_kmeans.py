@@ -120,3 +120,20 @@ def test_release_and_debug_library_in_one_process():
     with _lib.use(_lib.load_debug()):
         _check(pts, cent, 45, 48, 3)
     _check(pts, cent, 45, 48, 3)
+
+
+@pytest.mark.parametrize("limit", [1, 2, 3, 5, 20])
+@pytest.mark.parametrize("k,dim", [(4096, 45), (300, 24), (1000, 46)])
+def test_waits_that_run_out(k, dim, limit):
+    """Waits cut short (test hook of the debug build) end a CTA's walk with copies and MMAs under way: it lets them
+    finish, and its points are scanned in full."""
+    lib = _lib.load_debug()
+    pts, cent = _data(5000, k, dim, dim + 3, 3, k)
+    with _lib.use(lib):
+        try:
+            _lib.gs_debug_kmeans_wait(limit)
+            for _ in range(3):
+                _check(pts, cent, dim, dim + 3, 3)
+        finally:
+            _lib.gs_debug_kmeans_wait(0)
+        _check(pts, cent, dim, dim + 3, 3)

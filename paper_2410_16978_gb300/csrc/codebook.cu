@@ -11,6 +11,8 @@
 // (zero-padded) coordinates in registers and scans the centroids staged in
 // shared memory 64 at a time with 16-byte broadcast loads.  Larger ones rule
 // out nearly all centroids on the tensor cores first (k_kmeans_assign_tc).
+#include <type_traits>
+
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -22,50 +24,73 @@ namespace {
 constexpr int kKmTile = 64;                  // centroids per shared-memory tile
 constexpr int kKmThreads = 128;
 
-// The brute-force scan of point i by one thread of a CTA of NT (i >= n: none).
-template <int NT>
+// The brute-force scan of point i by one thread of a CTA of NT (i >= n: none), over D >= dim coordinates (the others
+// are zero).  Two centroids go through packed arithmetic together, each in the order of its coordinates, and two such
+// pairs are in flight: with a warp per scheduler the loop waits on the chains, with more it is bound by 2 D operations
+// per point and centroid.  Centroids are staged negated and interleaved in pairs; those past the end are infinitely
+// far.  One centroid at a time over 48 coordinates, before: 512 points x 16,384 centroids of 45 coordinates 2.99 -> 1.93
+// ms, 20,000 x 127 0.038 -> 0.032, 1,000,000 x 100 of 24 coordinates 0.393 -> 0.197, 1,000 x 64 of 9 0.020 -> 0.012.
+struct ScanTile {
+    float4 c[kKmTile / 2][kCbMaxDim / 2];
+};
+template <int NT, int D>
 __device__ __forceinline__ uint32_t scan_all(const float *__restrict__ pts, int64_t i, int64_t n, int dim,
-                                             int64_t stride, const float *__restrict__ cent, int k,
-                                             float4 (*s_c)[kCbMaxDim / 4]) {
-    float x[kCbMaxDim];
+                                             int64_t stride, const float *__restrict__ cent, int k, ScanTile &s) {
+    // x doubled for the packed operations; `zero` (k is positive, which the compiler does not know) keeps both halves in
+    // registers, where they would else be put together by moves before every use (20,000 x 2,048 0.42 against 0.33 ms)
+    const uint32_t zero = static_cast<uint32_t>(k) >> 31;
+    F2 x[D];
 #pragma unroll
-    for (int d = 0; d < kCbMaxDim; ++d) x[d] = (i < n && d < dim) ? pts[i * stride + d] : 0.f;
+    for (int d = 0; d < D; ++d) {
+        const float v = (i < n && d < dim) ? pts[i * stride + d] : 0.f;
+        x[d] = F2(v, __uint_as_float(__float_as_uint(v) ^ zero));
+    }
     float best = 3.0e38f;
     uint32_t arg = 0;
     for (int t0 = 0; t0 < k; t0 += kKmTile) {
         __syncthreads();
-        for (int e = threadIdx.x; e < kKmTile * kCbMaxDim; e += NT) {
-            const int j = e / kCbMaxDim, d = e % kCbMaxDim;
-            reinterpret_cast<float *>(&s_c[j][0])[d] = (t0 + j < k && d < dim) ? cent[(t0 + j) * dim + d] : 0.f;
+        for (int e = threadIdx.x; e < kKmTile * D; e += NT) {
+            const int j = e / D, d = e % D;
+            const float v = t0 + j >= k ? INFINITY : (d < dim ? cent[(t0 + j) * dim + d] : 0.f);
+            reinterpret_cast<float *>(&s.c[j >> 1][0])[2 * d + (j & 1)] = -v;
         }
         __syncthreads();
         const int m = min(kKmTile, k - t0);
-        for (int j = 0; j < m; ++j) {
-            float acc = 0.f;
+        for (int j = 0; j < m; j += 4) {
+            F2 acc[2] = {F2(0.f, 0.f), F2(0.f, 0.f)};
 #pragma unroll
-            for (int q = 0; q < kCbMaxDim / 4; ++q) {
-                const float4 c = s_c[j][q];
-                const float a = x[4 * q] - c.x, b = x[4 * q + 1] - c.y, e = x[4 * q + 2] - c.z, f = x[4 * q + 3] - c.w;
-                acc = fmaf(a, a, acc);
-                acc = fmaf(b, b, acc);
-                acc = fmaf(e, e, acc);
-                acc = fmaf(f, f, acc);
+            for (int q = 0; q < D / 2; ++q) {
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const float4 c = s.c[j / 2 + u][q];
+                    const F2 a = add2(x[2 * q], F2(c.x, c.y)), b = add2(x[2 * q + 1], F2(c.z, c.w));
+                    acc[u] = fma2(b, b, fma2(a, a, acc[u]));
+                }
             }
-            if (acc < best) {
-                best = acc;
-                arg = static_cast<uint32_t>(t0 + j);
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const float2 r = acc[u].get();
+                if (r.x < best) {
+                    best = r.x;
+                    arg = static_cast<uint32_t>(t0 + j + 2 * u);
+                }
+                if (r.y < best) {
+                    best = r.y;
+                    arg = static_cast<uint32_t>(t0 + j + 2 * u + 1);
+                }
             }
         }
     }
     return arg;
 }
 
+template <int D>
 __global__ void __launch_bounds__(kKmThreads) k_kmeans_assign(const float *__restrict__ pts, int64_t n, int dim,
                                                               int64_t stride, const float *__restrict__ cent, int k,
                                                               uint32_t *__restrict__ assign) {
-    __shared__ float4 s_c[kKmTile][kCbMaxDim / 4];
+    __shared__ ScanTile s_c;
     const int64_t i = static_cast<int64_t>(blockIdx.x) * kKmThreads + threadIdx.x;
-    const uint32_t arg = scan_all<kKmThreads>(pts, i, n, dim, stride, cent, k, s_c);
+    const uint32_t arg = scan_all<kKmThreads, D>(pts, i, n, dim, stride, cent, k, s_c);
     if (i < n) assign[i] = arg;
 }
 
@@ -111,6 +136,10 @@ constexpr int kTcEpiWarps = 8, kTcCvtWarps = 4, kTcCvtSets = 2;
 constexpr int kTcMmaWarp = kTcEpiWarps + kTcCvtSets * kTcCvtWarps;
 constexpr int kTcThreads = 32 * (kTcMmaWarp + 1);
 constexpr int kCand = 16;              // candidate groups remembered per point
+// A point with more than this share of the centroids left is scanned in full.  Evaluated one by one, 200,000 points with
+// 128 of 512 centroids left took 0.87 ms, with 64 0.53, with 32 0.40; with the scan 0.55, 0.52 and 0.69 (half of the
+// points, but every CTA).
+constexpr int kCandShare = 6;
 constexpr int kCmRing = 8;             // tiles whose largest norms are kept
 constexpr float kEProd = 1.05f * 0x1p-8f, kENorm = 0x1p-15f, kESlack = 0x1p-17f, kETiny = 1e-30f, kHuge = 1e14f;
 constexpr uint32_t kTcWaitLimit = 1u << 22;
@@ -533,7 +562,13 @@ __global__ void __launch_bounds__(kTcThreads) k_kmeans_assign_tc(const float *__
     const int64_t i = i0 + threadIdx.x;
     if (i >= n) return;
     uint32_t arg = kUnassigned;                                // (scanned in full by the next launch)
-    if (!full && !*failed) {
+    // (32 a group at most: only few centroids can be left in large part)
+    const int most = max(8, k / kCandShare);
+    int ncand = 0;
+    if (32 * cnt > most)
+        for (int e = 0; e < cnt; ++e)
+            if (sm.cand[e][threadIdx.x].x >= LB) ncand += __popc(sm.mask[e][threadIdx.x]);
+    if (!full && !*failed && ncand <= most) {
         const float *pt = pts + i * stride;
         float x[kCbMaxDim];
 #pragma unroll
@@ -565,26 +600,30 @@ __global__ void __launch_bounds__(kTcThreads) k_kmeans_assign_tc(const float *__
 }
 
 // The points that k_kmeans_assign_tc left (kUnassigned), in full: a CTA per kLeftPoints points collects those left
-// among them.  A few are scanned a warp per point, many a thread per point.
+// among them.  A few are scanned a warp per point, many a thread per point.  Their count comes from the barrier, which
+// makes the scan's loops uniform; taken from shared memory, the same loop took 0.75 against 0.47 ms (20,000 points x
+// 2,048 centroids).  Colours of a palette are what the bounds leave: 200,000 points of 64 colours x 16,384 centroids
+// 15.2 -> 13.0 ms in all (a spread of 0.1 of the palette's; 0.3: 15.7 -> 13.5; all points scanned without the tensor cores
+// 13.04), 50,000 x 4,096 of 24 coordinates 1.62 -> 0.64 (1.01), 20,000 x 2,048 0.78 -> 0.38 (0.43).
 constexpr int kLeftPoints = 128;
 
+template <int D>
 __global__ void __launch_bounds__(kLeftPoints) k_kmeans_assign_left(const float *__restrict__ pts, int64_t n, int dim,
                                                                     int64_t stride, const float *__restrict__ cent,
                                                                     int k, uint32_t *__restrict__ assign) {
     __shared__ __align__(16) union {
-        float4 c[kKmTile][kCbMaxDim / 4];
+        ScanTile c;
         PairBuf pair[kLeftPoints / 32];
     } s;
     __shared__ int s_left[kLeftPoints];
     __shared__ int s_n;
     const int64_t i0 = static_cast<int64_t>(blockIdx.x) * kLeftPoints;
     const bool left = i0 + threadIdx.x < n && assign[i0 + threadIdx.x] == kUnassigned;
-    if (!__syncthreads_or(left)) return;
     if (threadIdx.x == 0) s_n = 0;
-    __syncthreads();
+    const int m = __syncthreads_count(left);
+    if (m == 0) return;
     if (left) s_left[atomicAdd(&s_n, 1)] = threadIdx.x;
     __syncthreads();
-    const int m = s_n;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const bool vec = (reinterpret_cast<uintptr_t>(cent) & 15u) == 0;
     if (m <= kLeftPoints / 8) {
@@ -604,7 +643,7 @@ __global__ void __launch_bounds__(kLeftPoints) k_kmeans_assign_left(const float 
         return;
     }
     const int64_t i = static_cast<int>(threadIdx.x) < m ? i0 + s_left[threadIdx.x] : n;
-    const uint32_t arg = scan_all<kLeftPoints>(pts, i, n, dim, stride, cent, k, s.c);
+    const uint32_t arg = scan_all<kLeftPoints, D>(pts, i, n, dim, stride, cent, k, s.c);
     if (i < n) assign[i] = arg;
 }
 
@@ -667,6 +706,15 @@ __global__ void __launch_bounds__(256) k_sh_encode(const float *__restrict__ sh,
     }
 }
 
+// f(the scanned width as a constant): the least even one for the rows of SH degrees 1 to 3, 48 beyond.
+template <class F>
+void with_width(int dim, F f) {
+    if (dim <= 10) f(std::integral_constant<int, 10>{});
+    else if (dim <= 24) f(std::integral_constant<int, 24>{});
+    else if (dim <= 46) f(std::integral_constant<int, 46>{});
+    else f(std::integral_constant<int, kCbMaxDim>{});
+}
+
 // (In this namespace, so that the library has its own `attr`: a static of a template with a name for the linker is one
 // object of the process, also when a release and a debug library are loaded, each with kernels of its own.)
 template <int DIM>
@@ -695,12 +743,17 @@ cudaError_t launch_kmeans_assign(const float *pts, int64_t n, int dim, int64_t s
                               : dim == 9  ? launch_assign_tc<9>(pts, n, dim, stride, cent, k, assign, st)
                                           : launch_assign_tc<0>(pts, n, dim, stride, cent, k, assign, st);
         if (e != cudaSuccess) return e;
-        k_kmeans_assign_left<<<static_cast<unsigned>((n + kLeftPoints - 1) / kLeftPoints), kLeftPoints, 0, st>>>(
-            pts, n, dim, stride, cent, k, assign);
+        with_width(dim, [&](auto d) {
+            k_kmeans_assign_left<decltype(d)::value>
+                <<<static_cast<unsigned>((n + kLeftPoints - 1) / kLeftPoints), kLeftPoints, 0, st>>>(pts, n, dim, stride, cent,
+                                                                                                     k, assign);
+        });
         return cudaGetLastError();
     }
-    k_kmeans_assign<<<static_cast<unsigned>((n + kKmThreads - 1) / kKmThreads), kKmThreads, 0, st>>>(pts, n, dim, stride,
-                                                                                                  cent, k, assign);
+    with_width(dim, [&](auto d) {
+        k_kmeans_assign<decltype(d)::value><<<static_cast<unsigned>((n + kKmThreads - 1) / kKmThreads), kKmThreads, 0, st>>>(
+            pts, n, dim, stride, cent, k, assign);
+    });
     return cudaGetLastError();
 }
 

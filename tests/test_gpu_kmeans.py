@@ -137,3 +137,31 @@ def test_waits_that_run_out(k, dim, limit):
         finally:
             _lib.gs_debug_kmeans_wait(0)
         _check(pts, cent, dim, dim + 3, 3)
+
+
+@pytest.mark.parametrize("n,k", [(1, 1), (5, 2), (129, 3), (700, 5), (300, 63), (300, 64), (257, 65), (900, 127), (2000, 130),
+                                 (1500, 515)])
+@pytest.mark.parametrize("dim", [1, 2, 9, 10, 11, 24, 25, 45, 46, 47, 48])
+def test_whole_numbers(n, k, dim):
+    """Coordinates of -2 .. 2: every distance is exact in single precision and many are equal, so the assignment is
+    that of whole-number arithmetic, ties to the lower index, in the scan of every width and behind the tensor cores."""
+    rng = np.random.default_rng(1000 * dim + k)
+    x, c = rng.integers(-2, 3, (n, dim)), rng.integers(-2, 3, (k, dim))
+    want = ((x[:, None, :] - c[None]) ** 2).sum(2).argmin(1)
+    pts = torch.full((n, dim + 2), 7.0)
+    pts[:, 1:dim + 1] = torch.from_numpy(x).float()
+    pts = pts.cuda()
+    got = _assign(pts, torch.from_numpy(c).float().cuda(), dim, dim + 2, 1, 0, n)
+    assert np.array_equal(got.cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("colours,spread", [(64, 0.3), (64, 0.1), (8, 0.1), (4, 0.05), (1, 0.0)])
+@pytest.mark.parametrize("n,k,dim", [(6000, 2048, 45), (3000, 500, 24), (2100, 160, 9)])
+def test_palettes(n, k, dim, colours, spread):
+    """Points around a few colours: more candidates than a point remembers, or too large a share of the centroids."""
+    g = torch.Generator("cuda").manual_seed(colours + n)
+    pal = torch.randn((colours, dim + 3), generator=g, device="cuda") * 0.2
+    pts = pal[torch.randint(colours, (n,), generator=g, device="cuda")]
+    pts = pts + 0.2 * spread * torch.randn((n, dim + 3), generator=g, device="cuda")
+    cent = pts[torch.randperm(n, generator=g, device="cuda")[:k], 3:].contiguous()
+    _check(pts, cent, dim, dim + 3, 3)

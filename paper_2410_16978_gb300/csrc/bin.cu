@@ -201,7 +201,7 @@ template <int NV>
 __global__ void __launch_bounds__(256) k_bin_rows_count(const __grid_constant__ Views<BinView, NV> B) {
     chain_start();
     const BinView &V = B[blockIdx.y];
-    const uint32_t *__restrict__ order = V.order;
+    const uint32_t *order = V.order;               // (of the kernel before, as M, rows, rowlist and P below: see chain_start)
     const Rec *__restrict__ rec = V.rec;
     uint32_t *__restrict__ M = V.M;
     const Ctl *ctl = V.ctl;
@@ -267,8 +267,8 @@ __global__ void __launch_bounds__(256) k_bin_rows_write(const __grid_constant__ 
     const BinView &V = B[blockIdx.y];
     const uint32_t *__restrict__ order = V.order;
     const uint32_t *__restrict__ x01 = V.x01, *__restrict__ y01 = V.y01;
-    const uint32_t *__restrict__ M = V.M;
-    const RowInfo *__restrict__ rows = rows_of(V);
+    const uint32_t *M = V.M;
+    const RowInfo *rows = rows_of(V);
     uint2 *__restrict__ rowlist = V.rowlist;
     const Ctl *ctl = V.ctl;
     const int Ty = V.Ty;
@@ -471,7 +471,7 @@ template <int NV>
 __global__ void __launch_bounds__(256) k_bin_tiles_count(const __grid_constant__ Views<BinView, NV> B) {
     chain_start();
     const BinView &V = B[blockIdx.y];
-    const uint2 *__restrict__ rowlist = V.rowlist;
+    const uint2 *rowlist = V.rowlist;
     const RowInfo *__restrict__ rows = rows_of(V);
     uint32_t *__restrict__ P = V.P;
     const Ctl *ctl = V.ctl;
@@ -561,7 +561,7 @@ __global__ void __launch_bounds__(256) k_bin_tiles_write(const __grid_constant__
     const BinView &V = B[blockIdx.y];
     const uint2 *__restrict__ rowlist = V.rowlist;
     const RowInfo *__restrict__ rows = rows_of(V);
-    const uint32_t *__restrict__ P = V.P;
+    const uint32_t *P = V.P;
     uint32_t *__restrict__ list = V.list;
     const Ctl *ctl = V.ctl;
     const int Tx = V.Tx, Ty = V.Ty;

@@ -192,7 +192,11 @@ inline void with_views(const T *views, int n, F f) {
 // any return, so that a kernel's completion implies that of all before it;
 // the first kernel of a call is launched the ordinary way and therefore waits
 // for everything that precedes the call in the stream; and so does whatever
-// follows the call.
+// follows the call.  A kernel is resident while the one just before it still
+// writes, so it does not read what that one writes through the non-coherent path,
+// which is for data that stay the same for as long as a kernel lives: no
+// ld.global.nc and no const __restrict__ on such a pointer.  (What the kernels
+// further back write is complete before a kernel becomes resident.)
 __device__ __forceinline__ void chain_start() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -88,6 +88,12 @@ __device__ __forceinline__ float4 ld_now4(const void *p) {
     asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
     return v;
 }
+// (for the record gradient, which the kernel before writes: see chain_start)
+__device__ __forceinline__ float4 ld_written4(const void *p) {
+    float4 v;
+    asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    return v;
+}
 __device__ __forceinline__ float ld_now(const float *p) {
     float v;
     asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v) : "l"(p));
@@ -95,9 +101,9 @@ __device__ __forceinline__ float ld_now(const float *p) {
 }
 
 __device__ __forceinline__ void load_row(const SceneView &s, int i, const Geo *geo, const float4 *rec_grad, RowIn &r) {
-    r.ga = ld_now4(rec_grad + 3 * i);
-    r.gb = ld_now4(rec_grad + 3 * i + 1);
-    r.gc = ld_now4(rec_grad + 3 * i + 2);
+    r.ga = ld_written4(rec_grad + 3 * i);
+    r.gb = ld_written4(rec_grad + 3 * i + 1);
+    r.gc = ld_written4(rec_grad + 3 * i + 2);
     asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2];" : "=f"(r.A2), "=f"(r.beta) : "l"(&geo[i].a.z));
     r.G2 = ld_now(&geo[i].b.x);
 #pragma unroll
@@ -439,7 +445,7 @@ __global__ void __launch_bounds__(kBwdThreads, kBwdCtas) k_preprocess_bwd(SceneV
                                                                 const uint32_t *__restrict__ tiles,
                                                                 const uint32_t *__restrict__ vis_index,
                                                                 const Ctl *__restrict__ ctl, const Geo *__restrict__ geo,
-                                                                const float4 *__restrict__ rec_grad,
+                                                                const float4 *rec_grad,
                                                                 uint32_t grad_layer_mask, gs_grads g,
                                                                 float *__restrict__ contrib_sum, const ZeroRows zr) {
     chain_start();

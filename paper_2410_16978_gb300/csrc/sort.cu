@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(256) k_scan_reduce(F f, NSrc ns, uint32_t *__r
 }
 
 template <class F, class Out>
-__global__ void __launch_bounds__(256) k_scan_down(F f, NSrc ns, const uint32_t *__restrict__ partials, Out out,
+__global__ void __launch_bounds__(256) k_scan_down(F f, NSrc ns, const uint32_t *partials, Out out,
                                                    int64_t *__restrict__ n_total) {
     chain_start();
     __shared__ uint32_t s_w[8];
@@ -605,7 +605,7 @@ __global__ void __launch_bounds__(kPassThreads, kPassCtas) k_sort_pass(const __g
 
 // The shared order of two eyes: the other eye's visible list and counts, and an error of the sort (a wait that ran out
 // leaves the order unfinished, and the other eye bins in it too).
-__global__ void __launch_bounds__(256) k_share_order(const Ctl *from, const uint32_t *__restrict__ vis, Ctl *to,
+__global__ void __launch_bounds__(256) k_share_order(const Ctl *from, const uint32_t *vis, Ctl *to,
                                                      uint32_t *__restrict__ vis_to, uint32_t n) {
     chain_start();
     const uint32_t nv = from->n_vis;

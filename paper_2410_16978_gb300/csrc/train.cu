@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(kLossThreads) k_loss_maps(const float *__restr
 // strided share of the block sums in single precision, then a tree in shared
 // memory (scratch: 3 * kLossThreads floats).  The GB300's double-precision pipe is
 // narrow; converting and adding every block sum in double took 20 us.
-__device__ void loss_from_block_sums(const float *__restrict__ partials, int nb, size_t plane, float lam, float w_a,
+__device__ void loss_from_block_sums(const float *partials, int nb, size_t plane, float lam, float w_a,
                                      float *__restrict__ loss, float *scratch) {
     constexpr int NT = kLossThreads;
     const int tid = threadIdx.x;
@@ -236,9 +236,9 @@ __device__ void loss_from_block_sums(const float *__restrict__ partials, int nb,
 __global__ void __launch_bounds__(kLossThreads) k_loss_grad(const float *__restrict__ X, const float *__restrict__ A,
                                                             const float *__restrict__ Ct, const float *__restrict__ At,
                                                             float3 bg, int W, int H, const Win win, float lam,
-                                                            float w_a, const float *__restrict__ maps,
+                                                            float w_a, const float *maps,
                                                             float *__restrict__ dX, float *__restrict__ dA,
-                                                            const float *__restrict__ partials, float w_a_loss,
+                                                            const float *partials, float w_a_loss,
                                                             float *__restrict__ loss) {
     chain_start();
     __shared__ float2 s_ab[kRH][kSP];                      // maps (a, b)

@@ -39,27 +39,33 @@ bool make_layout(int64_t n, int W, int H, int64_t dup_cap, Layout *L) {
     o.geo = take(N * sizeof(Geo));
     o.tiles = take(N * 4);
     o.depth = take(N * 4);
+    o.vis_index = take(N * 4);
+    o.partials = take(kMaxSortBlocks * 4);
+    o.tile_order = take(static_cast<size_t>(o.Tn) * 16);
+    o.qdone = take(static_cast<size_t>(o.Tn) * 32);
+    o.seg_base = take(static_cast<size_t>(o.Tn) * 4);
+    o.list = take(D * 4);
+    // What the depth sort and the binning leave to one another, and in its place, from the compositor on, what the
+    // forward leaves to the backward.
+    const size_t shared = off;
     o.sort_k[0] = take(N * 4); o.sort_k[1] = take(N * 4);
     o.sort_v[0] = take(N * 4); o.sort_v[1] = take(N * 4);
     o.order = take(N * 4);
-    o.vis_index = take(N * 4);
     o.sort_cnt = take(sort_count_bytes(n));
     o.sort_status = take(sort_status_bytes(n));
     o.bin_m = take(static_cast<size_t>(kBinChunks) * o.Ty * 8);   // entries and pairs per (row, chunk)
     o.bin_p = take(bin_piece_bytes(dup_cap, o.Tx, o.Ty));
+    o.rowlist = take(D * 8);     // row entries <= pairs
+    const size_t front = off;
+    off = shared;
     o.t_final = take(P * 4);
     o.n_contrib = take(P * 4);
-    o.partials = take(kMaxSortBlocks * 4);
     o.rec_grad = take(N * sizeof(Rec));
-    o.tile_order = take(static_cast<size_t>(o.Tn) * 16);
-    o.qdone = take(static_cast<size_t>(o.Tn) * 32);
-    o.seg_base = take(static_cast<size_t>(o.Tn) * 4);
     o.qwork = take(static_cast<size_t>(o.Tn) * 16);
     const size_t segs = D / kSeg + static_cast<size_t>(o.Tn) + 1;   // >= sum over tiles of ceil(len / kSeg)
     o.ckpt = take(segs * kTilePix * sizeof(float4));
     o.items = take(4 * segs * sizeof(uint2));
-    o.rowlist = take(D * 8);     // row entries <= pairs
-    o.list = take(D * 4);
+    if (off < front) off = front;
     o.total = off;
     *L = o;
     return true;

@@ -302,7 +302,9 @@ int gs_gather_rows(const void *src, void *dst, int64_t row_bytes, const int32_t 
  * tests and debugging tools (host only, no device access).  out[k] for
  * k = 0..GS_LAYOUT_COUNT-1 in this order:
  *   0 status/control block   1 records (48 B per Gaussian: u, v, A2, beta,
- *   G2, opacity, r, g, b, depth, rect01, rect23)   2 tiles touched (u32)
+ *   G2, opacity, r, g, b, depth, rect01, rect23; from the next multiple of
+ *   256 bytes on 32 B per Gaussian: u, v, A2, beta, G2, opacity, r, g, the
+ *   copy that the compositors read)   2 tiles touched (u32)
  *   3 depth keys (u32 float bits, 0xFFFFFFFF when culled)   4 the pair list:
  *   Gaussian ids (u32) in tile order, depth order within a tile   5 tile
  *   ranges (u32 start, end per tile)   6 final transmittance (f32 per pixel)

@@ -36,7 +36,7 @@ bool make_layout(int64_t n, int W, int H, int64_t dup_cap, Layout *L) {
     o.tile_hist = take(kTileHistWords * 4);
     o.ranges = take(static_cast<size_t>(o.Tn) * 8);
     o.rec = take(N * sizeof(Rec));
-    o.geo = take(N * sizeof(Geo));
+    o.geo = take(N * sizeof(Geo));     // (behind the records: gs_workspace_layout says so)
     o.tiles = take(N * 4);
     o.depth = take(N * 4);
     o.vis_index = take(N * 4);

@@ -582,6 +582,7 @@ __global__ void __launch_bounds__(kFwdThreads) k_composite_fwd(const __grid_cons
         if constexpr (PX == 2) meet.settle(batch, lane);
         if (!ahead) take_next(q, nv);
     }
+    cp_async_wait<0>();                                 // (what the last item had staged beyond its stop)
     meet.settle(batch, lane);
 }
 

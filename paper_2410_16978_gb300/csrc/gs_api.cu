@@ -356,9 +356,9 @@ int front_preprocess(const FrontCtx *f, int n, cudaStream_t st) {
     PreView v[kMaxBatch];
     for (int i = 0; i < n; ++i) v[i] = f[i].pre;
     int rc;
+    Stage sg(GS_STAGE_PREPROCESS, st, 1);                    // (with the clearing kernel)
     if ((rc = cuda_check(launch_clear(v, n, st), "clear status")) != GS_OK) return rc;
     int launches = 0;
-    Stage sg(GS_STAGE_PREPROCESS, st, 1);                    // (with the clearing kernel)
     rc = cuda_check(launch_preprocess(v, n, st, &launches), "preprocess");
     g_launches += launches;
     return rc;

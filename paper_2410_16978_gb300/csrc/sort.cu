@@ -270,7 +270,10 @@ __device__ uint32_t look_back(uint64_t *status, uint32_t t, int c, uint32_t own,
         j -= used;
         if (waiting) {
             if (++spins > spin_limit) {
+                // What this kernel writes will have holes, keys that the digit histograms do not count: no tile for the
+                // kernels after it.  (Asking every CTA for the error status first cost 7 us for 3M Gaussians.)
                 ctl->st.error = GS_ERR_TIMEOUT;
+                for (int p = 1; p < 4; ++p) atomicOr(&ctl->sort_ticket[p], 0x80000000u);
                 break;
             }
             __nanosleep(64);
@@ -468,14 +471,12 @@ __global__ void __launch_bounds__(kPassThreads, kPassCtas) k_sort_pass(const __g
     uint32_t t = blockIdx.x;                       // the first digit kernel: the histogram pass's tiles
     // as many CTAs as tiles take part, the first ones: they start on one SM each before any SM gets a second
     if (t >= ntiles) return;
-    // (a wait that ran out leaves holes in what this kernel would read, keys that the histograms do not count: no tile)
-    if (!FIRST && threadIdx.x == 0)
-        s_ticket = ctl->st.error == GS_OK ? atomicAdd(&ctl->sort_ticket[pass], 1u) : 0xFFFFFFFFu;
+    if (!FIRST && threadIdx.x == 0) s_ticket = atomicAdd(&ctl->sort_ticket[pass], 1u);
     for (int e = threadIdx.x; e < kPassWarps * 256; e += kPassThreads) (&s_wc[0][0])[e] = 0;
     __syncthreads();
     if (!FIRST) {
         t = s_ticket;
-        if (t >= ntiles) return;
+        if (t >= ntiles) return;                   // (a wait of this or an earlier digit kernel ran out)
     }
 #ifdef GS_DEBUG
     const bool publish = !(pass == B.withhold && t == 0);

@@ -127,17 +127,19 @@ __device__ __forceinline__ void emit_group(uint32_t cov, V v, uint32_t (&pos)[kG
     }
 }
 
-// Sum over a block of 1024 threads, in every thread; synchronises the block.
+// Sum over a warp: three 32-bit reductions, which take 16, 16 and 32 bits of every value without an overflow.
+__device__ __forceinline__ unsigned long long warp_sum64(unsigned long long v) {
+    const uint32_t lo = static_cast<uint32_t>(v);
+    return __reduce_add_sync(FULL, lo & 0xFFFFu) + (static_cast<unsigned long long>(__reduce_add_sync(FULL, lo >> 16)) << 16) +
+           (static_cast<unsigned long long>(__reduce_add_sync(FULL, static_cast<uint32_t>(v >> 32))) << 32);
+}
+
+// Sum over a block of 1024 threads, for thread 0; synchronises the block.
 __device__ __forceinline__ unsigned long long block_sum64(unsigned long long v, unsigned long long *s_w) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
+    v = warp_sum64(v);
     if ((threadIdx.x & 31) == 0) s_w[threadIdx.x >> 5] = v;
     __syncthreads();
-    v = s_w[threadIdx.x & 31];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
-    __syncthreads();
-    return v;
+    return threadIdx.x < 32 ? warp_sum64(s_w[threadIdx.x]) : 0ull;
 }
 
 // In-place inclusive prefix sum of a[0..n) (shared memory) by one warp.
@@ -176,18 +178,9 @@ struct RowInfo {           // per tile row, in the workspace
     uint32_t pad_[5 - kRowParts];        // (32 bytes in all)
 };
 
-// Totals of a (row, part) of the row scan.  A chunk's pairs of a row fit 32 bits (at most 883,012 Gaussians of 256
-// tiles); a row's need not, and the frame's do not from 65,536 Gaussians that cover 4096 x 4096 on.
-struct PartTotal {
-    unsigned long long pairs;
-    uint32_t entries, pad_;
-};
-
-// The per-row info of a view, and behind it the totals of every (row, part) of the row scan.
+// The per-row info of a view, and behind it the (entries, pairs) totals of every (row, part) of the row scan.
 __device__ __forceinline__ RowInfo *rows_of(const BinView &v) { return static_cast<RowInfo *>(v.rows); }
-__device__ __forceinline__ PartTotal *part_totals_of(const BinView &v) {
-    return reinterpret_cast<PartTotal *>(rows_of(v) + v.Ty);
-}
+__device__ __forceinline__ uint2 *part_totals_of(const BinView &v) { return reinterpret_cast<uint2 *>(rows_of(v) + v.Ty); }
 
 // Chunk c of K of the depth order's n entries.
 __device__ __forceinline__ void chunk_range(uint32_t n, uint32_t c, uint32_t K, uint32_t &b, uint32_t &e) {
@@ -357,17 +350,19 @@ __global__ void __launch_bounds__(256) k_bin_rows_write(const __grid_constant__ 
 // coalesced loads and stores (each thread scans a contiguous run of counts);
 // the pair total needs only a sum, read coalesced.  The last CTA to finish
 // (a counter in the control block) then does the per-row work for the whole
-// frame: part bases, row totals, the row, pair and piece starts, the pair
-// total (in 64 bits) and the capacity check.  A frame that fits has at most
-// 2^32 - 1 pairs and no more entries than pairs, so its starts take 32 bits; after
-// an overflow nothing reads them.
+// frame: part bases, row totals, the row, pair and piece starts, and the capacity
+// check.  The pair total is added up in 64 bits in the status word: a chunk's pairs of
+// a row fit 32 (at most 883,012 Gaussians of 256 tiles), a frame's do not from 65,536
+// Gaussians that cover 4096 x 4096 on.  A frame that fits has at most 2^32 - 1 pairs and
+// no more entries than pairs, so its starts take 32 bits; after an overflow nothing reads
+// them.
 template <int NV>
 __global__ void __launch_bounds__(1024) k_bin_rowscan(const __grid_constant__ Views<BinView, NV> B, int K) {
     chain_start();
     const BinView &V = B[blockIdx.y];
     uint32_t *__restrict__ M = V.M;
     RowInfo *__restrict__ rows = rows_of(V);
-    PartTotal *__restrict__ part_tot = part_totals_of(V);
+    uint2 *__restrict__ part_tot = part_totals_of(V);
     Ctl *__restrict__ ctl = V.ctl;
     const uint64_t cap = V.cap;
     const int Tx = V.Tx, Ty = V.Ty;
@@ -406,7 +401,8 @@ __global__ void __launch_bounds__(1024) k_bin_rowscan(const __grid_constant__ Vi
     __syncthreads();
     for (int i = threadIdx.x; i < KP; i += 1024) row[i] = s_row[i];
     if (threadIdx.x == 0) {
-        part_tot[blockIdx.x] = PartTotal{ptot, tot, 0u};
+        part_tot[blockIdx.x] = make_uint2(tot, static_cast<uint32_t>(ptot));
+        atomicAdd(reinterpret_cast<unsigned long long *>(&ctl->st.n_dup), ptot);
         __threadfence();
         s_last = atomicAdd(&ctl->bin_scan_done, 1u) == static_cast<uint32_t>(Ty * kRowParts - 1);
     }
@@ -414,23 +410,22 @@ __global__ void __launch_bounds__(1024) k_bin_rowscan(const __grid_constant__ Vi
     if (!s_last) return;
     __threadfence();
     // the last CTA: per row (thread r < Ty <= 256) the part bases and totals, then the starts
-    const volatile PartTotal *pt = part_tot;
-    uint32_t ent = 0;
-    unsigned long long prs = 0;
+    const volatile uint2 *pt = part_tot;
+    const uint64_t pairs = *const_cast<const volatile uint64_t *>(&ctl->st.n_dup);
+    uint32_t ent = 0, prs = 0;
     if (threadIdx.x < Ty) {
         for (int p = 0; p < kRowParts; ++p) {
-            const uint32_t e = pt[threadIdx.x * kRowParts + p].entries;
+            const uint32_t e = pt[threadIdx.x * kRowParts + p].x;
             if (p > 0) rows[threadIdx.x].part_base[p - 1] = ent;
             ent += e;
-            prs += pt[threadIdx.x * kRowParts + p].pairs;
+            prs += pt[threadIdx.x * kRowParts + p].y;
         }
         rows[threadIdx.x].entries = ent;
     }
-    uint32_t te, tp32, tq;
+    uint32_t te, tp, tq;
     const bool in = threadIdx.x < Ty;
-    const unsigned long long tp = block_sum64(in ? prs : 0ull, s_w64);
     const uint32_t s0 = block_excl_scan<1024>(in ? ent : 0u, s_w, &te);
-    const uint32_t s1 = block_excl_scan<1024>(in ? static_cast<uint32_t>(prs) : 0u, s_w, &tp32);
+    const uint32_t s1 = block_excl_scan<1024>(in ? prs : 0u, s_w, &tp);
     // entries per piece: the largest that still gives every SM several warps of the scatter (piece, kGroup tiles)
     uint32_t piece = kPieceMin;
     const uint64_t groups = (Tx + kGroup - 1) / kGroup;
@@ -442,11 +437,10 @@ __global__ void __launch_bounds__(1024) k_bin_rowscan(const __grid_constant__ Vi
         rows[threadIdx.x].piece_start = s2;
     }
     if (threadIdx.x == 0) {
-        ctl->st.n_dup = tp;
         ctl->st.dup_capacity = cap;
         ctl->n_pieces = tq;
         ctl->bin_piece = piece;
-        if (tp > cap) ctl->st.error = GS_ERR_WORKSPACE;
+        if (pairs > cap) ctl->st.error = GS_ERR_WORKSPACE;
     }
 }
 
@@ -765,10 +759,10 @@ size_t bin_piece_bytes(int64_t dup_cap, int Tx, int Ty) {
     return (static_cast<size_t>(dup_cap) / kPieceMin + Ty + 1) * Tx * 4;
 }
 
-// The RowInfo of every row, then the totals of every (row, part) of the row scan.
+// The RowInfo of every row, then the (entries, pairs) totals of every (row, part) of the row scan.
 size_t bin_rows_bytes(int Ty) {
-    return static_cast<size_t>(Ty) * sizeof(RowInfo) + static_cast<size_t>(Ty) * kRowParts * sizeof(PartTotal);
+    return static_cast<size_t>(Ty) * sizeof(RowInfo) + static_cast<size_t>(Ty) * kRowParts * sizeof(uint2);
 }
-static_assert(sizeof(RowInfo) == 32 && sizeof(PartTotal) == 16, "RowInfo, PartTotal layout");
+static_assert(sizeof(RowInfo) == 32, "RowInfo layout");
 
 }  // namespace gs

@@ -9,8 +9,9 @@
 // sum_d (x_d - c_d)^2 (d in order, fused multiply-adds), ties to the lower
 // index.  Small calls scan brute force: a thread per point holds its
 // (zero-padded) coordinates in registers and scans the centroids staged in
-// shared memory 64 at a time with 16-byte broadcast loads.  Larger ones rule
-// out nearly all centroids on the tensor cores first (k_kmeans_assign_tc).
+// shared memory 64 at a time with 16-byte broadcast loads (scan_all).  Larger
+// ones rule out nearly all centroids on the tensor cores first
+// (k_kmeans_assign_tc).
 #include <type_traits>
 
 #include <cuda_bf16.h>
@@ -107,6 +108,8 @@ __global__ void __launch_bounds__(kKmThreads) k_kmeans_assign(const float *__res
 //    Cauchy-Schwarz over the coordinates), -|c|^2/2 enters as three bf16
 //    parts, and each of at most 64 accumulations errs by at most 2^-22 of the
 //    magnitudes added.  kEProd, kENorm round these up; kETiny covers underflow.
+//    (The last of the three is an assumption: the rounding of the accumulation is
+//    not documented.  The constants leave room for 2^-20.)
 //  * The scan's rounded distances err by at most (dim + 3) 2^-24 relative, so
 //    its winner has s within 2^-18 (|x| + |c|)^2 of the best; kESlack rounds up.
 //  * Per point, LB = max over groups of 32 centroids of (largest s~ - E) is a lower
@@ -117,20 +120,22 @@ __global__ void __launch_bounds__(kKmThreads) k_kmeans_assign(const float *__res
 //    finite or above kHuge, are scanned in full.
 //
 // A CTA takes 256 points (two 128-row A tiles, bf16, resident) and walks the
-// centroids in tiles of 128: four warps copy a tile's rows (cp.async) and convert
-// them to bf16 in the 128-byte swizzled K-major layout, one thread issues the
-// MMAs (M = N = 128, K = dim + 3 rounded up to 16) into one of two accumulator
-// sets in tensor memory, and eight warps read the other set back, one point per
-// thread.  Everything is staged by the CTA itself, as the entry point has no
-// workspace to hold converted centroids.
+// centroids in tiles of 128: two sets of four warps take the tiles in turn, each
+// tile's rows by one bulk copy, and convert them to bf16 in the 128-byte swizzled
+// K-major layout, one thread issues the MMAs (M = N = 128, K = dim + 3 rounded up
+// to 16) into one of two accumulator sets in tensor memory, and eight warps read
+// the other set back, one point per thread.  Everything is staged by the CTA
+// itself, as the entry point has no workspace to hold converted centroids.
 //
-// Bound by instruction issue: reading the accumulators back and the conversions
-// (the tensor pipe is 15% busy; K is only 48).  Measured, points x centroids of 45
-// coordinates: 200,000 x 16,384 13.0 -> 0.79 ms, 200,000 x 4,096 3.26 -> 0.32,
-// 1,200,000 x 16,384 71.9 -> 4.2, 20,000 x 256 0.060 -> 0.027; 20,000 x 16,384 of 9
-// coordinates 3.3 -> 0.13.  Found on the way: candidate groups scanned whole by a warp per
-// point (1.1 ms: a kilobyte-sized gather per point), one converter set (1.2 ms),
-// candidates told apart by 32 predicates (1.0 ms, the sign bits 0.79).
+// Bound by the latencies of that chain: half of the issue slots are used, the
+// tensor pipe is 19% busy (K is only 48), and what is waited for are the tile
+// hand-overs and the accumulators.  Measured, points x centroids of 45
+// coordinates against the scan of one centroid at a time: 200,000 x 16,384 13.0 -> 0.81
+// ms, 200,000 x 4,096 3.26 -> 0.32, 1,200,000 x 16,384 71.9 -> 4.2, 20,000 x 256 0.064 ->
+// 0.031; 20,000 x 16,384 of 9 coordinates 3.3 -> 0.13.  Found on the way: candidate groups
+// scanned whole by a warp per point (1.1 ms: a kilobyte-sized gather per point), one
+// converter set (1.2 ms), candidates told apart by 32 predicates (1.0 ms, the sign
+// bits 0.79).  Data of few colours leave many candidates: see k_kmeans_assign_left.
 constexpr int kTcPoints = 256, kTcTile = 128, kTcRow = 128;      // points per CTA, centroids per tile, bytes per row
 constexpr int kTcEpiWarps = 8, kTcCvtWarps = 4, kTcCvtSets = 2;
 constexpr int kTcMmaWarp = kTcEpiWarps + kTcCvtSets * kTcCvtWarps;

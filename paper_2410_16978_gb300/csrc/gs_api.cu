@@ -364,10 +364,6 @@ int front_preprocess(const FrontCtx *f, int n, cudaStream_t st) {
     return rc;
 }
 
-// Phase 2: the depth sort of the visible Gaussians of n views (depth order in
-// each view's workspace), or with `shared` one sort for views 0 and 1: a
-// Gaussian visible to either is kept and keyed by view 0's depth when view 0
-// sees it, else by view 1's.
 SortWork sort_work(void *ws, const Layout &L) {
     SortWork w;
     for (int k = 0; k < 2; ++k) {
@@ -383,6 +379,10 @@ SortWork sort_work(void *ws, const Layout &L) {
     return w;
 }
 
+// Phase 2: the depth sort of the visible Gaussians of n views (depth order in
+// each view's workspace), or with `shared` one sort for views 0 and 1: a
+// Gaussian visible to either is kept and keyed by view 0's depth when view 0
+// sees it, else by view 1's.
 int front_sort(FrontCtx *f, int n, bool shared, cudaStream_t st) {
     SortView v[kMaxBatch];
     for (int i = 0; i < n; ++i) {

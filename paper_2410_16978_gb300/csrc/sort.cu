@@ -234,8 +234,6 @@ struct SortJob {
     int withhold;
 };
 
-// One CTA per tile of the first digit kernel: the visible count, the key
-// range, the four digit histograms, and the tile's count of every first digit.
 // Exclusive prefix of counter c over the tiles before tile t (whose own count
 // `own` is already published as an aggregate unless t == 0); publishes the
 // inclusive prefix of tile t.  The predecessors are read kLookWindow at a time,
@@ -283,6 +281,8 @@ __device__ uint32_t look_back(uint64_t *status, uint32_t t, int c, uint32_t own,
     return excl;
 }
 
+// One CTA per tile of the first digit kernel: the visible count, the key
+// range, the four digit histograms, and the tile's count of every first digit.
 // Four Gaussians per thread: with sixteen the chain of a warp's shuffles and
 // votes set the time of small scenes (4,096 Gaussians 12.5 -> 7.8 us, 1.2M 16.5 -> 10.6,
 // 3M 24.9 -> 17.1).
